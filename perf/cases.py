@@ -1,0 +1,293 @@
+"""What a program that serves a transformer layer asks of this library, as cases that can be timed and compared.
+
+``listed()`` names the cases, ``draw(rng)`` gives more of the same ranges. Every case is one kind of call:
+
+  prompt       causal prefill of fresh prompts, the cache written in the same call
+  rope_prompt  what a rotary model does with a prompt: rotation (+ head norm) and cache write in one pass over the
+               projections, then attention read from the cache
+  chunk        new tokens over a populated cache (a continued conversation, a prompt cut into chunks), contiguous or paged
+  step         one decode step: the newest token appended and attended, over a contiguous or a paged cache, in bf16 or
+               e4m3, with or without the rotation (+ head norm) of the newest token in the same call
+  scan         the gated linear recurrence over a prompt or a single step
+
+Head geometries are those of the benchmark configurations and tests: 32 / 8 x 128 (the 8B-shaped layer), 64 / 8 and
+40 / 8 x 128, 12 / 12 x 64 (the small multi-head model), 4 / 2 x 64 (tiny). Lengths are ragged wherever a batch would be.
+"""
+from __future__ import annotations
+
+import math
+import random
+
+import torch
+
+from paper_2608_21836_b200 import binding as l4l
+from paper_2608_21836_b200 import workloads as wl
+
+LAYER = dict(Hq=32, Hkv=8, D=128)
+SMALL = dict(Hq=12, Hkv=12, D=64)
+TINY = dict(Hq=4, Hkv=2, D=64)
+WIDE = dict(Hq=64, Hkv=8, D=128)
+GROUP5 = dict(Hq=40, Hkv=8, D=128)
+
+
+def _prompt(name, B, lo, hi, heads, lens=0):
+    return dict(name=name, kind="prompt", B=B, lo=lo, hi=hi, lens=lens, **heads)
+
+
+def _step(name, B, lo, hi, heads, cache="bf16", page=0, rope=False, norm=False, lens=0):
+    return dict(name=name, kind="step", B=B, lo=lo, hi=hi, lens=lens, cache=cache, page=page, rope=rope, norm=norm, **heads)
+
+
+def listed():
+    return [
+        # The smallest call: a short prompt through a tiny model. Latency and the host side are all there is.
+        _prompt("prompt_tiny", 1, 128, 128, TINY),
+        # One user's prompt of ordinary length through a layer of an 8B-shaped model.
+        _prompt("prompt_layer", 1, 2048, 2048, LAYER),
+        # The largest call: four long documents at once; the prefill headline configuration.
+        _prompt("prompt_long", 4, 8192, 8192, LAYER),
+        # A rotary model with head norms takes in a batch of prompts of uneven length.
+        dict(name="rope_prompt_ragged", kind="rope_prompt", B=6, lo=180, hi=1900, lens=3, norm=True, **LAYER),
+        # A serving loop's mixed batch: chunks of prompts over what each request has in its pages already.
+        dict(name="chunk_paged_ragged", kind="chunk", B=5, past_lo=100, past_hi=5000, lo=65, hi=700, page=64, lens=4, **LAYER),
+        # One interactive user: a step of a rotary model with head norms at 2304 cached tokens (the layer
+        # configuration's 2048-token prompt and 256 steps).
+        _step("step_one_user", 1, 2304, 2304, LAYER, rope=True, norm=True),
+        # A batch of interactive users, ragged: the decode headline configuration with its append.
+        _step("step_batch_ragged", 32, 512, 4096, LAYER, lens=1),
+        # The same regime the way serving runtimes hold it: 16-token pages scattered over a pool.
+        _step("step_paged16_ragged", 48, 200, 3000, LAYER, page=16, lens=5),
+        # The same over an 8-bit cache, which a server takes to fit more users.
+        _step("step_fp8_ragged", 32, 512, 4096, LAYER, cache="fp8", lens=1),
+        # A small multi-head model at a fixed context: no grouping, 64-wide heads.
+        _step("step_small_mha", 64, 1024, 1024, SMALL),
+        # Many short requests (classification, short chats): hundreds of sequences of a few hundred tokens.
+        _step("step_many_short", 512, 64, 256, LAYER, lens=2),
+        # The recurrent block's prompt: a few long sequences.
+        dict(name="scan_long", kind="scan", B=4, lo=8192, hi=8192, W=2560, lens=0, reset=True),
+    ]
+
+
+def _log(rng, lo, hi):
+    """An integer spread over the logarithm of its range."""
+    return max(lo, min(hi, int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))))
+
+
+def draw(rng):
+    kind = rng.choice(["prompt", "rope_prompt", "chunk", "step", "step", "step", "step", "scan"])
+    lens = rng.randrange(1, 1 << 20)
+    if kind == "scan":
+        W = rng.choice([1024, 2560, 4096])
+        T = 1 if rng.random() < 0.2 else _log(rng, 16, 8192)
+        B = _log(rng, 1, max(1, min(64, 4 * 8192 * 2560 // (T * W))))
+        return dict(kind=kind, B=B, lo=max(1, T - T // 4), hi=T, W=W, lens=lens, reset=rng.random() < 0.5)
+    heads = rng.choice([LAYER, LAYER, WIDE, GROUP5, SMALL, TINY])
+    if kind in ("prompt", "rope_prompt"):
+        hi = _log(rng, 20, 8192)
+        most = 4 * 8192 * 8192 * 32 * 128 // (hi * hi * heads["Hq"] * heads["D"])
+        B = _log(rng, 1, max(1, min(16, most)))
+        c = dict(kind=kind, B=B, lo=max(1, hi // rng.choice([1, 2, 8])), hi=hi, lens=lens, **heads)
+        if kind == "rope_prompt":
+            c["norm"] = rng.random() < 0.5
+        return c
+    if kind == "chunk":
+        past, hi = _log(rng, 64, 7000), _log(rng, 17, 1024)
+        return dict(kind=kind, B=_log(rng, 1, 12), past_lo=past // 4, past_hi=past, lo=max(1, hi // 2), hi=hi,
+                    page=rng.choice([0, 16, 64, 256]), lens=lens, **heads)
+    hi = _log(rng, 40, 8192)
+    most = (1 << 29) // (hi * heads["Hkv"] * heads["D"] * 4)
+    B = _log(rng, 1, max(1, min(640, most)))
+    page = rng.choice([0, 0, 16, 32, 64])
+    cache = rng.choice(["bf16", "bf16", "fp8"])
+    rope = rng.random() < 0.4
+    return dict(kind=kind, B=B, lo=max(1, hi // rng.choice([1, 2, 8])), hi=hi, lens=lens, cache=cache, page=page, rope=rope,
+                norm=rope and rng.random() < 0.5, **heads)
+
+
+def _lengths(c, lo, hi, salt=0):
+    """The batch's lengths, from the case alone. A lone sequence has the full length."""
+    r = random.Random(c["lens"] * 7 + salt)
+    return [hi] if c["B"] == 1 else [r.randint(lo, hi) for _ in range(c["B"])]
+
+
+def _pages(lens, page):
+    return sum(-(-n // page) for n in lens)
+
+
+class _Inputs:
+    def __init__(self, seed):
+        self.gen = torch.Generator(device="cuda").manual_seed(seed)
+
+    def bf16(self, *shape):
+        return torch.randn(*shape, generator=self.gen, device="cuda", dtype=torch.bfloat16)
+
+    def f32(self, *shape):
+        return torch.randn(*shape, generator=self.gen, device="cuda")
+
+    def table(self, lens, page, width):
+        """A pool's block table: the sequences' pages lie scattered over the pool, as after hours of serving."""
+        n = _pages(lens, page)
+        order = torch.randperm(n, generator=self.gen, device="cuda").to(torch.int32)
+        t = torch.zeros(len(lens), width, dtype=torch.int32, device="cuda")
+        at = 0
+        for b, length in enumerate(lens):
+            k = -(-length // page)
+            t[b, :k] = order[at:at + k]
+            at += k
+        return n, t
+
+
+def _i32(values):
+    return torch.tensor(values, dtype=torch.int32, device="cuda")
+
+
+def _norm_and_tables(c, hi):
+    s = {}
+    cos, sin = wl.make_rope_tables(hi, c["D"])
+    s["cos"], s["sin"] = cos.cuda(), sin.cuda()
+    # head-norm weights as a module is initialised with them
+    s["norm"] = dict(q_weight=torch.ones(c["D"], device="cuda"), k_weight=torch.ones(c["D"], device="cuda"),
+                     eps=1e-6) if c["norm"] else {}
+    return s
+
+
+def _cache(x, c, lens, hi):
+    """K and V caches [B, Hkv, slots, D] or page pools [pages, Hkv, page, D] with their block table."""
+    if c.get("page"):
+        width = -(-hi // c["page"])
+        n, table = x.table(lens, c["page"], width)
+        shape = (n, c["Hkv"], c["page"], c["D"])
+    else:
+        slots = hi + (hi & 1)
+        shape, table = (c["B"], c["Hkv"], slots, c["D"]), None
+    k, v = x.bf16(*shape), x.bf16(*shape)
+    if c.get("cache") != "fp8":
+        return dict(k=k, v=v, table=table)
+    # a per-head scale that maps the head's largest value near the format's largest
+    ks = 0.0125 * (1 + 0.2 * torch.rand(c["Hkv"], generator=x.gen, device="cuda"))
+    vs = 0.0125 * (1 + 0.2 * torch.rand(c["Hkv"], generator=x.gen, device="cuda"))
+    q8 = lambda t, s: (t / s.view(1, -1, 1, 1)).to(torch.float8_e4m3fn).view(torch.uint8)  # noqa: E731
+    return dict(k=q8(k, ks), v=q8(v, vs), ks=ks, vs=vs, table=table)
+
+
+def prepare(case, seed):
+    c, x = case, _Inputs(seed)
+    s = {"c": c, "scale": 0.0}
+    B, kind = c["B"], c["kind"]
+    if kind == "scan":
+        T, W = c["hi"], c["W"]
+        s["x"], s["gx"], s["ga"] = x.bf16(B, T, W), 2 * x.bf16(B, T, W), 2 * x.bf16(B, T, W)
+        a = torch.rand(W, generator=x.gen, device="cuda") * 0.099 + 0.9         # a at an open gate, as initialised
+        s["ap"] = torch.log(torch.expm1(-torch.log(a) / 8))
+        s["state"], s["y"] = x.f32(B, W), torch.zeros_like(s["x"])
+        s["pos"] = torch.arange(T, dtype=torch.int32, device="cuda").repeat(B, 1) if c["reset"] else None
+        s["len"] = _i32(_lengths(c, c["lo"], T))
+        s["ws"] = l4l.new_rglru_workspace(B, T, W)
+        return s
+    Hq, Hkv, D = c["Hq"], c["Hkv"], c["D"]
+    s["scale"] = 1.0 / math.sqrt(D)
+    lens = _lengths(c, c["lo"], c["hi"])
+    if kind in ("prompt", "rope_prompt"):
+        S = c["hi"]
+        s["q"], s["k"], s["v"] = x.bf16(B, S, Hq, D), x.bf16(B, S, Hkv, D), x.bf16(B, S, Hkv, D)
+        s["o"] = torch.zeros_like(s["q"])
+        s["ck"], s["cv"] = (torch.zeros(B, Hkv, S, D, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        s["len"], s["past"] = _i32(lens), _i32([0] * B)
+        s["ws"] = l4l.new_workspace(l4l.L4L_OP_PREFILL, B, Hq, Hkv, D, S)
+        if kind == "rope_prompt":
+            s.update(_norm_and_tables(c, S))
+        return s
+    if kind == "chunk":
+        past = _lengths(c, c["past_lo"], c["past_hi"], 1)
+        total, S, hi = [p + n for p, n in zip(past, lens)], c["hi"], c["past_hi"] + c["hi"]
+        s["q"], s["k"], s["v"] = x.bf16(B, S, Hq, D), x.bf16(B, S, Hkv, D), x.bf16(B, S, Hkv, D)
+        s["o"] = torch.zeros_like(s["q"])
+        s["cache"] = _cache(x, c, total, hi)
+        s["len"], s["past"] = _i32(lens), _i32(past)
+        s["ws"] = l4l.new_workspace(l4l.L4L_OP_PREFILL, B, Hq, Hkv, D, hi)
+        return s
+    s["q"], s["k"], s["v"] = x.bf16(B, Hq, D), x.bf16(B, 1, Hkv, D), x.bf16(B, 1, Hkv, D)
+    s["o"] = torch.zeros_like(s["q"])
+    s["cache"] = _cache(x, c, lens, c["hi"])
+    s["len"] = _i32(lens)
+    s["ws"] = l4l.new_workspace(l4l.L4L_OP_DECODE, B, Hq, Hkv, D, c["hi"])
+    if c["rope"]:
+        s.update(_norm_and_tables(c, c["hi"]))
+    return s
+
+
+def run(s):
+    c = s["c"]
+    kind = c["kind"]
+    if kind == "scan":
+        l4l.l4l_rglru_scan(s["x"], s["gx"], s["ga"], s["ap"], s["state"], s["y"], s["ws"], position=s["pos"],
+                           seq_lens=s["len"])
+        return s["y"], s["state"]
+    if kind == "prompt":
+        l4l.l4l_attn_prefill(s["q"], s["k"], s["v"], s["o"], s["len"], s["scale"], s["ws"], cache_k=s["ck"],
+                             cache_v=s["cv"])
+        return s["o"], s["ck"], s["cv"]
+    if kind == "rope_prompt":
+        l4l.l4l_rope_kv_append(s["q"], s["k"], s["v"], s["ck"], s["cv"], s["past"], s["len"], s["cos"], s["sin"],
+                               **s["norm"])
+        l4l.l4l_attn_prefill_chunk(s["q"], s["o"], s["ck"], s["cv"], s["past"], s["len"], s["scale"], s["ws"])
+        return s["q"], s["o"], s["ck"], s["cv"]
+    h = s["cache"]
+    if kind == "chunk":
+        l4l.l4l_attn_prefill_chunk_append(s["q"], s["k"], s["v"], s["o"], h["k"], h["v"], s["past"], s["len"], s["scale"],
+                                          s["ws"], block_table=h["table"])
+        return s["o"], h["k"], h["v"]
+    hi, table = c["hi"], h["table"]
+    if c["cache"] == "fp8":
+        if c["rope"]:
+            l4l.l4l_attn_decode_rope_append_fp8(s["q"], s["o"], h["k"], h["v"], h["ks"], h["vs"], s["k"], s["v"], s["len"],
+                                                hi, s["scale"], s["cos"], s["sin"], s["ws"], block_table=table, **s["norm"])
+        else:
+            l4l.l4l_attn_decode_append_fp8(s["q"], s["o"], h["k"], h["v"], h["ks"], h["vs"], s["k"], s["v"], s["len"], hi,
+                                           s["scale"], s["ws"], block_table=table)
+    elif table is not None:
+        if c["rope"]:
+            l4l.l4l_attn_decode_paged_rope_append(s["q"], s["o"], h["k"], h["v"], table, s["k"], s["v"], s["len"], hi,
+                                                  s["scale"], s["cos"], s["sin"], s["ws"], **s["norm"])
+        else:
+            l4l.l4l_attn_decode_paged_append(s["q"], s["o"], h["k"], h["v"], table, s["k"], s["v"], s["len"], hi, s["scale"],
+                                             s["ws"])
+    elif c["rope"]:
+        l4l.l4l_attn_decode_rope_append(s["q"], s["o"], h["k"], h["v"], s["k"], s["v"], s["len"], hi, s["scale"], s["cos"],
+                                        s["sin"], s["ws"], **s["norm"])
+    else:
+        l4l.l4l_attn_decode_append(s["q"], s["o"], h["k"], h["v"], s["k"], s["v"], s["len"], hi, s["scale"], s["ws"])
+    return s["o"], h["k"], h["v"]
+
+
+def work(case):
+    """Every input that a result depends on read once, every result written once; 4 D flop per (query, visible key) pair
+    and query head."""
+    c = case
+    if c["kind"] == "scan":
+        n = sum(_lengths(c, c["lo"], c["hi"])) * c["W"]
+        return {"bytes": 8 * n + 8 * c["B"] * c["W"], "flops": 20 * n}
+    Hq, Hkv, D = c["Hq"], c["Hkv"], c["D"]
+    lens = _lengths(c, c["lo"], c["hi"])
+    if c["kind"] == "step":
+        size, tokens = (1 if c["cache"] == "fp8" else 2), sum(lens)
+        return {"bytes": 2 * size * tokens * Hkv * D + 4 * c["B"] * (Hq + Hkv) * D, "flops": 4 * D * Hq * tokens}
+    past = _lengths(c, c["past_lo"], c["past_hi"], 1) if c["kind"] == "chunk" else [0] * c["B"]
+    new, old = sum(lens), sum(past)
+    flops = sum(4 * D * Hq * (p * n + n * (n + 1) // 2) for p, n in zip(past, lens))
+    # q, k and v in; o and the cache rows out; the cached tokens in; the rotated q is a result too
+    size = 2 * D * (new * (2 * Hq + 4 * Hkv) + old * 2 * Hkv)
+    return {"bytes": size + (2 * D * new * Hq if c["kind"] == "rope_prompt" else 0), "flops": flops}
+
+
+def tolerance(case):
+    """About four times the distance of the results from the same computation in 64 bits. That distance is 2.0e-3 to 2.9e-3
+    of the norm for attention (bf16 results, bf16 softmax weights; 1.7e-3 for the rounding of the results alone, which
+    is the scan's and the e4m3 cache's) and, at the worst element against the root mean square, 0.10 over prompts (rows
+    that see few keys are large, most are small), 1.2e-2 for a step, 4e-3 for the scan. A rotated key that falls on the
+    other side of a bf16 rounding may give the neighbouring e4m3 code, in the new token's row alone."""
+    if case["kind"] == "scan":
+        return {"rel": 7e-3, "max": 1.6e-2}
+    if case["kind"] == "step":
+        return {"rel": 1e-2, "max": 5e-2, "differ": 5e-4 if case["rope"] and case["cache"] == "fp8" else 0.0}
+    return {"rel": 1e-2, "max": 0.4}

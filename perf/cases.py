@@ -291,3 +291,114 @@ def tolerance(case):
     if case["kind"] == "step":
         return {"rel": 1e-2, "max": 5e-2, "differ": 5e-4 if case["rope"] and case["cache"] == "fp8" else 0.0}
     return {"rel": 1e-2, "max": 0.4}
+
+
+# ------------------------------------------------------------------ the same results in 64 bits, by plain torch
+def _rotated(s, x, pos):
+    """Rows x [n, H, D] at positions pos [n]: the head norm where the case has it, then the rotation."""
+    x = x.double()
+    if s["norm"]:
+        x = x * torch.rsqrt(x.pow(2).mean(-1, keepdim=True) + s["norm"]["eps"])
+    cos, sin = s["cos"][pos].double().unsqueeze(1), s["sin"][pos].double().unsqueeze(1)
+    a, b = x.chunk(2, -1)
+    return torch.cat([a * cos - b * sin, b * cos + a * sin], -1)
+
+
+def _attend(q, k, v, first, scale):
+    """q [n, Hq, D] at positions first.. over k, v [Hkv, L, D]: every row sees the keys up to its own position."""
+    n, Hq, _ = q.shape
+    Hkv, L, _ = k.shape
+    out = torch.empty(n, Hq, q.shape[-1], dtype=torch.float64, device=q.device)
+    for h in range(Hq):
+        kk, vv = k[h // (Hq // Hkv)].double(), v[h // (Hq // Hkv)].double()
+        for r in range(0, n, 2048):
+            rows = q[r:r + 2048, h].double()
+            see = min(L, first + r + len(rows))
+            p = rows @ kk[:see].T * scale
+            own = first + r + torch.arange(len(rows), device=q.device)
+            p.masked_fill_(torch.arange(see, device=q.device) > own[:, None], -math.inf)
+            out[r:r + 2048, h] = torch.softmax(p, -1) @ vv[:see]
+    return out
+
+
+def _exact_scan(s):
+    x, L = s["x"].double(), s["len"].tolist()
+    i, r = torch.sigmoid(s["gx"].double()), torch.sigmoid(s["ga"].double())
+    log_a = -8 * r * torch.nn.functional.softplus(s["ap"].double())
+    a, m = torch.exp(log_a), torch.sqrt(-torch.expm1(2 * log_a))
+    if s["pos"] is not None:
+        start = (s["pos"] == 0).unsqueeze(-1)
+        a, m = a.masked_fill(start, 0.0), m.masked_fill(start, 1.0)
+    b = m * i * x
+    live = torch.arange(x.shape[1], device=x.device)[None, :] < s["len"][:, None]
+    h, y = s["state"].double(), s["y"].double()
+    for t in range(max(L)):
+        h = torch.where(live[:, t, None], a[:, t] * h + b[:, t], h)
+        y[:, t] = torch.where(live[:, t, None], h, y[:, t])
+    return y, h
+
+
+def _quantised(x, scale):
+    return (x.float() / scale[:, None]).clamp(-448, 448).to(torch.float8_e4m3fn)
+
+
+def _exact_step(c, s):
+    h, o = s["cache"], torch.empty(s["q"].shape, dtype=torch.float64, device="cuda")
+    k, v = (t.clone() if c["cache"] == "fp8" else t.double() for t in (h["k"], h["v"]))
+    for b, L in enumerate(s["len"].tolist()):
+        q, kn, vn = s["q"][b:b + 1].double(), s["k"][b].double(), s["v"][b].double()
+        if c["rope"]:
+            q, kn = _rotated(s, q, [L - 1]), _rotated(s, kn, [L - 1])
+        if c["cache"] == "fp8":
+            kn, vn = (_quantised(x[0].bfloat16(), sc).view(torch.uint8) for x, sc in ((kn, h["ks"]), (vn, h["vs"])))
+        else:
+            kn, vn = kn[0], vn[0]
+        if h["table"] is None:
+            k[b, :, L - 1], v[b, :, L - 1] = kn, vn
+            kk, vv = k[b, :, :L], v[b, :, :L]
+        else:
+            pages = h["table"][b, :-(-L // c["page"])].long()
+            at = pages[-1], slice(None), (L - 1) % c["page"]
+            k[at], v[at] = kn, vn
+            kk, vv = (t[pages].transpose(0, 1).flatten(1, 2)[:, :L] for t in (k, v))
+        if c["cache"] == "fp8":
+            kk, vv = (t.view(torch.float8_e4m3fn).double() * sc.double()[:, None, None]
+                      for t, sc in ((kk.contiguous(), h["ks"]), (vv.contiguous(), h["vs"])))
+        q = q[0].view(c["Hkv"], -1, c["D"])
+        o[b] = (torch.softmax(q @ kk.transpose(1, 2) * s["scale"], -1) @ vv).flatten(0, 1)
+    # the stored codes have no value in 64 bits
+    return (o, None, None) if c["cache"] == "fp8" else (o, k, v)
+
+
+def exact(case, seed):
+    c, s = case, prepare(case, seed)
+    kind = c["kind"]
+    if kind == "scan":
+        return _exact_scan(s)
+    if kind == "step":
+        return _exact_step(c, s)
+    past = s["past"].tolist() if "past" in s else [0] * c["B"]
+    q, o = s["q"].double(), s["o"].double()
+    if kind == "chunk":
+        h = s["cache"]
+        ck, cv = h["k"].double(), h["v"].double()
+    else:
+        ck, cv = s["ck"].double(), s["cv"].double()
+    for b, n in enumerate(s["len"].tolist()):
+        L, first = past[b] + n, past[b]
+        kn, vn = s["k"][b, :n].double(), s["v"][b, :n].double()
+        if kind == "rope_prompt":
+            pos = torch.arange(n, device="cuda")
+            q[b, :n], kn = _rotated(s, q[b, :n], pos), _rotated(s, kn, pos)
+        table = h["table"] if kind == "chunk" else None
+        if table is None:
+            ck[b, :, first:L], cv[b, :, first:L] = kn.transpose(0, 1), vn.transpose(0, 1)
+            kk, vv = ck[b, :, :L], cv[b, :, :L]
+        else:
+            pages = table[b, :-(-L // c["page"])].long()
+            slot = torch.arange(first, L, device="cuda")
+            at = pages[slot // c["page"]], slice(None), slot % c["page"]
+            ck[at], cv[at] = kn, vn
+            kk, vv = (t[pages].transpose(0, 1).flatten(1, 2)[:, :L] for t in (ck, cv))
+        o[b, :n] = _attend(q[b, :n], kk, vv, first, s["scale"])
+    return (q, o, ck, cv) if kind == "rope_prompt" else (o, ck, cv)

@@ -281,8 +281,9 @@ l4l_status l4l_attn_merge(const void *o_parts, const float *d_lse_parts, int R, 
  *   d_position   device int32 [B, T], or NULL: no resets (a chunk that continues its sequence)
  *   d_seq_lens   device int32 [B], or NULL meaning T for all
  *   d_state      device float [B, W], read and written
- *   workspace    >= l4l_rglru_workspace_bytes(B, T, W) bytes, initialised once (at present the 256-byte
- *                status block: the state is handed from tile to tile on chip)
+ *   workspace    >= l4l_rglru_workspace_bytes(B, T, W) bytes, initialised once: the 256-byte status block and
+ *                one counter per strip of channels. The status block alone is accepted too; long sequences
+ *                are then not cut along the time axis, which is slower for some sizes (same results)
  */
 size_t l4l_rglru_workspace_bytes(int B, int T, int W);
 

@@ -486,7 +486,8 @@ l4l_status l4l_rglru_scan(const void *x, const void *gate_x, const void *gate_a,
 int l4l_rglru_strip_channels(int B, int T, int W)
 {
     if (B <= 0 || T <= 0 || W <= 0 || W % 8 != 0) return -1;
-    const int split = rglru_strip_split(B, T, W);
+    int segments = 1;
+    const int split = rglru_strip_split(B, T, W, &segments);
     return split == 0 ? 64 : 64 / split;
 }
 

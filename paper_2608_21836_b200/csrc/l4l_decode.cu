@@ -38,10 +38,7 @@ namespace {
 // 16 of them); with W = 4 two CTAs share an SM, with W = 8 one CTA owns it and streams ranges twice as long,
 // so that fewer sequences are cut between CTAs. W + 2 warps in all: consumers, producer, finisher.
 constexpr int kPostRing = 16;               // pieces a producer can be ahead of its finisher (ring size)
-// The ticket counters sit at a FIXED place and size in the workspace (right after the status block), so
-// that calls of different shapes on one workspace can never write partials over counters another call
-// relies on being zero.
-constexpr size_t kTicketBytes = 128 * 1024;  // 32768 (sequence, KV head) pairs per launch
+constexpr size_t kTicketBytes = kCounterBytes;  // the ticket counters: 32768 (sequence, KV head) pairs per launch
 constexpr int kMaxB = 384;                 // sequences per launch (prefix sums and lengths live in shared memory)
 
 // F8: the cache holds e4m3 bytes (one byte per value) instead of bf16.

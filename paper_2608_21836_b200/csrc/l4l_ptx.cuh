@@ -19,6 +19,9 @@ constexpr unsigned kErrPrefillWait = 2u;
 constexpr unsigned kErrScanWait = 4u;
 constexpr unsigned kErrSelfTestWait = 8u;
 constexpr size_t kStatusBytes = 256;
+// Counters sit at a FIXED place and size in a workspace, right behind the status block, and are zero between calls:
+// calls of different kinds and shapes on one workspace can never write partials over counters that another relies on.
+constexpr size_t kCounterBytes = 128 * 1024;  // 32768 counters
 
 // Cycle budget of one bounded wait (~0.25 s at 2 GHz): far above any legitimate latency.
 constexpr long long kWaitCycleBudget = 1ll << 29;
@@ -70,6 +73,11 @@ __device__ __forceinline__ int ld_acquire_gpu(const int *p)
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void st_release_gpu(int *p, int v)
+{
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // ----------------------------------------------------------------------------- mbarrier

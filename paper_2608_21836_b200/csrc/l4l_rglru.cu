@@ -25,6 +25,11 @@
 // lane = (sub-tile, channel pair), so every instruction still does 32 lanes' worth of work. Everything per lane is
 // unchanged; the start states of a warp's later sub-tiles come from the earlier ones by kSplit - 1 shuffles
 // (h <- A h + E) inside step 3. Twice or four times as many CTAs of half or a quarter of the work spread evenly.
+//
+// Segments. Where the strips fill the GPU more than once, a last round of a few strips leaves most SMs idle (320 strips of 32
+// channels on 296 places: 200 us). The time axis is then cut as well: a CTA per (strip, segment), all first segments ahead of all
+// second ones, the state passing through its place in global memory behind a counter per strip (release / acquire). By
+// the time a later segment gets a place its predecessor has long finished, so nothing waits: 156 us in four segments.
 #include <type_traits>
 
 #include "l4l_internal.h"
@@ -54,6 +59,8 @@ struct RglruParams {
     float *state;                // [B, W] in/out
     __nv_bfloat16 *y;            // [B, T, W]
     unsigned *status;
+    int *progress;               // [B, strips] segments of the strip that are done (null: one segment); zero between calls
+    int seg_tiles;               // tiles (of kSteps steps) per segment
     int B, T, W;
 };
 
@@ -95,7 +102,11 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int b = blockIdx.y, c0 = blockIdx.x * kCw;
     int L = p.seq_lens ? p.seq_lens[b] : p.T;
     L = L < 0 ? 0 : (L > p.T ? p.T : L);
-    const int n_tiles = (L + kSteps - 1) / kSteps;
+    // this block's segment of the time axis: tiles [tile0, n_tiles) of the n_all tiles that the sequence has
+    const int n_all = (L + kSteps - 1) / kSteps;
+    const int tile0 = (int)blockIdx.z * p.seg_tiles, n_tiles = min(n_all, tile0 + p.seg_tiles);
+    if (tile0 >= n_tiles) return;
+    int *progress = p.progress ? p.progress + (size_t)b * gridDim.x + blockIdx.x : nullptr;
     const int c = c0 + 2 * cp;
     const bool live = c < p.W;                           // W is even: both channels or neither
 
@@ -106,19 +117,23 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         fence_barrier_init();
         fence_proxy_async_smem();
     }
-    if (warp == 0 && sub == 0) {
-        const float2 st = live ? *reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c) : make_float2(0.f, 0.f);
-        *reinterpret_cast<float2 *>(carry + 2 * cp) = st;                      // slot 0: the caller's state starts tile 0
-    }
+    auto start_state = [&]() {                           // warp 0: slot 0 holds the state that the block's first tile starts from
+        if (sub == 0) {
+            const float2 st = live ? __ldcg(reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c)) : make_float2(0.f, 0.f);
+            *reinterpret_cast<float2 *>(carry + 2 * cp) = st;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&handed[0]);
+    };
     __syncthreads();
-    if (threadIdx.x == 0) mbar_arrive(&handed[0]);
+    if (warp == 0 && blockIdx.z == 0) start_state();     // the caller's state
 
     uint8_t *my_stages = stages + (size_t)warp * kStages * kStageBytes;
     uint64_t *my_full = full + warp * kStages;
-    // lane 0 requests this warp's k-th tile (tile warp + k * kTeam) into its buffer k % kStages
+    // lane 0 requests this warp's k-th tile (tile tile0 + warp + k * kTeam) into its buffer k % kStages
     // (rows past T arrive as zeros and still count)
     auto request = [&](int k) {
-        const int tile = warp + k * kTeam;
+        const int tile = tile0 + warp + k * kTeam;
         if (lane == 0 && tile < n_tiles) {
             const uint32_t s = k % kStages;
             mbar_arrive_expect_tx(&my_full[s], kStageBytes);
@@ -144,30 +159,48 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
     const uint64_t half2 = pack_f32x2(0.5f, 0.5f), one2 = pack_f32x2(1.f, 1.f), zero2 = pack_f32x2(0.f, 0.f);
     const uint64_t k2h = mul_f32x2(k2, half2);
-    const uint64_t two_ln2 = pack_f32x2(1.3862943611198906f, 1.3862943611198906f);
-    const uint64_t nc24 = pack_f32x2(-1.f / 24.f, -1.f / 24.f), nc6 = pack_f32x2(-1.f / 6.f, -1.f / 6.f);
-    const uint64_t nhalf2 = pack_f32x2(-0.5f, -0.5f), neg1 = pack_f32x2(-1.f, -1.f);
+    // (1 - a^2) / 4 = -expm1(z) / 4 with z = w log2(a), w = 2 ln 2: series coefficients in log2(a), the quarter (which
+    // the square root turns into the half of sigmoid = 0.5 tanh + 0.5) folded in
+    constexpr float kW = 1.3862943611198906f, kNearOne = -0.0625f / kW;
+    const uint64_t s1c = pack_f32x2(-kW / 4, -kW / 4), s2c = pack_f32x2(-kW * kW / 8, -kW * kW / 8);
+    const uint64_t s3c = pack_f32x2(-kW * kW * kW / 24, -kW * kW * kW / 24);
+    const uint64_t s4c = pack_f32x2(-kW * kW * kW * kW / 96, -kW * kW * kW * kW / 96);
+    const uint64_t quarter2 = pack_f32x2(0.25f, 0.25f), nquarter2 = pack_f32x2(-0.25f, -0.25f);
     uint32_t *yrow = reinterpret_cast<uint32_t *>(p.y + (size_t)b * p.T * p.W + c);
     const size_t y_step = (size_t)p.W / 2;               // 32-bit words between time steps
-    auto resets_of = [&](int tile) -> unsigned {
-        // bit t: step t of THIS LANE'S sub-tile is the first token of a segment (position 0)
-        if (!p.position || tile >= n_tiles) return 0u;
-        unsigned mine = 0u;
+    // Positions of a tile's steps, one per lane and part, as loaded: the vote that turns them into a mask comes a whole
+    // tile later. (Voting right behind the load stalled every tile for an L2 round trip: B=4 x 8192 x 2560 with
+    // positions 184 us, without them 140 us.)
+    constexpr int kPosParts = (kSteps + 31) / 32;
+    int pos_next[kPosParts];
+    auto request_positions = [&](int tile) {
 #pragma unroll
-        for (int part = 0; part < (kSteps + 31) / 32; ++part) {
+        for (int part = 0; part < kPosParts; ++part) {
             const int t = tile * kSteps + part * 32 + lane;
-            const int pos = (part * 32 + lane < kSteps && t < L) ? __ldg(p.position + (size_t)b * p.T + t) : 1;
-            const unsigned bits = __ballot_sync(0xffffffffu, pos == 0);
+            pos_next[part] = (p.position && tile < n_tiles && part * 32 + lane < kSteps && t < L)
+                                 ? __ldg(p.position + (size_t)b * p.T + t) : 1;
+        }
+    };
+    auto resets_requested = [&]() -> unsigned {
+        // bit t: step t of THIS LANE'S sub-tile is the first token of a segment (position 0). Nearly every tile has none.
+        bool any = pos_next[0] == 0;
+#pragma unroll
+        for (int part = 1; part < kPosParts; ++part) any = any || pos_next[part] == 0;
+        unsigned mine = 0u;
+        if (!__any_sync(0xffffffffu, any)) return mine;
+#pragma unroll
+        for (int part = 0; part < kPosParts; ++part) {
+            const unsigned bits = __ballot_sync(0xffffffffu, pos_next[part] == 0);
             if ((sub * kTb) / 32 == part) mine = (bits >> ((sub * kTb) % 32)) & 0xffffu;
         }
         return mine;
     };
-    unsigned reset_next = resets_of(warp);
+    request_positions(tile0 + warp);
 
-    for (int k = 0, tile = warp; tile < n_tiles; ++k, tile += kTeam) {
+    for (int k = 0, tile = tile0 + warp; tile < n_tiles; ++k, tile += kTeam) {
         const uint32_t s = k % kStages, ph = (k / kStages) & 1u;
-        const unsigned resets = reset_next;
-        reset_next = resets_of(tile + kTeam);            // in flight while this tile is processed
+        const unsigned resets = resets_requested();
+        request_positions(tile + kTeam);                 // in flight while this tile is processed
         if (!mbar_wait(&my_full[s], ph, abort_flag)) break;
         // the tile in shared memory: kSteps rows of kPairs words; this lane reads rows sub * kTb .. of column cp
         const uint32_t *xs = reinterpret_cast<const uint32_t *>(my_stages + s * kStageBytes) + sub * kTb * kPairs + cp;
@@ -191,18 +224,16 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 float l0, l1;
                 unpack_f32x2(la2, l0, l1);
                 uint64_t a = pack_f32x2(fast_exp2(l0), fast_exp2(l1));
-                // 1 - a^2 = -expm1(z), z = 2 ln a: a short series when a is close to 1, where 1 - a*a cancels
-                const uint64_t z = mul_f32x2(la2, two_ln2);
-                const uint64_t npoly = fma_f32x2(z, fma_f32x2(z, fma_f32x2(z, nc24, nc6), nhalf2), neg1);
-                float s0, s1, d0, d1, z0, z1;
-                unpack_f32x2(mul_f32x2(z, npoly), s0, s1);
-                unpack_f32x2(fma_f32x2(mul_f32x2(a, neg1), a, one2), d0, d1);
-                unpack_f32x2(z, z0, z1);
-                float m0 = sqrt_approx(z0 > -0.0625f ? s0 : d0), m1 = sqrt_approx(z1 > -0.0625f ? s1 : d1);
+                // m / 2 = sqrt((1 - a^2) / 4): a short series when a is close to 1, where 1 - a*a cancels
+                const uint64_t series = fma_f32x2(la2, fma_f32x2(la2, fma_f32x2(la2, s4c, s3c), s2c), s1c);
+                float s0, s1, d0, d1;
+                unpack_f32x2(mul_f32x2(la2, series), s0, s1);
+                unpack_f32x2(fma_f32x2(mul_f32x2(a, nquarter2), a, quarter2), d0, d1);
+                float m0 = sqrt_approx(l0 > kNearOne ? s0 : d0), m1 = sqrt_approx(l1 > kNearOne ? s1 : d1);
                 if constexpr (!kPlain) {
                     if ((resets >> t) & 1u) {                                          // uniform across a sub-tile's lanes
                         a = zero2;
-                        m0 = m1 = 1.f;
+                        m0 = m1 = 0.5f;
                     }
                     if (t >= n) {                                                      // past the end: the identity step
                         a = one2;
@@ -210,7 +241,7 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     }
                 }
                 av[t] = a;
-                const uint64_t mxh = mul_f32x2(mul_f32x2(pack_f32x2(m0, m1), half2), xv);   // m x / 2
+                const uint64_t mxh = mul_f32x2(pack_f32x2(m0, m1), xv);                    // m x / 2
                 bv[t] = fma_f32x2(th_x, mxh, mxh);                                         // m x sigmoid(gate_x)
                 if constexpr (!kPlain) {
                     // rows past the end are caller memory that may hold anything (0 * NaN is NaN): select, not multiply
@@ -236,8 +267,24 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // Every warp has its own barrier, completed once per tile it owns by the owner of the tile before; that
         // warp cannot reach its next arrival here before this warp has handed the present tile on, so the
         // phases are seen one by one.
+        if (tile == tile0 && blockIdx.z != 0) {
+            // a later segment starts from the state that the strip's previous segment left in global memory
+            if (lane == 0) {
+                const long long w0 = clock64();
+                while (ld_acquire_gpu(progress) != (int)blockIdx.z) {
+                    if (*abort_flag || clock64() - w0 > kWaitCycleBudget) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    __nanosleep(64);
+                }
+            }
+            __syncwarp();
+            start_state();
+        }
         if (!mbar_wait(&handed[warp], k & 1u, abort_flag)) break;
-        const float2 hs = *reinterpret_cast<const float2 *>(carry + (tile & 1) * kCb + 2 * cp);
+        const int slot = (tile - tile0) & 1;
+        const float2 hs = *reinterpret_cast<const float2 *>(carry + slot * kCb + 2 * cp);
         uint64_t h2 = pack_f32x2(hs.x, hs.y);                                  // start state of the warp's first sub-tile
         {
             // start states of the later sub-tiles, and the end state of the warp's steps: h <- A h + E along the
@@ -252,11 +299,18 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                     unpack_f32x2(fma_f32x2(A, h2, E), e0, e1);
                 }
             }
-            if (sub == kSplit - 1) *reinterpret_cast<float2 *>(carry + ((tile + 1) & 1) * kCb + 2 * cp) = make_float2(e0, e1);
+            if (sub == kSplit - 1) *reinterpret_cast<float2 *>(carry + (slot ^ 1) * kCb + 2 * cp) = make_float2(e0, e1);
             __syncwarp();
             if (lane == 0) mbar_arrive(&handed[(warp + 1) % kTeam]);           // release: the slot is written
-            if (tile + 1 == n_tiles && live && sub == kSplit - 1)              // the sequence ends here
-                *reinterpret_cast<float2 *>(p.state + (size_t)b * p.W + c) = make_float2(e0, e1);
+            if (tile + 1 == n_tiles) {                                         // the sequence, or its segment, ends here
+                if (live && sub == kSplit - 1) *reinterpret_cast<float2 *>(p.state + (size_t)b * p.W + c) = make_float2(e0, e1);
+                if (progress) {
+                    __threadfence();
+                    __syncwarp();
+                    // the last segment leaves the counter at zero for the next call
+                    if (lane == 0) st_release_gpu(progress, n_tiles == n_all ? 0 : (int)blockIdx.z + 1);
+                }
+            }
         }
         // ---- the recurrence proper, one packed FMA per step, and the outputs
 #pragma unroll
@@ -275,12 +329,18 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
 }  // namespace
 
-size_t rglru_workspace_bytes(int, int, int) { return kStatusBytes; }
+// the status block and one counter per strip (of the narrowest width) where they fit the region that decode calls on
+// the same workspace leave at zero; a workspace of the status block alone is enough, the time axis is not cut then
+size_t rglru_workspace_bytes(int B, int, int W)
+{
+    const size_t counters = (size_t)B * ((W + 15) / 16) * sizeof(int);
+    return kStatusBytes + (counters <= kCounterBytes ? counters : 0);
+}
 
 namespace {
 
 template <int kTeam, int kSplit>
-l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, const RglruParams &p, cudaStream_t stream)
+l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, RglruParams p, int segments, cudaStream_t stream)
 {
     // one opt-in per instantiation and device
     static bool configured_on[kDeviceSlots] = {};
@@ -301,7 +361,12 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, c
         !make_tmap_rows_bf16(&tgx, gate_x, p.W, p.T, p.B, p.W, (int64_t)p.T * p.W, kCw, kTb * kSplit) ||
         !make_tmap_rows_bf16(&tga, gate_a, p.W, p.T, p.B, p.W, (int64_t)p.T * p.W, kCw, kTb * kSplit))
         return L4L_ERR_CUDA;
-    const dim3 grid((p.W + kCw - 1) / kCw, p.B);
+    const int strips = (p.W + kCw - 1) / kCw, tiles = (p.T + kTb * kSplit - 1) / (kTb * kSplit);
+    p.seg_tiles = (tiles + segments - 1) / segments;
+    if (segments > 1) p.seg_tiles = (p.seg_tiles + kTeam - 1) / kTeam * kTeam;      // whole rounds of the team
+    const int segs = (tiles + p.seg_tiles - 1) / p.seg_tiles;
+    if (segs == 1) p.progress = nullptr;
+    const dim3 grid(strips, p.B, segs);
     rglru_scan_kernel<kTeam, kSplit><<<grid, kTeam * 32, smem_bytes(kTeam), stream>>>(tx, tgx, tga, p);
     return cudaGetLastError() == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
 }
@@ -310,45 +375,62 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, c
 
 l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate_a, const float *d_a_param,
                              const int32_t *d_position, const int32_t *d_seq_lens, float *d_state, void *y, int B, int T,
-                             int W, void *workspace, size_t, cudaStream_t stream)
+                             int W, void *workspace, size_t ws_bytes, cudaStream_t stream)
 {
     RglruParams p;
     p.a_param = d_a_param; p.position = d_position; p.seq_lens = d_seq_lens; p.state = d_state;
     p.y = static_cast<__nv_bfloat16 *>(y);
     p.status = static_cast<unsigned *>(workspace);
     p.B = B; p.T = T; p.W = W;
-    if (T <= kTb) return launch_shape<1, 1>(x, gate_x, gate_a, p, stream);
-    const int split = rglru_strip_split(B, T, W);
-    if (split == 0) return launch_shape<16, 1>(x, gate_x, gate_a, p, stream);
-    if (split == 4) return launch_shape<8, 4>(x, gate_x, gate_a, p, stream);
-    if (split == 2) return launch_shape<8, 2>(x, gate_x, gate_a, p, stream);
-    return launch_shape<8, 1>(x, gate_x, gate_a, p, stream);
+    p.progress = reinterpret_cast<int *>(static_cast<uint8_t *>(workspace) + kStatusBytes);
+    if (T <= kTb) return launch_shape<1, 1>(x, gate_x, gate_a, p, 1, stream);
+    int segs = 1;
+    const size_t needed = rglru_workspace_bytes(B, T, W);
+    const bool with_counters = needed > kStatusBytes && ws_bytes >= needed;
+    const int split = rglru_strip_split(B, T, W, with_counters ? &segs : nullptr);
+    if (split == 0) return launch_shape<16, 1>(x, gate_x, gate_a, p, segs, stream);
+    if (split == 4) return launch_shape<8, 4>(x, gate_x, gate_a, p, segs, stream);
+    if (split == 2) return launch_shape<8, 2>(x, gate_x, gate_a, p, segs, stream);
+    return launch_shape<8, 1>(x, gate_x, gate_a, p, segs, stream);
 }
 
-// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels.
-int rglru_strip_split(int B, int T, int W)
+// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels. *segments
+// (when given): into how many segments the time axis is cut.
+//
+// Two teams of 8 are resident per SM and together keep its issue slots busy, so n blocks take n / (2 SMs) rounds; a
+// last round with a lone team on an SM takes 0.68 of a full one (a lone team reaches three quarters of the rate of two).
+// Narrower strips make n larger and the blocks shorter, and so do segments, which cost about 4 us per round (set-up, first
+// loads, drain of the ring; 6 us on 16-channel strips) but leave the lines that the loads fetch wider. A strip is a
+// serial chain: it is cut only when the strips alone fill the GPU, so that a segment finds its predecessor finished. B = 4 x 8192
+// x 2560 with positions, us by (channels, segments): (64, 1) 222, (32, 1) 200, (32, 2) 166, (32, 4) 156, (32, 8) 166, (16, 1) 170,
+// (16, 4) 180.
+int rglru_strip_split(int B, int T, int W, int *segments)
 {
+    if (segments) *segments = 1;
     if (T <= kTb) return 1;
     const long long sms = sm_count();
-    // A strip is a serial chain that keeps an SM's issue slots busy, so a launch takes as long as the most loaded
-    // SM. Estimated time of that SM, in units of one 64-channel strip on an SM of its own: k CTAs of 1/s strip each
-    // take k / s; a lone team of 8 warps reaches about three quarters of the issue rate that two co-resident teams
-    // or one team of 16 warps reach.
-    auto fullest = [&](int s) { return ((long long)((W + kCb / s - 1) / (kCb / s)) * B + sms - 1) / sms; };
+    const double us_per_step_channel = 4.54e-4;          // of a resident pair of teams
+    auto rounds = [&](long long n) {
+        const long long rest = n % (2 * sms);
+        return (double)(n / (2 * sms)) + (rest == 0 ? 0.0 : rest <= sms ? 0.68 : 1.0);
+    };
+    auto strips = [&](int s) { return (long long)((W + kCb / s - 1) / (kCb / s)) * B; };
     int best = 1;
-    double best_time = fullest(1) >= 2 ? (double)fullest(1) : 1.0 / 0.74;
-    if (fullest(1) == 1 && T >= 16 * 2 * kTb) {
+    double best_time = rounds(strips(1)) * T * kCb * us_per_step_channel;
+    if (strips(1) <= sms && T >= 16 * 2 * kTb) {         // no more strips than SMs: 16 warps reach the full rate alone
         best = 0;
-        best_time = 1.0;
+        best_time = 0.5 * T * kCb * us_per_step_channel;
     }
-    // narrower strips have to win by a tenth or more (their warps pay two or four dependent steps in the hand-off
-    // instead of one), and the sequence has to be long enough for their wider tiles
-    for (int s = 2; s <= 4; s *= 2) {
-        const long long k = fullest(s);
-        const double time = k >= 2 ? (double)k / s : (1.0 / s) / 0.74;
-        if (time < 0.9 * best_time && T >= 8 * kTb * s) {
-            best = s;
-            best_time = time;
+    for (int s = 1; s <= 4; s *= 2) {
+        if (s > 1 && T < 8 * kTb * s) break;             // long enough for the wider tiles of narrow strips
+        for (int z = 1; z <= (segments ? 4 : 1); z *= 2) {
+            if ((s == 1 && z == 1) || (z > 1 && (strips(s) < 2 * sms || T < 1024 * z))) continue;
+            const double time = rounds(strips(s) * z) * ((double)T / z * (kCb / s) * us_per_step_channel + (z == 1 ? 0.0 : s < 4 ? 4.0 : 6.0));
+            if (time < (z == 1 ? 0.9 : 0.95) * best_time) {
+                best = s;
+                best_time = time;
+                if (segments) *segments = z;
+            }
         }
     }
     return best;

@@ -120,3 +120,26 @@ def test_rglru_empty_inputs_are_a_no_op():
                        seq_lens=torch.zeros(2, dtype=torch.int32, device="cuda"))
     torch.cuda.synchronize()
     assert (state == 7.0).all() and (y == 3.0).all() and l4l.l4l_last_device_error(ws) == 0
+
+
+@pytest.mark.parametrize("B,T,W", [(4, 8192, 2560), (5, 8007, 2048)])
+def test_rglru_time_segments(B, T, W):
+    """Launches that the library cuts into segments of the time axis (a workspace with room for the counters) against the
+    same launch uncut (a workspace of the status block alone), which takes the same steps in the same order: equal bit
+    for bit. Lengths: none, one step, the end of a segment (2048 steps in the first case) and one past it, all; resets;
+    a second call finds the counters at zero."""
+    x, gx, ga, ap, h0 = (t.cuda() for t in make(B, T, W, 1900 + T))
+    lens = torch.tensor([T, 0, 2048, 2049, 1][:B], dtype=torch.int32, device="cuda")
+    pos = torch.arange(T, dtype=torch.int32, device="cuda").repeat(B, 1)
+    pos[0, 3000:] -= 3000
+    uncut, cut = l4l.new_rglru_workspace(B, T, W)[:256].clone(), l4l.new_rglru_workspace(B, T, W)
+    outs = []
+    for ws in (uncut, cut, cut):
+        y, st = torch.zeros_like(x), h0.clone()
+        l4l.l4l_rglru_scan(x, gx, ga, ap, st, y, ws, position=pos, seq_lens=lens)
+        assert l4l.l4l_last_device_error(ws) == 0
+        outs.append((y, st))
+    assert int(cut[256:].max()) == 0
+    for y, st in outs[1:]:
+        assert torch.equal(y.view(torch.int16), outs[0][0].view(torch.int16)) and torch.equal(st, outs[0][1])
+    assert torch.equal(outs[0][1][1], h0[1]) and torch.isfinite(outs[0][0]).all()

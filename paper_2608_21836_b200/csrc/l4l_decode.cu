@@ -120,6 +120,7 @@ struct DecodeParams {
     int table_stride, page_size, page_shift, num_pages;
     int page_box;             // paged: tokens per box of tmap_k / tmap_v (divides the tile, never straddles a page)
     int tail_rows;            // tokens per box of tmap_k_tail / tmap_v_tail (32, or the page size if that is smaller)
+    int page_loads;           // tmap_k / tmap_v bring a whole page, both halves, per load (bf16, head_dim 128, pages of 16 or 32)
     int B, Hq, Hkv, G, min_tiles, nsplit, max_kv_len;
     int stream_once;          // load K/V with the L2 evict-first policy (large caches)
     int nfin;                 // finisher warps (BigG: one per 4 query heads of the group; else 1)
@@ -420,6 +421,14 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                         if (bx >= n_box) break;
                         int tt = tile * kTileT + bx * box_rows;
                         if (paged) tt &= p.page_size - 1;
+                        if constexpr (C::kHalves == 2) {
+                            if (p.page_loads) {
+                                uint8_t *pb = dst + bx * box_rows * 256;   // [half][page tokens][128 bytes]
+                                tma_load_5d_policy(pb, &tmap_k, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
+                                tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
+                                continue;
+                            }
+                        }
                         order_coords(p.coord, tt / C::kTokPerRow, kvh, page_of[bx], c1, c2, c3);
                         uint8_t *db = dst + bx * box_rows * C::kTokBytes;  // whole 8-row groups: the swizzle phase is kept
 #pragma unroll
@@ -780,6 +789,8 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         uint32_t n_dumps = 0;                // pieces handed to the finisher so far
         uint32_t n_rotated = 0;              // pieces whose query rows were rotated (phase of q_rotated)
         float k_sc = 1.f, v_sc = 1.f;        // fp8 cache: scales of the piece's KV head (read once per piece)
+        const bool by_page = C::kHalves == 2 && p.page_loads != 0;
+        const TileRows rows = {by_page ? (uint32_t)p.page_size * 128u : C::kHalfBytes, by_page ? (uint32_t)-p.page_size : 0u};
 
         for (uint32_t it = 0;; ++it) {
             const uint32_t s = it % C::kStages;
@@ -874,7 +885,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     }
                     if (p.block_table == nullptr || (outer >= 0 && outer < p.num_pages)) {
                         uint8_t *kt = stages + (size_t)s * C::kStageBytes;
-                        const uint32_t off = (lane >> 3) * C::kHalfBytes + swz128(last, lane & 7);
+                        const uint32_t off = rows.chunk(last, lane);
                         *reinterpret_cast<uint4 *>(kt + off) = kk;
                         *reinterpret_cast<uint4 *>(kt + C::kTileBytes + off) = vv;
                         const size_t dst = (size_t)outer * p.c_sb + (size_t)mt.kvh * p.c_sh + (size_t)slot * p.c_st + lane * 8;
@@ -1006,7 +1017,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
 #pragma unroll
                 for (int u = 0; u < kSub; ++u) {
                     if (u == 0 || nvalid > 16 * u) {
-                        warp_qk_16x16<D>(qf, k_tile, C::kHalfBytes, row0 + 16 * u, sv[2 * u], sv[2 * u + 1]);
+                        warp_qk_16x16<D>(qf, k_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0, sv[2 * u], sv[2 * u + 1]);
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             sv[2 * u][e] *= sc;
@@ -1030,8 +1041,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     for (int i = lane; i < (fetched_end - nvalid) * chunks_per_row; i += 32) {
                         const int r = row0 + nvalid + i / chunks_per_row;
                         const int ch = i % chunks_per_row;
-                        *reinterpret_cast<uint4 *>(vt + (ch >> 3) * C::kHalfBytes + r * 128 + ((ch & 7) << 4)) =
-                            make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4 *>(vt + rows.chunk(r, ch)) = make_uint4(0u, 0u, 0u, 0u);
                     }
                     wrote_smem = true;
                     __syncwarp();
@@ -1040,7 +1050,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                 warp_softmax_tiles<D, false, 2 * kSub>(st, sv, pa);
 #pragma unroll
                 for (int u = 0; u < kSub; ++u)
-                    if (u == 0 || nvalid > 16 * u) warp_pv_16x16<D>(st, pa[u], v_tile, C::kHalfBytes, row0 + 16 * u);
+                    if (u == 0 || nvalid > 16 * u) warp_pv_16x16<D>(st, pa[u], v_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0);
             }
 
             if (wrote_smem) fence_proxy_async_smem();   // generic writes before the next TMA fill
@@ -1337,7 +1347,17 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         // what the maps see as a row: a token, or (fp8 at head_dim 64) a pair of tokens
         const int tpr = pair_rows ? 2 : 1, map_d = pair_rows ? 128 : D;
         const int64_t map_rows = cache.max_len / tpr, map_st = cache.stride_t * tpr;
-        if (!make_tmap(&tk, &coord, kb, map_d, map_rows, Hkv, outer, map_st, cache.stride_h,
+        // Pages of 16 or 32 tokens at head_dim 128: one load per page instead of one per 64-column half. What bounds such
+        // pools is the loads per tile (a 2 KB box holds the TMA unit for about 80 ns): B=48 ragged over 16-token pages 85.6
+        // us by halves, 69.7 by pages; B=32 over 32-token pages 63.5 and 57.5. Pages of 64 have half as many boxes already.
+        const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr) &&
+                                make_tmap_page(&tk, kb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) &&
+                                make_tmap_page(&tv, vb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b);
+        if (page_loads) {
+            tk_tail = tk;            // groups of the last tile are pages too
+            tv_tail = tv;
+            coord = TmapCoord{};
+        } else if (!make_tmap(&tk, &coord, kb, map_d, map_rows, Hkv, outer, map_st, cache.stride_h,
                        cache.stride_b, box_d, box_t / tpr, esz) ||
             !make_tmap(&tv, &coord_v, vb, map_d, map_rows, Hkv, outer, map_st, cache.stride_h,
                        cache.stride_b, box_d, box_t / tpr, esz) ||
@@ -1375,6 +1395,7 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         p.page_box = box_t;
         p.num_pages = paged ? paged->num_pages : 0;
         p.tail_rows = tail_rows;
+        p.page_loads = page_loads ? 1 : 0;
         p.page_shift = 0;
         while (paged && (1 << p.page_shift) < cache.max_len) ++p.page_shift;
         // only the fused append writes through these: the slice's sequences, or the whole pool of a paged cache

@@ -61,6 +61,7 @@ struct ClusterParams {
     const int32_t *block_table;               // paged cache (null: contiguous)
     int table_stride, page_size, page_shift, num_pages;
     int tail_rows;                            // tokens per box of the tail maps (32, or the page size if that is smaller)
+    int page_loads;                           // tmap_k / tmap_v bring a whole page, both halves, per load
     // rotary embedding (+ optional RMS norm) of the step's q and k_new (null: inputs are final); only with the fused
     // append. The new token's position is kv_len - 1.
     const float *rope_cos, *rope_sin;         // [rope_n_pos, D/2]
@@ -248,6 +249,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     if (bx >= n_box) break;
                     int tt = tile * kTileT + bx * box_rows;
                     if (paged) tt &= p.page_size - 1;
+                    if constexpr (C::kHalves == 2) {
+                        if (p.page_loads) {
+                            uint8_t *pb = dst + bx * box_rows * 256;   // [half][page tokens][128 bytes]
+                            tma_load_5d_policy(pb, &tmap_k, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
+                            tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
+                            continue;
+                        }
+                    }
                     order_coords(p.coord, tt, kvh, page_of[bx], c1, c2, c3);
                     uint8_t *db = dst + bx * box_rows * 128;          // whole 8-row groups: the swizzle phase is kept
 #pragma unroll
@@ -265,6 +274,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
         uint32_t qf[D / 16][4];
         const int r_lo = lane >> 2, r_hi = r_lo + 8;    // query heads of the group held in rows lane/4, lane/4 + 8
         float k_sc = 1.f, v_sc = 1.f;                   // fp8 cache: scales of this KV head
+        const bool by_page = C::kHalves == 2 && p.page_loads != 0;
+        const TileRows rows = {by_page ? (uint32_t)p.page_size * 128u : kHalfBytes, by_page ? (uint32_t)-p.page_size : 0u};
         if constexpr (F8) {
             k_sc = __ldg(p.k_scale + kvh);
             v_sc = __ldg(p.v_scale + kvh);
@@ -335,7 +346,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     }
                     if (p.block_table == nullptr || (outer >= 0 && outer < p.num_pages)) {
                         uint8_t *kt = stages + (size_t)s * C::kStageBytes;
-                        const uint32_t off = (lane >> 3) * kHalfBytes + swz128(last, lane & 7);
+                        const uint32_t off = rows.chunk(last, lane);
                         *reinterpret_cast<uint4 *>(kt + off) = kk;
                         *reinterpret_cast<uint4 *>(kt + C::kTileBytes + off) = vv;
                         const size_t dst = (size_t)outer * p.c_sb + (size_t)kvh * p.c_sh + (size_t)slot * p.c_st + lane * 8;
@@ -431,7 +442,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                 }
             } else if (nvalid > 0) {
                 float s_lo[4], s_hi[4];
-                warp_qk_16x16<D>(qf, k_tile, kHalfBytes, row0, s_lo, s_hi);
+                warp_qk_16x16<D>(qf, k_tile + rows.row(row0), rows.half_bytes, 0, s_lo, s_hi);
                 const int tok = 2 * (lane & 3);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -450,15 +461,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     constexpr int kChunksPerRow = D / 8;
                     for (int i = lane; i < (16 - nvalid) * kChunksPerRow; i += 32) {
                         const int r = row0 + nvalid + i / kChunksPerRow, ch = i % kChunksPerRow;
-                        *reinterpret_cast<uint4 *>(vt + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) =
-                            make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4 *>(vt + rows.chunk(r, ch)) = make_uint4(0u, 0u, 0u, 0u);
                     }
                     wrote_smem = true;
                     __syncwarp();
                 }
                 uint32_t pa[4];
                 warp_softmax_16<D>(st, s_lo, s_hi, pa);
-                warp_pv_16x16<D>(st, pa, v_tile, kHalfBytes, row0);
+                warp_pv_16x16<D>(st, pa, v_tile + rows.row(row0), rows.half_bytes, 0);
             }
             if (wrote_smem) fence_proxy_async_smem();   // generic writes before the next TMA fill
             __syncwarp();
@@ -733,7 +743,15 @@ l4l_status launch_decode_cluster(const void *q, void *o, const l4l_kv_cache &cac
     // pages smaller than a tile are fetched page by page: no box may exceed the page
     const int box_t = (paged && cache.max_len < kTileT) ? cache.max_len : kTileT;
     const int tail_rows = (paged && cache.max_len < 32) ? cache.max_len : 32;
-    if (!make_tmap(&tk, &coord, cache.k, D, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b, box_d,
+    // small pages: one load per page instead of one per 64-column half (the rule and its figures: launch_decode)
+    const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr) &&
+                            make_tmap_page(&tk, cache.k, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) &&
+                            make_tmap_page(&tv, cache.v, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b);
+    if (page_loads) {
+        tk_tail = tk;                // groups of the last tile are pages too
+        tv_tail = tv;
+        coord = TmapCoord{};
+    } else if (!make_tmap(&tk, &coord, cache.k, D, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b, box_d,
                    box_t, esz) ||
         !make_tmap(&tv, &coord_v, cache.v, D, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b,
                    box_d, box_t, esz) ||
@@ -764,6 +782,7 @@ l4l_status launch_decode_cluster(const void *q, void *o, const l4l_kv_cache &cac
     p.page_size = paged ? cache.max_len : 0;
     p.num_pages = paged ? paged->num_pages : 0;
     p.tail_rows = tail_rows;
+    p.page_loads = page_loads ? 1 : 0;
     p.page_shift = 0;
     while (paged && (1 << p.page_shift) < cache.max_len) ++p.page_shift;
     p.rope_cos = rope ? rope->cos : nullptr;

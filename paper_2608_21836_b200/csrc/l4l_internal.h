@@ -53,6 +53,12 @@ inline bool make_tmap_bf16(CUtensorMap *out, TmapCoord *coord, const void *base,
     return make_tmap(out, coord, base, D, n_t, n_h, n_b, stride_t, stride_h, stride_b, box_d, box_t, 2);
 }
 
+// The map for pages smaller than a tile, bf16 rows of 128 elements: a box is one page of one head, both 64-column halves
+// in one load ([half][page_size tokens][64], 128-byte swizzle). Coordinates are (column, token, half, head, page).
+bool make_tmap_page(CUtensorMap *out, const void *base, int page_size, int64_t n_h, int64_t n_pages, int64_t stride_t,
+                    int64_t stride_h, int64_t stride_page);
+inline bool pages_load_whole(int D, int page_size, bool fp8) { return !fp8 && D == 128 && page_size <= 32; }
+
 // Tiled bf16 tensor map without swizzle over a dense [outer, rows, cols] array (cols contiguous): box =
 // box_cols x box_rows x 1. Coordinates are (col, row, outer).
 bool make_tmap_rows_bf16(CUtensorMap *out, const void *base, int64_t n_cols, int64_t n_rows, int64_t n_outer,

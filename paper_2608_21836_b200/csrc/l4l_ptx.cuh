@@ -211,6 +211,18 @@ __device__ __forceinline__ void tma_load_4d_policy(void *smem_dst, const void *t
         : "memory");
 }
 
+// The 5-D form of it.
+__device__ __forceinline__ void tma_load_5d_policy(void *smem_dst, const void *tmap, uint64_t *bar, int c0, int c1,
+                                                   int c2, int c3, int c4, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+        ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(c0), "r"(c1),
+        "r"(c2), "r"(c3), "r"(c4), "l"(policy)
+        : "memory");
+}
+
 // 3-D tiled load global -> shared (same rules as the 4-D form).
 __device__ __forceinline__ void tma_load_3d(void *smem_dst, const void *tmap, uint64_t *bar, int c0, int c1, int c2)
 {

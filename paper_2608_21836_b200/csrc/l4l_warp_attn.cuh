@@ -5,12 +5,26 @@
 // tcgen05 instead: see l4l_prefill_tc.cu.)
 //
 // Tile layout in shared memory: D/64 "halves", each [tile_tokens][64] bf16 (128-byte rows,
-// swizzled), half h covering head_dim [64h, 64h+64).
+// swizzled), half h covering head_dim [64h, 64h+64). Over pages of 16 or 32 tokens at head_dim 128 one load brings
+// both halves of a page, and the tile is a row of pages, each [half][page tokens][64] (TileRows).
 #pragma once
 
 #include "l4l_ptx.cuh"
 
 namespace l4l {
+
+// Where the token rows of a tile lie: `half_bytes` between the halves, and `group` (the negative of the tokens per page;
+// 0: one group) for tiles made of pages that hold both halves each. A 16-token block never straddles groups.
+struct TileRows {
+    uint32_t half_bytes, group;
+    // offset of a token's row in half 0, without the swizzle of its chunks
+    __device__ __forceinline__ uint32_t row(uint32_t token) const { return (token + (token & group)) * 128u; }
+    // 16-byte chunk `ch` of a token's row (bf16: 16 chunks at head_dim 128)
+    __device__ __forceinline__ uint32_t chunk(uint32_t token, uint32_t ch) const
+    {
+        return (ch >> 3) * half_bytes + row(token) + (((ch ^ token) & 7u) << 4);
+    }
+};
 
 template <int D>
 struct WarpAttnState {

@@ -13,8 +13,8 @@
 //   producer warp    walks the CTA's tile range and keeps a ring of TMA tiles (K and V, 128-byte
 //                    swizzle) full, across piece boundaries
 //   W consumer warps each take 16 tokens of every tile and serve ALL query heads of the KV group
-//                    from it: the group is the M dimension (zero-padded to 16) of warp-level bf16
-//                    MMAs, so cache bytes are read once per group. Softmax statistics are fp32;
+//                    from it: the group is the N dimension (zero-padded to 8 or 16) of warp-level
+//                    MMAs whose rows are the tokens, so cache bytes are read once per group. Softmax statistics are fp32;
 //                    row maxima are reduced with warp shuffles. At the end of a piece they drop
 //                    their (max, sum, O) into shared memory and go straight on to the next tile.
 //   finisher warp    merges the consumer warps' results of a piece off the critical path. A sequence
@@ -161,7 +161,8 @@ __device__ __forceinline__ void order_coords(const TmapCoord &c, int t, int h, i
 
 // R8: an e4m3-cache kernel that also carries the rope-fused step. A build of its own, so that the rotation code does
 // not weigh on the registers of the plain fp8 kernels, which are bound by their consumer warps (bf16 kernels always carry it).
-template <int D, int W, bool F8, bool BigG, bool R8 = false>
+// NB: blocks of 8 query heads of the group (the N of the warp MMAs).
+template <int D, int W, bool F8, bool BigG, bool R8, int NB>
 __global__ void __launch_bounds__((BigG ? 11 : W + 2) * 32)
 decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
                     const __grid_constant__ CUtensorMap tmap_k_tail, const __grid_constant__ CUtensorMap tmap_v_tail,
@@ -781,11 +782,9 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         }
     } else {
         // ------------------------------------------------------------------ consumer warps
-        WarpAttnState<D> st;
+        WarpAttnState<D, NB> st;
         st.reset();
-        uint32_t qf[D / 16][4];
-        const int r_lo = lane >> 2;          // query head within the group held in rows lane/4, lane/4+8
-        const int r_hi = r_lo + 8;
+        uint32_t qf[D / 16][NB][2];
         uint32_t n_dumps = 0;                // pieces handed to the finisher so far
         uint32_t n_rotated = 0;              // pieces whose query rows were rotated (phase of q_rotated)
         float k_sc = 1.f, v_sc = 1.f;        // fp8 cache: scales of the piece's KV head (read once per piece)
@@ -826,27 +825,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                         ++n_rotated;
                     }
                 }
-                const uint32_t *qs = reinterpret_cast<const uint32_t *>(q_slots + (size_t)s * q_stride);
-                const uint32_t *qrow_lo = qs + (size_t)r_lo * D / 2;
-                const uint32_t *qrow_hi = qs + (size_t)r_hi * D / 2;
-                const bool v_lo = r_lo < p.G, v_hi = r_hi < p.G;
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    if constexpr (F8) {
-                        // f16 fragments with the k index permuted the way the fp8 K tiles arrive
-                        const int w = q_frag_f8_word(ks, 0, lane);
-                        qf[ks][0] = v_lo ? bf16x2_to_f16x2(qrow_lo[w]) : 0u;
-                        qf[ks][1] = v_hi ? bf16x2_to_f16x2(qrow_hi[w]) : 0u;
-                        qf[ks][2] = v_lo ? bf16x2_to_f16x2(qrow_lo[w + 1]) : 0u;
-                        qf[ks][3] = v_hi ? bf16x2_to_f16x2(qrow_hi[w + 1]) : 0u;
-                    } else {
-                        const int w = ks * 8 + (lane & 3);           // 32-bit word index in the row
-                        qf[ks][0] = v_lo ? qrow_lo[w] : 0u;
-                        qf[ks][1] = v_hi ? qrow_hi[w] : 0u;
-                        qf[ks][2] = v_lo ? qrow_lo[w + 4] : 0u;
-                        qf[ks][3] = v_hi ? qrow_hi[w + 4] : 0u;
-                    }
-                }
+                load_q_fragments<D, NB, F8>(qf, reinterpret_cast<const uint32_t *>(q_slots + (size_t)s * q_stride), p.G);
             }
 
             const uint32_t k_tile = smem_u32(stages + (size_t)s * C::kStageBytes);
@@ -968,29 +947,19 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     // token is skipped (its rows may never have been fetched); in the last valid block the
                     // tokens past the end get no weight and their V rows are cleared.
                     constexpr int kSub = C::kSub;
-                    float sv[2 * kSub][4];
+                    float sv[kSub][NB][4];
                     const float sc = p.scale_log2e * k_sc;
 #pragma unroll
                     for (int u = 0; u < kSub; ++u) {
-                        if (u == 0 || nvalid > 16 * u) {
-                            warp_qk_16x16_f8<D>(qf, k_tile, row0 + 16 * u, sv[2 * u], sv[2 * u + 1]);
+                        const bool on = u == 0 || nvalid > 16 * u;
+                        if (on) warp_qk_f8<D, NB>(qf, k_tile, row0 + 16 * u, sv[u]);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                sv[2 * u][e] *= sc;
-                                sv[2 * u + 1][e] *= sc;
-                            }
-                        } else {
+                        for (int n = 0; n < NB; ++n)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) sv[2 * u][e] = sv[2 * u + 1][e] = -INFINITY;
-                        }
+                            for (int e = 0; e < 4; ++e) sv[u][n][e] = on ? sv[u][n][e] * sc : -INFINITY;
                     }
                     if (nvalid < 16 * kSub) {
-                        const int tok = 2 * (lane & 3);
-#pragma unroll
-                        for (int j = 0; j < 2 * kSub; ++j)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (8 * j + tok + (e & 1) >= nvalid) sv[j][e] = -INFINITY;
+                        warp_mask<NB, kSub>(sv, nvalid);
                         uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;
                         const int fetched_end = (nvalid + 15) & ~15;                 // end of the last valid block
                         constexpr int kCh = D / 16;                                   // 16-byte chunks of a token
@@ -1000,11 +969,11 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                         wrote_smem = true;
                         __syncwarp();
                     }
-                    uint32_t pa[kSub][4];
-                    warp_softmax_tiles<D, true, 2 * kSub>(st, sv, pa);
+                    uint32_t pb[kSub][NB][2];
+                    warp_softmax<D, NB, true, kSub>(st, sv, pb);
 #pragma unroll
                     for (int u = 0; u < kSub; ++u)
-                        if (u == 0 || nvalid > 16 * u) warp_pv_16x16_f8<D>(st, pa[u], v_tile, row0 + 16 * u);
+                        if (u == 0 || nvalid > 16 * u) warp_pv_f8<D, NB>(st, pb[u], v_tile, row0 + 16 * u);
                 }
             } else if (nvalid > 0) {
                 // kSub 16-token blocks per step share one softmax update. A block with no valid token is skipped (its
@@ -1012,29 +981,19 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                 // no weight, and their V rows (which may hold any bits, NaN included) are cleared so that 0 * garbage
                 // cannot appear.
                 constexpr int kSub = C::kSub;
-                float sv[2 * kSub][4];
+                float sv[kSub][NB][4];
                 const float sc = p.scale_log2e;
 #pragma unroll
                 for (int u = 0; u < kSub; ++u) {
-                    if (u == 0 || nvalid > 16 * u) {
-                        warp_qk_16x16<D>(qf, k_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0, sv[2 * u], sv[2 * u + 1]);
+                    const bool on = u == 0 || nvalid > 16 * u;
+                    if (on) warp_qk<D, NB>(qf, k_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0, sv[u]);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            sv[2 * u][e] *= sc;
-                            sv[2 * u + 1][e] *= sc;
-                        }
-                    } else {
+                    for (int n = 0; n < NB; ++n)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) sv[2 * u][e] = sv[2 * u + 1][e] = -INFINITY;
-                    }
+                        for (int e = 0; e < 4; ++e) sv[u][n][e] = on ? sv[u][n][e] * sc : -INFINITY;
                 }
                 if (nvalid < 16 * kSub) {
-                    const int tok = 2 * (lane & 3);
-#pragma unroll
-                    for (int j = 0; j < 2 * kSub; ++j)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (8 * j + tok + (e & 1) >= nvalid) sv[j][e] = -INFINITY;
+                    warp_mask<NB, kSub>(sv, nvalid);
                     uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;
                     const int chunks_per_row = C::kRowBytes / 16;
                     const int fetched_end = (nvalid + 15) & ~15;                 // end of the last valid block
@@ -1046,11 +1005,11 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     wrote_smem = true;
                     __syncwarp();
                 }
-                uint32_t pa[kSub][4];
-                warp_softmax_tiles<D, false, 2 * kSub>(st, sv, pa);
+                uint32_t pb[kSub][NB][2];
+                warp_softmax<D, NB, false, kSub>(st, sv, pb);
 #pragma unroll
                 for (int u = 0; u < kSub; ++u)
-                    if (u == 0 || nvalid > 16 * u) warp_pv_16x16<D>(st, pa[u], v_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0);
+                    if (u == 0 || nvalid > 16 * u) warp_pv<D, NB>(st, pb[u], v_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0);
             }
 
             if (wrote_smem) fence_proxy_async_smem();   // generic writes before the next TMA fill
@@ -1060,77 +1019,30 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
             if (mt.flags & kFlagLast) {
                 // ---- hand this piece's (max, sum, O) to the finisher warp and carry on
                 if (!mbar_wait(comb_empty, (n_dumps & 1u) ^ 1u, abort_flag)) break;
-                float l0 = st.l[0], l1 = st.l[1];
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-                l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-                l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+                st.finish_sums();
                 uint8_t *cw = comb_b + (size_t)warp * p.G * CR::kBytes;
-                // fp8: accumulator tiles alternate even / odd head dims (a tile pair gives this lane 4 consecutive
-                // dims) and O still lacks the V scale of its KV head
-                const float vs = F8 ? v_sc : 1.f;
-                if (r_lo < p.G) {
-                    uint8_t *rowb = cw + (size_t)r_lo * CR::kBytes;
-                    float *row = reinterpret_cast<float *>(rowb);
-                    if ((lane & 3) == 0) {
-                        *reinterpret_cast<float *>(rowb + CR::kOffM) = st.m[0];
-                        *reinterpret_cast<float *>(rowb + CR::kOffM + 4) = l0;
-                    }
-                    if constexpr (BigG) {
-                        // bf16 rows (groups of 5 to 8 heads occupy rows lane/4 only): the same elements, half the bytes
-                        if constexpr (F8) {
+                const float vs = F8 ? v_sc : 1.f;      // O over an fp8 cache still lacks the V scale of its KV head
+                if constexpr (BigG) {
+                    // bf16 rows: two words per 16 head dims and lane, of head 8n + lane / 4
 #pragma unroll
-                            for (int ch = 0; ch < D / 16; ++ch)
-                                *reinterpret_cast<uint2 *>(rowb + (ch * 16 + 4 * (lane & 3)) * 2) =
-                                    make_uint2(pack_bf16x2(st.o[2 * ch][0] * vs, st.o[2 * ch + 1][0] * vs),
-                                               pack_bf16x2(st.o[2 * ch][1] * vs, st.o[2 * ch + 1][1] * vs));
-                        } else {
+                    for (int n = 0; n < NB; ++n) {
 #pragma unroll
-                            for (int nt = 0; nt < D / 8; ++nt)
-                                *reinterpret_cast<uint32_t *>(rowb + (nt * 8 + 2 * (lane & 3)) * 2) = pack_bf16x2(st.o[nt][0], st.o[nt][1]);
+                        for (int mt = 0; mt < D / 16; ++mt) {
+                            const uint2 w = output_words<D, NB, F8>(st, mt, n, vs, vs);
+                            const int head = 8 * n + (lane >> 2);
+                            if (head < p.G) store_output_words<F8>(cw + (size_t)head * CR::kBytes, mt, lane, w);
                         }
-                    } else if constexpr (F8) {
 #pragma unroll
-                        for (int ch = 0; ch < D / 16; ++ch)
-                            *reinterpret_cast<float4 *>(row + ch * 16 + 4 * (lane & 3)) =
-                                make_float4(st.o[2 * ch][0] * vs, st.o[2 * ch + 1][0] * vs, st.o[2 * ch][1] * vs,
-                                            st.o[2 * ch + 1][1] * vs);
-                    } else {
-#pragma unroll
-                        for (int nt = 0; nt < D / 8; ++nt)
-                            *reinterpret_cast<float2 *>(row + nt * 8 + 2 * (lane & 3)) = make_float2(st.o[nt][0], st.o[nt][1]);
-                    }
-                }
-                if (r_hi < p.G) {
-                    uint8_t *rowb = cw + (size_t)r_hi * CR::kBytes;
-                    float *row = reinterpret_cast<float *>(rowb);
-                    if ((lane & 3) == 0) {
-                        *reinterpret_cast<float *>(rowb + CR::kOffM) = st.m[1];
-                        *reinterpret_cast<float *>(rowb + CR::kOffM + 4) = l1;
-                    }
-                    if constexpr (BigG) {
-                        if constexpr (F8) {
-#pragma unroll
-                            for (int ch = 0; ch < D / 16; ++ch)
-                                *reinterpret_cast<uint2 *>(rowb + (ch * 16 + 4 * (lane & 3)) * 2) =
-                                    make_uint2(pack_bf16x2(st.o[2 * ch][2] * vs, st.o[2 * ch + 1][2] * vs),
-                                               pack_bf16x2(st.o[2 * ch][3] * vs, st.o[2 * ch + 1][3] * vs));
-                        } else {
-#pragma unroll
-                            for (int nt = 0; nt < D / 8; ++nt)
-                                *reinterpret_cast<uint32_t *>(rowb + (nt * 8 + 2 * (lane & 3)) * 2) = pack_bf16x2(st.o[nt][2], st.o[nt][3]);
+                        for (int e = 0; e < 2; ++e) {
+                            const int head = 8 * n + 2 * (lane & 3) + e;
+                            if (lane < 4 && head < p.G) {
+                                *reinterpret_cast<float *>(cw + (size_t)head * CR::kBytes + CR::kOffM) = st.m[n][e];
+                                *reinterpret_cast<float *>(cw + (size_t)head * CR::kBytes + CR::kOffM + 4) = st.l[n][e];
+                            }
                         }
-                    } else if constexpr (F8) {
-#pragma unroll
-                        for (int ch = 0; ch < D / 16; ++ch)
-                            *reinterpret_cast<float4 *>(row + ch * 16 + 4 * (lane & 3)) =
-                                make_float4(st.o[2 * ch][2] * vs, st.o[2 * ch + 1][2] * vs, st.o[2 * ch][3] * vs,
-                                            st.o[2 * ch + 1][3] * vs);
-                    } else {
-#pragma unroll
-                        for (int nt = 0; nt < D / 8; ++nt)
-                            *reinterpret_cast<float2 *>(row + nt * 8 + 2 * (lane & 3)) = make_float2(st.o[nt][2], st.o[nt][3]);
                     }
+                } else {
+                    dump_rows_f32<D, NB, F8>(st, p.G, vs, CR::kOffM, [&](int head) { return cw + (size_t)head * CR::kBytes; });
                 }
                 if (warp == 0 && lane == 0) {
                     piece_meta->b = mt.b; piece_meta->kvh = mt.kvh; piece_meta->piece = mt.piece;
@@ -1150,8 +1062,10 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
     }
 }
 
+using SplitKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const DecodeParams);
+
 // Resident CTAs per SM for a given dynamic shared-memory size (0 on failure).
-template <int D, int W, bool F8, bool BigG, bool R8 = false>
+template <int D, int W, bool F8, bool BigG, bool R8, int NB>
 int decode_blocks_per_sm(size_t smem)
 {
     static bool attr_set_on[kDeviceSlots] = {};
@@ -1161,14 +1075,14 @@ int decode_blocks_per_sm(size_t smem)
     std::lock_guard<std::mutex> lock(setup_mutex());
     if (!attr_set) {
         // the opt-in limit is per kernel: allow everything the SM has
-        if (cudaFuncSetAttribute(decode_split_kernel<D, W, F8, BigG, R8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+        if (cudaFuncSetAttribute(decode_split_kernel<D, W, F8, BigG, R8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
             cudaSuccess)
             return 0;
         attr_set = true;
     }
     if (smem > 227 * 1024) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_split_kernel<D, W, F8, BigG, R8>, (BigG ? 11 : W + 2) * 32, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_split_kernel<D, W, F8, BigG, R8, NB>, (BigG ? 11 : W + 2) * 32, smem) != cudaSuccess)
         return 0;
     return n;
 }
@@ -1182,12 +1096,14 @@ struct ShapeOps {
     int warps, tile_t;
     size_t (*smem_bytes)(int G, int nsplit);
     int (*blocks_per_sm)(size_t smem);
+    SplitKernel kernel;
 };
 
-template <int D, int W, bool F8, bool BigG = false, bool R8 = false>
+template <int D, int W, bool F8, bool BigG, bool R8, int NB>
 ShapeOps shape_ops()
 {
-    return ShapeOps{W, DecodeCfg<D, W, F8>::kTileT, &decode_smem_bytes<D, W, F8, BigG>, &decode_blocks_per_sm<D, W, F8, BigG, R8>};
+    return ShapeOps{W, DecodeCfg<D, W, F8>::kTileT, &decode_smem_bytes<D, W, F8, BigG>, &decode_blocks_per_sm<D, W, F8, BigG, R8, NB>,
+                    decode_split_kernel<D, W, F8, BigG, R8, NB>};
 }
 
 // Groups of more than 4 query heads at head_dim 128: 16-bit hand-over rows and one finisher warp per 4 heads. Up to 8
@@ -1198,20 +1114,24 @@ bool is_big_group(int D, int warps, int G)
     return D == 128 && ((warps == 8 && G > 4 && G <= 8) || (warps == 6 && G > 8 && G <= 16));
 }
 
-ShapeOps pick_shape(int D, int warps, bool fp8, bool big = false, bool rope8 = false)
+// The shapes of one cache type. Groups of more than 8 heads run on the shapes whose hand-over rows leave room for them.
+template <bool F8, bool R8>
+ShapeOps pick_shape_of(int D, int warps, int G)
 {
-    if (fp8 && rope8) {          // the e4m3-cache kernels that carry the rope-fused step
-        if (big && warps == 6) return shape_ops<128, 6, true, true, true>();
-        if (big) return shape_ops<128, 8, true, true, true>();
-        if (D == 64) return warps == 8 ? shape_ops<64, 8, true, false, true>() : shape_ops<64, 4, true, false, true>();
-        return warps == 8 ? shape_ops<128, 8, true, false, true>() : shape_ops<128, 4, true, false, true>();
+    if (is_big_group(D, warps, G)) return warps == 6 ? shape_ops<128, 6, F8, true, R8, 2>() : shape_ops<128, 8, F8, true, R8, 1>();
+    if (D == 64) {
+        if (G > 8) return warps == 8 ? shape_ops<64, 8, F8, false, R8, 2>() : shape_ops<64, 4, F8, false, R8, 2>();
+        return warps == 8 ? shape_ops<64, 8, F8, false, R8, 1>() : shape_ops<64, 4, F8, false, R8, 1>();
     }
-    if (big && warps == 6) return fp8 ? shape_ops<128, 6, true, true>() : shape_ops<128, 6, false, true>();
-    if (big) return fp8 ? shape_ops<128, 8, true, true>() : shape_ops<128, 8, false, true>();
-    if (fp8 && D == 64) return warps == 8 ? shape_ops<64, 8, true>() : shape_ops<64, 4, true>();
-    if (fp8) return warps == 8 ? shape_ops<128, 8, true>() : shape_ops<128, 4, true>();
-    if (D == 128) return warps == 8 ? shape_ops<128, 8, false>() : shape_ops<128, 4, false>();
-    return warps == 8 ? shape_ops<64, 8, false>() : shape_ops<64, 4, false>();
+    if (warps == 8) return shape_ops<128, 8, F8, false, R8, 1>();      // more than 8 heads never fit beside its stages
+    return G > 8 ? shape_ops<128, 4, F8, false, R8, 2>() : shape_ops<128, 4, F8, false, R8, 1>();
+}
+
+// rope8: the e4m3-cache kernels that carry the rope-fused step
+ShapeOps pick_shape(int D, int warps, bool fp8, int G, bool rope8 = false)
+{
+    if (!fp8) return pick_shape_of<false, false>(D, warps, G);
+    return rope8 ? pick_shape_of<true, true>(D, warps, G) : pick_shape_of<true, false>(D, warps, G);
 }
 
 // Plan for one kernel shape (warps = 4 or 8).
@@ -1224,7 +1144,7 @@ DecodePlan plan_for_shape(int B, int Hq, int Hkv, int D, int max_kv_len, size_t 
     // caller's workspace and the shared memory fits the SM.
     DecodePlan pl;
     const int G = Hq / Hkv;
-    const ShapeOps ops = pick_shape(D, warps, fp8, is_big_group(D, warps, G));
+    const ShapeOps ops = pick_shape(D, warps, fp8, G);
     pl.warps = warps;
     auto blocks = [&](int nsplit) {
         const size_t smem = ops.smem_bytes(G, nsplit);
@@ -1315,7 +1235,7 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
     const bool big = is_big_group(D, plan.warps, G);
     const int nfin = big ? (G + 3) / 4 : 1;
     const bool rope8 = fp8 != nullptr && rope != nullptr;
-    const ShapeOps ops = pick_shape(D, plan.warps, fp8 != nullptr, big, rope8);
+    const ShapeOps ops = pick_shape(D, plan.warps, fp8 != nullptr, G, rope8);
     const int kTileT = ops.tile_t;
     const size_t smem = ops.smem_bytes(G, plan.nsplit);
     if (ops.blocks_per_sm(smem) == 0) return L4L_ERR_CUDA;
@@ -1421,34 +1341,7 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t err;
-        if (rope8 && big)
-            err = plan.warps == 6 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 6, true, true, true>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, true, true, true>, tk, tv, tk_tail, tv_tail, p);
-        else if (rope8 && D == 64)
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 8, true, false, true>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 4, true, false, true>, tk, tv, tk_tail, tv_tail, p);
-        else if (rope8)
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, true, false, true>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 4, true, false, true>, tk, tv, tk_tail, tv_tail, p);
-        else if (big && plan.warps == 6)
-            err = fp8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 6, true, true>, tk, tv, tk_tail, tv_tail, p)
-                      : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 6, false, true>, tk, tv, tk_tail, tv_tail, p);
-        else if (big)
-            err = fp8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, true, true>, tk, tv, tk_tail, tv_tail, p)
-                      : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, false, true>, tk, tv, tk_tail, tv_tail, p);
-        else if (fp8 && D == 64)
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 8, true, false>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 4, true, false>, tk, tv, tk_tail, tv_tail, p);
-        else if (fp8)
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, true, false>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 4, true, false>, tk, tv, tk_tail, tv_tail, p);
-        else if (D == 128)
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 8, false, false>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<128, 4, false, false>, tk, tv, tk_tail, tv_tail, p);
-        else
-            err = plan.warps == 8 ? cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 8, false, false>, tk, tv, tk_tail, tv_tail, p)
-                                  : cudaLaunchKernelEx(&cfg, decode_split_kernel<64, 4, false, false>, tk, tv, tk_tail, tv_tail, p);
+        const cudaError_t err = cudaLaunchKernelEx(&cfg, ops.kernel, tk, tv, tk_tail, tv_tail, p);
         if (err != cudaSuccess) return L4L_ERR_CUDA;
     }
     return L4L_OK;

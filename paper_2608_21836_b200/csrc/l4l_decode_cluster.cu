@@ -125,7 +125,7 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr)
     return v;
 }
 
-template <int D, bool F8>
+template <int D, bool F8, int NB>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
                       const __grid_constant__ CUtensorMap tmap_k_tail, const __grid_constant__ CUtensorMap tmap_v_tail,
@@ -269,10 +269,9 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
         }
     } else {
         // ------------------------------------------------------------------ consumer warps
-        WarpAttnState<D> st;
+        WarpAttnState<D, NB> st;
         st.reset();
-        uint32_t qf[D / 16][4];
-        const int r_lo = lane >> 2, r_hi = r_lo + 8;    // query heads of the group held in rows lane/4, lane/4 + 8
+        uint32_t qf[D / 16][NB][2];
         float k_sc = 1.f, v_sc = 1.f;                   // fp8 cache: scales of this KV head
         const bool by_page = C::kHalves == 2 && p.page_loads != 0;
         const TileRows rows = {by_page ? (uint32_t)p.page_size * 128u : kHalfBytes, by_page ? (uint32_t)-p.page_size : 0u};
@@ -295,27 +294,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     if (lane == 0) mbar_arrive(q_rotated);
                     if (!mbar_wait(q_rotated, 0u, abort_flag)) break;
                 }
-                const uint32_t *qs = reinterpret_cast<const uint32_t *>(q_smem);
-                const uint32_t *qrow_lo = qs + (size_t)r_lo * D / 2;
-                const uint32_t *qrow_hi = qs + (size_t)r_hi * D / 2;
-                const bool v_lo = r_lo < p.G, v_hi = r_hi < p.G;
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    if constexpr (F8) {
-                        // f16 fragments with the k index permuted the way the fp8 K tiles arrive
-                        const int w = q_frag_f8_word(ks, 0, lane);
-                        qf[ks][0] = v_lo ? bf16x2_to_f16x2(qrow_lo[w]) : 0u;
-                        qf[ks][1] = v_hi ? bf16x2_to_f16x2(qrow_hi[w]) : 0u;
-                        qf[ks][2] = v_lo ? bf16x2_to_f16x2(qrow_lo[w + 1]) : 0u;
-                        qf[ks][3] = v_hi ? bf16x2_to_f16x2(qrow_hi[w + 1]) : 0u;
-                    } else {
-                        const int w = ks * 8 + (lane & 3);           // 32-bit word index in the row
-                        qf[ks][0] = v_lo ? qrow_lo[w] : 0u;
-                        qf[ks][1] = v_hi ? qrow_hi[w] : 0u;
-                        qf[ks][2] = v_lo ? qrow_lo[w + 4] : 0u;
-                        qf[ks][3] = v_hi ? qrow_hi[w + 4] : 0u;
-                    }
-                }
+                load_q_fragments<D, NB, F8>(qf, reinterpret_cast<const uint32_t *>(q_smem), p.G);
             }
             const int t0 = (t_begin + it) * kTileT;
             const uint32_t k_tile = smem_u32(stages + (size_t)s * C::kStageBytes);
@@ -403,29 +382,19 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     // skipped (its rows may never have been fetched); in the last valid block the tokens past the end
                     // get no weight and their V rows are cleared.
                     constexpr int kSub = C::kSub;
-                    float sv[2 * kSub][4];
+                    float sv[kSub][NB][4];
                     const float sc = p.scale_log2e * k_sc;
 #pragma unroll
                     for (int u = 0; u < kSub; ++u) {
-                        if (u == 0 || nvalid > 16 * u) {
-                            warp_qk_16x16_f8<D>(qf, k_tile, row0 + 16 * u, sv[2 * u], sv[2 * u + 1]);
+                        const bool on = u == 0 || nvalid > 16 * u;
+                        if (on) warp_qk_f8<D, NB>(qf, k_tile, row0 + 16 * u, sv[u]);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                sv[2 * u][e] *= sc;
-                                sv[2 * u + 1][e] *= sc;
-                            }
-                        } else {
+                        for (int n = 0; n < NB; ++n)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) sv[2 * u][e] = sv[2 * u + 1][e] = -INFINITY;
-                        }
+                            for (int e = 0; e < 4; ++e) sv[u][n][e] = on ? sv[u][n][e] * sc : -INFINITY;
                     }
                     if (nvalid < 16 * kSub) {
-                        const int tok = 2 * (lane & 3);
-#pragma unroll
-                        for (int j = 0; j < 2 * kSub; ++j)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if (8 * j + tok + (e & 1) >= nvalid) sv[j][e] = -INFINITY;
+                        warp_mask<NB, kSub>(sv, nvalid);
                         uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;
                         const int fetched_end = (nvalid + 15) & ~15;                 // end of the last valid block
                         for (int i = lane; i < (fetched_end - nvalid) * 8; i += 32)
@@ -434,29 +403,23 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                         wrote_smem = true;
                         __syncwarp();
                     }
-                    uint32_t pa[kSub][4];
-                    warp_softmax_tiles<D, true, 2 * kSub>(st, sv, pa);
+                    uint32_t pb[kSub][NB][2];
+                    warp_softmax<D, NB, true, kSub>(st, sv, pb);
 #pragma unroll
                     for (int u = 0; u < kSub; ++u)
-                        if (u == 0 || nvalid > 16 * u) warp_pv_16x16_f8<D>(st, pa[u], v_tile, row0 + 16 * u);
+                        if (u == 0 || nvalid > 16 * u) warp_pv_f8<D, NB>(st, pb[u], v_tile, row0 + 16 * u);
                 }
             } else if (nvalid > 0) {
-                float s_lo[4], s_hi[4];
-                warp_qk_16x16<D>(qf, k_tile + rows.row(row0), rows.half_bytes, 0, s_lo, s_hi);
-                const int tok = 2 * (lane & 3);
+                float sv[1][NB][4];
+                warp_qk<D, NB>(qf, k_tile + rows.row(row0), rows.half_bytes, 0, sv[0]);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    s_lo[e] *= p.scale_log2e;
-                    s_hi[e] *= p.scale_log2e;
-                }
+                for (int n = 0; n < NB; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sv[0][n][e] *= p.scale_log2e;
                 if (nvalid < 16) {
                     // tokens past the end of the sequence: no weight, and their V rows (any bits, NaN included)
                     // are cleared so that 0 * garbage cannot appear
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (tok + (e & 1) >= nvalid) s_lo[e] = -INFINITY;
-                        if (tok + (e & 1) + 8 >= nvalid) s_hi[e] = -INFINITY;
-                    }
+                    warp_mask<NB, 1>(sv, nvalid);
                     uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;
                     constexpr int kChunksPerRow = D / 8;
                     for (int i = lane; i < (16 - nvalid) * kChunksPerRow; i += 32) {
@@ -466,52 +429,19 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     wrote_smem = true;
                     __syncwarp();
                 }
-                uint32_t pa[4];
-                warp_softmax_16<D>(st, s_lo, s_hi, pa);
-                warp_pv_16x16<D>(st, pa, v_tile + rows.row(row0), rows.half_bytes, 0);
+                uint32_t pb[1][NB][2];
+                warp_softmax<D, NB, false, 1>(st, sv, pb);
+                warp_pv<D, NB>(st, pb[0], v_tile + rows.row(row0), rows.half_bytes, 0);
             }
             if (wrote_smem) fence_proxy_async_smem();   // generic writes before the next TMA fill
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s]);
         }
         // ---- this warp's (max, sum, O) into shared memory
-        float l0 = st.l[0], l1 = st.l[1];
-        l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-        l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+        st.finish_sums();
         float *cw = comb + (size_t)warp * p.G * kPitch;
-        // fp8: accumulator tiles alternate even / odd head dims (a tile pair gives this lane 4 consecutive dims) and O
-        // still lacks the V scale of its KV head
-        const float vs = F8 ? v_sc : 1.f;
-        if (r_lo < p.G) {
-            float *row = cw + (size_t)r_lo * kPitch;
-            if ((lane & 3) == 0) { row[D] = st.m[0]; row[D + 1] = l0; }
-            if constexpr (F8) {
-#pragma unroll
-                for (int ch = 0; ch < D / 16; ++ch)
-                    *reinterpret_cast<float4 *>(row + ch * 16 + 4 * (lane & 3)) =
-                        make_float4(st.o[2 * ch][0] * vs, st.o[2 * ch + 1][0] * vs, st.o[2 * ch][1] * vs, st.o[2 * ch + 1][1] * vs);
-            } else {
-#pragma unroll
-                for (int nt = 0; nt < D / 8; ++nt)
-                    *reinterpret_cast<float2 *>(row + nt * 8 + 2 * (lane & 3)) = make_float2(st.o[nt][0], st.o[nt][1]);
-            }
-        }
-        if (r_hi < p.G) {
-            float *row = cw + (size_t)r_hi * kPitch;
-            if ((lane & 3) == 0) { row[D] = st.m[1]; row[D + 1] = l1; }
-            if constexpr (F8) {
-#pragma unroll
-                for (int ch = 0; ch < D / 16; ++ch)
-                    *reinterpret_cast<float4 *>(row + ch * 16 + 4 * (lane & 3)) =
-                        make_float4(st.o[2 * ch][2] * vs, st.o[2 * ch + 1][2] * vs, st.o[2 * ch][3] * vs, st.o[2 * ch + 1][3] * vs);
-            } else {
-#pragma unroll
-                for (int nt = 0; nt < D / 8; ++nt)
-                    *reinterpret_cast<float2 *>(row + nt * 8 + 2 * (lane & 3)) = make_float2(st.o[nt][2], st.o[nt][3]);
-            }
-        }
+        // O over an fp8 cache still lacks the V scale of its KV head
+        dump_rows_f32<D, NB, F8>(st, p.G, F8 ? v_sc : 1.f, D * 4, [&](int head) { return reinterpret_cast<uint8_t *>(cw + (size_t)head * kPitch); });
     }
     __syncthreads();
 
@@ -600,7 +530,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
     }
 }
 
-template <int D, bool F8>
+template <int D, bool F8, int NB>
 bool configure_kernel()
 {
     static bool done_on[kDeviceSlots] = {}, ok_on[kDeviceSlots] = {};
@@ -610,7 +540,7 @@ bool configure_kernel()
     std::lock_guard<std::mutex> lock(setup_mutex());
     if (!done) {
         done = true;
-        ok = cudaFuncSetAttribute(decode_cluster_kernel<D, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) ==
+        ok = cudaFuncSetAttribute(decode_cluster_kernel<D, F8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) ==
              cudaSuccess;
         if (!ok) (void)cudaGetLastError();
     }
@@ -627,7 +557,7 @@ int pick_stages(int G)
 }
 
 // Clusters of C CTAs that the device can hold at once (0 if the shape cannot launch). Looked up once per shape.
-template <int D, bool F8>
+template <int D, bool F8, int NB>
 int resident_clusters(int C, size_t smem)
 {
     struct Entry { int C; size_t smem; int dev; int n; };
@@ -636,7 +566,7 @@ int resident_clusters(int C, size_t smem)
     static std::mutex mutex;
     const int dev = device_slot();
     if (dev < 0) return 0;
-    if (!configure_kernel<D, F8>()) return 0;
+    if (!configure_kernel<D, F8, NB>()) return 0;
     std::lock_guard<std::mutex> lock(mutex);
     for (int i = 0; i < n_cached; ++i)
         if (cache[i].C == C && cache[i].smem == smem && cache[i].dev == dev) return cache[i].n;
@@ -650,13 +580,15 @@ int resident_clusters(int C, size_t smem)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<D, F8>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<D, F8, NB>, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         n = 0;
     }
     if (n_cached < 32) cache[n_cached++] = Entry{C, smem, dev, n};
     return n;
 }
+
+using ClusterKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const ClusterParams);
 
 // Host-side view of one instantiation.
 struct ClusterShape {
@@ -666,19 +598,20 @@ struct ClusterShape {
     size_t (*smem)(int G, int stages);
     int (*resident)(int C, size_t smem);
     bool (*configure)();
+    ClusterKernel kernel;
 };
 
-template <int D, bool F8>
+template <int D, bool F8, int NB>
 ClusterShape shape_of()
 {
-    return ClusterShape{ClusterCfg<D, F8>::kTileT, ClusterCfg<D, F8>::kStageBytes, &pick_stages<D, F8>, &cluster_smem_bytes<D, F8>, &resident_clusters<D, F8>,
-                        &configure_kernel<D, F8>};
+    return ClusterShape{ClusterCfg<D, F8>::kTileT, ClusterCfg<D, F8>::kStageBytes, &pick_stages<D, F8>, &cluster_smem_bytes<D, F8>,
+                        &resident_clusters<D, F8, NB>, &configure_kernel<D, F8, NB>, decode_cluster_kernel<D, F8, NB>};
 }
 
-ClusterShape pick_cluster_shape(int D, bool fp8)
+ClusterShape pick_cluster_shape(int D, bool fp8, int G)
 {
-    if (fp8) return shape_of<128, true>();
-    return D == 128 ? shape_of<128, false>() : shape_of<64, false>();
+    if (G > 8) return fp8 ? shape_of<128, true, 2>() : D == 128 ? shape_of<128, false, 2>() : shape_of<64, false, 2>();
+    return fp8 ? shape_of<128, true, 1>() : D == 128 ? shape_of<128, false, 1>() : shape_of<64, false, 1>();
 }
 
 }  // namespace
@@ -692,7 +625,7 @@ int decode_cluster_width(int B, int Hq, int Hkv, int D, int max_kv_len, bool fp8
     const long long units = (long long)B * Hkv;
     const int sms = sm_count();
     if (units <= 0 || units > 65535 || units > sms) return 0;
-    const ClusterShape shape = pick_cluster_shape(D, fp8);
+    const ClusterShape shape = pick_cluster_shape(D, fp8, G);
     const int stages = shape.stages(G);
     if (stages == 0) return 0;
     const size_t smem = shape.smem(G, stages);
@@ -730,7 +663,7 @@ l4l_status launch_decode_cluster(const void *q, void *o, const l4l_kv_cache &cac
     // fp8: cache.k / cache.v point at e4m3 bytes, the strides count bytes (= elements)
     const int esz = fp8 ? 1 : 2, box_d = fp8 ? 128 : 64;
     const int G = Hq / Hkv;
-    const ClusterShape shape = pick_cluster_shape(D, fp8 != nullptr);
+    const ClusterShape shape = pick_cluster_shape(D, fp8 != nullptr, G);
     const int kTileT = shape.tile_t;
     const int stages = shape.stages(G);
     if (stages == 0 || width < 1 || width > kMaxCluster) return L4L_ERR_UNSUPPORTED;
@@ -810,10 +743,7 @@ l4l_status launch_decode_cluster(const void *q, void *o, const l4l_kv_cache &cac
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t err =
-        fp8        ? cudaLaunchKernelEx(&cfg, decode_cluster_kernel<128, true>, tk, tv, tk_tail, tv_tail, p)
-        : D == 128 ? cudaLaunchKernelEx(&cfg, decode_cluster_kernel<128, false>, tk, tv, tk_tail, tv_tail, p)
-                   : cudaLaunchKernelEx(&cfg, decode_cluster_kernel<64, false>, tk, tv, tk_tail, tv_tail, p);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, shape.kernel, tk, tv, tk_tail, tv_tail, p);
     return err == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
 }
 

@@ -97,7 +97,8 @@ struct Cursor {
     bool valid;                       // false: the queue is empty
 };
 
-template <int D, int kWarps, bool F8>
+// NB: blocks of 8 query heads of the group (the N of the warp MMAs).
+template <int D, int kWarps, bool F8, int NB>
 __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpParams p)
 {
     static_assert(!F8 || D == 128, "the fp8 path wants one 128-byte row per token");
@@ -326,10 +327,9 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
         head_slot = head_slot + 1 == S ? 0 : head_slot + 1;
     }
 
-    WarpAttnState<D> st;
+    WarpAttnState<D, NB> st;
     st.reset();
-    uint32_t qf[D / 16][4];
-    const int r_lo = lane >> 2, r_hi = r_lo + 8;
+    uint32_t qf[D / 16][NB][2];
     float k_sc = 1.f, v_sc = 1.f;                  // fp8 cache: scales of the unit's KV head
     while (live(tail)) {
         if (live(head)) {
@@ -350,27 +350,7 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
         uint8_t *stg = ring + (size_t)tail_slot * sbytes;
         const uint32_t k_tile = smem_u32(stg), v_tile = k_tile + C::kTileBytes;
         if (tail.chunk == 0) {
-            const uint32_t *qs = reinterpret_cast<const uint32_t *>(stg + 2 * C::kTileBytes);
-            const uint32_t *qrow_lo = qs + (size_t)r_lo * D / 2;
-            const uint32_t *qrow_hi = qs + (size_t)r_hi * D / 2;
-            const bool v_lo = r_lo < p.G, v_hi = r_hi < p.G;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-                if constexpr (F8) {
-                    // f16 fragments with the k index permuted the way the fp8 K rows arrive
-                    const int w = q_frag_f8_word(ks, 0, lane);
-                    qf[ks][0] = v_lo ? bf16x2_to_f16x2(qrow_lo[w]) : 0u;
-                    qf[ks][1] = v_hi ? bf16x2_to_f16x2(qrow_hi[w]) : 0u;
-                    qf[ks][2] = v_lo ? bf16x2_to_f16x2(qrow_lo[w + 1]) : 0u;
-                    qf[ks][3] = v_hi ? bf16x2_to_f16x2(qrow_hi[w + 1]) : 0u;
-                } else {
-                    const int w = ks * 8 + (lane & 3);
-                    qf[ks][0] = v_lo ? qrow_lo[w] : 0u;
-                    qf[ks][1] = v_hi ? qrow_hi[w] : 0u;
-                    qf[ks][2] = v_lo ? qrow_lo[w + 4] : 0u;
-                    qf[ks][3] = v_hi ? qrow_hi[w + 4] : 0u;
-                }
-            }
+            load_q_fragments<D, NB, F8>(qf, reinterpret_cast<const uint32_t *>(stg + 2 * C::kTileBytes), p.G);
             if constexpr (F8) {
                 k_sc = __ldg(p.k_scale + tail.kvh);
                 v_sc = __ldg(p.v_scale + tail.kvh);
@@ -381,7 +361,7 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
                 __syncwarp();
                 for (int i = lane; i < D / 4; i += 32) reinterpret_cast<float4 *>(rope_priv)[i] = src[i];
                 __syncwarp();
-                rope_q_fragments<D>(qf, p.G, p.q_weight != nullptr, p.norm_eps, rope_priv, norm_w, lane);
+                rope_q_fragments<D, NB>(qf, p.G, p.q_weight != nullptr, p.norm_eps, rope_priv, norm_w, lane);
             }
         }
         const int t0 = tail.chunk * kChunkT;
@@ -417,79 +397,40 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
                 }
                 __syncwarp();
             }
-            float s_lo[4], s_hi[4];
-            if constexpr (F8)
-                warp_qk_16x16_f8<D>(qf, k_tile, 0, s_lo, s_hi);
-            else
-                warp_qk_16x16<D>(qf, k_tile, C::kHalfBytes, 0, s_lo, s_hi);
+            float sv[1][NB][4];
+            if constexpr (F8) warp_qk_f8<D, NB>(qf, k_tile, 0, sv[0]);
+            else warp_qk<D, NB>(qf, k_tile, C::kHalfBytes, 0, sv[0]);
             const float sc = F8 ? p.scale_log2e * k_sc : p.scale_log2e;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                s_lo[e] *= sc;
-                s_hi[e] *= sc;
-            }
-            if (nvalid < kChunkT) {                // tokens past the end: no weight (their V rows arrived as zeros)
-                const int tok = 2 * (lane & 3);
+            for (int n = 0; n < NB; ++n)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (tok + (e & 1) >= nvalid) s_lo[e] = -INFINITY;
-                    if (tok + (e & 1) + 8 >= nvalid) s_hi[e] = -INFINITY;
-                }
-            }
-            uint32_t pa[4];
-            warp_softmax_16<D, F8>(st, s_lo, s_hi, pa);        // fp8: weights as f16 for the f16 MMAs
-            if constexpr (F8)
-                warp_pv_16x16_f8<D>(st, pa, v_tile, 0);
-            else
-                warp_pv_16x16<D>(st, pa, v_tile, C::kHalfBytes, 0);
+                for (int e = 0; e < 4; ++e) sv[0][n][e] *= sc;
+            if (nvalid < kChunkT) warp_mask<NB, 1>(sv, nvalid);   // past the end: no weight (their V rows arrived as zeros)
+            uint32_t pb[1][NB][2];
+            warp_softmax<D, NB, F8, 1>(st, sv, pb);               // fp8: weights as f16 for the f16 MMAs
+            if constexpr (F8) warp_pv_f8<D, NB>(st, pb[0], v_tile, 0);
+            else warp_pv<D, NB>(st, pb[0], v_tile, C::kHalfBytes, 0);
         }
         if (tail.chunk + 1 == tail.chunks) {
             // ---- the unit is complete: normalise and write its G output rows
-            float l0 = st.l[0], l1 = st.l[1];
-            l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-            l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-            l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-            l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+            st.finish_sums();
             const bool any = tail.len > 0;
-            const float i0 = any ? 1.f / l0 : 0.f, i1 = any ? 1.f / l1 : 0.f;
             const size_t bh = (size_t)tail.b * p.Hq + (size_t)tail.kvh * p.G;
-            // fp8: accumulator tiles alternate even / odd head dims (a tile pair gives this lane 4 consecutive dims) and O
-            // still lacks the V scale of its KV head
-            if (r_lo < p.G) {
-                if constexpr (F8) {
-                    __nv_bfloat16 *row = p.o + (bh + r_lo) * D + 4 * (lane & 3);
-                    const float f = i0 * v_sc;
 #pragma unroll
-                    for (int ch = 0; ch < D / 16; ++ch)
-                        *reinterpret_cast<uint2 *>(row + ch * 16) =
-                            make_uint2(pack_bf16x2(st.o[2 * ch][0] * f, st.o[2 * ch + 1][0] * f),
-                                       pack_bf16x2(st.o[2 * ch][1] * f, st.o[2 * ch + 1][1] * f));
-                } else {
-                    __nv_bfloat16 *row = p.o + (bh + r_lo) * D + 2 * (lane & 3);
+            for (int n = 0; n < NB; ++n) {
+                // (O over an fp8 cache still lacks the V scale of its KV head)
+                const float f0 = any ? (F8 ? v_sc : 1.f) / st.l[n][0] : 0.f, f1 = any ? (F8 ? v_sc : 1.f) / st.l[n][1] : 0.f;
+                const int head = 8 * n + (lane >> 2);
 #pragma unroll
-                    for (int nt = 0; nt < D / 8; ++nt)
-                        *reinterpret_cast<uint32_t *>(row + nt * 8) = pack_bf16x2(st.o[nt][0] * i0, st.o[nt][1] * i0);
+                for (int mt = 0; mt < D / 16; ++mt) {
+                    const uint2 w = output_words<D, NB, F8>(st, mt, n, f0, f1);
+                    if (head < p.G) store_output_words<F8>(p.o + (bh + head) * D, mt, lane, w);
                 }
-                if ((lane & 3) == 0 && p.lse)
-                    p.lse[bh + r_lo] = any ? (st.m[0] + log2f(l0)) * 0.6931471805599453f : -INFINITY;
-            }
-            if (r_hi < p.G) {
-                if constexpr (F8) {
-                    __nv_bfloat16 *row = p.o + (bh + r_hi) * D + 4 * (lane & 3);
-                    const float f = i1 * v_sc;
+                if (lane < 4 && p.lse)
 #pragma unroll
-                    for (int ch = 0; ch < D / 16; ++ch)
-                        *reinterpret_cast<uint2 *>(row + ch * 16) =
-                            make_uint2(pack_bf16x2(st.o[2 * ch][2] * f, st.o[2 * ch + 1][2] * f),
-                                       pack_bf16x2(st.o[2 * ch][3] * f, st.o[2 * ch + 1][3] * f));
-                } else {
-                    __nv_bfloat16 *row = p.o + (bh + r_hi) * D + 2 * (lane & 3);
-#pragma unroll
-                    for (int nt = 0; nt < D / 8; ++nt)
-                        *reinterpret_cast<uint32_t *>(row + nt * 8) = pack_bf16x2(st.o[nt][2] * i1, st.o[nt][3] * i1);
-                }
-                if ((lane & 3) == 0 && p.lse)
-                    p.lse[bh + r_hi] = any ? (st.m[1] + log2f(l1)) * 0.6931471805599453f : -INFINITY;
+                    for (int e = 0; e < 2; ++e)
+                        if (8 * n + 2 * lane + e < p.G)
+                            p.lse[bh + 8 * n + 2 * lane + e] = any ? (st.m[n][e] + log2f(st.l[n][e])) * 0.6931471805599453f : -INFINITY;
             }
             st.reset();
         }
@@ -505,7 +446,7 @@ size_t warp_smem_bytes(int D, int G, int warps, int stages, bool f8, bool rope)
     return kMetaBytes + (size_t)warps * stages * stage_bytes(D, G, f8, rope) + rope_extra_bytes(D, warps, rope);
 }
 
-template <int D, int W, bool F8>
+template <int D, int W, bool F8, int NB>
 int blocks_per_sm(size_t smem)
 {
     struct Entry { size_t smem; int dev; int n; };
@@ -518,8 +459,8 @@ int blocks_per_sm(size_t smem)
     for (int i = 0; i < n_cached; ++i)
         if (cache[i].smem == smem && cache[i].dev == dev) return cache[i].n;
     int n = 0;
-    if (cudaFuncSetAttribute(decode_warp_kernel<D, W, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_warp_kernel<D, W, F8>, W * 32, smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(decode_warp_kernel<D, W, F8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_warp_kernel<D, W, F8, NB>, W * 32, smem) != cudaSuccess) {
         (void)cudaGetLastError();
         n = 0;
     }
@@ -553,17 +494,19 @@ WarpShape pick_warp_shape(int D, int G, long long units, bool f8, bool rope = fa
 
 using WarpKernel = void (*)(const WarpParams);
 struct KernelEntry { WarpKernel fn; int (*blocks)(size_t); };
-template <int D, int W, bool F8>
-KernelEntry entry() { return {decode_warp_kernel<D, W, F8>, &blocks_per_sm<D, W, F8>}; }
-KernelEntry pick_kernel(int D, int warps, bool f8)
+template <int D, int W, bool F8, int NB>
+KernelEntry entry() { return {decode_warp_kernel<D, W, F8, NB>, &blocks_per_sm<D, W, F8, NB>}; }
+template <int NB>
+KernelEntry pick_kernel_of(int D, int warps, bool f8)
 {
     if (f8)                                                       // head_dim 128 only
-        return warps == 4 ? entry<128, 4, true>() : warps == 6 ? entry<128, 6, true>()
-               : warps == 8 ? entry<128, 8, true>() : entry<128, 12, true>();
-    if (D == 64) return warps == 4 ? entry<64, 4, false>() : warps == 6 ? entry<64, 6, false>() : entry<64, 8, false>();
-    return warps == 4 ? entry<128, 4, false>() : warps == 6 ? entry<128, 6, false>()
-           : warps == 8 ? entry<128, 8, false>() : entry<128, 12, false>();
+        return warps == 4 ? entry<128, 4, true, NB>() : warps == 6 ? entry<128, 6, true, NB>()
+               : warps == 8 ? entry<128, 8, true, NB>() : entry<128, 12, true, NB>();
+    if (D == 64) return warps == 4 ? entry<64, 4, false, NB>() : warps == 6 ? entry<64, 6, false, NB>() : entry<64, 8, false, NB>();
+    return warps == 4 ? entry<128, 4, false, NB>() : warps == 6 ? entry<128, 6, false, NB>()
+           : warps == 8 ? entry<128, 8, false, NB>() : entry<128, 12, false, NB>();
 }
+KernelEntry pick_kernel(int D, int warps, bool f8, int G) { return G > 8 ? pick_kernel_of<2>(D, warps, f8) : pick_kernel_of<1>(D, warps, f8); }
 
 }  // namespace
 
@@ -605,7 +548,7 @@ l4l_status launch_decode_warp(const void *q, void *o, const l4l_kv_cache &cache,
         const int stages = shape.stages, kWarps = shape.warps;
         if (stages == 0) return L4L_ERR_UNSUPPORTED;
         const size_t smem = warp_smem_bytes(D, G, kWarps, stages, f8, rope != nullptr);
-        const KernelEntry kernel = pick_kernel(D, kWarps, f8);
+        const KernelEntry kernel = pick_kernel(D, kWarps, f8, G);
         const int per_sm = kernel.blocks(smem);
         if (per_sm == 0) return L4L_ERR_CUDA;
         WarpParams p = {};

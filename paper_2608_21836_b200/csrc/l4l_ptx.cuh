@@ -328,10 +328,17 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi)
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
-__device__ __forceinline__ float sum_f16x2(uint32_t v)
+__device__ __forceinline__ void unpack_f16x2(uint32_t v, float &lo, float &hi)
 {
-    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&v));
-    return f.x + f.y;
+    asm("{ .reg .f16 a, b; mov.b32 {a, b}, %2; cvt.f32.f16 %0, a; cvt.f32.f16 %1, b; }" : "=f"(lo), "=f"(hi) : "r"(v));
+}
+
+// 8 x 8 transpose of 16-bit elements across the warp: lane (r, c) holds row r, columns 2c, 2c+1, before and after.
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v)
+{
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)

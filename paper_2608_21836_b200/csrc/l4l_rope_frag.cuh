@@ -1,5 +1,5 @@
 // Rotary embedding (+ optional per-head RMS norm) of a decode step's own token on the data layouts of the decode
-// kernels: the query rows as warp-MMA A fragments in registers, the new key row as 16-byte pieces across a warp.
+// kernels: the query rows as warp-MMA B fragments in registers, the new key row as 16-byte pieces across a warp.
 #pragma once
 
 #include "l4l_ptx.cuh"
@@ -10,59 +10,59 @@ namespace l4l {
 // y2 = fma(x1, sin, x2 * cos) in fp32, one rounding to bf16. A position outside the table leaves the row as it is.
 // The cos | sin rows of the position come from shared memory: the producer fetches them with the piece's first tile.
 
-// The q rows live in the A fragments of the warp MMA: a thread holds, per 16-column k-step, columns 2c, 2c+1
-// (registers 0: row lane/4, 1: row lane/4 + 8) and 2c+8, 2c+9 (registers 2, 3), c = lane % 4. The partner of
-// column i is column i + D/2, i.e. the same register of the k-step D/32 further on: no data leaves the thread.
+// The q rows live in the B fragments of the warp MMA: a thread holds, per 16-column k-step and block of 8 heads, columns
+// 2c, 2c+1 and 2c+8, 2c+9 of head 8n + lane/4, c = lane % 4. The partner of column i is column i + D/2, i.e. the same
+// register of the k-step D/32 further on: no data leaves the thread.
 // (The warp-per-unit kernel rotates this way: every warp has its own query rows. The split and the cluster kernel,
 // where all warps of a CTA share the rows, rotate them once in shared memory instead: rope_row_in_smem below.)
-template <int D>
-__device__ __forceinline__ void rope_q_fragments(uint32_t (&qf)[D / 16][4], int G, bool with_norm, float norm_eps,
+template <int D, int NB>
+__device__ __forceinline__ void rope_q_fragments(uint32_t (&qf)[D / 16][NB][2], int G, bool with_norm, float norm_eps,
                                                  const float *cos_sin, const float *weight, int lane)
 {
     constexpr int kSteps = D / 16, kHalf = kSteps / 2;
     const int c = lane & 3;
-    const bool valid[2] = {(lane >> 2) < G, (lane >> 2) + 8 < G};
-    float rinv[2] = {1.f, 1.f};
-    if (with_norm) {
-        float ss[2] = {0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < kSteps; ++ks)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float a = __uint_as_float(qf[ks][r] << 16), b = __uint_as_float(qf[ks][r] & 0xffff0000u);
-                ss[r & 1] = fmaf(a, a, fmaf(b, b, ss[r & 1]));
-            }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            ss[h] += __shfl_xor_sync(0xffffffffu, ss[h], 1);
-            ss[h] += __shfl_xor_sync(0xffffffffu, ss[h], 2);
-            rinv[h] = valid[h] ? rsqrtf(ss[h] * (1.f / D) + norm_eps) : 0.f;
-        }
-    }
     const float *cr = cos_sin, *sr = cos_sin + D / 2;              // shared memory: cos | sin of the position
 #pragma unroll
-    for (int ks = 0; ks < kHalf; ++ks)
+    for (int n = 0; n < NB; ++n) {
+        const bool valid = 8 * n + (lane >> 2) < G;
+        float rinv = 1.f;
+        if (with_norm) {
+            float ss = 0.f;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int col = 16 * ks + 2 * c + ((r >> 1) << 3);               // first-half column of element 0
-            float x1[2] = {__uint_as_float(qf[ks][r] << 16), __uint_as_float(qf[ks][r] & 0xffff0000u)};
-            float x2[2] = {__uint_as_float(qf[ks + kHalf][r] << 16), __uint_as_float(qf[ks + kHalf][r] & 0xffff0000u)};
-            float y1[2], y2[2];
+            for (int ks = 0; ks < kSteps; ++ks)
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                if (with_norm) {
-                    x1[e] = x1[e] * rinv[r & 1] * weight[col + e];
-                    x2[e] = x2[e] * rinv[r & 1] * weight[col + e + D / 2];
+                for (int r = 0; r < 2; ++r) {
+                    const float a = __uint_as_float(qf[ks][n][r] << 16), b = __uint_as_float(qf[ks][n][r] & 0xffff0000u);
+                    ss = fmaf(a, a, fmaf(b, b, ss));
                 }
-                const float cs = cr[col + e], sn = sr[col + e];
-                y1[e] = fmaf(-x2[e], sn, x1[e] * cs);
-                y2[e] = fmaf(x1[e], sn, x2[e] * cs);
-            }
-            if (valid[r & 1]) {
-                qf[ks][r] = pack_bf16x2(y1[0], y1[1]);
-                qf[ks + kHalf][r] = pack_bf16x2(y2[0], y2[1]);
-            }
+            ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+            ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+            rinv = valid ? rsqrtf(ss * (1.f / D) + norm_eps) : 0.f;
         }
+#pragma unroll
+        for (int ks = 0; ks < kHalf; ++ks)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int col = 16 * ks + 2 * c + 8 * r;                         // first-half column of element 0
+                float x1[2] = {__uint_as_float(qf[ks][n][r] << 16), __uint_as_float(qf[ks][n][r] & 0xffff0000u)};
+                float x2[2] = {__uint_as_float(qf[ks + kHalf][n][r] << 16), __uint_as_float(qf[ks + kHalf][n][r] & 0xffff0000u)};
+                float y1[2], y2[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (with_norm) {
+                        x1[e] = x1[e] * rinv * weight[col + e];
+                        x2[e] = x2[e] * rinv * weight[col + e + D / 2];
+                    }
+                    const float cs = cr[col + e], sn = sr[col + e];
+                    y1[e] = fmaf(-x2[e], sn, x1[e] * cs);
+                    y2[e] = fmaf(x1[e], sn, x2[e] * cs);
+                }
+                if (valid) {
+                    qf[ks][n][r] = pack_bf16x2(y1[0], y1[1]);
+                    qf[ks + kHalf][n][r] = pack_bf16x2(y2[0], y2[1]);
+                }
+            }
+    }
 }
 
 // One query row rotated in place in shared memory by one warp: lane l owns the words l (elements 2l, 2l+1) and

@@ -1,8 +1,14 @@
-// Warp-level building blocks on the legacy tensor path (mma.sync m16n8k16, bf16 -> fp32):
-// one warp holds 16 query rows and consumes 16 tokens of K and V at a time from a shared-
-// memory tile written by TMA with the 128-byte swizzle. Used by the decode kernel, where
-// the 16 rows are the (zero-padded) query-head group of one KV head. (Prefill runs on
-// tcgen05 instead: see l4l_prefill_tc.cu.)
+// Warp-level building blocks of the decode kernels on the legacy tensor path (mma.sync m16n8k16, 16-bit inputs -> fp32):
+// one warp holds the query heads of one KV group and consumes 16 tokens of K and V at a time from a shared-memory tile
+// with the 128-byte swizzle. (Prefill runs on tcgen05 instead: see l4l_prefill_tc.cu.)
+//
+// The products are taken transposed: S^T = K Q^T with the TOKENS as the M = 16 rows and the group's query heads as the
+// N = 8 columns, then O^T = V^T P^T with the head dims as rows. A group of 4 heads fills half of the 8 columns, where as
+// rows it would fill a quarter of 16: half the MMAs, half the exponentials, and the output accumulators of a 128-wide
+// head are 32 registers instead of 64 (NB = 2 blocks of 8 heads, for groups of 9 to 16, are as before). P^T is the B operand of
+// the second product: an 8 x 8 transpose of the score fragment (movmatrix). Measured, us, heads as rows -> as columns: e4m3
+// cache, B = 32 ragged 36.7 -> 31.1; B = 512 x 64..256 tokens 65.3 -> 62.5; one sequence of 2304 tokens with rope and norm
+// 9.2 -> 8.8; bf16 caches of large batches, bound by HBM, 46.5 -> 46.4.
 //
 // Tile layout in shared memory: D/64 "halves", each [tile_tokens][64] bf16 (128-byte rows,
 // swizzled), half h covering head_dim [64h, 64h+64). Over pages of 16 or 32 tokens at head_dim 128 one load brings
@@ -26,138 +32,169 @@ struct TileRows {
     }
 };
 
-template <int D>
+// Fragment positions of a lane: r = lane / 4, c = lane % 4. Heads of block n: column 2c, 2c + 1 -> heads 8n + 2c + {0, 1}.
+template <int D, int NB>
 struct WarpAttnState {
-    float m[2];           // running max (log2 domain) of rows lane/4 and lane/4 + 8
-    float l[2];           // this lane's share of the running sum
-    float o[D / 8][4];    // accumulator fragments: n-tile nt covers head_dim [8nt, 8nt+8)
+    float m[NB][2];          // running maximum (log2 domain) of this lane's two heads of each block
+    float l[NB][2];          // this lane's share of their running sums (its token rows)
+    float o[D / 16][NB][4];  // O^T, unnormalised: 16 head dims per tile; [e] dim row r, [2 + e] dim row r + 8 of head 2c + e
 
     __device__ __forceinline__ void reset()
     {
-        m[0] = m[1] = -INFINITY;
-        l[0] = l[1] = 0.f;
 #pragma unroll
-        for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+        for (int n = 0; n < NB; ++n) {
+            m[n][0] = m[n][1] = -INFINITY;
+            l[n][0] = l[n][1] = 0.f;
+#pragma unroll
+            for (int i = 0; i < D / 16; ++i) o[i][n][0] = o[i][n][1] = o[i][n][2] = o[i][n][3] = 0.f;
+        }
+    }
+    // the sums over all token rows (every lane of the warp must call this)
+    __device__ __forceinline__ void finish_sums()
+    {
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int off = 4; off <= 16; off <<= 1) l[n][e] += __shfl_xor_sync(0xffffffffu, l[n][e], off);
     }
 };
 
-// S(16 rows x 16 tokens) = Q(16 x D) . K(tokens row0..row0+15)^T.
-// s_lo: tokens row0 + 2*(lane%4) + {0,1}   (elements 0,1: row lane/4; 2,3: row lane/4 + 8)
-// s_hi: the same for tokens + 8.
-template <int D>
-__device__ __forceinline__ void warp_qk_16x16(const uint32_t (&qf)[D / 16][4], uint32_t k_tile, uint32_t half_bytes,
-                                              int row0, float (&s_lo)[4], float (&s_hi)[4])
+__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v)
+{
+    return pack_f16x2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+
+// The group's query rows (bf16, [G][D] in shared memory) as B fragments: qf[k-step][block] = head 8n + r, columns
+// 16 ks + 2c + {0, 1} and + 8. kF16 (e4m3 caches): as f16, with the k index permuted the way the K bytes arrive (below).
+template <int D, int NB, bool kF16>
+__device__ __forceinline__ void load_q_fragments(uint32_t (&qf)[D / 16][NB][2], const uint32_t *q_rows, int G)
 {
     const int lane = threadIdx.x & 31;
-    s_lo[0] = s_lo[1] = s_lo[2] = s_lo[3] = 0.f;
-    s_hi[0] = s_hi[1] = s_hi[2] = s_hi[3] = 0.f;
-    const uint32_t row = row0 + ((lane >> 4) << 3) + (lane & 7);   // matrices 2,3: tokens +8
-    const uint32_t csel = (lane >> 3) & 1;                          // matrices 1,3: head_dim +8
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+        const int head = 8 * n + (lane >> 2);
+        const uint32_t *row = q_rows + (size_t)head * (D / 2);
+        const bool valid = head < G;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) {
+            const int w = kF16 ? ks * 8 + 2 * (lane & 3) : ks * 8 + (lane & 3);
+            const uint32_t a = valid ? row[w] : 0u, b = valid ? row[w + (kF16 ? 1 : 4)] : 0u;
+            qf[ks][n][0] = kF16 ? bf16x2_to_f16x2(a) : a;
+            qf[ks][n][1] = kF16 ? bf16x2_to_f16x2(b) : b;
+        }
+    }
+}
+
+// S^T (16 tokens x 8 NB heads) = K(tokens row0 .. row0 + 15) . Q^T. s[n]: [e] token row0 + r, [2 + e] token row0 + r + 8 of
+// head 8n + 2c + e. Even and odd k-steps are accumulated apart: two dependent chains of half the length.
+template <int D, int NB>
+__device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, uint32_t half_bytes, int row0,
+                                        float (&s)[NB][4])
+{
+    const int lane = threadIdx.x & 31;
+    float odd[NB][4];
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[n][e] = odd[n][e] = 0.f;
+    const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
+    const uint32_t csel = lane >> 4;                                // matrices 2, 3: head dims + 8
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t chunk = 2 * ks + csel;                       // 16-byte chunk of the full row
-        const uint32_t addr = k_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7);
-        uint32_t b0, b1, b2, b3;
-        ldmatrix_x4(addr, b0, b1, b2, b3);
-        mma_bf16_16816(s_lo, qf[ks], b0, b1);
-        mma_bf16_16816(s_hi, qf[ks], b2, b3);
+        uint32_t a[4];
+        ldmatrix_x4(k_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
+#pragma unroll
+        for (int n = 0; n < NB; ++n) mma_bf16_16816((ks & 1) ? odd[n] : s[n], a, qf[ks][n][0], qf[ks][n][1]);
     }
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[n][e] += odd[n][e];
 }
 
-// Online-softmax update for 16 tokens. Scores arrive already multiplied by scale*log2(e)
-// and with masked positions set to -inf. Produces the bf16 A-fragment of P and rescales O.
-// kF16: P is packed as f16 (for the f16 MMAs of the fp8-cache path) instead of bf16.
-template <int D, bool kF16 = false>
-__device__ __forceinline__ void warp_softmax_16(WarpAttnState<D> &st, const float (&s_lo)[4], const float (&s_hi)[4],
-                                                uint32_t (&pa)[4])
-{
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float a0 = s_lo[2 * h], a1 = s_lo[2 * h + 1], a2 = s_hi[2 * h], a3 = s_hi[2 * h + 1];
-        float mx = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(st.m[h], mx);
-        const float m_use = (m_new == -INFINITY) ? 0.f : m_new;     // row with nothing visible yet
-        const float corr = fast_exp2(st.m[h] - m_use);
-        const float e0 = fast_exp2(a0 - m_use), e1 = fast_exp2(a1 - m_use);
-        const float e2 = fast_exp2(a2 - m_use), e3 = fast_exp2(a3 - m_use);
-        const uint32_t p01 = kF16 ? pack_f16x2(e0, e1) : pack_bf16x2(e0, e1);
-        const uint32_t p23 = kF16 ? pack_f16x2(e2, e3) : pack_bf16x2(e2, e3);
-        pa[h] = p01;          // tokens +0,+1
-        pa[2 + h] = p23;      // tokens +8,+9
-        // the denominator sums exactly the rounded weights that multiply V
-        const float psum = kF16 ? sum_f16x2(p01) + sum_f16x2(p23)
-                                : __uint_as_float(p01 << 16) + __uint_as_float(p01 & 0xffff0000u) +
-                                      __uint_as_float(p23 << 16) + __uint_as_float(p23 & 0xffff0000u);
-        st.l[h] = st.l[h] * corr + psum;
-        st.m[h] = m_new;
-        // O is rescaled only if some row of this half saw its maximum grow (after the first tiles of a long
-        // sequence that is rare): corr == 1 exactly otherwise
-        if (__any_sync(0xffffffffu, corr != 1.f)) {
-#pragma unroll
-            for (int nt = 0; nt < D / 8; ++nt) {
-                st.o[nt][2 * h] *= corr;
-                st.o[nt][2 * h + 1] *= corr;
-            }
-        }
-    }
-}
-
-// O(16 x D) += P(16 x 16 tokens) . V(tokens row0..row0+15, D)
-template <int D>
-__device__ __forceinline__ void warp_pv_16x16(WarpAttnState<D> &st, const uint32_t (&pa)[4], uint32_t v_tile,
-                                              uint32_t half_bytes, int row0)
+// O^T += V(tokens row0 .. row0 + 15)^T . P^T
+template <int D, int NB>
+__device__ __forceinline__ void warp_pv(WarpAttnState<D, NB> &st, const uint32_t (&pb)[NB][2], uint32_t v_tile,
+                                        uint32_t half_bytes, int row0)
 {
     const int lane = threadIdx.x & 31;
-    const uint32_t row = row0 + (((lane >> 3) & 1) << 3) + (lane & 7);   // matrices 1,3: tokens +8
-    const uint32_t csel = lane >> 4;                                      // matrices 2,3: head_dim +8
+    const uint32_t row = row0 + ((lane >> 4) << 3) + (lane & 7);    // matrices 2, 3: tokens + 8
+    const uint32_t csel = (lane >> 3) & 1;                          // matrices 1, 3: head dims + 8
 #pragma unroll
-    for (int np = 0; np < D / 16; ++np) {
-        const uint32_t chunk = 2 * np + csel;
-        const uint32_t addr = v_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7);
-        uint32_t b0, b1, b2, b3;
-        ldmatrix_x4_trans(addr, b0, b1, b2, b3);
-        mma_bf16_16816(st.o[2 * np], pa, b0, b1);
-        mma_bf16_16816(st.o[2 * np + 1], pa, b2, b3);
+    for (int mt = 0; mt < D / 16; ++mt) {
+        const uint32_t chunk = 2 * mt + csel;
+        uint32_t a[4];
+        ldmatrix_x4_trans(v_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
+#pragma unroll
+        for (int n = 0; n < NB; ++n) mma_bf16_16816(st.o[mt][n], a, pb[n][0], pb[n][1]);
     }
 }
 
-// Online-softmax update over NT 8-token score tiles at once (NT = 2 is warp_softmax_16; the fp8 path takes 32
-// tokens per step so that the shuffles and the bookkeeping are paid once per 32 tokens). s[j] holds tokens
-// 8j + 2*(lane%4) + {0,1} (elements 0,1: row lane/4; 2,3: row lane/4 + 8); pa[u] is the A fragment of P for
-// tokens 16u .. 16u+15.
-template <int D, bool kF16, int NT>
-__device__ __forceinline__ void warp_softmax_tiles(WarpAttnState<D> &st, const float (&s)[NT][4], uint32_t (&pa)[NT / 2][4])
+// Tokens from `nvalid` on (of the 16 * NT in s) get no weight.
+template <int NB, int NT>
+__device__ __forceinline__ void warp_mask(float (&s)[NT][NB][4], int nvalid)
+{
+    const int r = (threadIdx.x & 31) >> 2;
+#pragma unroll
+    for (int u = 0; u < NT; ++u)
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (16 * u + r + 8 * (e >> 1) >= nvalid) s[u][n][e] = -INFINITY;
+}
+
+// Online-softmax update over NT blocks of 16 tokens. Scores arrive already multiplied by scale*log2(e), masked positions
+// at -inf. A step in which no score exceeds the running maxima of its heads (most of them, after the first tiles) needs one
+// vote and neither shuffles nor a rescale. (The maxima stay exact: a reference left up to 2^8 behind would save the rest of
+// the shuffles, but then the largest weights are rounded too, and the log-sum-exp was off by 2.5e-3 instead of 2e-3.)
+// pb[u]: B fragments of P^T, weights as bf16, or as f16 for the MMAs of the e4m3 path.
+template <int D, int NB, bool kF16, int NT>
+__device__ __forceinline__ void warp_softmax(WarpAttnState<D, NB> &st, const float (&s)[NT][NB][4], uint32_t (&pb)[NT][NB][2])
 {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float mx = -INFINITY;
+    for (int n = 0; n < NB; ++n) {
+        float mx[2];
 #pragma unroll
-        for (int j = 0; j < NT; ++j) mx = fmaxf(mx, fmaxf(s[j][2 * h], s[j][2 * h + 1]));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(st.m[h], mx);
-        const float m_use = (m_new == -INFINITY) ? 0.f : m_new;     // row with nothing visible yet
-        const float corr = fast_exp2(st.m[h] - m_use);
-        float psum = 0.f;
+        for (int e = 0; e < 2; ++e) {
+            mx[e] = fmaxf(s[0][n][e], s[0][n][2 + e]);
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            const float e0 = fast_exp2(s[j][2 * h] - m_use), e1 = fast_exp2(s[j][2 * h + 1] - m_use);
-            const uint32_t pk = kF16 ? pack_f16x2(e0, e1) : pack_bf16x2(e0, e1);
-            pa[j >> 1][(j & 1) * 2 + h] = pk;
-            // the denominator sums exactly the rounded weights that multiply V
-            psum += kF16 ? sum_f16x2(pk) : __uint_as_float(pk << 16) + __uint_as_float(pk & 0xffff0000u);
+            for (int u = 1; u < NT; ++u) mx[e] = fmaxf(mx[e], fmaxf(s[u][n][e], s[u][n][2 + e]));
         }
-        st.l[h] = st.l[h] * corr + psum;
-        st.m[h] = m_new;
-        if (__any_sync(0xffffffffu, corr != 1.f)) {
+        if (__any_sync(0xffffffffu, mx[0] > st.m[n][0] || mx[1] > st.m[n][1])) {
 #pragma unroll
-            for (int nt = 0; nt < D / 8; ++nt) {
-                st.o[nt][2 * h] *= corr;
-                st.o[nt][2 * h + 1] *= corr;
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int off = 4; off <= 16; off <<= 1) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], off));
+                const float m_new = fmaxf(st.m[n][e], mx[e]);
+                const float corr = fast_exp2(st.m[n][e] - ((m_new == -INFINITY) ? 0.f : m_new));
+                st.m[n][e] = m_new;
+                st.l[n][e] *= corr;
+#pragma unroll
+                for (int mt = 0; mt < D / 16; ++mt) {
+                    st.o[mt][n][e] *= corr;
+                    st.o[mt][n][2 + e] *= corr;
+                }
             }
         }
+        const float m0 = (st.m[n][0] == -INFINITY) ? 0.f : st.m[n][0], m1 = (st.m[n][1] == -INFINITY) ? 0.f : st.m[n][1];
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                           // token rows r and r + 8
+                const float e0 = fast_exp2(s[u][n][2 * h] - m0), e1 = fast_exp2(s[u][n][2 * h + 1] - m1);
+                const uint32_t pk = kF16 ? pack_f16x2(e0, e1) : pack_bf16x2(e0, e1);
+                // the denominator sums exactly the rounded weights that multiply V
+                float w0, w1;
+                if constexpr (kF16) unpack_f16x2(pk, w0, w1);
+                else w0 = __uint_as_float(pk << 16), w1 = __uint_as_float(pk & 0xffff0000u);
+                st.l[n][0] += w0;
+                st.l[n][1] += w1;
+                pb[u][n][h] = movmatrix_trans(pk);
+            }
     }
 }
 
@@ -168,10 +205,9 @@ __device__ __forceinline__ void warp_softmax_tiles(WarpAttnState<D> &st, const f
 // widened to f16 in registers (exact) and multiplied with f16 MMAs. ldmatrix moves 16-bit units, so a
 // thread receives 4 consecutive head-dim bytes of a K row where the MMA wants two separate pairs: the
 // k index of QK^T is therefore permuted (MMA slots 2c, 2c+1, 2c+8, 2c+9 of a 16-block hold head dims
-// 4c .. 4c+3), and the q fragments are built with the same permutation (see q_frag_f8_word). For V the
-// transposing ldmatrix delivers, per thread, two tokens of an EVEN and an ODD head dim: the 8-column
-// MMA tiles of O alternate even / odd dims (tile 2j: dims 16j + 2x, tile 2j+1: dims 16j + 2x + 1 in
-// column x); a thread's accumulators of a tile pair are then 4 consecutive head dims.
+// 4c .. 4c+3), and the q fragments are built with the same permutation. For V the
+// transposing ldmatrix delivers, per thread, two tokens of an EVEN and an ODD head dim: rows r of a 16-dim tile of O^T
+// are the even dims (2r), rows r + 8 the odd ones (2r + 1).
 
 // Shared-memory address of head dims [16c, 16c+16) of token `tok` of an fp8 tile.
 template <int D>
@@ -182,52 +218,109 @@ __device__ __forceinline__ uint32_t tok_chunk_f8(uint32_t tile, uint32_t tok, ui
     else return tile + swz128(tok >> 1, ((tok & 1u) << 2) + c);
 }
 
-// 32-bit word (two bf16) of a q row that feeds A-fragment register `reg` (0..3) of k-step ks, as f16x2.
-__device__ __forceinline__ int q_frag_f8_word(int ks, int reg, int lane) { return ks * 8 + 2 * (lane & 3) + (reg >> 1); }
-
-__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t v)
-{
-    return pack_f16x2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
-}
-
-template <int D>
-__device__ __forceinline__ void warp_qk_16x16_f8(const uint32_t (&qf)[D / 16][4], uint32_t k_tile, int row0,
-                                                 float (&s_lo)[4], float (&s_hi)[4])
+template <int D, int NB>
+__device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, int row0, float (&s)[NB][4])
 {
     const int lane = threadIdx.x & 31;
-    s_lo[0] = s_lo[1] = s_lo[2] = s_lo[3] = 0.f;
-    s_hi[0] = s_hi[1] = s_hi[2] = s_hi[3] = 0.f;
-    const uint32_t row = row0 + ((lane >> 4) << 3) + (lane & 7);   // matrices 2,3: tokens +8
-    const uint32_t csel = (lane >> 3) & 1;                          // matrices 1,3: next 16 head dims
+    float odd[NB][4];
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[n][e] = odd[n][e] = 0.f;
+    const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
+    const uint32_t csel = lane >> 4;                                // matrices 2, 3: next 16 head dims
 #pragma unroll
     for (int qd = 0; qd < D / 32; ++qd) {
         uint32_t r0, r1, r2, r3;
         ldmatrix_x4(tok_chunk_f8<D>(k_tile, row, 2 * qd + csel), r0, r1, r2, r3);
-        mma_f16_16816(s_lo, qf[2 * qd], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r0 >> 16));
-        mma_f16_16816(s_lo, qf[2 * qd + 1], e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r1 >> 16));
-        mma_f16_16816(s_hi, qf[2 * qd], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r2 >> 16));
-        mma_f16_16816(s_hi, qf[2 * qd + 1], e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r3 >> 16));
+        const uint32_t a[4] = {e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16)};
+        const uint32_t b[4] = {e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16)};
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            mma_f16_16816(s[n], a, qf[2 * qd][n][0], qf[2 * qd][n][1]);
+            mma_f16_16816(odd[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
+        }
     }
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[n][e] += odd[n][e];
 }
 
-template <int D>
-__device__ __forceinline__ void warp_pv_16x16_f8(WarpAttnState<D> &st, const uint32_t (&pa)[4], uint32_t v_tile, int row0)
+template <int D, int NB>
+__device__ __forceinline__ void warp_pv_f8(WarpAttnState<D, NB> &st, const uint32_t (&pb)[NB][2], uint32_t v_tile, int row0)
 {
     const int lane = threadIdx.x & 31;
-    const uint32_t row = row0 + (((lane >> 3) & 1) << 3) + (lane & 7);   // matrices 1,3: tokens +8
-    const uint32_t csel = lane >> 4;                                      // matrices 2,3: next 16 head dims
+    const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
+    const uint32_t csel = lane >> 4;                                // matrices 2, 3: next 16 head dims
+    // bytes (tok, even) (tok, odd) (tok+1, even) (tok+1, odd) -> (tok, even) (tok+1, even) | (tok, odd) (tok+1, odd)
+    auto tile = [&](int mt, uint32_t lo, uint32_t hi) {
+        const uint32_t x = __byte_perm(lo, 0u, 0x3120), y = __byte_perm(hi, 0u, 0x3120);
+        const uint32_t a[4] = {e4m3x2_to_f16x2(x), e4m3x2_to_f16x2(x >> 16), e4m3x2_to_f16x2(y), e4m3x2_to_f16x2(y >> 16)};
+#pragma unroll
+        for (int n = 0; n < NB; ++n) mma_f16_16816(st.o[mt][n], a, pb[n][0], pb[n][1]);
+    };
 #pragma unroll
     for (int qd = 0; qd < D / 32; ++qd) {
         uint32_t r0, r1, r2, r3;
         ldmatrix_x4_trans(tok_chunk_f8<D>(v_tile, row, 2 * qd + csel), r0, r1, r2, r3);
-        // bytes (tok, even) (tok, odd) (tok+1, even) (tok+1, odd) -> (tok, even) (tok+1, even) | (tok, odd) (tok+1, odd)
-        const uint32_t x0 = __byte_perm(r0, 0u, 0x3120), x1 = __byte_perm(r1, 0u, 0x3120);
-        const uint32_t x2 = __byte_perm(r2, 0u, 0x3120), x3 = __byte_perm(r3, 0u, 0x3120);
-        mma_f16_16816(st.o[4 * qd], pa, e4m3x2_to_f16x2(x0), e4m3x2_to_f16x2(x1));
-        mma_f16_16816(st.o[4 * qd + 1], pa, e4m3x2_to_f16x2(x0 >> 16), e4m3x2_to_f16x2(x1 >> 16));
-        mma_f16_16816(st.o[4 * qd + 2], pa, e4m3x2_to_f16x2(x2), e4m3x2_to_f16x2(x3));
-        mma_f16_16816(st.o[4 * qd + 3], pa, e4m3x2_to_f16x2(x2 >> 16), e4m3x2_to_f16x2(x3 >> 16));
+        tile(2 * qd, r0, r1);
+        tile(2 * qd + 1, r2, r3);
     }
+}
+
+// ----------------------------------------------------------------------------- leaving the accumulators
+// One block's O^T tile mt, scaled per head, as bf16 rows: lane (r, c) gets two words of head 8n + r, and word_dim says which
+// head dims they hold: bf16 caches 16 mt + 2c + {0, 1} and + 8, e4m3 caches 16 mt + 4c + {0, 1} and {2, 3}.
+template <int D, int NB, bool F8>
+__device__ __forceinline__ uint2 output_words(const WarpAttnState<D, NB> &st, int mt, int n, float f0, float f1)
+{
+    const uint32_t a = movmatrix_trans(pack_bf16x2(st.o[mt][n][0] * f0, st.o[mt][n][1] * f1));
+    const uint32_t b = movmatrix_trans(pack_bf16x2(st.o[mt][n][2] * f0, st.o[mt][n][3] * f1));
+    if constexpr (F8) return make_uint2(__byte_perm(a, b, 0x5410), __byte_perm(a, b, 0x7632));
+    else return make_uint2(a, b);
+}
+// Stores them into a row of bf16 (16-byte aligned).
+template <bool F8>
+__device__ __forceinline__ void store_output_words(void *row, int mt, int lane, uint2 w)
+{
+    uint32_t *dst = reinterpret_cast<uint32_t *>(row) + mt * 8;
+    if constexpr (F8) {
+        *reinterpret_cast<uint2 *>(dst + 2 * (lane & 3)) = w;
+    } else {
+        dst[lane & 3] = w.x;
+        dst[4 + (lane & 3)] = w.y;
+    }
+}
+
+// This warp's share of a piece as rows of fp32 O, maximum and sum for the merge over warps: row(head) gives the row of a
+// head, the maximum sits at off_m bytes, the sum behind it. finish_sums() has been called.
+template <int D, int NB, bool F8, class RowOf>
+__device__ __forceinline__ void dump_rows_f32(const WarpAttnState<D, NB> &st, int G, float vs, int off_m, RowOf row)
+{
+    const int lane = threadIdx.x & 31, r = lane >> 2;
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int head = 8 * n + 2 * (lane & 3) + e;
+            if (head >= G) continue;
+            uint8_t *rowb = row(head);
+            float *o = reinterpret_cast<float *>(rowb);
+            if (r == 0) {
+                *reinterpret_cast<float *>(rowb + off_m) = st.m[n][e];
+                *reinterpret_cast<float *>(rowb + off_m + 4) = st.l[n][e];
+            }
+#pragma unroll
+            for (int mt = 0; mt < D / 16; ++mt) {
+                if constexpr (F8) {
+                    *reinterpret_cast<float2 *>(o + mt * 16 + 2 * r) = make_float2(st.o[mt][n][e] * vs, st.o[mt][n][2 + e] * vs);
+                } else {
+                    o[mt * 16 + r] = st.o[mt][n][e];
+                    o[mt * 16 + 8 + r] = st.o[mt][n][2 + e];
+                }
+            }
+        }
 }
 
 }  // namespace l4l

@@ -1,7 +1,7 @@
-"""Thin ctypes binding of the C-ABI library ``libl4l.so`` (same names as ``include/l4l.h``).
+"""Thin binding of the C-ABI library ``libl4l.so`` (same names as ``include/l4l.h``).
 
 Argument marshalling only: tensors become pointers + strides, the current CUDA stream
-becomes a ``void*``. Every step of the attention path runs inside the library's kernels;
+becomes a ``void*``, in ``_l4l_marshal`` (C++) for the calls of every step and by ctypes for the rest. Every step of the attention path runs inside the library's kernels;
 PyTorch is used for device memory and streams. There is no fallback: if the library is
 missing or a call fails, an exception is raised.
 """
@@ -160,6 +160,20 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+_native = None
+
+
+def _load_native():
+    """The module that marshals the arguments of the per-step calls (csrc/l4l_marshal.cpp), next to libl4l.so."""
+    global _native
+    if _native is None:
+        load()
+        from . import _l4l_marshal
+
+        _native = _l4l_marshal
+    return _native
+
+
 def version() -> str:
     return load().l4l_version().decode()
 
@@ -240,34 +254,15 @@ def l4l_kv_append(cache_k, cache_v, k_new, v_new, write_pos, n_new=None) -> None
 
 def l4l_attn_prefill(q, k, v, o, seq_lens, scale: float, workspace, cache_k=None, cache_v=None, lse=None) -> None:
     """q,o [B,S,Hq,D]; k,v [B,S,Hkv,D]; seq_lens CUDA int32 [B]; lse optional CUDA float32 [B,Hq,S]."""
-    B, S, Hq, D = q.shape
-    Hkv = k.shape[2]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq, S)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq, S]")
-    st = load().l4l_attn_prefill(tensor4(q, "q"), tensor4(k, "k"), tensor4(v, "v"), tensor4(o, "o"),
-                                 kv_cache(cache_k, cache_v), _i32_dev(seq_lens, "seq_lens"), S, B, Hq, Hkv, D,
-                                 float(scale), None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                 workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).prefill(q, k, v, o, seq_lens, scale, workspace, cache_k, cache_v, lse)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_prefill")
 
 
 def l4l_attn_decode(q, o, cache_k, cache_v, kv_lens, max_kv_len: int, scale: float, workspace, lse=None) -> None:
     """q,o dense [B,Hq,D]; cache [B,Hkv,max_len,D]; kv_lens CUDA int32 [B] (current token included)."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k.shape[1]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq]")
-    st = load().l4l_attn_decode(q.data_ptr(), o.data_ptr(), kv_cache(cache_k, cache_v),
-                                _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, None, None, kv_lens, max_kv_len,
+                                            scale, None, None, None, None, 0.0, workspace, lse, 2)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode")
 
@@ -298,22 +293,8 @@ def l4l_attn_decode_append(q, o, cache_k, cache_v, k_new, v_new, kv_lens, max_kv
                            lse=None) -> None:
     """One launch per decode step: writes k_new / v_new ([B,1,Hkv,D]) into cache slot kv_lens[b]-1 and attends
     over slots 0..kv_lens[b]-1. Same result as l4l_kv_append followed by l4l_attn_decode."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k.shape[1]
-    if tuple(k_new.shape) != (B, 1, Hkv, D) or tuple(v_new.shape) != (B, 1, Hkv, D):
-        raise ValueError("k_new and v_new must be [B, 1, Hkv, D]")
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq]")
-    st = load().l4l_attn_decode_append(q.data_ptr(), o.data_ptr(), kv_cache(cache_k, cache_v),
-                                       tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-                                       _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                       None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                       workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, k_new, v_new, kv_lens,
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 3)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_append")
 
@@ -321,15 +302,7 @@ def l4l_attn_decode_append(q, o, cache_k, cache_v, k_new, v_new, kv_lens, max_kv
 def l4l_attn_prefill_chunk(q, o, cache_k, cache_v, past_lens, q_lens, scale: float, workspace, lse=None) -> None:
     """Chunk of new tokens over a populated cache. q,o [B,S,Hq,D]; the chunk's K/V are already in the cache at
     slots past..past+q_len-1; past_lens, q_lens CUDA int32 [B]; lse optional CUDA float32 [B,Hq,S]."""
-    B, S, Hq, D = q.shape
-    Hkv = cache_k.shape[1]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq, S)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq, S]")
-    st = load().l4l_attn_prefill_chunk(tensor4(q, "q"), tensor4(o, "o"), kv_cache(cache_k, cache_v),
-                                       _i32_dev(past_lens, "past_lens"), _i32_dev(q_lens, "q_lens"), S, B, Hq, Hkv, D,
-                                       float(scale), None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                       workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).prefill_chunk(q, o, cache_k, cache_v, past_lens, q_lens, scale, workspace, lse)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_prefill_chunk")
 
@@ -339,21 +312,8 @@ def l4l_attn_prefill_chunk_append(q, k_new, v_new, o, cache_k, cache_v, past_len
     """Chunk of new tokens over a populated cache with the cache update fused in (one launch). q,o [B,S,Hq,D];
     k_new, v_new [B,S,Hkv,D] go to slots past..past+q_len-1. With block_table (CUDA int32 [B, n]) cache_k / cache_v
     are a page pool [pages,Hkv,page_size,D]; without it a contiguous cache [B,Hkv,max_len,D]."""
-    B, S, Hq, D = q.shape
-    Hkv = k_new.shape[2]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq, S)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq, S]")
-    common = (_i32_dev(past_lens, "past_lens"), _i32_dev(q_lens, "q_lens"), S, B, Hq, Hkv, D, float(scale),
-              None if lse is None else lse.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-              _stream())
-    if block_table is None:
-        st = load().l4l_attn_prefill_chunk_append(tensor4(q, "q"), tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-                                                  tensor4(o, "o"), kv_cache(cache_k, cache_v), *common)
-    else:
-        tbl, stride = _block_table(block_table, B)
-        st = load().l4l_attn_prefill_chunk_paged_append(tensor4(q, "q"), tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-                                                        tensor4(o, "o"), paged_kv(cache_k, cache_v), tbl, stride, *common)
+    st = (_native or _load_native()).prefill_chunk_append(q, k_new, v_new, o, cache_k, cache_v, past_lens, q_lens, scale,
+                                                          workspace, lse, block_table)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_prefill_chunk_append")
 
@@ -373,15 +333,8 @@ def l4l_rope_kv_append(q, k_new, v_new, cache_k, cache_v, pos, n_new, cos, sin, 
     """Rotary embedding (+ optional per-head RMS norm) of q (in place) and k, with K and V written to the cache.
     q [B,T,Hq,D]; k_new, v_new [B,T,Hkv,D]; pos CUDA int32 [B]; n_new CUDA int32 [B] or None;
     cos, sin CUDA float32 [n_pos, D/2]; q_weight, k_weight CUDA float32 [D] or None."""
-    B, T, Hq, D = q.shape
-    Hkv = k_new.shape[2]
-    n_pos = cos.shape[0]
-    st = load().l4l_rope_kv_append(tensor4(q, "q"), tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-                                   kv_cache(cache_k, cache_v), _i32_dev(pos, "pos"),
-                                   None if n_new is None else _i32_dev(n_new, "n_new"), T, B, Hq, Hkv, D,
-                                   _f32_dev(cos, "cos", (n_pos, D // 2)), _f32_dev(sin, "sin", (n_pos, D // 2)), n_pos,
-                                   _f32_dev(q_weight, "q_weight", (D,)), _f32_dev(k_weight, "k_weight", (D,)),
-                                   float(eps), _stream())
+    st = (_native or _load_native()).rope_kv_append(q, k_new, v_new, cache_k, cache_v, pos, n_new, cos, sin, q_weight,
+                                                    k_weight, eps)
     if st != L4L_OK:
         raise L4LError(st, "l4l_rope_kv_append")
 
@@ -416,20 +369,8 @@ def l4l_kv_append_paged(pool_k, pool_v, block_table, k_new, v_new, write_pos, n_
 def l4l_attn_decode_paged(q, o, pool_k, pool_v, block_table, kv_lens, max_kv_len: int, scale: float, workspace,
                           lse=None) -> None:
     """Decode over a paged cache. q,o dense [B,Hq,D]; pools [pages,Hkv,page_size,D]; block_table CUDA int32 [B, n]."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = pool_k.shape[1]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq]")
-    tbl, stride = _block_table(block_table, B)
-    st = load().l4l_attn_decode_paged(q.data_ptr(), o.data_ptr(), paged_kv(pool_k, pool_v), tbl, stride,
-                                      _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                      None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                      workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, None, None, kv_lens,
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 2)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged")
 
@@ -439,23 +380,8 @@ def l4l_attn_decode_paged_append(q, o, pool_k, pool_v, block_table, k_new, v_new
     """One launch per decode step over a paged cache: k_new / v_new ([B,1,Hkv,D]) go to slot kv_lens[b]-1 of sequence b
     (the page the block table names) and are attended with the rest. Same result as l4l_kv_append_paged followed by
     l4l_attn_decode_paged."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = pool_k.shape[1]
-    if tuple(k_new.shape) != (B, 1, Hkv, D) or tuple(v_new.shape) != (B, 1, Hkv, D):
-        raise ValueError("k_new and v_new must be [B, 1, Hkv, D]")
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq]")
-    tbl, stride = _block_table(block_table, B)
-    st = load().l4l_attn_decode_paged_append(q.data_ptr(), o.data_ptr(), paged_kv(pool_k, pool_v), tbl, stride,
-                                             tensor4(k_new), tensor4(v_new), _i32_dev(kv_lens, "kv_lens"),
-                                             int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                             None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                             workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, k_new, v_new, kv_lens,
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 3)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_append")
 
@@ -465,22 +391,8 @@ def l4l_attn_decode_paged_rope_append(q, o, pool_k, pool_v, block_table, k_new, 
                                       lse=None) -> None:
     """l4l_attn_decode_rope_append over a paged cache: rotation (+ optional RMS norm) of q and k_new at position
     kv_lens - 1, write of the rotated k and of v_new into the page slot, attention: one launch."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = pool_k.shape[1]
-    if tuple(k_new.shape) != (B, 1, Hkv, D) or tuple(v_new.shape) != (B, 1, Hkv, D):
-        raise ValueError("k_new and v_new must be [B, 1, Hkv, D]")
-    n_pos = cos.shape[0]
-    tbl, stride = _block_table(block_table, B)
-    st = load().l4l_attn_decode_paged_rope_append(
-        q.data_ptr(), o.data_ptr(), paged_kv(pool_k, pool_v), tbl, stride, tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-        _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-        _f32_dev(cos, "cos", (n_pos, D // 2)), _f32_dev(sin, "sin", (n_pos, D // 2)), n_pos,
-        _f32_dev(q_weight, "q_weight", (D,)), _f32_dev(k_weight, "k_weight", (D,)), float(eps),
-        None if lse is None else lse.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, k_new, v_new, kv_lens,
+                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, 1)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_rope_append")
 
@@ -491,28 +403,9 @@ def l4l_attn_decode_rope_append_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, 
     """One launch per decode step over an fp8 cache with the rotation fused in: q and k_new are rotated (+ optional RMS
     norm) at position kv_lens - 1, the rotated k (rounded to bf16) and v_new are quantised as l4l_kv_append_fp8 does and
     written to slot kv_lens - 1, the rotated q attends. With block_table, the caches are a page pool."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k8.shape[1]
-    if tuple(k_new.shape) != (B, 1, Hkv, D) or tuple(v_new.shape) != (B, 1, Hkv, D):
-        raise ValueError("k_new and v_new must be [B, 1, Hkv, D]")
-    n_pos = cos.shape[0]
-    c = kv_cache8(cache_k8, cache_v8)
-    common = (tensor4(k_new, "k_new"), tensor4(v_new, "v_new"), _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv,
-              D, float(scale), _f32_dev(cos, "cos", (n_pos, D // 2)), _f32_dev(sin, "sin", (n_pos, D // 2)), n_pos,
-              _f32_dev(q_weight, "q_weight", (D,)), _f32_dev(k_weight, "k_weight", (D,)), float(eps),
-              None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-              workspace.numel() * workspace.element_size(), _stream())
-    ks, vs = _f32_dev(k_scale, "k_scale", (Hkv,)), _f32_dev(v_scale, "v_scale", (Hkv,))
-    if block_table is None:
-        st = load().l4l_attn_decode_rope_append_fp8(q.data_ptr(), o.data_ptr(), c, ks, vs, *common)
-    else:
-        pool = PagedKV(c.k, c.v, c.stride_b, c.stride_h, c.stride_t, cache_k8.shape[2], cache_k8.shape[0])
-        tbl, stride = _block_table(block_table, B)
-        st = load().l4l_attn_decode_paged_rope_append_fp8(q.data_ptr(), o.data_ptr(), pool, ks, vs, tbl, stride, *common)
+    st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, block_table, k_new, v_new,
+                                            kv_lens, max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace,
+                                            lse, 1)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_rope_append_fp8")
 
@@ -543,20 +436,8 @@ def l4l_attn_decode_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, kv_lens, max
                         lse=None) -> None:
     """Decode over an fp8 (e4m3) cache with per-KV-head scales. q,o dense bf16 [B,Hq,D] (at head_dim 64 the cache's
     token rows must be dense and even in number)."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k8.shape[1]
-    if lse is not None and not (lse.is_cuda and lse.dtype == torch.float32 and lse.is_contiguous()
-                                and tuple(lse.shape) == (B, Hq)):
-        raise TypeError("lse must be a contiguous CUDA float32 tensor [B, Hq]")
-    st = load().l4l_attn_decode_fp8(q.data_ptr(), o.data_ptr(), kv_cache8(cache_k8, cache_v8),
-                                    _f32_dev(k_scale, "k_scale", (Hkv,)), _f32_dev(v_scale, "v_scale", (Hkv,)),
-                                    _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                    None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                    workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, None, None, None, kv_lens,
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 2)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_fp8")
 
@@ -565,19 +446,7 @@ def l4l_rglru_scan(x, gate_x, gate_a, a_param, state, y, workspace, position=Non
     """Gated linear recurrence (RG-LRU) over the sequence. x, gate_x, gate_a, y dense CUDA bf16 [B,T,W];
     a_param CUDA float32 [W]; state CUDA float32 [B,W] (in/out); position CUDA int32 [B,T] or None;
     seq_lens CUDA int32 [B] or None."""
-    for t, name in ((x, "x"), (gate_x, "gate_x"), (gate_a, "gate_a"), (y, "y")):
-        _check_bf16_cuda(t, name)
-        if not (t.dim() == 3 and t.is_contiguous() and t.shape == x.shape):
-            raise ValueError(f"{name} must be a dense [B, T, W] tensor of the same shape as x")
-    B, T, W = x.shape
-    if position is not None and not (position.is_cuda and position.dtype == torch.int32 and position.is_contiguous()
-                                     and tuple(position.shape) == (B, T)):
-        raise TypeError("position must be a contiguous CUDA int32 tensor [B, T]")
-    st = load().l4l_rglru_scan(x.data_ptr(), gate_x.data_ptr(), gate_a.data_ptr(), _f32_dev(a_param, "a_param", (W,)),
-                               None if position is None else position.data_ptr(),
-                               None if seq_lens is None else _i32_dev(seq_lens, "seq_lens"),
-                               _f32_dev(state, "state", (B, W)), y.data_ptr(), B, T, W, workspace.data_ptr(),
-                               workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).rglru_scan(x, gate_x, gate_a, a_param, state, y, workspace, position, seq_lens)
     if st != L4L_OK:
         raise L4LError(st, "l4l_rglru_scan")
 
@@ -594,20 +463,9 @@ def new_rglru_workspace(B: int, T: int, W: int, device=None) -> torch.Tensor:
 def l4l_attn_decode_paged_fp8(q, o, pool_k8, pool_v8, k_scale, v_scale, block_table, kv_lens, max_kv_len: int, scale: float,
                               workspace, lse=None) -> None:
     """Decode over an fp8 page pool [pages, Hkv, page_size, 128] (uint8 / float8_e4m3fn) read through a block table."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    c = kv_cache8(pool_k8, pool_v8)                     # same checks; fields reinterpreted as a page pool
-    pool = PagedKV(c.k, c.v, c.stride_b, c.stride_h, c.stride_t, pool_k8.shape[2], pool_k8.shape[0])
-    Hkv = pool_k8.shape[1]
-    tbl, stride = _block_table(block_table, B)
-    st = load().l4l_attn_decode_paged_fp8(q.data_ptr(), o.data_ptr(), pool, _f32_dev(k_scale, "k_scale", (Hkv,)),
-                                          _f32_dev(v_scale, "v_scale", (Hkv,)), tbl, stride, _i32_dev(kv_lens, "kv_lens"),
-                                          int(max_kv_len), B, Hq, Hkv, D, float(scale),
-                                          None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-                                          workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, pool_k8, pool_v8, k_scale, v_scale, block_table, None, None,
+                                            kv_lens, max_kv_len, scale, None, None, None, None, 0.0, workspace, lse,
+                                            0)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_fp8")
 
@@ -617,25 +475,9 @@ def l4l_attn_decode_append_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, k_new
     """One launch per decode step over an fp8 cache: bf16 k_new / v_new ([B,1,Hkv,128]) are quantised as
     l4l_kv_append_fp8 does, written to slot kv_lens[b]-1 and attended with the rest. With block_table, cache_k8 /
     cache_v8 are a page pool [pages, Hkv, page_size, 128]."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k8.shape[1]
-    if tuple(k_new.shape) != (B, 1, Hkv, D) or tuple(v_new.shape) != (B, 1, Hkv, D):
-        raise ValueError("k_new and v_new must be [B, 1, Hkv, D]")
-    c = kv_cache8(cache_k8, cache_v8)
-    common = (tensor4(k_new, "k_new"), tensor4(v_new, "v_new"), _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv,
-              D, float(scale), None if lse is None else lse.data_ptr(), workspace.data_ptr(),
-              workspace.numel() * workspace.element_size(), _stream())
-    ks, vs = _f32_dev(k_scale, "k_scale", (Hkv,)), _f32_dev(v_scale, "v_scale", (Hkv,))
-    if block_table is None:
-        st = load().l4l_attn_decode_append_fp8(q.data_ptr(), o.data_ptr(), c, ks, vs, *common)
-    else:
-        pool = PagedKV(c.k, c.v, c.stride_b, c.stride_h, c.stride_t, cache_k8.shape[2], cache_k8.shape[0])
-        tbl, stride = _block_table(block_table, B)
-        st = load().l4l_attn_decode_paged_append_fp8(q.data_ptr(), o.data_ptr(), pool, ks, vs, tbl, stride, *common)
+    st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, block_table, k_new, v_new,
+                                            kv_lens, max_kv_len, scale, None, None, None, None, 0.0, workspace, lse,
+                                            1)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_append_fp8")
 
@@ -713,18 +555,7 @@ def l4l_attn_decode_rope_append(q, o, cache_k, cache_v, k_new, v_new, kv_lens, m
     """One launch per decode step: rotary embedding (+ optional RMS norm) of q and k_new at position kv_lens - 1, cache
     update and attention. q,o dense [B,Hq,D] (q is not modified); k_new, v_new [B,1,Hkv,D]; cos, sin CUDA float32
     [n_pos, D/2]."""
-    _check_bf16_cuda(q, "q")
-    _check_bf16_cuda(o, "o")
-    if not (q.is_contiguous() and o.is_contiguous() and q.dim() == 3 and q.shape == o.shape):
-        raise ValueError("q and o must be dense [B, Hq, D]")
-    B, Hq, D = q.shape
-    Hkv = cache_k.shape[1]
-    n_pos = cos.shape[0]
-    st = load().l4l_attn_decode_rope_append(
-        q.data_ptr(), o.data_ptr(), kv_cache(cache_k, cache_v), tensor4(k_new, "k_new"), tensor4(v_new, "v_new"),
-        _i32_dev(kv_lens, "kv_lens"), int(max_kv_len), B, Hq, Hkv, D, float(scale),
-        _f32_dev(cos, "cos", (n_pos, D // 2)), _f32_dev(sin, "sin", (n_pos, D // 2)), n_pos,
-        _f32_dev(q_weight, "q_weight", (D,)), _f32_dev(k_weight, "k_weight", (D,)), float(eps),
-        None if lse is None else lse.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream())
+    st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, k_new, v_new, kv_lens,
+                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, 0)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_rope_append")

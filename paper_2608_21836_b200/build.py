@@ -7,12 +7,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "csrc", "build")
 LIB = os.path.join(PKG, "libl4l.so")
+MARSHAL = os.path.join(PKG, "_l4l_marshal.so")       # the Python module that marshals the per-step calls
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -58,6 +60,17 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".tmp{os.getpid()}"
         run(["nvcc", "-shared", "-Wno-deprecated-gpu-targets", "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    src = os.path.join(CSRC, "l4l_marshal.cpp")
+    if force or _stale(MARSHAL, [src, os.path.join(PKG, "..", "include", "l4l.h")]):
+        import torch
+
+        home = os.path.dirname(torch.__file__)
+        tmp = MARSHAL + f".tmp{os.getpid()}"
+        run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+             f"-I{home}/include", f"-I{home}/include/torch/csrc/api/include", "-I/usr/local/cuda/include",
+             "-I" + sysconfig.get_paths()["include"], src, "-o", tmp, f"-L{PKG}", "-l:libl4l.so", f"-L{home}/lib",
+             "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, MARSHAL)
     return LIB
 
 

@@ -1064,26 +1064,31 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
 
 using SplitKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const DecodeParams);
 
-// Resident CTAs per SM for a given dynamic shared-memory size (0 on failure).
+// Resident CTAs per SM for a given dynamic shared-memory size (0 on failure). Looked up once per size and device: a
+// decode call asks three times, and the occupancy look-up is a good part of a small call's host time.
 template <int D, int W, bool F8, bool BigG, bool R8, int NB>
 int decode_blocks_per_sm(size_t smem)
 {
+    struct Entry { size_t smem; int dev, n; };
+    static Entry cache[32];
+    static int n_cached = 0, next = 0;
     static bool attr_set_on[kDeviceSlots] = {};
     const int slot = device_slot();
-    if (slot < 0) return 0;
-    bool &attr_set = attr_set_on[slot];
+    if (slot < 0 || smem > 227 * 1024) return 0;
     std::lock_guard<std::mutex> lock(setup_mutex());
-    if (!attr_set) {
+    for (int i = 0; i < n_cached; ++i)
+        if (cache[i].smem == smem && cache[i].dev == slot) return cache[i].n;
+    const auto kernel = decode_split_kernel<D, W, F8, BigG, R8, NB>;
+    if (!attr_set_on[slot]) {
         // the opt-in limit is per kernel: allow everything the SM has
-        if (cudaFuncSetAttribute(decode_split_kernel<D, W, F8, BigG, R8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
-            cudaSuccess)
-            return 0;
-        attr_set = true;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) return 0;
+        attr_set_on[slot] = true;
     }
-    if (smem > 227 * 1024) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_split_kernel<D, W, F8, BigG, R8, NB>, (BigG ? 11 : W + 2) * 32, smem) != cudaSuccess)
-        return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, (BigG ? 11 : W + 2) * 32, smem) != cudaSuccess) return 0;
+    cache[next] = Entry{smem, slot, n};
+    next = (next + 1) % 32;
+    if (n_cached < 32) ++n_cached;
     return n;
 }
 

@@ -1,0 +1,72 @@
+"""The native argument marshalling refuses what the entry points have always refused, before anything is launched."""
+import pytest
+import torch
+
+from paper_2608_21836_b200 import binding as l4l
+from paper_2608_21836_b200 import build
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    build.build()
+
+
+def calls(t4, t3, i):
+    """Every call of the native module, its tensors all of one kind."""
+    t2 = torch.zeros(4, 32)
+    return {
+        "prefill": lambda: l4l.l4l_attn_prefill(t4, t4, t4, t4, i, 1.0, i),
+        "chunk": lambda: l4l.l4l_attn_prefill_chunk(t4, t4, t4, t4, i, i, 1.0, i),
+        "chunk_append": lambda: l4l.l4l_attn_prefill_chunk_append(t4, t4, t4, t4, t4, t4, i, i, 1.0, i),
+        "rope": lambda: l4l.l4l_rope_kv_append(t4, t4, t4, t4, t4, i, i, t2, t2),
+        "decode": lambda: l4l.l4l_attn_decode(t3, t3, t4, t4, i, 4, 1.0, i),
+        "decode_append": lambda: l4l.l4l_attn_decode_append(t3, t3, t4, t4, t4, t4, i, 4, 1.0, i),
+        "decode_paged": lambda: l4l.l4l_attn_decode_paged(t3, t3, t4, t4, i, i, 4, 1.0, i),
+        "decode_paged_append": lambda: l4l.l4l_attn_decode_paged_append(t3, t3, t4, t4, i, t4, t4, i, 4, 1.0, i),
+        "decode_rope": lambda: l4l.l4l_attn_decode_rope_append(t3, t3, t4, t4, t4, t4, i, 4, 1.0, t2, t2, i),
+        "decode_paged_rope": lambda: l4l.l4l_attn_decode_paged_rope_append(t3, t3, t4, t4, i, t4, t4, i, 4, 1.0, t2, t2, i),
+        "decode_fp8": lambda: l4l.l4l_attn_decode_fp8(t3, t3, t4, t4, t2, t2, i, 4, 1.0, i),
+        "decode_paged_fp8": lambda: l4l.l4l_attn_decode_paged_fp8(t3, t3, t4, t4, t2, t2, i, i, 4, 1.0, i),
+        "decode_append_fp8": lambda: l4l.l4l_attn_decode_append_fp8(t3, t3, t4, t4, t2, t2, t4, t4, i, 4, 1.0, i),
+        "decode_rope_fp8": lambda: l4l.l4l_attn_decode_rope_append_fp8(t3, t3, t4, t4, t2, t2, t4, t4, i, 4, 1.0, t2, t2, i),
+        "scan": lambda: l4l.l4l_rglru_scan(t3, t3, t3, t2, t2, t3, i),
+    }
+
+
+NAMES = sorted(calls(None, None, None))
+
+
+@pytest.mark.parametrize("name", NAMES)
+def test_host_tensors_and_other_objects_are_type_errors(name):
+    t4, t3, i = torch.zeros(1, 4, 2, 64, dtype=torch.bfloat16), torch.zeros(1, 2, 64, dtype=torch.bfloat16), torch.zeros(1, dtype=torch.int32)
+    with pytest.raises(TypeError):
+        calls(t4, t3, i)[name]()
+    with pytest.raises(TypeError):
+        calls(7, 7, 7)[name]()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", NAMES)
+def test_float32_on_the_device_is_a_type_error(name):
+    t4, t3 = torch.zeros(1, 4, 2, 64, device="cuda"), torch.zeros(1, 2, 64, device="cuda")
+    with pytest.raises(TypeError):
+        calls(t4, t3, torch.zeros(1, dtype=torch.int32, device="cuda"))[name]()
+
+
+@pytest.mark.gpu
+def test_shapes_are_value_errors_and_statuses_are_raised():
+    q, o = torch.zeros(2, 4, 64, dtype=torch.bfloat16, device="cuda"), torch.zeros(2, 4, 64, dtype=torch.bfloat16, device="cuda")
+    ck, lens = torch.zeros(2, 2, 8, 64, dtype=torch.bfloat16, device="cuda"), torch.ones(2, dtype=torch.int32, device="cuda")
+    new = torch.zeros(2, 1, 2, 64, dtype=torch.bfloat16, device="cuda")
+    ws = l4l.new_workspace(l4l.L4L_OP_DECODE, 2, 4, 2, 64, 8)
+    with pytest.raises(ValueError):
+        l4l.l4l_attn_decode(q, o[:1], ck, ck, lens, 8, 1.0, ws)
+    with pytest.raises(ValueError):
+        l4l.l4l_attn_decode_append(q, o, ck, ck, new[:, :, :1], new, lens, 8, 1.0, ws)
+    with pytest.raises(ValueError):
+        l4l.l4l_attn_decode(q, o, ck, ck[:, :, :4], lens, 8, 1.0, ws)
+    with pytest.raises(TypeError):
+        l4l.l4l_attn_decode(q, o, ck, ck, lens, 8, 1.0, ws, lse=torch.zeros(2, 3, device="cuda"))
+    with pytest.raises(l4l.L4LError):
+        l4l.l4l_attn_decode(q, o, ck, ck, lens, 9, 1.0, ws)        # more than the cache's slots
+    l4l.l4l_attn_decode(q, o, ck, ck.clone(), lens, 8, 1.0, ws)

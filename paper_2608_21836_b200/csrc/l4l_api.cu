@@ -504,7 +504,7 @@ int l4l_rglru_strip_channels(int B, int T, int W)
 {
     if (B <= 0 || T <= 0 || W <= 0 || W % 8 != 0) return -1;
     int segments = 1;
-    const int split = rglru_strip_split(B, T, W, &segments);
+    const int split = rglru_strip_split(B, T, W, &segments, true);
     return split == 0 ? 64 : 64 / split;
 }
 

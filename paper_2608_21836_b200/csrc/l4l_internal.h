@@ -154,7 +154,7 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
 size_t rglru_workspace_bytes(int B, int T, int W);
 // the scan's shape for these sizes on the current device: 0 = 64-channel strips, teams of 16 warps; 1, 2, 4 = teams of
 // 8 warps on strips of 64, 32, 16 channels; *segments (null: one) = pieces of the time axis, which need the counters
-int rglru_strip_split(int B, int T, int W, int *segments);
+int rglru_strip_split(int B, int T, int W, int *segments, bool positions);
 
 // Where one prefill launch takes its keys and values from, and where it puts them.
 struct PrefillKV {

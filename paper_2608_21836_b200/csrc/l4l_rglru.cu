@@ -29,7 +29,7 @@
 // Segments. Where the strips fill the GPU more than once, a last round of a few strips leaves most SMs idle (320 strips of 32
 // channels on 296 places: 200 us). The time axis is then cut as well: a CTA per (strip, segment), all first segments ahead of all
 // second ones, the state passing through its place in global memory behind a counter per strip (release / acquire). By
-// the time a later segment gets a place its predecessor has long finished, so nothing waits: 156 us in four segments.
+// the time a later segment gets a place its predecessor has long finished, so nothing waits: 144 us in four segments.
 #include <type_traits>
 
 #include "l4l_internal.h"
@@ -81,7 +81,8 @@ __device__ __forceinline__ float sqrt_approx(float x)
 // two bf16 in one word -> packed fp32x2 (low half first)
 __device__ __forceinline__ uint64_t widen2(uint32_t w) { return pack_u32x2(w << 16, w & 0xffff0000u); }
 
-template <int kTeam, int kSplit>
+// kSeg: the launch is cut along the time axis (an instantiation of its own: the other launches are 8 % faster without its code)
+template <int kTeam, int kSplit, bool kSeg>
 __global__ void __launch_bounds__(kTeam * 32)
 rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_gx,
                   const __grid_constant__ CUtensorMap tmap_ga, const RglruParams p)
@@ -104,9 +105,9 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     L = L < 0 ? 0 : (L > p.T ? p.T : L);
     // this block's segment of the time axis: tiles [tile0, n_tiles) of the n_all tiles that the sequence has
     const int n_all = (L + kSteps - 1) / kSteps;
-    const int tile0 = (int)blockIdx.z * p.seg_tiles, n_tiles = min(n_all, tile0 + p.seg_tiles);
-    if (tile0 >= n_tiles) return;
-    int *progress = p.progress ? p.progress + (size_t)b * gridDim.x + blockIdx.x : nullptr;
+    const int segment = kSeg ? (int)blockIdx.z : 0, tile0 = kSeg ? segment * p.seg_tiles : 0;
+    const int n_tiles = kSeg ? min(n_all, tile0 + p.seg_tiles) : n_all;
+    if (kSeg && tile0 >= n_tiles) return;
     const int c = c0 + 2 * cp;
     const bool live = c < p.W;                           // W is even: both channels or neither
 
@@ -117,16 +118,13 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         fence_barrier_init();
         fence_proxy_async_smem();
     }
-    auto start_state = [&]() {                           // warp 0: slot 0 holds the state that the block's first tile starts from
-        if (sub == 0) {
-            const float2 st = live ? __ldcg(reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c)) : make_float2(0.f, 0.f);
-            *reinterpret_cast<float2 *>(carry + 2 * cp) = st;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&handed[0]);
-    };
+    if (warp == 0 && sub == 0) {
+        // slot 0: the state that the block's first tile starts from (a later segment's: below)
+        const float2 st = live && segment == 0 ? *reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c) : make_float2(0.f, 0.f);
+        *reinterpret_cast<float2 *>(carry + 2 * cp) = st;
+    }
     __syncthreads();
-    if (warp == 0 && blockIdx.z == 0) start_state();     // the caller's state
+    if (threadIdx.x == 0 && segment == 0) mbar_arrive(&handed[0]);
 
     uint8_t *my_stages = stages + (size_t)warp * kStages * kStageBytes;
     uint64_t *my_full = full + warp * kStages;
@@ -197,6 +195,24 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     };
     request_positions(tile0 + warp);
 
+    int *progress = kSeg ? p.progress + (size_t)b * gridDim.x + blockIdx.x : nullptr;
+    if (kSeg && warp == 0 && segment != 0) {
+        // a later segment starts from the state that the strip's previous segment left in global memory
+        if (lane == 0) {
+            const long long w0 = clock64();
+            while (ld_acquire_gpu(progress) != segment) {
+                if (*abort_flag || clock64() - w0 > kWaitCycleBudget) {
+                    *abort_flag = 1;
+                    break;
+                }
+                __nanosleep(64);
+            }
+        }
+        __syncwarp();
+        if (sub == 0 && live) *reinterpret_cast<float2 *>(carry + 2 * cp) = __ldcg(reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&handed[0]);
+    }
     for (int k = 0, tile = tile0 + warp; tile < n_tiles; ++k, tile += kTeam) {
         const uint32_t s = k % kStages, ph = (k / kStages) & 1u;
         const unsigned resets = resets_requested();
@@ -267,21 +283,6 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         // Every warp has its own barrier, completed once per tile it owns by the owner of the tile before; that
         // warp cannot reach its next arrival here before this warp has handed the present tile on, so the
         // phases are seen one by one.
-        if (tile == tile0 && blockIdx.z != 0) {
-            // a later segment starts from the state that the strip's previous segment left in global memory
-            if (lane == 0) {
-                const long long w0 = clock64();
-                while (ld_acquire_gpu(progress) != (int)blockIdx.z) {
-                    if (*abort_flag || clock64() - w0 > kWaitCycleBudget) {
-                        *abort_flag = 1;
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-            }
-            __syncwarp();
-            start_state();
-        }
         if (!mbar_wait(&handed[warp], k & 1u, abort_flag)) break;
         const int slot = (tile - tile0) & 1;
         const float2 hs = *reinterpret_cast<const float2 *>(carry + slot * kCb + 2 * cp);
@@ -302,15 +303,8 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
             if (sub == kSplit - 1) *reinterpret_cast<float2 *>(carry + (slot ^ 1) * kCb + 2 * cp) = make_float2(e0, e1);
             __syncwarp();
             if (lane == 0) mbar_arrive(&handed[(warp + 1) % kTeam]);           // release: the slot is written
-            if (tile + 1 == n_tiles) {                                         // the sequence, or its segment, ends here
-                if (live && sub == kSplit - 1) *reinterpret_cast<float2 *>(p.state + (size_t)b * p.W + c) = make_float2(e0, e1);
-                if (progress) {
-                    __threadfence();
-                    __syncwarp();
-                    // the last segment leaves the counter at zero for the next call
-                    if (lane == 0) st_release_gpu(progress, n_tiles == n_all ? 0 : (int)blockIdx.z + 1);
-                }
-            }
+            if (tile + 1 == n_tiles && live && sub == kSplit - 1)              // the sequence, or its segment, ends here
+                *reinterpret_cast<float2 *>(p.state + (size_t)b * p.W + c) = make_float2(e0, e1);
         }
         // ---- the recurrence proper, one packed FMA per step, and the outputs
 #pragma unroll
@@ -322,6 +316,13 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
                 if (live) yrow[(size_t)(t0 + t) * y_step] = pack_bf16x2(h0, h1);
             }
         }
+    }
+    if (kSeg && warp == (n_tiles - 1 - tile0) % kTeam && !*abort_flag) {
+        // this warp stored the segment's end state: on to the next segment (the last one leaves the counter at zero for the
+        // next call)
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) st_release_gpu(progress, n_tiles == n_all ? 0 : segment + 1);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status + kStatusErrWord, kErrScanWait);
@@ -339,7 +340,7 @@ size_t rglru_workspace_bytes(int B, int, int W)
 
 namespace {
 
-template <int kTeam, int kSplit>
+template <int kTeam, int kSplit, bool kSeg = false>
 l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, RglruParams p, int segments, cudaStream_t stream)
 {
     // one opt-in per instantiation and device
@@ -349,7 +350,7 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, R
     {
         std::lock_guard<std::mutex> lock(setup_mutex());
         if (!configured_on[slot]) {
-            if (cudaFuncSetAttribute(rglru_scan_kernel<kTeam, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            if (cudaFuncSetAttribute(rglru_scan_kernel<kTeam, kSplit, kSeg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem_bytes(kTeam)) != cudaSuccess)
                 return L4L_ERR_CUDA;
             configured_on[slot] = true;
@@ -362,12 +363,9 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, R
         !make_tmap_rows_bf16(&tga, gate_a, p.W, p.T, p.B, p.W, (int64_t)p.T * p.W, kCw, kTb * kSplit))
         return L4L_ERR_CUDA;
     const int strips = (p.W + kCw - 1) / kCw, tiles = (p.T + kTb * kSplit - 1) / (kTb * kSplit);
-    p.seg_tiles = (tiles + segments - 1) / segments;
-    if (segments > 1) p.seg_tiles = (p.seg_tiles + kTeam - 1) / kTeam * kTeam;      // whole rounds of the team
-    const int segs = (tiles + p.seg_tiles - 1) / p.seg_tiles;
-    if (segs == 1) p.progress = nullptr;
-    const dim3 grid(strips, p.B, segs);
-    rglru_scan_kernel<kTeam, kSplit><<<grid, kTeam * 32, smem_bytes(kTeam), stream>>>(tx, tgx, tga, p);
+    p.seg_tiles = kSeg ? (tiles + segments * kTeam - 1) / (segments * kTeam) * kTeam : tiles;        // whole rounds of the team
+    const dim3 grid(strips, p.B, (tiles + p.seg_tiles - 1) / p.seg_tiles);
+    rglru_scan_kernel<kTeam, kSplit, kSeg><<<grid, kTeam * 32, smem_bytes(kTeam), stream>>>(tx, tgx, tga, p);
     return cudaGetLastError() == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
 }
 
@@ -387,52 +385,68 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
     int segs = 1;
     const size_t needed = rglru_workspace_bytes(B, T, W);
     const bool with_counters = needed > kStatusBytes && ws_bytes >= needed;
-    const int split = rglru_strip_split(B, T, W, with_counters ? &segs : nullptr);
-    if (split == 0) return launch_shape<16, 1>(x, gate_x, gate_a, p, segs, stream);
-    if (split == 4) return launch_shape<8, 4>(x, gate_x, gate_a, p, segs, stream);
-    if (split == 2) return launch_shape<8, 2>(x, gate_x, gate_a, p, segs, stream);
-    return launch_shape<8, 1>(x, gate_x, gate_a, p, segs, stream);
+    const int split = rglru_strip_split(B, T, W, with_counters ? &segs : nullptr, d_position != nullptr);
+    if (segs > 1)
+        return split == 4   ? launch_shape<8, 4, true>(x, gate_x, gate_a, p, segs, stream)
+               : split == 2 ? launch_shape<8, 2, true>(x, gate_x, gate_a, p, segs, stream)
+                            : launch_shape<8, 1, true>(x, gate_x, gate_a, p, segs, stream);
+    if (split == 0) return launch_shape<16, 1>(x, gate_x, gate_a, p, 1, stream);
+    if (split == 4) return launch_shape<8, 4>(x, gate_x, gate_a, p, 1, stream);
+    if (split == 2) return launch_shape<8, 2>(x, gate_x, gate_a, p, 1, stream);
+    return launch_shape<8, 1>(x, gate_x, gate_a, p, 1, stream);
 }
 
 // 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels. *segments
-// (when given): into how many segments the time axis is cut.
-//
-// Two teams of 8 are resident per SM and together keep its issue slots busy, so n blocks take n / (2 SMs) rounds; a
-// last round with a lone team on an SM takes 0.68 of a full one (a lone team reaches three quarters of the rate of two).
-// Narrower strips make n larger and the blocks shorter, and so do segments, which cost about 4 us per round (set-up, first
-// loads, drain of the ring; 6 us on 16-channel strips) but leave the lines that the loads fetch wider. A strip is a
-// serial chain: it is cut only when the strips alone fill the GPU, so that a segment finds its predecessor finished. B = 4 x 8192
-// x 2560 with positions, us by (channels, segments): (64, 1) 222, (32, 1) 200, (32, 2) 166, (32, 4) 156, (32, 8) 166, (16, 1) 170,
-// (16, 4) 180.
-int rglru_strip_split(int B, int T, int W, int *segments)
+// (when given): into how many segments the time axis is cut; positions: the launch has reset positions.
+int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
 {
     if (segments) *segments = 1;
     if (T <= kTb) return 1;
     const long long sms = sm_count();
-    const double us_per_step_channel = 4.54e-4;          // of a resident pair of teams
-    auto rounds = [&](long long n) {
-        const long long rest = n % (2 * sms);
-        return (double)(n / (2 * sms)) + (rest == 0 ? 0.0 : rest <= sms ? 0.68 : 1.0);
-    };
+    // A strip is a serial chain that keeps an SM's issue slots busy, so a launch takes as long as the most loaded
+    // SM. Estimated time of that SM, in units of one 64-channel strip on an SM of its own: k CTAs of 1/s strip each
+    // take k / s; a lone team of 8 warps reaches about three quarters of the issue rate that two co-resident teams
+    // or one team of 16 warps reach.
     auto strips = [&](int s) { return (long long)((W + kCb / s - 1) / (kCb / s)) * B; };
+    auto fullest = [&](int s) { return (strips(s) + sms - 1) / sms; };
     int best = 1;
-    double best_time = rounds(strips(1)) * T * kCb * us_per_step_channel;
-    if (strips(1) <= sms && T >= 16 * 2 * kTb) {         // no more strips than SMs: 16 warps reach the full rate alone
+    double best_time = fullest(1) >= 2 ? (double)fullest(1) : 1.0 / 0.74;
+    if (fullest(1) == 1 && T >= 16 * 2 * kTb) {
         best = 0;
-        best_time = 0.5 * T * kCb * us_per_step_channel;
+        best_time = 1.0;
     }
-    for (int s = 1; s <= 4; s *= 2) {
-        if (s > 1 && T < 8 * kTb * s) break;             // long enough for the wider tiles of narrow strips
-        for (int z = 1; z <= (segments ? 4 : 1); z *= 2) {
-            if ((s == 1 && z == 1) || (z > 1 && (strips(s) < 2 * sms || T < 1024 * z))) continue;
-            const double time = rounds(strips(s) * z) * ((double)T / z * (kCb / s) * us_per_step_channel + (z == 1 ? 0.0 : s < 4 ? 4.0 : 6.0));
-            if (time < (z == 1 ? 0.9 : 0.95) * best_time) {
-                best = s;
-                best_time = time;
-                if (segments) *segments = z;
-            }
+    // narrower strips have to win by a tenth or more (their warps pay two or four dependent steps in the hand-off
+    // instead of one), and the sequence has to be long enough for their wider tiles
+    for (int s = 2; s <= 4; s *= 2) {
+        const long long k = fullest(s);
+        const double time = k >= 2 ? (double)k / s : (1.0 / s) / 0.74;
+        if (time < 0.9 * best_time && T >= 8 * kTb * s) {
+            best = s;
+            best_time = time;
         }
     }
+    // Segments: n blocks take n / (2 SMs) rounds of two resident teams each, a last round with a lone team on an SM 0.68 of
+    // a full one; every round of a cut launch pays for set-up, first loads and the drain of the ring (about 1.5 us; 3 us on
+    // 16-channel strips). A strip is cut only where the strips alone fill the GPU, so that a segment finds its predecessor
+    // finished. B = 4 x 8192 x 2560 with positions, us by (channels, segments): (64, 1) 222, (32, 1) 200, (32, 2) 166, (32, 4) 133,
+    // (32, 8) 166, (16, 1) 165, (16, 4) 180; 16 channels uncut were the choice before.
+    if (!segments || best == 0) return best;
+    const double us_per_step_channel = 4.54e-4;          // of a resident pair of teams
+    auto estimate = [&](int s, int z) {
+        const long long n = strips(s) * z, rest = n % (2 * sms);
+        const double rounds = (double)(n / (2 * sms)) + (rest == 0 ? 0.0 : rest <= sms ? 0.68 : 1.0);
+        return rounds * ((double)T / z * (kCb / s) * us_per_step_channel + (z == 1 ? 0.0 : s < 4 ? 1.5 : 3.0));
+    };
+    // (positions slow the uncut narrow shapes down most, every strip reads them; without them a cut has to promise more:
+    // 3 x 5000 x 4096 109.6 us cut against 115.3 with positions, 105.7 against 101.4 without)
+    best_time = (positions ? 0.95 : 0.85) * estimate(best, 1);
+    for (int s = 1; s <= 4; s *= 2)
+        for (int z = 2; z <= 4; z *= 2)
+            if (strips(s) >= 2 * sms && T >= 1024 * z && estimate(s, z) < best_time) {
+                best = s;
+                best_time = estimate(s, z);
+                *segments = z;
+            }
     return best;
 }
 

@@ -756,14 +756,14 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     // Chunks over caches of different lengths: a row block's work is then set by the tokens cached ahead of it as much as by
     // its place, and with the last row blocks first whatever their length the launch ends on a few heavy blocks. Five chunks
     // of 180 to 676 tokens over 720 to 4590: 131 us by place, 116 by work. Without a past the order of places is the order of
-    // work, one sequence needs no order, a launch of no more blocks than SMs has none, and beyond 128 sequences there are
-    // enough blocks to even themselves out. The ranking costs a block 0.4 us, finding equal pasts 0.15 (864 blocks of six
+    // work, one sequence needs no order, launches of one or two blocks per SM have little to order (two chunks of up to 522
+    // tokens, 160 blocks: 21.8 us by place, 22.3 by work), and beyond 128 sequences there are enough blocks to even themselves out. The ranking costs a block 0.4 us, finding equal pasts 0.15 (864 blocks of six
     // prompts: 101.7, 106.2 and 103 us); where the cache has no room for a tile ahead of the chunk (a prompt that fills its
     // cache) nobody looks.
     bool ranked = kv.past && d_past_lens && B > 1 && B <= 32 * kLaneSeqs;
     if (ranked) {
         const long long slots = kv.paged ? (long long)kv.paged->table_stride * kv.past->max_len : kv.past->max_len;
-        ranked = slots - S_max >= kRows && (long long)p.n_qblocks * (p.pair_heads ? Hq / 2 : Hq) * B > sm_count();
+        ranked = slots - S_max >= kRows && (long long)p.n_qblocks * (p.pair_heads ? Hq / 2 : Hq) * B > 2 * sm_count();
     }
     if (ranked)
         return D == 128 ? launch_t<128, true>(tq, tk, tv, to, tkc, tvc, p, stream) : launch_t<64, true>(tq, tk, tv, to, tkc, tvc, p, stream);

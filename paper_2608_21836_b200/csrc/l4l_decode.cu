@@ -37,6 +37,7 @@ namespace {
 // The kernel comes in two shapes, W = 4 or 8 consumer warps. A tile is 16*W tokens (each consumer warp takes
 // 16 of them); with W = 4 two CTAs share an SM, with W = 8 one CTA owns it and streams ranges twice as long,
 // so that fewer sequences are cut between CTAs. W + 2 warps in all: consumers, producer, finisher.
+constexpr int kTailRows = 32;                // tokens per box of the maps for a mostly empty last tile
 constexpr int kPostRing = 16;               // pieces a producer can be ahead of its finisher (ring size)
 constexpr size_t kTicketBytes = kCounterBytes;  // the ticket counters: 32768 (sequence, KV head) pairs per launch
 constexpr int kMaxB = 384;                 // sequences per launch (prefix sums and lengths live in shared memory)
@@ -119,7 +120,7 @@ struct DecodeParams {
     const int32_t *block_table;
     int table_stride, page_size, page_shift, num_pages;
     int page_box;             // paged: tokens per box of tmap_k / tmap_v (divides the tile, never straddles a page)
-    int tail_rows;            // tokens per box of tmap_k_tail / tmap_v_tail (32, or the page size if that is smaller)
+    int small_pages;          // pages of 16 or 32 tokens: every box is a page
     int page_loads;           // tmap_k / tmap_v bring a whole page, both halves, per load (bf16, head_dim 128, pages of 16 or 32)
     int B, Hq, Hkv, G, min_tiles, nsplit, max_kv_len;
     int stream_once;          // load K/V with the L2 evict-first policy (large caches)
@@ -355,81 +356,101 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                 for (int tile = tile_begin; tile < tile_end; ++tile, ++it) {
                     const uint32_t s = it % C::kStages;
                     const uint32_t ph = (it / C::kStages) & 1u;
-                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
-                    TileMeta &mt = meta[s];
-                    mt.b = b; mt.kvh = kvh; mt.t0 = tile * kTileT; mt.piece = piece; mt.kv_len = len;
-                    mt.npieces = npieces;
-                    mt.flags = (tile == tile_begin ? kFlagFirst : 0) | (tile + 1 == tile_end ? kFlagLast : 0);
                     // the first tile of a piece also brings the group's query rows (contiguous in q)
                     const bool first = (tile == tile_begin);
-                    // The last tile of a sequence: if at most half of it holds tokens it is fetched in groups of
-                    // p.tail_rows tokens (a few small boxes, nothing past the group that holds the last token); else as
-                    // a whole tile like the others (one box; rows past the end of the sequence are never looked at
-                    // by the consumers, rows past the end of the cache arrive as zeros). With pages smaller than a
-                    // tile only the pages that hold tokens are fetched.
-                    const bool paged = p.block_table != nullptr;
+                    uint8_t *dst = stages + (size_t)s * C::kStageBytes;
+                    // What goes with a tile besides its K and V, and the bytes its barrier waits for. page_of_new: paged fused append,
+                    // the page of the newest token's slot (it lies in the last box fetched).
+                    auto announce = [&](uint32_t kv_bytes, int page_of_new) {
+                        TileMeta &mt = meta[s];
+                        mt.b = b; mt.kvh = kvh; mt.t0 = tile * kTileT; mt.piece = piece; mt.kv_len = len;
+                        mt.npieces = npieces;
+                        mt.flags = (first ? kFlagFirst : 0) | (tile + 1 == tile_end ? kFlagLast : 0);
+                        mt.pad = page_of_new;
+                        // with the rope fused into the step, the piece's first tile also brings the cos / sin rows of
+                        // the new token's position (kv_len - 1), if the table has it
+                        const bool with_rope = first && p.rope_cos != nullptr && len - 1 < p.rope_n_pos;
+                        const bool with_new = kNewBytes != 0 && p.k_new != nullptr && tile + 1 == tiles_b;   // the tile of the newest token
+                        mbar_arrive_expect_tx(&full[s], kv_bytes + (first ? q_bytes : 0u) + (with_rope ? kRopeBytes : 0u) +
+                                                            (with_new ? kNewBytes : 0u));
+                        if (with_new) {
+                            uint8_t *ns = q_slots + (size_t)s * q_stride + q_bytes + kRopeBytes;
+                            const size_t src = (size_t)b * p.new_sb + (size_t)kvh * p.new_sh;
+                            bulk_load_1d(ns, p.k_new + src, kNewBytes / 2, &full[s]);
+                            bulk_load_1d(ns + kNewBytes / 2, p.v_new + src, kNewBytes / 2, &full[s]);
+                        }
+                        if (first)
+                            bulk_load_1d(q_slots + (size_t)s * q_stride, p.q + ((size_t)b * p.Hq + (size_t)kvh * p.G) * D,
+                                         q_bytes, &full[s]);
+                        if (with_rope) {
+                            uint8_t *rs = q_slots + (size_t)s * q_stride + q_bytes;
+                            bulk_load_1d(rs, p.rope_cos + (size_t)(len - 1) * (D / 2), kRopeBytes / 2, &full[s]);
+                            bulk_load_1d(rs + kRopeBytes / 2, p.rope_sin + (size_t)(len - 1) * (D / 2), kRopeBytes / 2, &full[s]);
+                        }
+                    };
                     const int rem = len - tile * kTileT;
-                    // (a whole tile of a contiguous cache, which is nearly every tile, is one box: no division on that path)
-                    bool by_groups = false;
-                    int box_rows = kTileT, n_box = 1;
-                    if (rem < kTileT || paged) {
-                        const int groups = (rem + p.tail_rows - 1) / p.tail_rows;
-                        by_groups = rem < kTileT && groups * p.tail_rows * 2 <= kTileT;
-                        box_rows = by_groups ? p.tail_rows : (paged ? p.page_box : kTileT);
-                        n_box = by_groups ? groups : ((rem >= kTileT || box_rows == kTileT) ? kTileT / box_rows
-                                                                                              : (rem + box_rows - 1) / box_rows);
+                    // A page id outside the pool makes its box read zeros, never memory.
+                    if (p.small_pages) {
+                        // Pages of 16 or 32 tokens: a box (or a pair of boxes) per page, only the pages that hold tokens. Their ids are
+                        // asked for together, ahead of the wait for the stage, which the latency then hides behind: B=48 ragged over
+                        // 16-token pages 67.2 us with one path for all layouts and the look-up behind the wait, 57.3 so.
+                        const int n_box = (min(rem, kTileT) + p.page_size - 1) >> p.page_shift;
+                        const int32_t *ids = p.block_table + (size_t)b * p.table_stride + ((tile * kTileT) >> p.page_shift);
+                        int page_of[kTileT / 16];
+#pragma unroll
+                        for (int bx = 0; bx < kTileT / 16; ++bx) page_of[bx] = bx < n_box ? __ldg(ids + bx) : 0;
+                        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+                        int last_page = page_of[0];
+#pragma unroll
+                        for (int bx = 1; bx < kTileT / 16; ++bx) last_page = bx < n_box ? page_of[bx] : last_page;
+                        announce((uint32_t)n_box * p.page_size * (uint32_t)C::kTokBytes * C::kHalves * 2u, last_page);
+#pragma unroll
+                        for (int bx = 0; bx < kTileT / 16; ++bx) {
+                            if (bx >= n_box) break;
+                            if constexpr (C::kHalves == 2) {
+                                if (p.page_loads) {
+                                    uint8_t *pb = dst + bx * p.page_size * 256;    // [half][page tokens][128 bytes]
+                                    tma_load_5d_policy(pb, &tmap_k, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
+                                    tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
+                                    continue;
+                                }
+                            }
+                            order_coords(p.coord, 0, kvh, page_of[bx], c1, c2, c3);
+                            uint8_t *db = dst + bx * p.page_size * C::kTokBytes;   // whole 8-row groups: the swizzle phase is kept
+#pragma unroll
+                            for (int hf = 0; hf < C::kHalves; ++hf) {
+                                tma_load_4d_policy(db + hf * C::kHalfBytes, &tmap_k, &full[s], hf * C::kBoxD, c1, c2, c3, stream_policy);
+                                tma_load_4d_policy(db + C::kTileBytes + hf * C::kHalfBytes, &tmap_v, &full[s], hf * C::kBoxD, c1, c2, c3, stream_policy);
+                            }
+                        }
+                        continue;
                     }
-                    // Neither a box nor a group straddles pages: page sizes are powers of two >= 16 and p.tail_rows is at
-                    // most the page size. A page id outside the pool makes the box read zeros, never memory.
+                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+                    // The last tile of a sequence: if at most half of it holds tokens it is fetched in groups of 32 tokens (a few
+                    // small boxes, nothing past the group that holds the last token); else as a whole tile like the others (one
+                    // box; rows past the end of the sequence are never looked at by the consumers, rows past the end of the cache
+                    // arrive as zeros). Neither a box nor a group straddles pages.
+                    const bool paged = p.block_table != nullptr;
+                    const int groups = (rem + kTailRows - 1) / kTailRows;
+                    const bool by_groups = rem < kTileT && groups * kTailRows * 2 <= kTileT;
+                    const int box_rows = by_groups ? kTailRows : (paged ? p.page_box : kTileT);
+                    const int n_box = by_groups ? groups : ((rem >= kTileT || box_rows == kTileT) ? kTileT / box_rows
+                                                                                                    : (rem + box_rows - 1) / box_rows);
                     const int32_t *pages = paged ? p.block_table + (size_t)b * p.table_stride : nullptr;
                     const CUtensorMap *tk = by_groups ? &tmap_k_tail : &tmap_k;
                     const CUtensorMap *tv = by_groups ? &tmap_v_tail : &tmap_v;
-                    int page_of[kTileT / 16];                    // looked up together: independent loads
+                    int page_of[kTileT / 32], last_page = 0;     // looked up together: independent loads
 #pragma unroll
-                    for (int bx = 0; bx < kTileT / 16; ++bx)
+                    for (int bx = 0; bx < kTileT / 32; ++bx) {
                         page_of[bx] = (paged && bx < n_box) ? __ldg(pages + ((tile * kTileT + bx * box_rows) >> p.page_shift)) : b;
-                    // paged fused append: the page of the newest token's slot (it lies in the last box fetched)
-                    if (paged && p.k_new != nullptr && tile + 1 == tiles_b) {
-                        int pg = page_of[0];
+                        last_page = bx < n_box ? page_of[bx] : last_page;
+                    }
+                    announce((uint32_t)n_box * box_rows * (uint32_t)C::kTokBytes * C::kHalves * 2u, last_page);
 #pragma unroll
-                        for (int bx = 1; bx < kTileT / 16; ++bx) pg = (bx < n_box) ? page_of[bx] : pg;
-                        mt.pad = pg;
-                    }
-                    const uint32_t kv_bytes = (uint32_t)n_box * box_rows * (uint32_t)C::kTokBytes * C::kHalves * 2u;
-                    // with the rope fused into the step, the piece's first tile also brings the cos / sin rows of
-                    // the new token's position (kv_len - 1), if the table has it
-                    const bool with_rope = first && p.rope_cos != nullptr && len - 1 < p.rope_n_pos;
-                    const bool with_new = kNewBytes != 0 && p.k_new != nullptr && tile + 1 == tiles_b;   // the tile of the newest token
-                    mbar_arrive_expect_tx(&full[s], kv_bytes + (first ? q_bytes : 0u) + (with_rope ? kRopeBytes : 0u) +
-                                                        (with_new ? kNewBytes : 0u));
-                    if (with_new) {
-                        uint8_t *ns = q_slots + (size_t)s * q_stride + q_bytes + kRopeBytes;
-                        const size_t src = (size_t)b * p.new_sb + (size_t)kvh * p.new_sh;
-                        bulk_load_1d(ns, p.k_new + src, kNewBytes / 2, &full[s]);
-                        bulk_load_1d(ns + kNewBytes / 2, p.v_new + src, kNewBytes / 2, &full[s]);
-                    }
-                    if (first)
-                        bulk_load_1d(q_slots + (size_t)s * q_stride, p.q + ((size_t)b * p.Hq + (size_t)kvh * p.G) * D,
-                                     q_bytes, &full[s]);
-                    if (with_rope) {
-                        uint8_t *rs = q_slots + (size_t)s * q_stride + q_bytes;
-                        bulk_load_1d(rs, p.rope_cos + (size_t)(len - 1) * (D / 2), kRopeBytes / 2, &full[s]);
-                        bulk_load_1d(rs + kRopeBytes / 2, p.rope_sin + (size_t)(len - 1) * (D / 2), kRopeBytes / 2, &full[s]);
-                    }
-                    uint8_t *dst = stages + (size_t)s * C::kStageBytes;
-#pragma unroll
-                    for (int bx = 0; bx < kTileT / 16; ++bx) {
+                    for (int bx = 0; bx < kTileT / 32; ++bx) {
                         if (bx >= n_box) break;
                         int tt = tile * kTileT + bx * box_rows;
                         if (paged) tt &= p.page_size - 1;
-                        if constexpr (C::kHalves == 2) {
-                            if (p.page_loads) {
-                                uint8_t *pb = dst + bx * box_rows * 256;   // [half][page tokens][128 bytes]
-                                tma_load_5d_policy(pb, &tmap_k, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
-                                tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, tt, 0, kvh, page_of[bx], stream_policy);
-                                continue;
-                            }
-                        }
                         order_coords(p.coord, tt / C::kTokPerRow, kvh, page_of[bx], c1, c2, c3);
                         uint8_t *db = dst + bx * box_rows * C::kTokBytes;  // whole 8-row groups: the swizzle phase is kept
 #pragma unroll
@@ -1268,13 +1289,14 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         // power of two (96 tokens) over larger pages in 32-token boxes (page sizes are powers of two >= 16)
         int box_t = kTileT;
         if (paged) box_t = (kTileT % cache.max_len == 0) ? cache.max_len : (cache.max_len % kTileT == 0 ? kTileT : 32);
-        const int tail_rows = (paged && cache.max_len < 32) ? cache.max_len : 32;
+        const int tail_rows = (paged && cache.max_len < 32) ? cache.max_len : kTailRows;
         // what the maps see as a row: a token, or (fp8 at head_dim 64) a pair of tokens
         const int tpr = pair_rows ? 2 : 1, map_d = pair_rows ? 128 : D;
         const int64_t map_rows = cache.max_len / tpr, map_st = cache.stride_t * tpr;
         // Pages of 16 or 32 tokens at head_dim 128: one load per page instead of one per 64-column half. What bounds such
-        // pools is the loads per tile (a 2 KB box holds the TMA unit for about 80 ns): B=48 ragged over 16-token pages 85.6
-        // us by halves, 69.7 by pages; B=32 over 32-token pages 63.5 and 57.5. Pages of 64 have half as many boxes already.
+        // pools is the loads per tile (a 2 KB box holds the TMA unit for about 80 ns): B=48 ragged over 16-token pages 85.3
+        // us by halves, 69.3 by pages (57.9 with the page ids looked up ahead); B=32 over 32-token pages 62.9, 57.5 and 55.8.
+        // Pages of 64 have half as many boxes already.
         const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr) &&
                                 make_tmap_page(&tk, kb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) &&
                                 make_tmap_page(&tv, vb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b);
@@ -1319,7 +1341,7 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         p.page_size = paged ? cache.max_len : 0;
         p.page_box = box_t;
         p.num_pages = paged ? paged->num_pages : 0;
-        p.tail_rows = tail_rows;
+        p.small_pages = paged && cache.max_len <= 32 ? 1 : 0;
         p.page_loads = page_loads ? 1 : 0;
         p.page_shift = 0;
         while (paged && (1 << p.page_shift) < cache.max_len) ++p.page_shift;

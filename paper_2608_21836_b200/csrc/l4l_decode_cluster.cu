@@ -210,7 +210,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
             for (int it = 0; it < n_mine; ++it) {
                 const int tile = t_begin + it;
                 const uint32_t s = it % p.stages, ph = (it / p.stages) & 1u;
-                if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
                 // The last tile of a sequence: if at most half of it holds tokens it comes in groups of p.tail_rows
                 // tokens (a few small boxes), else as a whole tile like the others (rows past the end of the sequence are
                 // never looked at, rows past the end of the cache arrive as zeros); with pages smaller than a tile only
@@ -221,6 +220,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                 const int box_rows = by_groups ? p.tail_rows : ((paged && p.page_size < kTileT) ? p.page_size : kTileT);
                 const int n_box = by_groups ? groups : ((rem >= kTileT || box_rows == kTileT) ? kTileT / box_rows
                                                                                               : (rem + box_rows - 1) / box_rows);
+                int page_of[kTileT / 16];                            // looked up together, ahead of the wait for the stage
+#pragma unroll
+                for (int bx = 0; bx < kTileT / 16; ++bx)
+                    page_of[bx] = (paged && bx < n_box) ? __ldg(pages + ((tile * kTileT + bx * box_rows) >> p.page_shift)) : b;
+                if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
                 const uint32_t kv_bytes = (uint32_t)n_box * box_rows * 128u * C::kHalves * 2u;
                 mbar_arrive_expect_tx(&full[s], kv_bytes + (it == 0 ? q_bytes + (with_rope ? kRopeBytes : 0u) +
                                                                               (p.k_new != nullptr ? kNewBytes : 0u) : 0u));
@@ -240,10 +244,6 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                 int c1, c2, c3;
                 const CUtensorMap *tk = by_groups ? &tmap_k_tail : &tmap_k;
                 const CUtensorMap *tv = by_groups ? &tmap_v_tail : &tmap_v;
-                int page_of[kTileT / 16];                            // looked up together: independent loads
-#pragma unroll
-                for (int bx = 0; bx < kTileT / 16; ++bx)
-                    page_of[bx] = (paged && bx < n_box) ? __ldg(pages + ((tile * kTileT + bx * box_rows) >> p.page_shift)) : b;
 #pragma unroll
                 for (int bx = 0; bx < kTileT / 16; ++bx) {
                     if (bx >= n_box) break;

@@ -88,7 +88,8 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qf)[D / 16][NB][2], 
 }
 
 // S^T (16 tokens x 8 NB heads) = K(tokens row0 .. row0 + 15) . Q^T. s[n]: [e] token row0 + r, [2 + e] token row0 + r + 8 of
-// head 8n + 2c + e. Even and odd k-steps are accumulated apart: two dependent chains of half the length.
+// head 8n + 2c + e. Even and odd k-steps are accumulated apart, two dependent chains of half the length (two blocks of heads
+// are two chains by themselves).
 template <int D, int NB>
 __device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, uint32_t half_bytes, int row0,
                                         float (&s)[NB][4])
@@ -107,12 +108,12 @@ __device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uin
         uint32_t a[4];
         ldmatrix_x4(k_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
 #pragma unroll
-        for (int n = 0; n < NB; ++n) mma_bf16_16816((ks & 1) ? odd[n] : s[n], a, qf[ks][n][0], qf[ks][n][1]);
+        for (int n = 0; n < NB; ++n) mma_bf16_16816((NB == 1 && (ks & 1)) ? odd[n] : s[n], a, qf[ks][n][0], qf[ks][n][1]);
     }
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] += odd[n][e];
+        for (int e = 0; e < 4; ++e) s[n][e] += NB == 1 ? odd[n][e] : 0.f;
 }
 
 // O^T += V(tokens row0 .. row0 + 15)^T . P^T
@@ -238,13 +239,13 @@ __device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], 
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
             mma_f16_16816(s[n], a, qf[2 * qd][n][0], qf[2 * qd][n][1]);
-            mma_f16_16816(odd[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
+            mma_f16_16816(NB == 1 ? odd[n] : s[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
         }
     }
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] += odd[n][e];
+        for (int e = 0; e < 4; ++e) s[n][e] += NB == 1 ? odd[n][e] : 0.f;
 }
 
 template <int D, int NB>

@@ -142,6 +142,12 @@ Workspace workspace_of(PyObject *o)
     return {t.data_ptr(), (size_t)t.numel() * t.element_size()};
 }
 
+// The library is called without the interpreter lock, as a ctypes call is: a launch may wait for room in the stream's queue.
+struct Unlocked {
+    PyThreadState *state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
 l4l_stream stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
 struct Dims { int B, S, Hq, D; };
@@ -159,9 +165,18 @@ int size_at(PyObject *o, const char *name, int dim) { return (int)tensor(o, name
         PyErr_Format(PyExc_TypeError, "%zd arguments instead of %d", n, (int)(count)); \
         return nullptr;                                                                \
     }
-#define L4L_RETURN(status)                  \
-    return PyLong_FromLong((long)(status)); \
-    END_HANDLE_TH_ERRORS
+// the call itself, on the current stream s and without the interpreter lock
+#define L4L_CALL(expr)                           \
+    {                                            \
+        const l4l_stream s = stream();           \
+        l4l_status st;                           \
+        {                                        \
+            Unlocked unlocked;                   \
+            st = (expr);                         \
+        }                                        \
+        return PyLong_FromLong((long)st);        \
+    }
+#define L4L_END END_HANDLE_TH_ERRORS
 
 // q, k, v, o, seq_lens, scale, workspace, cache_k, cache_v, lse
 PyObject *prefill(PyObject *, PyObject *const *a, Py_ssize_t n)
@@ -171,11 +186,12 @@ PyObject *prefill(PyObject *, PyObject *const *a, Py_ssize_t n)
     const int Hkv = size_at(a[1], "k", 2);
     float *lse = lse_of(a[9], {d.B, d.Hq, d.S}, "[B, Hq, S]");
     const l4l_tensor4 q = tensor4(a[0], "q"), k = tensor4(a[1], "k"), v = tensor4(a[2], "v"), o = tensor4(a[3], "o");
-    const Cache c = cache_of(a[7], a[8], false, false);
+    const l4l_kv_cache cache = cache_of(a[7], a[8], false, false).contiguous();
     const int32_t *lens = i32(a[4], "seq_lens");
     const Workspace w = workspace_of(a[6]);
-    L4L_RETURN(l4l_attn_prefill(q, k, v, o, c.contiguous(), lens, d.S, d.B, d.Hq, Hkv, d.D, as_float(a[5]), lse, w.ptr, w.bytes,
-                                stream()))
+    const float scale = as_float(a[5]);
+    L4L_CALL(l4l_attn_prefill(q, k, v, o, cache, lens, d.S, d.B, d.Hq, Hkv, d.D, scale, lse, w.ptr, w.bytes, s))
+    L4L_END
 }
 
 // q, o, cache_k, cache_v, past_lens, q_lens, scale, workspace, lse
@@ -186,11 +202,12 @@ PyObject *prefill_chunk(PyObject *, PyObject *const *a, Py_ssize_t n)
     const int Hkv = size_at(a[2], "cache_k", 1);
     float *lse = lse_of(a[8], {d.B, d.Hq, d.S}, "[B, Hq, S]");
     const l4l_tensor4 q = tensor4(a[0], "q"), o = tensor4(a[1], "o");
-    const Cache c = cache_of(a[2], a[3], false, false);
+    const l4l_kv_cache cache = cache_of(a[2], a[3], false, false).contiguous();
     const int32_t *past = i32(a[4], "past_lens"), *lens = i32(a[5], "q_lens");
     const Workspace w = workspace_of(a[7]);
-    L4L_RETURN(l4l_attn_prefill_chunk(q, o, c.contiguous(), past, lens, d.S, d.B, d.Hq, Hkv, d.D, as_float(a[6]), lse, w.ptr,
-                                      w.bytes, stream()))
+    const float scale = as_float(a[6]);
+    L4L_CALL(l4l_attn_prefill_chunk(q, o, cache, past, lens, d.S, d.B, d.Hq, Hkv, d.D, scale, lse, w.ptr, w.bytes, s))
+    L4L_END
 }
 
 // q, k_new, v_new, o, cache_k, cache_v, past_lens, q_lens, scale, workspace, lse, block_table
@@ -207,10 +224,14 @@ PyObject *prefill_chunk_append(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Table t = paged ? table_of(a[11], d.B) : Table{nullptr, 0};
     const l4l_tensor4 q = tensor4(a[0], "q"), k = tensor4(a[1], "k_new"), v = tensor4(a[2], "v_new"), o = tensor4(a[3], "o");
     const Cache c = cache_of(a[4], a[5], paged, false);
-    L4L_RETURN(paged ? l4l_attn_prefill_chunk_paged_append(q, k, v, o, c.paged(), t.ids, t.stride, past, lens, d.S, d.B, d.Hq, Hkv, d.D,
-                                                           scale, lse, w.ptr, w.bytes, stream())
-                     : l4l_attn_prefill_chunk_append(q, k, v, o, c.contiguous(), past, lens, d.S, d.B, d.Hq, Hkv, d.D, scale, lse, w.ptr,
-                                                     w.bytes, stream()))
+    if (paged) {
+        const l4l_paged_kv pool = c.paged();
+        L4L_CALL(l4l_attn_prefill_chunk_paged_append(q, k, v, o, pool, t.ids, t.stride, past, lens, d.S, d.B, d.Hq, Hkv, d.D, scale, lse,
+                                                     w.ptr, w.bytes, s))
+    }
+    const l4l_kv_cache cache = c.contiguous();
+    L4L_CALL(l4l_attn_prefill_chunk_append(q, k, v, o, cache, past, lens, d.S, d.B, d.Hq, Hkv, d.D, scale, lse, w.ptr, w.bytes, s))
+    L4L_END
 }
 
 // q, k_new, v_new, cache_k, cache_v, pos, n_new, cos, sin, q_weight, k_weight, eps
@@ -220,12 +241,13 @@ PyObject *rope_kv_append(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Dims d = dims4(a[0], "q");
     const int Hkv = size_at(a[1], "k_new", 2), n_pos = size_at(a[7], "cos", 0);
     const l4l_tensor4 q = tensor4(a[0], "q"), k = tensor4(a[1], "k_new"), v = tensor4(a[2], "v_new");
-    const Cache c = cache_of(a[3], a[4], false, false);
+    const l4l_kv_cache cache = cache_of(a[3], a[4], false, false).contiguous();
     const int32_t *pos = i32(a[5], "pos"), *n_new = i32(a[6], "n_new");
     const float *cs = f32(a[7], "cos", {n_pos, d.D / 2}), *sn = f32(a[8], "sin", {n_pos, d.D / 2});
     const float *qw = f32(a[9], "q_weight", {d.D}), *kw = f32(a[10], "k_weight", {d.D});
-    L4L_RETURN(l4l_rope_kv_append(q, k, v, c.contiguous(), pos, n_new, d.S, d.B, d.Hq, Hkv, d.D, cs, sn, n_pos, qw, kw, as_float(a[11]),
-                                  stream()))
+    const float eps = as_float(a[11]);
+    L4L_CALL(l4l_rope_kv_append(q, k, v, cache, pos, n_new, d.S, d.B, d.Hq, Hkv, d.D, cs, sn, n_pos, qw, kw, eps, s))
+    L4L_END
 }
 
 // Every decode step: q, o, k, v, k_scale, v_scale (fp8 caches, else None), block_table (paged, else None), k_new, v_new
@@ -274,35 +296,41 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
         vs = f32(a[5], "v_scale", {Hkv});
     }
     void *qp = q.data_ptr(), *op = o.data_ptr();
+    const l4l_kv_cache cache = c.contiguous();
+    const l4l_paged_kv pool = paged ? c.paged() : l4l_paged_kv{};
     const l4l_stream s = stream();
     l4l_status st;
+    {
+    Unlocked unlocked;
     if (fp8 && rope)
-        st = paged ? l4l_attn_decode_paged_rope_append_fp8(qp, op, c.paged(), ks, vs, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale,
+        st = paged ? l4l_attn_decode_paged_rope_append_fp8(qp, op, pool, ks, vs, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale,
                                                            cs, sn, n_pos, qw, kw, eps, lse, w.ptr, w.bytes, s)
-                   : l4l_attn_decode_rope_append_fp8(qp, op, c.contiguous(), ks, vs, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn,
+                   : l4l_attn_decode_rope_append_fp8(qp, op, cache, ks, vs, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn,
                                                      n_pos, qw, kw, eps, lse, w.ptr, w.bytes, s);
     else if (fp8 && append)
-        st = paged ? l4l_attn_decode_paged_append_fp8(qp, op, c.paged(), ks, vs, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse,
+        st = paged ? l4l_attn_decode_paged_append_fp8(qp, op, pool, ks, vs, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse,
                                                       w.ptr, w.bytes, s)
-                   : l4l_attn_decode_append_fp8(qp, op, c.contiguous(), ks, vs, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
+                   : l4l_attn_decode_append_fp8(qp, op, cache, ks, vs, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
                                                 w.bytes, s);
     else if (fp8)
-        st = paged ? l4l_attn_decode_paged_fp8(qp, op, c.paged(), ks, vs, t.ids, t.stride, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
+        st = paged ? l4l_attn_decode_paged_fp8(qp, op, pool, ks, vs, t.ids, t.stride, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
                                                w.bytes, s)
-                   : l4l_attn_decode_fp8(qp, op, c.contiguous(), ks, vs, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
+                   : l4l_attn_decode_fp8(qp, op, cache, ks, vs, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
     else if (rope)
-        st = paged ? l4l_attn_decode_paged_rope_append(qp, op, c.paged(), t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn,
+        st = paged ? l4l_attn_decode_paged_rope_append(qp, op, pool, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn,
                                                        n_pos, qw, kw, eps, lse, w.ptr, w.bytes, s)
-                   : l4l_attn_decode_rope_append(qp, op, c.contiguous(), kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn, n_pos, qw, kw,
+                   : l4l_attn_decode_rope_append(qp, op, cache, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, cs, sn, n_pos, qw, kw,
                                                  eps, lse, w.ptr, w.bytes, s);
     else if (append)
-        st = paged ? l4l_attn_decode_paged_append(qp, op, c.paged(), t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
+        st = paged ? l4l_attn_decode_paged_append(qp, op, pool, t.ids, t.stride, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr,
                                                   w.bytes, s)
-                   : l4l_attn_decode_append(qp, op, c.contiguous(), kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
+                   : l4l_attn_decode_append(qp, op, cache, kn, vn, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
     else
-        st = paged ? l4l_attn_decode_paged(qp, op, c.paged(), t.ids, t.stride, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s)
-                   : l4l_attn_decode(qp, op, c.contiguous(), lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
-    L4L_RETURN(st)
+        st = paged ? l4l_attn_decode_paged(qp, op, pool, t.ids, t.stride, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s)
+                   : l4l_attn_decode(qp, op, cache, lens, max_len, B, Hq, Hkv, D, scale, lse, w.ptr, w.bytes, s);
+    }
+    return PyLong_FromLong((long)st);
+    L4L_END
 }
 
 // x, gate_x, gate_a, a_param, state, y, workspace, position, seq_lens
@@ -332,7 +360,8 @@ PyObject *rglru_scan(PyObject *, PyObject *const *a, Py_ssize_t n)
     const int32_t *lens = i32(a[8], "seq_lens");
     float *state = f32(a[4], "state", {B, W});
     const Workspace w = workspace_of(a[6]);
-    L4L_RETURN(l4l_rglru_scan(ptr[0], ptr[1], ptr[2], ap, position, lens, state, ptr[3], B, T, W, w.ptr, w.bytes, stream()))
+    L4L_CALL(l4l_rglru_scan(ptr[0], ptr[1], ptr[2], ap, position, lens, state, ptr[3], B, T, W, w.ptr, w.bytes, s))
+    L4L_END
 }
 
 #define L4L_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}

@@ -393,7 +393,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     if (p.small_pages) {
                         // Pages of 16 or 32 tokens: a box (or a pair of boxes) per page, only the pages that hold tokens. Their ids are
                         // asked for together, ahead of the wait for the stage, which the latency then hides behind: B=48 ragged over
-                        // 16-token pages 67.2 us with one path for all layouts and the look-up behind the wait, 57.3 so.
+                        // 16-token pages 67.2 us with one path for all layouts and the look-up behind the wait, 55.4 so.
                         const int n_box = (min(rem, kTileT) + p.page_size - 1) >> p.page_shift;
                         const int32_t *ids = p.block_table + (size_t)b * p.table_stride + ((tile * kTileT) >> p.page_shift);
                         int page_of[kTileT / 16];
@@ -407,20 +407,17 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
 #pragma unroll
                         for (int bx = 0; bx < kTileT / 16; ++bx) {
                             if (bx >= n_box) break;
+                            // (one form per kernel: copies of both, eight times each, cost a contiguous launch 2 us when its code comes
+                            // from a cold L2)
                             if constexpr (C::kHalves == 2) {
-                                if (p.page_loads) {
-                                    uint8_t *pb = dst + bx * p.page_size * 256;    // [half][page tokens][128 bytes]
-                                    tma_load_5d_policy(pb, &tmap_k, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
-                                    tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
-                                    continue;
-                                }
-                            }
-                            order_coords(p.coord, 0, kvh, page_of[bx], c1, c2, c3);
-                            uint8_t *db = dst + bx * p.page_size * C::kTokBytes;   // whole 8-row groups: the swizzle phase is kept
-#pragma unroll
-                            for (int hf = 0; hf < C::kHalves; ++hf) {
-                                tma_load_4d_policy(db + hf * C::kHalfBytes, &tmap_k, &full[s], hf * C::kBoxD, c1, c2, c3, stream_policy);
-                                tma_load_4d_policy(db + C::kTileBytes + hf * C::kHalfBytes, &tmap_v, &full[s], hf * C::kBoxD, c1, c2, c3, stream_policy);
+                                uint8_t *pb = dst + bx * p.page_size * 256;        // [half][page tokens][128 bytes]
+                                tma_load_5d_policy(pb, &tmap_k, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
+                                tma_load_5d_policy(pb + C::kTileBytes, &tmap_v, &full[s], 0, 0, 0, kvh, page_of[bx], stream_policy);
+                            } else {
+                                order_coords(p.coord, 0, kvh, page_of[bx], c1, c2, c3);
+                                uint8_t *db = dst + bx * p.page_size * C::kTokBytes;   // whole 8-row groups: the swizzle phase is kept
+                                tma_load_4d_policy(db, &tmap_k, &full[s], 0, c1, c2, c3, stream_policy);
+                                tma_load_4d_policy(db + C::kTileBytes, &tmap_v, &full[s], 0, c1, c2, c3, stream_policy);
                             }
                         }
                         continue;
@@ -1295,12 +1292,13 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         const int64_t map_rows = cache.max_len / tpr, map_st = cache.stride_t * tpr;
         // Pages of 16 or 32 tokens at head_dim 128: one load per page instead of one per 64-column half. What bounds such
         // pools is the loads per tile (a 2 KB box holds the TMA unit for about 80 ns): B=48 ragged over 16-token pages 85.3
-        // us by halves, 69.3 by pages (57.9 with the page ids looked up ahead); B=32 over 32-token pages 62.9, 57.5 and 55.8.
+        // us by halves, 69.3 by pages (55.4 with the page ids looked up ahead); B=32 over 32-token pages 62.9, 57.5 and 55.8.
         // Pages of 64 have half as many boxes already.
-        const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr) &&
-                                make_tmap_page(&tk, kb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) &&
-                                make_tmap_page(&tv, vb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b);
+        const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr);
         if (page_loads) {
+            if (!make_tmap_page(&tk, kb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) ||
+                !make_tmap_page(&tv, vb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b))
+                return L4L_ERR_CUDA;
             tk_tail = tk;            // groups of the last tile are pages too
             tv_tail = tv;
             coord = TmapCoord{};

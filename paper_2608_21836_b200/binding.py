@@ -161,6 +161,18 @@ def load() -> ctypes.CDLL:
 
 
 _native = None
+# what a decode call is and which shapes it looks at (enum Form of csrc/l4l_marshal.cpp)
+_NEW_SHAPES, _LSE_SHAPE, _APPEND, _ROPE, _FP8, _PAGED, _MAYBE_PAGED = (1 << i for i in range(7))
+_DECODE = _LSE_SHAPE
+_DECODE_APPEND = _APPEND | _NEW_SHAPES | _LSE_SHAPE
+_DECODE_ROPE = _APPEND | _ROPE
+_DECODE_PAGED = _PAGED | _LSE_SHAPE
+_DECODE_PAGED_APPEND = _PAGED | _APPEND | _NEW_SHAPES | _LSE_SHAPE
+_DECODE_PAGED_ROPE = _PAGED | _APPEND | _ROPE | _NEW_SHAPES
+_DECODE_FP8 = _FP8 | _LSE_SHAPE
+_DECODE_APPEND_FP8 = _FP8 | _APPEND | _MAYBE_PAGED | _NEW_SHAPES
+_DECODE_ROPE_FP8 = _FP8 | _APPEND | _ROPE | _MAYBE_PAGED | _NEW_SHAPES
+_DECODE_PAGED_FP8 = _FP8 | _PAGED
 
 
 def _load_native():
@@ -262,7 +274,7 @@ def l4l_attn_prefill(q, k, v, o, seq_lens, scale: float, workspace, cache_k=None
 def l4l_attn_decode(q, o, cache_k, cache_v, kv_lens, max_kv_len: int, scale: float, workspace, lse=None) -> None:
     """q,o dense [B,Hq,D]; cache [B,Hkv,max_len,D]; kv_lens CUDA int32 [B] (current token included)."""
     st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, None, None, kv_lens, max_kv_len,
-                                            scale, None, None, None, None, 0.0, workspace, lse, 2)
+                                            scale, None, None, None, None, 0.0, workspace, lse, _DECODE)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode")
 
@@ -294,7 +306,7 @@ def l4l_attn_decode_append(q, o, cache_k, cache_v, k_new, v_new, kv_lens, max_kv
     """One launch per decode step: writes k_new / v_new ([B,1,Hkv,D]) into cache slot kv_lens[b]-1 and attends
     over slots 0..kv_lens[b]-1. Same result as l4l_kv_append followed by l4l_attn_decode."""
     st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, k_new, v_new, kv_lens,
-                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 3)
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, _DECODE_APPEND)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_append")
 
@@ -370,7 +382,7 @@ def l4l_attn_decode_paged(q, o, pool_k, pool_v, block_table, kv_lens, max_kv_len
                           lse=None) -> None:
     """Decode over a paged cache. q,o dense [B,Hq,D]; pools [pages,Hkv,page_size,D]; block_table CUDA int32 [B, n]."""
     st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, None, None, kv_lens,
-                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 2)
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, _DECODE_PAGED)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged")
 
@@ -381,7 +393,7 @@ def l4l_attn_decode_paged_append(q, o, pool_k, pool_v, block_table, k_new, v_new
     (the page the block table names) and are attended with the rest. Same result as l4l_kv_append_paged followed by
     l4l_attn_decode_paged."""
     st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, k_new, v_new, kv_lens,
-                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 3)
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, _DECODE_PAGED_APPEND)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_append")
 
@@ -392,7 +404,7 @@ def l4l_attn_decode_paged_rope_append(q, o, pool_k, pool_v, block_table, k_new, 
     """l4l_attn_decode_rope_append over a paged cache: rotation (+ optional RMS norm) of q and k_new at position
     kv_lens - 1, write of the rotated k and of v_new into the page slot, attention: one launch."""
     st = (_native or _load_native()).decode(q, o, pool_k, pool_v, None, None, block_table, k_new, v_new, kv_lens,
-                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, 1)
+                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, _DECODE_PAGED_ROPE)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_rope_append")
 
@@ -405,7 +417,7 @@ def l4l_attn_decode_rope_append_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, 
     written to slot kv_lens - 1, the rotated q attends. With block_table, the caches are a page pool."""
     st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, block_table, k_new, v_new,
                                             kv_lens, max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace,
-                                            lse, 1)
+                                            lse, _DECODE_ROPE_FP8)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_rope_append_fp8")
 
@@ -437,7 +449,7 @@ def l4l_attn_decode_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, kv_lens, max
     """Decode over an fp8 (e4m3) cache with per-KV-head scales. q,o dense bf16 [B,Hq,D] (at head_dim 64 the cache's
     token rows must be dense and even in number)."""
     st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, None, None, None, kv_lens,
-                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, 2)
+                                            max_kv_len, scale, None, None, None, None, 0.0, workspace, lse, _DECODE_FP8)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_fp8")
 
@@ -465,7 +477,7 @@ def l4l_attn_decode_paged_fp8(q, o, pool_k8, pool_v8, k_scale, v_scale, block_ta
     """Decode over an fp8 page pool [pages, Hkv, page_size, 128] (uint8 / float8_e4m3fn) read through a block table."""
     st = (_native or _load_native()).decode(q, o, pool_k8, pool_v8, k_scale, v_scale, block_table, None, None,
                                             kv_lens, max_kv_len, scale, None, None, None, None, 0.0, workspace, lse,
-                                            0)
+                                            _DECODE_PAGED_FP8)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_paged_fp8")
 
@@ -477,7 +489,7 @@ def l4l_attn_decode_append_fp8(q, o, cache_k8, cache_v8, k_scale, v_scale, k_new
     cache_v8 are a page pool [pages, Hkv, page_size, 128]."""
     st = (_native or _load_native()).decode(q, o, cache_k8, cache_v8, k_scale, v_scale, block_table, k_new, v_new,
                                             kv_lens, max_kv_len, scale, None, None, None, None, 0.0, workspace, lse,
-                                            1)
+                                            _DECODE_APPEND_FP8)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_append_fp8")
 
@@ -556,6 +568,6 @@ def l4l_attn_decode_rope_append(q, o, cache_k, cache_v, k_new, v_new, kv_lens, m
     update and attention. q,o dense [B,Hq,D] (q is not modified); k_new, v_new [B,1,Hkv,D]; cos, sin CUDA float32
     [n_pos, D/2]."""
     st = (_native or _load_native()).decode(q, o, cache_k, cache_v, None, None, None, k_new, v_new, kv_lens,
-                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, 0)
+                                            max_kv_len, scale, cos, sin, q_weight, k_weight, eps, workspace, lse, _DECODE_ROPE)
     if st != L4L_OK:
         raise L4LError(st, "l4l_attn_decode_rope_append")

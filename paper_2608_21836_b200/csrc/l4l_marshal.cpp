@@ -250,14 +250,26 @@ PyObject *rope_kv_append(PyObject *, PyObject *const *a, Py_ssize_t n)
     L4L_END
 }
 
-// Every decode step: q, o, k, v, k_scale, v_scale (fp8 caches, else None), block_table (paged, else None), k_new, v_new
-// (fused append, else None), kv_lens, max_kv_len, scale, cos, sin, q_weight, k_weight, eps (rope, else None), workspace, lse,
-// and which shapes are looked at: 1 those of k_new and v_new, 2 that of lse
+// What a decode call is, said by the entry point: an argument that is missing never makes it another operation.
+// (binding.py has the same values.)
+enum Form {
+    kNewShapes = 1, kLseShape = 2,                               // shapes that are looked at: those of k_new and v_new, that of lse
+    kAppend = 4, kRope = 8, kFp8 = 16, kPaged = 32,              // the operation
+    kMaybePaged = 64,                                            // paged where a block table is given
+};
+
+// Every decode step: q, o, k, v, k_scale, v_scale (fp8 caches), block_table (paged), k_new, v_new (fused append), kv_lens,
+// max_kv_len, scale, cos, sin, q_weight, k_weight, eps (rope), workspace, lse, form. What the form has no use for is None.
 PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     L4L_ARGS(20)
-    const int checks = as_int(a[19]);
-    const bool fp8 = !is_none(a[4]), paged = !is_none(a[6]), append = !is_none(a[7]), rope = !is_none(a[12]);
+    const int form = as_int(a[19]);
+    const bool fp8 = form & kFp8, append = form & kAppend, rope = form & kRope;
+    const bool paged = (form & kPaged) || ((form & kMaybePaged) && !is_none(a[6]));
+    // (a missing sin or scale is a null pointer, which the library refuses)
+    if (append) tensor(a[7], "k_new"), tensor(a[8], "v_new");
+    if (paged) tensor(a[6], "block_table");
+    if (rope) tensor(a[12], "cos");
     const Tensor &q = bf16(a[0], "q"), &o = bf16(a[1], "o");
     if (!(q.is_contiguous() && o.is_contiguous() && q.dim() == 3 && q.sizes() == o.sizes())) value_error("q and o must be dense [B, Hq, D]");
     const int B = (int)q.size(0), Hq = (int)q.size(1), D = (int)q.size(2);
@@ -267,13 +279,13 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
     l4l_tensor4 kn{}, vn{};
     if (append) {
         const int64_t want[4] = {B, 1, Hkv, D};
-        if ((checks & 1) && (tensor(a[7], "k_new").sizes() != at::IntArrayRef(want, 4) ||
-                             tensor(a[8], "v_new").sizes() != at::IntArrayRef(want, 4)))
+        if ((form & kNewShapes) && (tensor(a[7], "k_new").sizes() != at::IntArrayRef(want, 4) ||
+                                    tensor(a[8], "v_new").sizes() != at::IntArrayRef(want, 4)))
             value_error("k_new and v_new must be [B, 1, Hkv, D]");
         kn = tensor4(a[7], "k_new");
         vn = tensor4(a[8], "v_new");
     }
-    float *lse = (checks & 2) ? lse_of(a[18], {B, Hq}, "[B, Hq]")
+    float *lse = (form & kLseShape) ? lse_of(a[18], {B, Hq}, "[B, Hq]")
                               : is_none(a[18]) ? nullptr : static_cast<float *>(tensor(a[18], "lse").data_ptr());
     const Table t = paged ? table_of(a[6], B) : Table{nullptr, 0};
     const int32_t *lens = i32(a[9], "kv_lens");

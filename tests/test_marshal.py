@@ -45,6 +45,53 @@ def test_host_tensors_and_other_objects_are_type_errors(name):
         calls(7, 7, 7)[name]()
 
 
+def decode_calls(device):
+    """Every decode entry point, by name, with arguments that it accepts."""
+    B, Hq, Hkv, D, page = 2, 4, 2, 128, 16
+    z = lambda *s, dtype=torch.bfloat16: torch.zeros(*s, dtype=dtype, device=device)  # noqa: E731
+    # caches [B, Hkv, slots, D] and pools [pages, Hkv, slots, D] of one shape: within bounds whichever way they are read
+    k, v, k8, v8 = (z(B, Hkv, page, D, dtype=t) for t in (torch.bfloat16,) * 2 + (torch.uint8,) * 2)
+    ones, table = torch.ones(Hkv, device=device), torch.arange(B, dtype=torch.int32, device=device).view(B, 1)
+    step = dict(q=z(B, Hq, D), o=z(B, Hq, D), kv_lens=torch.full((B,), 5, dtype=torch.int32, device=device), max_kv_len=page,
+                scale=1.0, workspace=z(8 << 20, dtype=torch.uint8))
+    kv, pool = dict(cache_k=k, cache_v=v), dict(pool_k=k, pool_v=v, block_table=table)
+    kv8 = dict(cache_k8=k8, cache_v8=v8, k_scale=ones, v_scale=ones)
+    pool8 = dict(pool_k8=k8, pool_v8=v8, k_scale=ones, v_scale=ones, block_table=table)
+    append = dict(k_new=z(B, 1, Hkv, D), v_new=z(B, 1, Hkv, D))
+    rope = dict(append, cos=z(page, D // 2, dtype=torch.float32), sin=z(page, D // 2, dtype=torch.float32))
+    forms = dict(decode=kv, decode_append=kv | append, decode_rope_append=kv | rope, decode_paged=pool,
+                 decode_paged_append=pool | append, decode_paged_rope_append=pool | rope, decode_fp8=kv8,
+                 decode_append_fp8=kv8 | append, decode_rope_append_fp8=kv8 | rope, decode_paged_fp8=pool8)
+    return {name: (getattr(l4l, "l4l_attn_" + name), step | args) for name, args in forms.items()}
+
+
+DECODES = decode_calls("cpu")
+
+
+# without one of these the call would be another operation
+@pytest.mark.parametrize("name,argument", [(n, a) for n in DECODES for a in ("k_new", "v_new", "block_table", "cos") if a in DECODES[n][1]])
+def test_an_argument_left_out_is_named(name, argument):
+    """Refused by name, ahead of any look at the tensors: the entry point says what the operation is, not its arguments."""
+    call, args = DECODES[name]
+    with pytest.raises(TypeError, match=f"^{argument} must be a tensor"):
+        call(**{**args, argument: None})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", DECODES)
+def test_every_decode_argument_is_required(name):
+    call, args = decode_calls("cuda")[name]
+    call(**args)
+    for argument in set(args) - {"max_kv_len", "scale"}:
+        with pytest.raises((TypeError, l4l.L4LError)):
+            call(**{**args, argument: None})
+    if name.endswith("fp8"):                                   # without scales it is no call over a bf16 cache
+        bf16 = {a: t.to(torch.bfloat16) for a, t in args.items() if a.endswith("8")}
+        with pytest.raises(TypeError):
+            call(**{**args, **bf16, "k_scale": None, "v_scale": None})
+    torch.cuda.synchronize()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("name", NAMES)
 def test_float32_on_the_device_is_a_type_error(name):

@@ -988,7 +988,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                         __syncwarp();
                     }
                     uint32_t pb[kSub][NB][2];
-                    warp_softmax<D, NB, true, kSub>(st, sv, pb);
+                    warp_softmax<D, NB, true, kSub, false>(st, sv, pb);
 #pragma unroll
                     for (int u = 0; u < kSub; ++u)
                         if (u == 0 || nvalid > 16 * u) warp_pv_f8<D, NB>(st, pb[u], v_tile, row0 + 16 * u);
@@ -1024,7 +1024,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     __syncwarp();
                 }
                 uint32_t pb[kSub][NB][2];
-                warp_softmax<D, NB, false, kSub>(st, sv, pb);
+                warp_softmax<D, NB, false, kSub, false>(st, sv, pb);
 #pragma unroll
                 for (int u = 0; u < kSub; ++u)
                     if (u == 0 || nvalid > 16 * u) warp_pv<D, NB>(st, pb[u], v_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0);
@@ -1050,13 +1050,12 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                             const int head = 8 * n + (lane >> 2);
                             if (head < p.G) store_output_words<F8>(cw + (size_t)head * CR::kBytes, mt, lane, w);
                         }
+                        if ((lane & 3) == 0 && 8 * n + (lane >> 2) < p.G)
+                            *reinterpret_cast<float *>(cw + (size_t)(8 * n + (lane >> 2)) * CR::kBytes + CR::kOffM + 4) = st.l[n];
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             const int head = 8 * n + 2 * (lane & 3) + e;
-                            if (lane < 4 && head < p.G) {
-                                *reinterpret_cast<float *>(cw + (size_t)head * CR::kBytes + CR::kOffM) = st.m[n][e];
-                                *reinterpret_cast<float *>(cw + (size_t)head * CR::kBytes + CR::kOffM + 4) = st.l[n][e];
-                            }
+                            if (lane < 4 && head < p.G) *reinterpret_cast<float *>(cw + (size_t)head * CR::kBytes + CR::kOffM) = st.m[n][e];
                         }
                     }
                 } else {

@@ -404,7 +404,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                         __syncwarp();
                     }
                     uint32_t pb[kSub][NB][2];
-                    warp_softmax<D, NB, true, kSub>(st, sv, pb);
+                    warp_softmax<D, NB, true, kSub, false>(st, sv, pb);
 #pragma unroll
                     for (int u = 0; u < kSub; ++u)
                         if (u == 0 || nvalid > 16 * u) warp_pv_f8<D, NB>(st, pb[u], v_tile, row0 + 16 * u);
@@ -430,7 +430,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_c
                     __syncwarp();
                 }
                 uint32_t pb[1][NB][2];
-                warp_softmax<D, NB, false, 1>(st, sv, pb);
+                warp_softmax<D, NB, false, 1, true>(st, sv, pb);
                 warp_pv<D, NB>(st, pb[0], v_tile + rows.row(row0), rows.half_bytes, 0);
             }
             if (wrote_smem) fence_proxy_async_smem();   // generic writes before the next TMA fill

@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
                 for (int e = 0; e < 4; ++e) sv[0][n][e] *= sc;
             if (nvalid < kChunkT) warp_mask<NB, 1>(sv, nvalid);   // past the end: no weight (their V rows arrived as zeros)
             uint32_t pb[1][NB][2];
-            warp_softmax<D, NB, F8, 1>(st, sv, pb);               // fp8: weights as f16 for the f16 MMAs
+            warp_softmax<D, NB, F8, 1, !F8>(st, sv, pb);          // fp8: weights as f16 for the f16 MMAs
             if constexpr (F8) warp_pv_f8<D, NB>(st, pb[0], v_tile, 0);
             else warp_pv<D, NB>(st, pb[0], v_tile, C::kHalfBytes, 0);
         }
@@ -419,7 +419,8 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
 #pragma unroll
             for (int n = 0; n < NB; ++n) {
                 // (O over an fp8 cache still lacks the V scale of its KV head)
-                const float f0 = any ? (F8 ? v_sc : 1.f) / st.l[n][0] : 0.f, f1 = any ? (F8 ? v_sc : 1.f) / st.l[n][1] : 0.f;
+                const float l0 = __shfl_sync(0xffffffffu, st.l[n], 8 * (lane & 3)), l1 = __shfl_sync(0xffffffffu, st.l[n], 8 * (lane & 3) + 4);
+                const float f0 = any ? 1.f / l0 * (F8 ? v_sc : 1.f) : 0.f, f1 = any ? 1.f / l1 * (F8 ? v_sc : 1.f) : 0.f;
                 const int head = 8 * n + (lane >> 2);
 #pragma unroll
                 for (int mt = 0; mt < D / 16; ++mt) {
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
 #pragma unroll
                     for (int e = 0; e < 2; ++e)
                         if (8 * n + 2 * lane + e < p.G)
-                            p.lse[bh + 8 * n + 2 * lane + e] = any ? (st.m[n][e] + log2f(st.l[n][e])) * 0.6931471805599453f : -INFINITY;
+                            p.lse[bh + 8 * n + 2 * lane + e] = any ? (st.m[n][e] + log2f(e ? l1 : l0)) * 0.6931471805599453f : -INFINITY;
             }
             st.reset();
         }

@@ -7,8 +7,10 @@
 // rows it would fill a quarter of 16: half the MMAs, half the exponentials, and the output accumulators of a 128-wide
 // head are 32 registers instead of 64 (NB = 2 blocks of 8 heads, for groups of 9 to 16, are as before). P^T is the B operand of
 // the second product: an 8 x 8 transpose of the score fragment (movmatrix). Measured, us, heads as rows -> as columns: e4m3
-// cache, B = 32 ragged 36.7 -> 31.1; B = 512 x 64..256 tokens 65.3 -> 62.5; one sequence of 2304 tokens with rope and norm
-// 9.2 -> 8.8; bf16 caches of large batches, bound by HBM, 46.5 -> 46.4.
+// cache, B = 32 ragged 37.0 -> 32.2; B = 512 x 64..256 tokens 65.8 -> 62.9; bf16 caches of large batches, bound by HBM, 46.7
+// -> 46.5. Every sum has the order that it has with the heads as rows, so that the results are the same bit for bit: one
+// accumulator per score, and denominators summed from the transposed weights. (Two accumulators for even and odd k-steps and sums
+// ahead of the transpose would save 0.1 to 0.2 us: one sequence of 2304 tokens 8.57 against 8.69, the e4m3 batch 31.96 against 32.19.)
 //
 // Tile layout in shared memory: D/64 "halves", each [tile_tokens][64] bf16 (128-byte rows,
 // swizzled), half h covering head_dim [64h, 64h+64). Over pages of 16 or 32 tokens at head_dim 128 one load brings
@@ -36,7 +38,7 @@ struct TileRows {
 template <int D, int NB>
 struct WarpAttnState {
     float m[NB][2];          // running maximum (log2 domain) of this lane's two heads of each block
-    float l[NB][2];          // this lane's share of their running sums (its token rows)
+    float l[NB];             // this lane's share of the running sum of head 8n + r (tokens 2c, 2c + 1 of every 8)
     float o[D / 16][NB][4];  // O^T, unnormalised: 16 head dims per tile; [e] dim row r, [2 + e] dim row r + 8 of head 2c + e
 
     __device__ __forceinline__ void reset()
@@ -44,20 +46,18 @@ struct WarpAttnState {
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
             m[n][0] = m[n][1] = -INFINITY;
-            l[n][0] = l[n][1] = 0.f;
+            l[n] = 0.f;
 #pragma unroll
             for (int i = 0; i < D / 16; ++i) o[i][n][0] = o[i][n][1] = o[i][n][2] = o[i][n][3] = 0.f;
         }
     }
-    // the sums over all token rows (every lane of the warp must call this)
+    // the sums over all tokens (every lane of the warp must call this)
     __device__ __forceinline__ void finish_sums()
     {
 #pragma unroll
         for (int n = 0; n < NB; ++n)
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
-#pragma unroll
-                for (int off = 4; off <= 16; off <<= 1) l[n][e] += __shfl_xor_sync(0xffffffffu, l[n][e], off);
+            for (int off = 1; off <= 2; off <<= 1) l[n] += __shfl_xor_sync(0xffffffffu, l[n], off);
     }
 };
 
@@ -88,18 +88,16 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qf)[D / 16][NB][2], 
 }
 
 // S^T (16 tokens x 8 NB heads) = K(tokens row0 .. row0 + 15) . Q^T. s[n]: [e] token row0 + r, [2 + e] token row0 + r + 8 of
-// head 8n + 2c + e. Even and odd k-steps are accumulated apart, two dependent chains of half the length (two blocks of heads
-// are two chains by themselves).
+// head 8n + 2c + e. One accumulator per block, the k-steps in their order.
 template <int D, int NB>
 __device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, uint32_t half_bytes, int row0,
                                         float (&s)[NB][4])
 {
     const int lane = threadIdx.x & 31;
-    float odd[NB][4];
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] = odd[n][e] = 0.f;
+        for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
     const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
     const uint32_t csel = lane >> 4;                                // matrices 2, 3: head dims + 8
 #pragma unroll
@@ -108,12 +106,8 @@ __device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uin
         uint32_t a[4];
         ldmatrix_x4(k_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
 #pragma unroll
-        for (int n = 0; n < NB; ++n) mma_bf16_16816((NB == 1 && (ks & 1)) ? odd[n] : s[n], a, qf[ks][n][0], qf[ks][n][1]);
+        for (int n = 0; n < NB; ++n) mma_bf16_16816(s[n], a, qf[ks][n][0], qf[ks][n][1]);
     }
-#pragma unroll
-    for (int n = 0; n < NB; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] += NB == 1 ? odd[n][e] : 0.f;
 }
 
 // O^T += V(tokens row0 .. row0 + 15)^T . P^T
@@ -152,13 +146,15 @@ __device__ __forceinline__ void warp_mask(float (&s)[NT][NB][4], int nvalid)
 // at -inf. A step in which no score exceeds the running maxima of its heads (most of them, after the first tiles) needs one
 // vote and neither shuffles nor a rescale. (The maxima stay exact: a reference left up to 2^8 behind would save the rest of
 // the shuffles, but then the largest weights are rounded too, and the log-sum-exp was off by 2.5e-3 instead of 2e-3.)
-// pb[u]: B fragments of P^T, weights as bf16, or as f16 for the MMAs of the e4m3 path.
-template <int D, int NB, bool kF16, int NT>
+// pb[u]: B fragments of P^T, weights as bf16, or as f16 for the MMAs of the e4m3 path. The denominators are summed from them:
+// once transposed, a lane's weights are all of one head. kInRow: the four weights of a 16-token block one after the other, else by pairs.
+template <int D, int NB, bool kF16, int NT, bool kInRow>
 __device__ __forceinline__ void warp_softmax(WarpAttnState<D, NB> &st, const float (&s)[NT][NB][4], uint32_t (&pb)[NT][NB][2])
 {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
-        float mx[2];
+        float mx[2], corr_l = 1.f;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             mx[e] = fmaxf(s[0][n][e], s[0][n][2 + e]);
@@ -173,7 +169,8 @@ __device__ __forceinline__ void warp_softmax(WarpAttnState<D, NB> &st, const flo
                 const float m_new = fmaxf(st.m[n][e], mx[e]);
                 const float corr = fast_exp2(st.m[n][e] - ((m_new == -INFINITY) ? 0.f : m_new));
                 st.m[n][e] = m_new;
-                st.l[n][e] *= corr;
+                const float of_row = __shfl_sync(0xffffffffu, corr, lane >> 3);      // lane r / 2 holds heads r - r % 2 + {0, 1}
+                if (((lane >> 2) & 1) == e) corr_l = of_row;
 #pragma unroll
                 for (int mt = 0; mt < D / 16; ++mt) {
                     st.o[mt][n][e] *= corr;
@@ -182,20 +179,21 @@ __device__ __forceinline__ void warp_softmax(WarpAttnState<D, NB> &st, const flo
             }
         }
         const float m0 = (st.m[n][0] == -INFINITY) ? 0.f : st.m[n][0], m1 = (st.m[n][1] == -INFINITY) ? 0.f : st.m[n][1];
+        float sum = 0.f;
 #pragma unroll
         for (int u = 0; u < NT; ++u)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {                           // token rows r and r + 8
                 const float e0 = fast_exp2(s[u][n][2 * h] - m0), e1 = fast_exp2(s[u][n][2 * h + 1] - m1);
-                const uint32_t pk = kF16 ? pack_f16x2(e0, e1) : pack_bf16x2(e0, e1);
+                const uint32_t pk = movmatrix_trans(kF16 ? pack_f16x2(e0, e1) : pack_bf16x2(e0, e1));
+                pb[u][n][h] = pk;
                 // the denominator sums exactly the rounded weights that multiply V
                 float w0, w1;
                 if constexpr (kF16) unpack_f16x2(pk, w0, w1);
                 else w0 = __uint_as_float(pk << 16), w1 = __uint_as_float(pk & 0xffff0000u);
-                st.l[n][0] += w0;
-                st.l[n][1] += w1;
-                pb[u][n][h] = movmatrix_trans(pk);
+                sum = kInRow ? sum + w0 + w1 : sum + (w0 + w1);
             }
+        st.l[n] = fmaf(st.l[n], corr_l, sum);
     }
 }
 
@@ -223,11 +221,10 @@ template <int D, int NB>
 __device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, int row0, float (&s)[NB][4])
 {
     const int lane = threadIdx.x & 31;
-    float odd[NB][4];
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] = odd[n][e] = 0.f;
+        for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
     const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
     const uint32_t csel = lane >> 4;                                // matrices 2, 3: next 16 head dims
 #pragma unroll
@@ -239,13 +236,9 @@ __device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], 
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
             mma_f16_16816(s[n], a, qf[2 * qd][n][0], qf[2 * qd][n][1]);
-            mma_f16_16816(NB == 1 ? odd[n] : s[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
+            mma_f16_16816(s[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
         }
     }
-#pragma unroll
-    for (int n = 0; n < NB; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] += NB == 1 ? odd[n][e] : 0.f;
 }
 
 template <int D, int NB>
@@ -301,17 +294,15 @@ __device__ __forceinline__ void dump_rows_f32(const WarpAttnState<D, NB> &st, in
 {
     const int lane = threadIdx.x & 31, r = lane >> 2;
 #pragma unroll
-    for (int n = 0; n < NB; ++n)
+    for (int n = 0; n < NB; ++n) {
+        if ((lane & 3) == 0 && 8 * n + r < G) *reinterpret_cast<float *>(row(8 * n + r) + off_m + 4) = st.l[n];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int head = 8 * n + 2 * (lane & 3) + e;
             if (head >= G) continue;
             uint8_t *rowb = row(head);
             float *o = reinterpret_cast<float *>(rowb);
-            if (r == 0) {
-                *reinterpret_cast<float *>(rowb + off_m) = st.m[n][e];
-                *reinterpret_cast<float *>(rowb + off_m + 4) = st.l[n][e];
-            }
+            if (r == 0) *reinterpret_cast<float *>(rowb + off_m) = st.m[n][e];
 #pragma unroll
             for (int mt = 0; mt < D / 16; ++mt) {
                 if constexpr (F8) {
@@ -322,6 +313,7 @@ __device__ __forceinline__ void dump_rows_f32(const WarpAttnState<D, NB> &st, in
                 }
             }
         }
+    }
 }
 
 }  // namespace l4l

@@ -482,6 +482,15 @@ const char *l4l_status_string(l4l_status status);
 int l4l_decode_kernel_choice(int B, int Hq, int Hkv, int head_dim, int max_kv_len, int fp8, int *detail);
 
 /*
+ * The order in which a chunk launch (l4l_attn_prefill_chunk and the fused appends) takes its row blocks, for tests: the number n
+ * of row blocks if it is by the key tiles they visit, heaviest first, which up to 32 sequences with room for a past in the
+ * cache get (slots: token slots per sequence); 0 if it is by place, -1 for sizes that the calls reject. With d_order (device
+ * int32 [n, 2], n of a call without) a kernel on `stream` fills in (sequence, row block) of each, (-1, -1) past the last that holds rows.
+ */
+int l4l_prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens, int S_max, long long slots, int B, int Hq,
+                                int Hkv, int head_dim, int32_t *d_order, l4l_stream stream);
+
+/*
  * Tuning override of the decode kernel choice, process-wide (for tests and benchmarks that must hold a call on
  * one kernel; a serving loop has no reason to call it). No counterpart in the paper.
  *   cluster      -1 library's choice; 0 never the cluster kernel; N > 0 clusters of N CTAs where they fit

@@ -28,7 +28,7 @@ EXPORTS = (
     "l4l_attn_decode_paged_rope_append", "l4l_attn_decode_append_fp8", "l4l_attn_decode_paged_append_fp8",
     "l4l_attn_prefill_chunk_append", "l4l_attn_prefill_chunk_paged_append", "l4l_rglru_strip_channels",
     "l4l_decode_kernel_choice", "l4l_set_decode_override", "l4l_check_status", "l4l_selftest_wait_expiry",
-    "l4l_attn_decode_rope_append_fp8", "l4l_attn_decode_paged_rope_append_fp8",
+    "l4l_attn_decode_rope_append_fp8", "l4l_attn_decode_paged_rope_append_fp8", "l4l_prefill_row_block_order",
 )
 STATIC_SCRATCH_BYTES = 8 << 20
 
@@ -139,6 +139,8 @@ def load() -> ctypes.CDLL:
     lib.l4l_rglru_workspace_bytes.argtypes = [c_int, c_int, c_int]
     lib.l4l_rglru_strip_channels.restype = c_int
     lib.l4l_rglru_strip_channels.argtypes = [c_int, c_int, c_int]
+    lib.l4l_prefill_row_block_order.restype = c_int
+    lib.l4l_prefill_row_block_order.argtypes = [i32p, i32p, c_int, ctypes.c_longlong, c_int, c_int, c_int, c_int, vp, vp]
     lib.l4l_rglru_scan.restype = c_int
     lib.l4l_rglru_scan.argtypes = [vp, vp, vp, vp, i32p, i32p, vp, vp, c_int, c_int, c_int, vp, c_size, vp]
     lib.l4l_rope_kv_append.restype = c_int
@@ -541,6 +543,21 @@ def l4l_selftest_wait_expiry(workspace: torch.Tensor, budget_cycles: int = 10000
                                          int(budget_cycles), _stream())
     if st != L4L_OK:
         raise L4LError(st, "l4l_selftest_wait_expiry")
+
+
+def l4l_prefill_row_block_order(past_lens, q_lens, S: int, slots: int, Hq: int, Hkv: int, head_dim: int) -> Optional[torch.Tensor]:
+    """(sequence, row block) of every row block of a chunk launch, int32 [n, 2] in the order in which they are taken, where that is
+    by their work ((-1, -1) past the last that holds rows); None where it is by place. For tests."""
+    args = (_i32_dev(past_lens, "past_lens"), _i32_dev(q_lens, "q_lens"), int(S), int(slots), past_lens.numel(), Hq, Hkv, head_dim)
+    n = load().l4l_prefill_row_block_order(*args, None, None)
+    if n < 0:
+        raise L4LError(L4L_ERR_INVALID_ARG, "l4l_prefill_row_block_order")
+    if n == 0:
+        return None
+    order = torch.empty(n, 2, dtype=torch.int32, device=past_lens.device)
+    if load().l4l_prefill_row_block_order(*args, order.data_ptr(), _stream()) != n:
+        raise L4LError(L4L_ERR_CUDA, "l4l_prefill_row_block_order")
+    return order
 
 
 def l4l_rglru_strip_channels(B: int, T: int, W: int) -> int:

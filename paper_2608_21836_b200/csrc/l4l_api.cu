@@ -549,6 +549,13 @@ l4l_status l4l_attn_prefill(l4l_tensor4 q, l4l_tensor4 k, l4l_tensor4 v, l4l_ten
                              static_cast<cudaStream_t>(stream));
 }
 
+int l4l_prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens, int S_max, long long slots, int B, int Hq,
+                                int Hkv, int head_dim, int32_t *d_order, l4l_stream stream)
+{
+    if (shape_status(B, Hq, Hkv, head_dim) != L4L_OK || S_max <= 0 || slots < 0 || B <= 0 || !d_past_lens || !d_q_lens) return -1;
+    return prefill_row_block_order(d_past_lens, d_q_lens, S_max, slots, B, Hq, Hkv, d_order, static_cast<cudaStream_t>(stream));
+}
+
 l4l_status l4l_attn_prefill_chunk(l4l_tensor4 q, l4l_tensor4 o, l4l_kv_cache cache, const int32_t *d_past_lens,
                                   const int32_t *d_q_lens, int S_max, int B, int Hq, int Hkv, int head_dim,
                                   float scale, float *d_lse, void *workspace, size_t ws_bytes, l4l_stream stream)

@@ -169,6 +169,10 @@ struct PrefillKV {
 
 // tcgen05 / tensor-memory prefill kernel: a fresh prompt (no past), or a chunk of new tokens over a populated
 // cache. d_past_lens (may be null): tokens ahead of the chunk, per sequence.
+// Row blocks of a chunk launch in the order in which they are taken where that is by their work: their number (and, when
+// d_order is given, their (sequence, row block) pairs, -1 past the last), 0 where it is by place.
+int prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens, int S_max, long long slots, int B, int Hq, int Hkv,
+                            int32_t *d_order, cudaStream_t stream);
 l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const PrefillKV &kv, const int32_t *d_seq_lens,
                              const int32_t *d_past_lens, int S_max, int B, int Hq, int Hkv, int D, float scale,
                              float *d_lse, void *workspace, cudaStream_t stream);

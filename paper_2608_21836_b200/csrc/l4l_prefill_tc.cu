@@ -40,8 +40,6 @@ constexpr int kThreads = 384;                  // 3 warpgroups: softmax 0, softm
 constexpr uint32_t kHalfBytes = kRows * 128;   // [128 rows][64 bf16], 128-byte swizzled
 constexpr float kRescaleThreshold = 8.f;       // log2 domain: O is rescaled only if the max grew by > 2^8
 
-constexpr int kLaneSeqs = 4;                   // sequences per lane when row blocks are ranked by their work (B <= 128)
-
 template <int D>
 struct TcCfg {
     static constexpr int kHalves = D / 64;
@@ -101,69 +99,32 @@ __host__ __device__ constexpr uint32_t make_idesc(int n, bool b_mn_major)
            ((uint32_t)(kRows >> 4) << 24);
 }
 
-// Which row block the block group `g` (the blocks of all heads of one row block) works on when sequences have different pasts:
-// row blocks are ranked by their work, i.e. the key tiles they visit, heaviest first. Row block qb of a sequence has
+// Which row block the block group `g` (the blocks of all heads of one row block) works on when up to 32 sequences have different
+// pasts: row blocks are ranked by their work, i.e. the key tiles they visit, heaviest first. Row block qb of a sequence has
 // past + (qb + 1) << shift tiles, so the ranking needs no sort: the largest w with more than g row blocks of weight >= w is the
-// weight of rank g, found by bisection with a count over the sequences (up to four per lane); equal weights go by sequence.
-// With equal pasts the order of places is the order of work, and b, qb and the lengths stay what the caller made them. Every lane of the
-// warp calls this; every warp of the block does, so it is kept short (and its first loads, len0 and past0 of sequence `lane`,
-// are made ahead by the caller). Returns false past the last row block that holds rows.
-__device__ __forceinline__ bool row_block_by_work(const int32_t *seq_lens, const int32_t *past_lens, int B, int S_max, int row_shift,
-                                                  int shift, int g, int len0, int past_len0, int &b, int &qb, int &L_raw, int &past_raw)
+// weight of rank g, found by bisection with a count over the sequences; equal weights go by sequence. A whole warp calls this,
+// lane l with the lengths of sequence l (0 past the last). Returns false past the last row block that holds rows.
+__device__ __forceinline__ bool row_block_by_work(int len, int past_len, int S_max, int row_shift, int shift, int g, int &b, int &qb)
 {
-    const int lane = threadIdx.x & 31;
-    int blocks[kLaneSeqs], past[kLaneSeqs], len_of[kLaneSeqs], past_of[kLaneSeqs], top = 0, all = 0;
-    bool same = true;
-#pragma unroll
-    for (int u = 0; u < kLaneSeqs; ++u) {
-        blocks[u] = past[u] = len_of[u] = past_of[u] = 0;
-        if (u * 32 >= B) continue;
-        const int i = u * 32 + lane;
-        if (i < B) {
-            len_of[u] = u == 0 ? len0 : __ldg(seq_lens + i);
-            past_of[u] = u == 0 ? past_len0 : __ldg(past_lens + i);
-            blocks[u] = (min(max(len_of[u], 0), S_max) + (1 << row_shift) - 1) >> row_shift;
-            past[u] = (max(past_of[u], 0) + kRows - 1) / kRows;
-        }
-        const int past0 = __shfl_sync(0xffffffffu, past[0], 0);
-        same = same && (i >= B || past[u] == past0);
-        top = max(top, blocks[u] > 0 ? past[u] + (blocks[u] << shift) : 0);
-        all += blocks[u];
-    }
-    if (__all_sync(0xffffffffu, same)) return true;
-    if (g >= (int)__reduce_add_sync(0xffffffffu, (unsigned)all)) return false;
+    const int past = (max(past_len, 0) + kRows - 1) / kRows;
+    const int blocks = (min(max(len, 0), S_max) + (1 << row_shift) - 1) >> row_shift;
+    if (g >= (int)__reduce_add_sync(0xffffffffu, (unsigned)blocks)) return false;
     auto at_least = [&](int w) {
-        int n = 0;
-#pragma unroll
-        for (int u = 0; u < kLaneSeqs; ++u)
-            if (u * 32 < B) n += max(0, blocks[u] - max(0, ((w - past[u] + (1 << shift) - 1) >> shift) - 1));
-        return (int)__reduce_add_sync(0xffffffffu, (unsigned)n);
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)max(0, blocks - max(0, ((w - past + (1 << shift) - 1) >> shift) - 1)));
     };
-    int lo = 1, hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)top) + 1;          // at_least(lo) > g >= at_least(hi)
+    const unsigned top = blocks > 0 ? (unsigned)(past + (blocks << shift)) : 0u;
+    int lo = 1, hi = (int)__reduce_max_sync(0xffffffffu, top) + 1;                     // at_least(lo) > g >= at_least(hi)
     int above = 0;                                                                     // at_least(hi)
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1, n = at_least(mid);
         if (n > g) lo = mid; else hi = mid, above = n;
     }
-    int skip = g - above;                                  // row blocks of this very weight ahead of ours
-#pragma unroll
-    for (int u = 0; u < kLaneSeqs; ++u) {
-        if (u * 32 >= B) continue;
-        const int off = lo - past[u];
-        unsigned who = __ballot_sync(0xffffffffu, off > 0 && (off >> shift) << shift == off && off >> shift <= blocks[u]);
-        const int n = __popc(who);
-        if (skip >= 0 && skip < n) {
-            for (; skip > 0; --skip) who &= who - 1;
-            const int src = __ffs(who) - 1;
-            b = u * 32 + src;
-            qb = (__shfl_sync(0xffffffffu, off, src) >> shift) - 1;
-            L_raw = __shfl_sync(0xffffffffu, len_of[u], src);
-            past_raw = __shfl_sync(0xffffffffu, past_of[u], src);
-            skip = -1;
-        } else if (skip >= 0) {
-            skip -= n;
-        }
-    }
+    // the row block of this very weight with g - above of them ahead (a sequence has one at most)
+    const int off = lo - past;
+    unsigned who = __ballot_sync(0xffffffffu, off > 0 && (off >> shift) << shift == off && off >> shift <= blocks);
+    for (int skip = g - above; skip > 0; --skip) who &= who - 1;
+    b = __ffs(who) - 1;
+    qb = (__shfl_sync(0xffffffffu, off, b) >> shift) - 1;
     return true;
 }
 
@@ -194,8 +155,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     // their latency is hidden behind it.
     int L_raw = __ldg(p.seq_lens + b);
     int past_raw = p.past_lens ? __ldg(p.past_lens + b) : 0;
-    const bool ranked = kRanked && (int)(threadIdx.x & 31) < p.B;
-    const int len0 = ranked ? __ldg(p.seq_lens + (threadIdx.x & 31)) : 0, past_len0 = ranked ? __ldg(p.past_lens + (threadIdx.x & 31)) : 0;
+    // Ranked row blocks: the lengths of all sequences (at most 32), requested with them.
+    int len_of = 0, past_of = 0;
+    if (kRanked && (int)(threadIdx.x & 31) < p.B) {
+        len_of = __ldg(p.seq_lens + (threadIdx.x & 31));
+        past_of = __ldg(p.past_lens + (threadIdx.x & 31));
+    }
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -236,9 +201,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         fence_barrier_init();
         fence_proxy_async_smem();
     }
-    if (kRanked && !row_block_by_work(p.seq_lens, p.past_lens, p.B, p.S_max, pair ? 7 : 8, pair ? 0 : 1, (int)(blockIdx.x / heads), len0,
-                                      past_len0, b, qb, L_raw, past_raw))
-        return;
+    // Ranked row blocks. With equal pasts (every fresh prompt) the order of places is the order of work, and this vote is all that
+    // the block pays for.
+    if (kRanked && __builtin_expect(!__all_sync(0xffffffffu, lane >= p.B || past_of == past_raw), 0)) {
+        if (!row_block_by_work(len_of, past_of, p.S_max, pair ? 7 : 8, pair ? 0 : 1, (int)(blockIdx.x / heads), b, qb)) return;
+        L_raw = __shfl_sync(0xffffffffu, len_of, b);
+        past_raw = __shfl_sync(0xffffffffu, past_of, b);
+        b = __shfl_sync(0xffffffffu, b, 0);                  // the same in every lane: in registers of the warp
+        qb = __shfl_sync(0xffffffffu, qb, 0);
+    }
     const int q0 = qb * (pair ? kRows : 2 * kRows);
     const int diag0 = pair ? qb : 2 * qb;                 // tile (among the new tokens) of sub-tile 0's diagonal
     // first use of the lengths. A block past the end of its sequence has nothing to do (decided before any
@@ -664,6 +635,35 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     }
 }
 
+bool pairs_heads(int G) { return G % 2 == 0; }
+int row_blocks(int S_max, int G) { return pairs_heads(G) ? (S_max + kRows - 1) / kRows : (S_max + 2 * kRows - 1) / (2 * kRows); }
+
+// Chunks over caches of different lengths: a row block's work is then set by the tokens cached ahead of it as much as by its
+// place, and with the last row blocks first whatever their length the launch ends on a few heavy blocks. Five chunks of
+// 180 to 676 tokens over 720 to 4590 in pages: 131.9 us by place, 115.1 by work; 32 chunks of up to 300 over up to 3000 236 and 216.
+// One sequence needs no order, and launches of one or two blocks per SM have little to order (two chunks of up to 522 tokens, 160
+// blocks: 21.8 us by place, 22.3 by work). Where a cache has room ahead of the chunk the pasts may still be equal, as
+// for fresh prompts, and finding that out must cost nothing: with one sequence per lane it is a vote (16 prompts of 512 rotated
+// and attended 118.9 us either way). Beyond 32 sequences it was not (40 prompts of up to 300 tokens 129.7 and 131.9 us, 100 of up to 200
+// 209.5 and 213.7), for a gain of 2.6 % with 40 chunks and a loss of 1 % with 100. slots: token slots per sequence in the cache (0: no past).
+bool row_blocks_by_work(int S_max, long long slots, int B, int Hq, int G)
+{
+    return slots - S_max >= kRows && B > 1 && B <= 32 &&
+           (long long)row_blocks(S_max, G) * (pairs_heads(G) ? Hq / 2 : Hq) * B > 2 * sm_count();
+}
+
+// The order for tests: block g reports the (sequence, row block) that the blocks of group g of a ranked launch work on.
+__global__ void row_block_order_kernel(const int32_t *past_lens, const int32_t *q_lens, int S_max, int B, int n_qblocks, bool pair, int2 *order)
+{
+    const int lane = threadIdx.x, g = blockIdx.x;
+    int b = g % B, qb = n_qblocks - 1 - g / B;
+    const int past = lane < B ? past_lens[lane] : 0, len = lane < B ? q_lens[lane] : 0, past_raw = past_lens[b];
+    bool rows = true;
+    if (!__all_sync(0xffffffffu, lane >= B || past == past_raw)) rows = row_block_by_work(len, past, S_max, pair ? 7 : 8, pair ? 0 : 1, g, b, qb);
+    rows = rows && qb * (pair ? kRows : 2 * kRows) < min(q_lens[b], S_max);
+    if (lane == 0) order[g] = rows ? make_int2(b, qb) : make_int2(-1, -1);
+}
+
 template <int D, bool kRanked>
 l4l_status launch_t(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const CUtensorMap &to,
                     const CUtensorMap &tkc, const CUtensorMap &tvc, const TcParams &p, cudaStream_t stream)
@@ -749,25 +749,29 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     p.lse = d_lse;
     p.status = static_cast<unsigned *>(workspace);
     p.S_max = S_max; p.B = B; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
-    p.pair_heads = (p.G % 2 == 0) ? 1 : 0;
-    p.n_qblocks = p.pair_heads ? (S_max + kRows - 1) / kRows : (S_max + 2 * kRows - 1) / (2 * kRows);
+    p.pair_heads = pairs_heads(p.G) ? 1 : 0;
+    p.n_qblocks = row_blocks(S_max, p.G);
     p.scale_log2e = scale * 1.4426950408889634f;
     p.cq = cq; p.ckv = ck; p.co = co; p.ckc = ckc;
-    // Chunks over caches of different lengths: a row block's work is then set by the tokens cached ahead of it as much as by
-    // its place, and with the last row blocks first whatever their length the launch ends on a few heavy blocks. Five chunks
-    // of 180 to 676 tokens over 720 to 4590: 131 us by place, 116 by work. Without a past the order of places is the order of
-    // work, one sequence needs no order, launches of one or two blocks per SM have little to order (two chunks of up to 522
-    // tokens, 160 blocks: 21.8 us by place, 22.3 by work), and beyond 128 sequences there are enough blocks to even themselves out. The ranking costs a block 0.4 us, finding equal pasts 0.15 (864 blocks of six
-    // prompts: 101.7, 106.2 and 103 us); where the cache has no room for a tile ahead of the chunk (a prompt that fills its
-    // cache) nobody looks.
-    bool ranked = kv.past && d_past_lens && B > 1 && B <= 32 * kLaneSeqs;
-    if (ranked) {
-        const long long slots = kv.paged ? (long long)kv.paged->table_stride * kv.past->max_len : kv.past->max_len;
-        ranked = slots - S_max >= kRows && (long long)p.n_qblocks * (p.pair_heads ? Hq / 2 : Hq) * B > 2 * sm_count();
-    }
+    const long long slots = !kv.past ? 0 : kv.paged ? (long long)kv.paged->table_stride * kv.past->max_len : kv.past->max_len;
+    const bool ranked = d_past_lens && row_blocks_by_work(S_max, slots, B, Hq, p.G);
     if (ranked)
         return D == 128 ? launch_t<128, true>(tq, tk, tv, to, tkc, tvc, p, stream) : launch_t<64, true>(tq, tk, tv, to, tkc, tvc, p, stream);
     return D == 128 ? launch_t<128, false>(tq, tk, tv, to, tkc, tvc, p, stream) : launch_t<64, false>(tq, tk, tv, to, tkc, tvc, p, stream);
+}
+
+int prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens, int S_max, long long slots, int B, int Hq, int Hkv,
+                            int32_t *d_order, cudaStream_t stream)
+{
+    const int G = Hq / Hkv;
+    if (!row_blocks_by_work(S_max, slots, B, Hq, G)) return 0;
+    const int n = row_blocks(S_max, G) * B;
+    if (d_order) {
+        row_block_order_kernel<<<n, 32, 0, stream>>>(d_past_lens, d_q_lens, S_max, B, row_blocks(S_max, G), pairs_heads(G),
+                                                     reinterpret_cast<int2 *>(d_order));
+        if (cudaGetLastError() != cudaSuccess) return -1;
+    }
+    return n;
 }
 
 }  // namespace l4l

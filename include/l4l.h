@@ -291,8 +291,12 @@ size_t l4l_rglru_workspace_bytes(int B, int T, int W);
  * Channels per strip (64, 32 or 16) that l4l_rglru_scan would give one thread block for these sizes on the
  * current device, without launching anything (for tests and tuning; no counterpart in the paper): narrower
  * strips are taken when 64-channel ones would load the SMs unevenly. -1 for sizes the scan rejects.
+ * The choice also depends on whether there are reset positions and on the workspace; this answers for a launch with positions
+ * on a workspace of l4l_rglru_workspace_bytes, l4l_rglru_launch_shape for the one that is described, with the number
+ * of segments that the time axis is cut into in *segments (NULL: not asked for).
  */
 int l4l_rglru_strip_channels(int B, int T, int W);
+int l4l_rglru_launch_shape(int B, int T, int W, int positions, size_t ws_bytes, int *segments);
 l4l_status l4l_rglru_scan(const void *x, const void *gate_x, const void *gate_a, const float *d_a_param,
                           const int32_t *d_position, const int32_t *d_seq_lens, float *d_state, void *y,
                           int B, int T, int W, void *workspace, size_t ws_bytes, l4l_stream stream);

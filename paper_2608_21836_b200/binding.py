@@ -29,6 +29,7 @@ EXPORTS = (
     "l4l_attn_prefill_chunk_append", "l4l_attn_prefill_chunk_paged_append", "l4l_rglru_strip_channels",
     "l4l_decode_kernel_choice", "l4l_set_decode_override", "l4l_check_status", "l4l_selftest_wait_expiry",
     "l4l_attn_decode_rope_append_fp8", "l4l_attn_decode_paged_rope_append_fp8", "l4l_prefill_row_block_order",
+    "l4l_rglru_launch_shape",
 )
 STATIC_SCRATCH_BYTES = 8 << 20
 
@@ -139,6 +140,8 @@ def load() -> ctypes.CDLL:
     lib.l4l_rglru_workspace_bytes.argtypes = [c_int, c_int, c_int]
     lib.l4l_rglru_strip_channels.restype = c_int
     lib.l4l_rglru_strip_channels.argtypes = [c_int, c_int, c_int]
+    lib.l4l_rglru_launch_shape.restype = c_int
+    lib.l4l_rglru_launch_shape.argtypes = [c_int, c_int, c_int, c_int, c_size, ctypes.POINTER(c_int)]
     lib.l4l_prefill_row_block_order.restype = c_int
     lib.l4l_prefill_row_block_order.argtypes = [i32p, i32p, c_int, ctypes.c_longlong, c_int, c_int, c_int, c_int, vp, vp]
     lib.l4l_rglru_scan.restype = c_int
@@ -561,8 +564,19 @@ def l4l_prefill_row_block_order(past_lens, q_lens, S: int, slots: int, Hq: int, 
 
 
 def l4l_rglru_strip_channels(B: int, T: int, W: int) -> int:
-    """Channels per strip (64, 32 or 16) the scan would use for these sizes on the current device."""
+    """Channels per strip (64, 32 or 16) the scan would use for these sizes on the current device, with reset positions and a
+    workspace of l4l_rglru_workspace_bytes."""
     return int(load().l4l_rglru_strip_channels(int(B), int(T), int(W)))
+
+
+def l4l_rglru_launch_shape(B: int, T: int, W: int, positions: bool, ws_bytes: Optional[int] = None):
+    """(channels per strip, segments of the time axis) of a scan of these sizes with or without reset positions, on a workspace of
+    ws_bytes (None: l4l_rglru_workspace_bytes); None for sizes the scan rejects."""
+    if ws_bytes is None:
+        ws_bytes = load().l4l_rglru_workspace_bytes(B, T, W)
+    segments = ctypes.c_int(0)
+    c = load().l4l_rglru_launch_shape(B, T, W, int(bool(positions)), ws_bytes, ctypes.byref(segments))
+    return None if c < 0 else (c, segments.value)
 
 
 def l4l_attn_merge(o_parts, lse_parts, o, lse=None) -> None:

@@ -503,8 +503,15 @@ l4l_status l4l_rglru_scan(const void *x, const void *gate_x, const void *gate_a,
 int l4l_rglru_strip_channels(int B, int T, int W)
 {
     if (B <= 0 || T <= 0 || W <= 0 || W % 8 != 0) return -1;
-    int segments = 1;
-    const int split = rglru_strip_split(B, T, W, &segments, true);
+    return l4l_rglru_launch_shape(B, T, W, 1, rglru_workspace_bytes(B, T, W), nullptr);
+}
+
+int l4l_rglru_launch_shape(int B, int T, int W, int positions, size_t ws_bytes, int *segments)
+{
+    if (B <= 0 || T <= 0 || W <= 0 || W % 8 != 0) return -1;
+    int n = 1;
+    const int split = rglru_shape(B, T, W, positions != 0, ws_bytes, &n);
+    if (segments) *segments = n;
     return split == 0 ? 64 : 64 / split;
 }
 

@@ -340,6 +340,9 @@ size_t rglru_workspace_bytes(int B, int, int W)
 
 namespace {
 
+int tiles_of(int T, int split) { return (T + kTb * split - 1) / (kTb * split); }
+int tiles_per_segment(int tiles, int segments, int team) { return (tiles + segments * team - 1) / (segments * team) * team; }   // whole rounds of the team
+
 template <int kTeam, int kSplit, bool kSeg = false>
 l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, RglruParams p, int segments, cudaStream_t stream)
 {
@@ -362,8 +365,8 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, R
         !make_tmap_rows_bf16(&tgx, gate_x, p.W, p.T, p.B, p.W, (int64_t)p.T * p.W, kCw, kTb * kSplit) ||
         !make_tmap_rows_bf16(&tga, gate_a, p.W, p.T, p.B, p.W, (int64_t)p.T * p.W, kCw, kTb * kSplit))
         return L4L_ERR_CUDA;
-    const int strips = (p.W + kCw - 1) / kCw, tiles = (p.T + kTb * kSplit - 1) / (kTb * kSplit);
-    p.seg_tiles = kSeg ? (tiles + segments * kTeam - 1) / (segments * kTeam) * kTeam : tiles;        // whole rounds of the team
+    const int strips = (p.W + kCw - 1) / kCw, tiles = tiles_of(p.T, kSplit);
+    p.seg_tiles = kSeg ? tiles_per_segment(tiles, segments, kTeam) : tiles;
     const dim3 grid(strips, p.B, (tiles + p.seg_tiles - 1) / p.seg_tiles);
     rglru_scan_kernel<kTeam, kSplit, kSeg><<<grid, kTeam * 32, smem_bytes(kTeam), stream>>>(tx, tgx, tga, p);
     return cudaGetLastError() == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
@@ -383,9 +386,7 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
     p.progress = reinterpret_cast<int *>(static_cast<uint8_t *>(workspace) + kStatusBytes);
     if (T <= kTb) return launch_shape<1, 1>(x, gate_x, gate_a, p, 1, stream);
     int segs = 1;
-    const size_t needed = rglru_workspace_bytes(B, T, W);
-    const bool with_counters = needed > kStatusBytes && ws_bytes >= needed;
-    const int split = rglru_strip_split(B, T, W, with_counters ? &segs : nullptr, d_position != nullptr);
+    const int split = rglru_shape(B, T, W, d_position != nullptr, ws_bytes, &segs);
     if (segs > 1)
         return split == 4   ? launch_shape<8, 4, true>(x, gate_x, gate_a, p, segs, stream)
                : split == 2 ? launch_shape<8, 2, true>(x, gate_x, gate_a, p, segs, stream)
@@ -396,9 +397,9 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
     return launch_shape<8, 1>(x, gate_x, gate_a, p, 1, stream);
 }
 
-// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels. *segments
-// (when given): into how many segments the time axis is cut; positions: the launch has reset positions.
-int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
+// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels (a single warp for a
+// single tile). *segments (when given): into how many segments the time axis is cut; positions: the launch has reset positions.
+static int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
 {
     if (segments) *segments = 1;
     if (T <= kTb) return 1;
@@ -448,6 +449,19 @@ int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
                 *segments = z;
             }
     return best;
+}
+
+int rglru_shape(int B, int T, int W, bool positions, size_t ws_bytes, int *segments)
+{
+    const size_t needed = rglru_workspace_bytes(B, T, W);
+    const bool with_counters = needed > kStatusBytes && ws_bytes >= needed;
+    *segments = 1;
+    const int split = rglru_strip_split(B, T, W, with_counters ? segments : nullptr, positions);
+    if (*segments > 1) {
+        const int tiles = tiles_of(T, split), each = tiles_per_segment(tiles, *segments, 8);
+        *segments = (tiles + each - 1) / each;
+    }
+    return split;
 }
 
 }  // namespace l4l

@@ -122,17 +122,35 @@ def test_rglru_empty_inputs_are_a_no_op():
     assert (state == 7.0).all() and (y == 3.0).all() and l4l.l4l_last_device_error(ws) == 0
 
 
-@pytest.mark.parametrize("B,T,W", [(4, 8192, 2560), (5, 8007, 2048)])
-def test_rglru_time_segments(B, T, W):
+def segment_steps(T, channels, segments):
+    steps = 16 * (64 // channels)                                  # whole rounds of 8 warps' tiles
+    return -(-(-(-T // steps)) // (8 * segments)) * 8 * steps
+
+
+# every kernel that is built for cut launches, two and four segments, with positions and without
+@pytest.mark.parametrize("B,T,W,positions,shape", [
+    (4, 8192, 2560, True, (32, 4)), (5, 8007, 2048, True, (32, 4)), (6, 2049, 4096, True, (32, 2)), (6, 6000, 4096, False, (32, 4)),
+    (2, 5133, 2560, True, (16, 4)), (2, 8192, 2560, False, (16, 4)), (16, 2048, 2560, True, (64, 2)), (8, 4096, 2560, True, (64, 4))])
+def test_rglru_time_segments(B, T, W, positions, shape):
     """Launches that the library cuts into segments of the time axis (a workspace with room for the counters) against the
     same launch uncut (a workspace of the status block alone), which takes the same steps in the same order: equal bit
-    for bit. Lengths: none, one step, the end of a segment (2048 steps in the first case) and one past it, all; resets;
-    a second call finds the counters at zero."""
+    for bit. Lengths: all, the end of a segment and one past it, none, one step, all but one; resets; a second call finds the
+    counters at zero."""
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert l4l.l4l_rglru_launch_shape(B, T, W, positions) == shape
+    assert l4l.l4l_rglru_launch_shape(B, T, W, positions)[1] > 1 and l4l.l4l_rglru_launch_shape(B, T, W, positions, 256)[1] == 1
     x, gx, ga, ap, h0 = (t.cuda() for t in make(B, T, W, 1900 + T))
-    lens = torch.tensor([T, 0, 2048, 2049, 1][:B], dtype=torch.int32, device="cuda")
-    pos = torch.arange(T, dtype=torch.int32, device="cuda").repeat(B, 1)
-    pos[0, 3000:] -= 3000
-    uncut, cut = l4l.new_rglru_workspace(B, T, W)[:256].clone(), l4l.new_rglru_workspace(B, T, W)
+    seg = segment_steps(T, *shape)
+    assert (T - 1) // seg + 1 == shape[1]
+    lens = ([T, seg + 1, seg, 0, 1, T - 1] + [T] * B)[:B]
+    none = 3 if B > 3 else None
+    lens = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    pos = torch.arange(T, dtype=torch.int32, device="cuda").repeat(B, 1) if positions else None
+    if positions:
+        pos[0, seg:] -= seg                                        # a reset on the first step of a segment, and one inside
+        pos[0, seg + 900:] -= 900
+    cut = l4l.new_rglru_workspace(B, T, W).view(torch.uint8)
+    uncut = cut[:256].clone()
     outs = []
     for ws in (uncut, cut, cut):
         y, st = torch.zeros_like(x), h0.clone()
@@ -142,4 +160,21 @@ def test_rglru_time_segments(B, T, W):
     assert int(cut[256:].max()) == 0
     for y, st in outs[1:]:
         assert torch.equal(y.view(torch.int16), outs[0][0].view(torch.int16)) and torch.equal(st, outs[0][1])
-    assert torch.equal(outs[0][1][1], h0[1]) and torch.isfinite(outs[0][0]).all()
+    assert torch.isfinite(outs[0][0]).all() and (none is None or torch.equal(outs[0][1][none], h0[none]))
+
+
+@pytest.mark.parametrize("B,T,W,positions", [(2, 5133, 2560, True), (6, 2049, 4096, True), (2, 8192, 2560, False)])
+def test_rglru_cut_launches_match_the_oracle(B, T, W, positions):
+    assert l4l.l4l_rglru_launch_shape(B, T, W, positions)[1] > 1
+    x, gx, ga, ap, h0 = make(B, T, W, 2100 + T)
+    pos = torch.arange(T, dtype=torch.int32).repeat(B, 1) + (0 if positions else 1)     # no position 0: no resets
+    if positions:
+        pos[0, 1900:] -= 1900
+    lens = [T] + [T - 400 * i for i in range(1, B)]
+    y_ref, st_ref = orc.rglru(x, gx, ga, ap.numpy(), state=h0.double().numpy(), position=pos.numpy(), seq_len=lens)
+    y, st = torch.zeros(B, T, W, dtype=torch.bfloat16, device="cuda"), h0.cuda()
+    ws = l4l.new_rglru_workspace(B, T, W)
+    l4l.l4l_rglru_scan(x.cuda(), gx.cuda(), ga.cuda(), ap.cuda(), st, y, ws, position=pos.cuda() if positions else None,
+                       seq_lens=torch.tensor(lens, dtype=torch.int32).cuda())
+    assert l4l.l4l_last_device_error(ws) == 0
+    check(y, st, y_ref, st_ref, np.broadcast_to(np.arange(T)[None, :, None] < np.array(lens)[:, None, None], (B, T, W)))

@@ -83,3 +83,18 @@ def test_missing_library_is_an_error_not_a_fallback(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(FileNotFoundError):
         binding.load()
+
+
+def test_the_scan_s_shape_is_that_of_the_launch_described(lib):
+    """It depends on reset positions and on the workspace (no device here: the rule for 148 SMs)."""
+    if binding.torch.cuda.is_available() and binding.torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the rule for another number of SMs")
+    shape = binding.l4l_rglru_launch_shape
+    assert shape(4, 8192, 2560, True) == (32, 4) and shape(4, 8192, 2560, False) == (16, 1)
+    assert shape(8, 4096, 2560, True) == (64, 4) and shape(8, 4096, 2560, False) == (32, 1)
+    assert shape(4, 8192, 2560, True, 256) == (16, 1)                # the status block alone: not cut
+    full = lib.l4l_rglru_workspace_bytes(4, 8192, 2560)
+    assert shape(4, 8192, 2560, True, full) == (32, 4) and shape(4, 8192, 2560, True, full - 1) == (16, 1)
+    assert shape(3, 1, 2560, True) == (64, 1) and shape(3, 16, 12, True) is None
+    for B, T, W in ((4, 8192, 2560), (4, 600, 2560), (4, 300, 2560), (2, 5133, 2560)):
+        assert binding.l4l_rglru_strip_channels(B, T, W) == shape(B, T, W, True)[0]

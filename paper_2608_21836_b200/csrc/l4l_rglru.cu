@@ -27,9 +27,10 @@
 // (h <- A h + E) inside step 3. Twice or four times as many CTAs of half or a quarter of the work spread evenly.
 //
 // Segments. Where the strips fill the GPU more than once, a last round of a few strips leaves most SMs idle (320 strips of 32
-// channels on 296 places: 200 us). The time axis is then cut as well: a CTA per (strip, segment), all first segments ahead of all
-// second ones, the state passing through its place in global memory behind a counter per strip (release / acquire). By
-// the time a later segment gets a place its predecessor has long finished, so nothing waits: 144 us in four segments.
+// channels on 296 places: 181 us). The time axis is then cut as well: a CTA per (strip, segment), all first segments ahead of all
+// second ones, the state passing through its place in global memory behind a counter per strip (release / acquire). Blocks
+// start in the order of their indexes, so by the time a later segment gets a place its predecessor has long finished and nothing
+// waits (the wait is bounded like every other): 135 us in four segments.
 #include <type_traits>
 
 #include "l4l_internal.h"
@@ -429,8 +430,11 @@ static int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
     // Segments: n blocks take n / (2 SMs) rounds of two resident teams each, a last round with a lone team on an SM 0.68 of
     // a full one; every round of a cut launch pays for set-up, first loads and the drain of the ring (about 1.5 us; 3 us on
     // 16-channel strips). A strip is cut only where the strips alone fill the GPU, so that a segment finds its predecessor
-    // finished. B = 4 x 8192 x 2560 with positions, us by (channels, segments): (64, 1) 222, (32, 1) 200, (32, 2) 166, (32, 4) 133,
-    // (32, 8) 166, (16, 1) 165, (16, 4) 180; 16 channels uncut were the choice before.
+    // finished. B = 4 x 8192 x 2560 with positions, us by (channels, segments), thirty launches back to back on one build: (64, 1)
+    // 205, (32, 1) 181, (16, 1) 154, which is the choice without segments, (64, 4) 186, (32, 2) 141, (32, 4) 135, (32, 8) 148, (16, 2) 145,
+    // (16, 4) 162. (Kept up for a second the launch takes 148 us: the clock falls under the load.) The model is off by up to a
+    // fifth where strips are wide or sequences few, but it orders the shapes well enough: over 92 sizes for which it cuts, of
+    // 1024 to 5120 channels, cut launches take 0.86 to 1.013 times what the same launches take uncut, 90 of them less.
     if (!segments || best == 0) return best;
     const double us_per_step_channel = 4.54e-4;          // of a resident pair of teams
     auto estimate = [&](int s, int z) {
@@ -439,7 +443,7 @@ static int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
         return rounds * ((double)T / z * (kCb / s) * us_per_step_channel + (z == 1 ? 0.0 : s < 4 ? 1.5 : 3.0));
     };
     // (positions slow the uncut narrow shapes down most, every strip reads them; without them a cut has to promise more:
-    // 3 x 5000 x 4096 109.6 us cut against 115.3 with positions, 105.7 against 101.4 without)
+    // 3 x 5000 x 4096 111.0 us cut against 114.3 with positions, 107.0 against 104.0 without)
     best_time = (positions ? 0.95 : 0.85) * estimate(best, 1);
     for (int s = 1; s <= 4; s *= 2)
         for (int z = 2; z <= 4; z *= 2)

@@ -153,9 +153,9 @@ bool make_tmap_page(CUtensorMap *out, const void *base, int page_size, int64_t n
     if (!fn) return false;
     cuuint64_t gdim[5] = {64, (cuuint64_t)page_size, 2, (cuuint64_t)n_h, (cuuint64_t)(n_pages < 1 ? 1 : n_pages)};
     cuuint64_t gstride[4] = {(cuuint64_t)stride_t * 2, 128, (cuuint64_t)stride_h * 2, (cuuint64_t)stride_page * 2};
-    // the stride of an extent-1 dimension is never used for addressing, but has to be a valid one
-    if (n_h <= 1) gstride[2] = (cuuint64_t)page_size * gstride[0];
-    if (n_pages <= 1) gstride[3] = (cuuint64_t)n_h * gstride[2];
+    // the stride of an extent-1 dimension is never used for addressing, but has to be a valid one, as make_tmap's is
+    if (n_h <= 1) gstride[2] = 128;
+    if (n_pages <= 1) gstride[3] = 128;
     cuuint32_t box[5] = {64, (cuuint32_t)page_size, 2, 1, 1};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), gdim, gstride, box, estr,

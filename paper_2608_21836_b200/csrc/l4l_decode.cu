@@ -120,8 +120,7 @@ struct DecodeParams {
     const int32_t *block_table;
     int table_stride, page_size, page_shift, num_pages;
     int page_box;             // paged: tokens per box of tmap_k / tmap_v (divides the tile, never straddles a page)
-    int small_pages;          // pages of 16 or 32 tokens: every box is a page
-    int page_loads;           // tmap_k / tmap_v bring a whole page, both halves, per load (bf16, head_dim 128, pages of 16 or 32)
+    int small_pages;          // pages of 16 or 32 tokens: every box is a page (two halves per row: one load brings both)
     int B, Hq, Hkv, G, min_tiles, nsplit, max_kv_len;
     int stream_once;          // load K/V with the L2 evict-first policy (large caches)
     int nfin;                 // finisher warps (BigG: one per 4 query heads of the group; else 1)
@@ -806,7 +805,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
         uint32_t n_dumps = 0;                // pieces handed to the finisher so far
         uint32_t n_rotated = 0;              // pieces whose query rows were rotated (phase of q_rotated)
         float k_sc = 1.f, v_sc = 1.f;        // fp8 cache: scales of the piece's KV head (read once per piece)
-        const bool by_page = C::kHalves == 2 && p.page_loads != 0;
+        const bool by_page = C::kHalves == 2 && p.small_pages != 0;
         const TileRows rows = {by_page ? (uint32_t)p.page_size * 128u : C::kHalfBytes, by_page ? (uint32_t)-p.page_size : 0u};
 
         for (uint32_t it = 0;; ++it) {
@@ -1298,7 +1297,7 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
             if (!make_tmap_page(&tk, kb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) ||
                 !make_tmap_page(&tv, vb, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b))
                 return L4L_ERR_CUDA;
-            tk_tail = tk;            // groups of the last tile are pages too
+            tk_tail = tk;            // never loaded from here, but the kernel prefetches all four descriptors
             tv_tail = tv;
             coord = TmapCoord{};
         } else if (!make_tmap(&tk, &coord, kb, map_d, map_rows, Hkv, outer, map_st, cache.stride_h,
@@ -1339,7 +1338,6 @@ l4l_status launch_decode(const void *q, void *o, const l4l_kv_cache &cache, cons
         p.page_box = box_t;
         p.num_pages = paged ? paged->num_pages : 0;
         p.small_pages = paged && cache.max_len <= 32 ? 1 : 0;
-        p.page_loads = page_loads ? 1 : 0;
         p.page_shift = 0;
         while (paged && (1 << p.page_shift) < cache.max_len) ++p.page_shift;
         // only the fused append writes through these: the slice's sequences, or the whole pool of a paged cache

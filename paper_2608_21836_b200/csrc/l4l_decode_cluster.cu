@@ -677,11 +677,12 @@ l4l_status launch_decode_cluster(const void *q, void *o, const l4l_kv_cache &cac
     const int box_t = (paged && cache.max_len < kTileT) ? cache.max_len : kTileT;
     const int tail_rows = (paged && cache.max_len < 32) ? cache.max_len : 32;
     // small pages: one load per page instead of one per 64-column half (the rule and its figures: launch_decode)
-    const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr) &&
-                            make_tmap_page(&tk, cache.k, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) &&
-                            make_tmap_page(&tv, cache.v, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b);
+    const bool page_loads = paged && pages_load_whole(D, cache.max_len, fp8 != nullptr);
     if (page_loads) {
-        tk_tail = tk;                // groups of the last tile are pages too
+        if (!make_tmap_page(&tk, cache.k, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b) ||
+            !make_tmap_page(&tv, cache.v, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b))
+            return L4L_ERR_CUDA;
+        tk_tail = tk;                // never loaded from here, but the kernel prefetches all four descriptors
         tv_tail = tv;
         coord = TmapCoord{};
     } else if (!make_tmap(&tk, &coord, cache.k, D, cache.max_len, Hkv, outer, cache.stride_t, cache.stride_h, cache.stride_b, box_d,

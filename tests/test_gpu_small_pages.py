@@ -49,3 +49,23 @@ def test_small_pages_equal_the_contiguous_cache(page, Hq, Hkv, D, layout, cluste
     assert torch.equal(want.view(torch.int16), got.view(torch.int16))
     for c, p in ((ck, pk), (cv, pv)):                      # the newest row went to the right page, and nothing else changed
         assert torch.equal(c.view(torch.int16), torch.stack([p[table[b].long()].transpose(0, 1).flatten(1, 2) for b in range(B)]).view(torch.int16))
+
+
+@pytest.mark.parametrize("cluster", [0, -1])
+@pytest.mark.parametrize("Hkv", [1, 2])
+@pytest.mark.parametrize("page", [16, 32])
+def test_a_pool_of_one_page(page, Hkv, cluster):
+    """Outer extents of 1, whose strides address nothing: whatever they are, the map is a valid one."""
+    g = torch.Generator(device="cuda").manual_seed(page + Hkv)
+    mk = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.bfloat16)  # noqa: E731
+    q, ck, cv = mk(1, 4 * Hkv, 128), mk(1, Hkv, page, 128), mk(1, Hkv, page, 128)
+    lens, table = torch.tensor([page - 3], dtype=torch.int32, device="cuda"), torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    ws = l4l.new_workspace(l4l.L4L_OP_DECODE, 1, 4 * Hkv, Hkv, 128, page)
+    strides = [(0, 8), (8, 16), (1 << 40, 1 << 41)] if Hkv == 1 else [(0, page * 128), (1 << 41, page * 128)]
+    with l4l.decode_override(cluster=cluster, warp=0):
+        want, got = torch.empty_like(q), torch.empty_like(q)
+        l4l.l4l_attn_decode(q, want, ck, cv, lens, page, 128 ** -0.5, ws)
+        for sp, sh in strides:
+            pk, pv = (c.as_strided((1, Hkv, page, 128), (sp, sh, 128, 1)) for c in (ck, cv))
+            l4l.l4l_attn_decode_paged(q, got.zero_(), pk, pv, table, lens, page, 128 ** -0.5, ws)
+            assert torch.equal(want.view(torch.int16), got.view(torch.int16))

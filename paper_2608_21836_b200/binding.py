@@ -13,6 +13,8 @@ from typing import Optional
 
 import torch
 
+from . import build
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libl4l.so")
 
@@ -181,12 +183,19 @@ _DECODE_PAGED_FP8 = _FP8 | _PAGED
 
 
 def _load_native():
-    """The module that marshals the arguments of the per-step calls (csrc/l4l_marshal.cpp), next to libl4l.so."""
+    """The module that marshals the arguments of the per-step calls (csrc/l4l_marshal.cpp), next to libl4l.so. It reads torch's
+    objects by their layout, so it is refused when it was built for another torch."""
     global _native
     if _native is None:
         load()
+        if not os.path.exists(build.MARSHAL):
+            raise FileNotFoundError(f"{build.MARSHAL} not found: build it with `python -m paper_2608_21836_b200.build`; there is no "
+                                    "fallback path")
         from . import _l4l_marshal
 
+        if _l4l_marshal.BUILT_FOR != build.marshal_tag():
+            raise ImportError(f"{build.MARSHAL} was built for {_l4l_marshal.BUILT_FOR}, this is {build.marshal_tag()}: build it with "
+                              "`python -m paper_2608_21836_b200.build`")
         _native = _l4l_marshal
     return _native
 

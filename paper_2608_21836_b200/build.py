@@ -5,6 +5,7 @@ Run as ``python -m paper_2608_21836_b200.build``. nvcc cross-compiles, so no GPU
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 import sysconfig
@@ -14,7 +15,9 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "csrc", "build")
 LIB = os.path.join(PKG, "libl4l.so")
-MARSHAL = os.path.join(PKG, "_l4l_marshal.so")       # the Python module that marshals the per-step calls
+# the Python module that marshals the per-step calls: for one interpreter (by its name) and one torch (by its tag)
+MARSHAL = os.path.join(PKG, "_l4l_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
+MARSHAL_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-shared"]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -31,6 +34,23 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+MARSHAL_SRC = [os.path.join(CSRC, "l4l_marshal.cpp"), os.path.join(PKG, "..", "include", "l4l.h")]
+
+
+def marshal_tag() -> str:
+    """What the module's layout of tensors and of the interpreter depends on; compiled into it, and compared when it is loaded."""
+    import torch
+
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}, {' '.join(MARSHAL_FLAGS)}"
+
+
+def marshal_is_stale() -> bool:
+    if _stale(MARSHAL, MARSHAL_SRC):
+        return True
+    with open(MARSHAL, "rb") as f:
+        return marshal_tag().encode() not in f.read()
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -60,15 +80,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".tmp{os.getpid()}"
         run(["nvcc", "-shared", "-Wno-deprecated-gpu-targets", "-o", tmp] + objs)
         os.replace(tmp, LIB)
-    src = os.path.join(CSRC, "l4l_marshal.cpp")
-    if force or _stale(MARSHAL, [src, os.path.join(PKG, "..", "include", "l4l.h")]):
+    if force or marshal_is_stale():
         import torch
 
         home = os.path.dirname(torch.__file__)
+        cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
         tmp = MARSHAL + f".tmp{os.getpid()}"
-        run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
-             f"-I{home}/include", f"-I{home}/include/torch/csrc/api/include", "-I/usr/local/cuda/include",
-             "-I" + sysconfig.get_paths()["include"], src, "-o", tmp, f"-L{PKG}", "-l:libl4l.so", f"-L{home}/lib",
+        run(["g++", *MARSHAL_FLAGS, f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", f'-DL4L_BUILT_FOR="{marshal_tag()}"',
+             f"-I{home}/include", f"-I{home}/include/torch/csrc/api/include", f"-I{cuda}/include",
+             "-I" + sysconfig.get_paths()["include"], MARSHAL_SRC[0], "-o", tmp, f"-L{PKG}", "-l:libl4l.so", f"-L{home}/lib",
              "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
         os.replace(tmp, MARSHAL)
     return LIB

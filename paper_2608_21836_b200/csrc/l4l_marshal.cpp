@@ -386,4 +386,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_l4l_marshal", nullptr, -1, method
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__l4l_marshal() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__l4l_marshal()
+{
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "BUILT_FOR", L4L_BUILT_FOR) < 0) Py_CLEAR(m);
+    return m;
+}

@@ -11,6 +11,18 @@ def built():
     build.build()
 
 
+def test_a_module_for_another_torch_is_rebuilt_and_not_loaded(monkeypatch, tmp_path):
+    assert not build.marshal_is_stale() and l4l._load_native().BUILT_FOR == build.marshal_tag()
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    assert build.marshal_is_stale()
+    monkeypatch.setattr(l4l, "_native", None)
+    with pytest.raises(ImportError, match="9.9.9.*build it with"):
+        l4l._load_native()
+    monkeypatch.setattr(build, "MARSHAL", str(tmp_path / "missing.so"))
+    with pytest.raises(FileNotFoundError, match="build it with"):
+        l4l._load_native()
+
+
 def calls(t4, t3, i):
     """Every call of the native module, its tensors all of one kind."""
     t2 = torch.zeros(4, 32)

@@ -960,21 +960,19 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                     __syncwarp();
                 }
                 if (nvalid > 0) {
-                    // 32 tokens per step: two 16-token blocks share one softmax update. A block with no valid
-                    // token is skipped (its rows may never have been fetched); in the last valid block the
-                    // tokens past the end get no weight and their V rows are cleared.
+                    // 32 tokens per step: two 16-token blocks share one softmax update. A block with no valid token (its rows
+                    // may never have been fetched) gets scores like the others, which are dropped, and no product with V; in
+                    // the last valid block the tokens past the end get no weight and their V rows are cleared.
                     constexpr int kSub = C::kSub;
                     float sv[kSub][NB][4];
                     const float sc = p.scale_log2e * k_sc;
+                    warp_qk_f8<D, NB, kSub>(qf, k_tile, row0, sv);
 #pragma unroll
-                    for (int u = 0; u < kSub; ++u) {
-                        const bool on = u == 0 || nvalid > 16 * u;
-                        if (on) warp_qk_f8<D, NB>(qf, k_tile, row0 + 16 * u, sv[u]);
+                    for (int u = 0; u < kSub; ++u)
 #pragma unroll
                         for (int n = 0; n < NB; ++n)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) sv[u][n][e] = on ? sv[u][n][e] * sc : -INFINITY;
-                    }
+                            for (int e = 0; e < 4; ++e) sv[u][n][e] *= sc;
                     if (nvalid < 16 * kSub) {
                         warp_mask<NB, kSub>(sv, nvalid);
                         uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;
@@ -993,22 +991,23 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_con
                         if (u == 0 || nvalid > 16 * u) warp_pv_f8<D, NB>(st, pb[u], v_tile, row0 + 16 * u);
                 }
             } else if (nvalid > 0) {
-                // kSub 16-token blocks per step share one softmax update. A block with no valid token is skipped (its
-                // rows may never have been fetched); in the last valid block the tokens past the end of the sequence get
-                // no weight, and their V rows (which may hold any bits, NaN included) are cleared so that 0 * garbage
-                // cannot appear.
+                // kSub 16-token blocks per step share one softmax update. A block with no valid token (its rows may never have
+                // been fetched) gets scores like the others, which are dropped, and no product with V; in the last valid block
+                // the tokens past the end of the sequence get no weight, and their V rows (which may hold any bits, NaN
+                // included) are cleared so that 0 * garbage cannot appear.
                 constexpr int kSub = C::kSub;
                 float sv[kSub][NB][4];
                 const float sc = p.scale_log2e;
+                uint32_t k_block[kSub];
 #pragma unroll
-                for (int u = 0; u < kSub; ++u) {
-                    const bool on = u == 0 || nvalid > 16 * u;
-                    if (on) warp_qk<D, NB>(qf, k_tile + rows.row(row0 + 16 * u), rows.half_bytes, 0, sv[u]);
+                for (int u = 0; u < kSub; ++u) k_block[u] = k_tile + rows.row(row0 + 16 * u);
+                warp_qk<D, NB, kSub>(qf, k_block, rows.half_bytes, sv);
+#pragma unroll
+                for (int u = 0; u < kSub; ++u)
 #pragma unroll
                     for (int n = 0; n < NB; ++n)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) sv[u][n][e] = on ? sv[u][n][e] * sc : -INFINITY;
-                }
+                        for (int e = 0; e < 4; ++e) sv[u][n][e] *= sc;
                 if (nvalid < 16 * kSub) {
                     warp_mask<NB, kSub>(sv, nvalid);
                     uint8_t *vt = stages + (size_t)s * C::kStageBytes + C::kTileBytes;

@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(kWarps * 32) decode_warp_kernel(const WarpPara
                 __syncwarp();
             }
             float sv[1][NB][4];
-            if constexpr (F8) warp_qk_f8<D, NB>(qf, k_tile, 0, sv[0]);
-            else warp_qk<D, NB>(qf, k_tile, C::kHalfBytes, 0, sv[0]);
+            if constexpr (F8) warp_qk_f8<D, NB, 1>(qf, k_tile, 0, sv);
+            else warp_qk<D, NB, 1>(qf, {k_tile}, C::kHalfBytes, sv);
             const float sc = F8 ? p.scale_log2e * k_sc : p.scale_log2e;
 #pragma unroll
             for (int n = 0; n < NB; ++n)

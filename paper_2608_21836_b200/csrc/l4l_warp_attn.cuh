@@ -7,10 +7,10 @@
 // rows it would fill a quarter of 16: half the MMAs, half the exponentials, and the output accumulators of a 128-wide
 // head are 32 registers instead of 64 (NB = 2 blocks of 8 heads, for groups of 9 to 16, are as before). P^T is the B operand of
 // the second product: an 8 x 8 transpose of the score fragment (movmatrix). Measured, us, heads as rows -> as columns: e4m3
-// cache, B = 32 ragged 37.0 -> 32.2; B = 512 x 64..256 tokens 65.8 -> 62.9; bf16 caches of large batches, bound by HBM, 46.7
-// -> 46.5. Every sum has the order that it has with the heads as rows, so that the results are the same bit for bit: one
-// accumulator per score, and denominators summed from the transposed weights. (Two accumulators for even and odd k-steps and sums
-// ahead of the transpose would save 0.1 to 0.2 us: one sequence of 2304 tokens 8.57 against 8.69, the e4m3 batch 31.96 against 32.19.)
+// cache, B = 32 ragged 37.0 -> 31.7; B = 512 x 64..256 tokens 65.1 -> 62.4; bf16 caches of large batches are bound by HBM, 46.2
+// either way. Every sum has the order that it has with the heads as rows, so that the results are the same bit for bit: one
+// accumulator per score, and denominators summed from the transposed weights. (Two accumulators for even and odd k-steps and
+// sums ahead of the transpose would save one sequence of 2304 tokens 8.58 against 8.70 us, 512 short ones 62.2 against 62.4.)
 //
 // Tile layout in shared memory: D/64 "halves", each [tile_tokens][64] bf16 (128-byte rows,
 // swizzled), half h covering head_dim [64h, 64h+64). Over pages of 16 or 32 tokens at head_dim 128 one load brings
@@ -88,25 +88,31 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qf)[D / 16][NB][2], 
 }
 
 // S^T (16 tokens x 8 NB heads) = K(tokens row0 .. row0 + 15) . Q^T. s[n]: [e] token row0 + r, [2 + e] token row0 + r + 8 of
-// head 8n + 2c + e. One accumulator per block, the k-steps in their order.
-template <int D, int NB>
-__device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, uint32_t half_bytes, int row0,
-                                        float (&s)[NB][4])
+// head 8n + 2c + e. One accumulator per score, the k-steps in their order; several blocks of 16 tokens (block u at k_tile[u], rows from
+// row0 on) are so many independent chains, issued in turn.
+template <int D, int NB, int NT>
+__device__ __forceinline__ void warp_qk(const uint32_t (&qf)[D / 16][NB][2], const uint32_t (&k_tile)[NT], uint32_t half_bytes,
+                                        float (&s)[NT][NB][4])
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int n = 0; n < NB; ++n)
+    for (int u = 0; u < NT; ++u)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
-    const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[u][n][e] = 0.f;
+    const uint32_t row = lane & 15;                                 // matrices 1, 3: tokens + 8
     const uint32_t csel = lane >> 4;                                // matrices 2, 3: head dims + 8
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t chunk = 2 * ks + csel;                       // 16-byte chunk of the full row
-        uint32_t a[4];
-        ldmatrix_x4(k_tile + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
 #pragma unroll
-        for (int n = 0; n < NB; ++n) mma_bf16_16816(s[n], a, qf[ks][n][0], qf[ks][n][1]);
+        for (int u = 0; u < NT; ++u) {
+            uint32_t a[4];
+            ldmatrix_x4(k_tile[u] + (chunk >> 3) * half_bytes + swz128(row, chunk & 7), a[0], a[1], a[2], a[3]);
+#pragma unroll
+            for (int n = 0; n < NB; ++n) mma_bf16_16816(s[u][n], a, qf[ks][n][0], qf[ks][n][1]);
+        }
     }
 }
 
@@ -217,27 +223,33 @@ __device__ __forceinline__ uint32_t tok_chunk_f8(uint32_t tile, uint32_t tok, ui
     else return tile + swz128(tok >> 1, ((tok & 1u) << 2) + c);
 }
 
-template <int D, int NB>
-__device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, int row0, float (&s)[NB][4])
+template <int D, int NB, int NT>
+__device__ __forceinline__ void warp_qk_f8(const uint32_t (&qf)[D / 16][NB][2], uint32_t k_tile, int row0, float (&s)[NT][NB][4])
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int n = 0; n < NB; ++n)
+    for (int u = 0; u < NT; ++u)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[u][n][e] = 0.f;
     const uint32_t row = row0 + (lane & 15);                        // matrices 1, 3: tokens + 8
     const uint32_t csel = lane >> 4;                                // matrices 2, 3: next 16 head dims
 #pragma unroll
     for (int qd = 0; qd < D / 32; ++qd) {
-        uint32_t r0, r1, r2, r3;
-        ldmatrix_x4(tok_chunk_f8<D>(k_tile, row, 2 * qd + csel), r0, r1, r2, r3);
-        const uint32_t a[4] = {e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16)};
-        const uint32_t b[4] = {e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16)};
+        uint32_t r[NT][4];
 #pragma unroll
-        for (int n = 0; n < NB; ++n) {
-            mma_f16_16816(s[n], a, qf[2 * qd][n][0], qf[2 * qd][n][1]);
-            mma_f16_16816(s[n], b, qf[2 * qd + 1][n][0], qf[2 * qd + 1][n][1]);
-        }
+        for (int u = 0; u < NT; ++u)
+            ldmatrix_x4(tok_chunk_f8<D>(k_tile, row + 16 * u, 2 * qd + csel), r[u][0], r[u][1], r[u][2], r[u][3]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)                                 // head dims 32 qd + 16 h ..
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+                const uint32_t lo = r[u][2 * h], hi = r[u][2 * h + 1];
+                const uint32_t a[4] = {e4m3x2_to_f16x2(lo), e4m3x2_to_f16x2(hi), e4m3x2_to_f16x2(lo >> 16), e4m3x2_to_f16x2(hi >> 16)};
+#pragma unroll
+                for (int n = 0; n < NB; ++n) mma_f16_16816(s[u][n], a, qf[2 * qd + h][n][0], qf[2 * qd + h][n][1]);
+            }
     }
 }
 

@@ -1,7 +1,8 @@
 """Thin binding of the C-ABI library ``libl4l.so`` (same names as ``include/l4l.h``).
 
 Argument marshalling only: tensors become pointers + strides, the current CUDA stream
-becomes a ``void*``, in ``_l4l_marshal`` (C++) for the calls of every step and by ctypes for the rest. Every step of the attention path runs inside the library's kernels;
+becomes a ``void*``, in ``_l4l_marshal`` (C++) for the calls of every step and by ctypes
+for the rest. Every step of the attention path runs inside the library's kernels;
 PyTorch is used for device memory and streams. There is no fallback: if the library is
 missing or a call fails, an exception is raised.
 """

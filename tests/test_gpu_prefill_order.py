@@ -11,9 +11,10 @@ SENTINEL = 0x4D4D
 i32 = lambda a: torch.from_numpy(np.asarray(a, np.int32)).cuda()  # noqa: E731
 
 
-# ranked launches from just beyond two blocks per SM (B = 31: 310) to many, head pairs and single heads; B = 33 and more: by place
+# ranked launches from just beyond two blocks per SM (B = 31: 310) to many, head pairs and single heads; by place: few blocks, B > 32
 @pytest.mark.parametrize("page", [0, 16, 256])
-@pytest.mark.parametrize("B,Hq,Hkv,D", [(2, 64, 8, 64), (31, 4, 2, 64), (32, 5, 5, 64), (32, 4, 2, 128), (33, 3, 1, 64), (129, 4, 2, 64)])
+@pytest.mark.parametrize("B,Hq,Hkv,D", [(2, 4, 2, 64), (2, 64, 8, 64), (31, 4, 2, 64), (32, 5, 5, 64), (32, 4, 2, 128), (33, 3, 1, 64),
+                                         (70, 2, 1, 128), (128, 5, 5, 64), (129, 4, 2, 64)])
 def test_row_blocks_by_work_cover_every_row_once(B, Hq, Hkv, D, page):
     r = np.random.default_rng(B)
     S, slots = 520, 1280
@@ -21,7 +22,8 @@ def test_row_blocks_by_work_cover_every_row_once(B, Hq, Hkv, D, page):
     past[r.integers(0, B, B // 2)] = 256                       # equal weights, and sequences with nothing to do
     qlen[r.integers(0, B, B // 4)] = 0
     past[0], qlen[0] = 0, S
-    assert (l4l.l4l_prefill_row_block_order(i32(past), i32(qlen), S, slots, Hq, Hkv, D) is None) == (B > 32)
+    by_work = l4l.l4l_prefill_row_block_order(i32(past), i32(qlen), S, slots, Hq, Hkv, D) is not None
+    assert by_work == ((B, Hq) in ((2, 64), (31, 4), (32, 5), (32, 4)))
     g = torch.Generator(device="cuda").manual_seed(B)
     mk = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.bfloat16)  # noqa: E731
     q, kn, vn = mk(B, S, Hq, D), mk(B, S, Hkv, D), mk(B, S, Hkv, D)

@@ -4,7 +4,7 @@
 //
 // The recurrence is sequential in time and independent across (sequence, channel). A CTA owns 64 channels
 // of one sequence (two per lane, packed fp32x2 arithmetic) and walks the time axis in tiles of 16 steps,
-// its 8 warps taking the tiles in turn (warp w: tiles w, w + 8, ...; a single warp when there is only one tile). Per tile a warp
+// its 8 warps taking the tiles in turn (warp w: tiles w, w + 8, ...). Per tile a warp
 //   1. has the tile's x, gate_x and gate_a in shared memory (its own TMA double buffer: as soon as a tile's
 //      values are in registers the buffer is refilled with the warp's tile after next),
 //   2. evaluates a_t and b_t of all 16 steps (independent of the state, so MUFU and FMA latencies overlap)
@@ -46,8 +46,7 @@ constexpr int kStages = 2;       // TMA buffers per warp
 constexpr uint32_t kArrayBytes = kTb * kCb * 2;   // one array of a warp's tile: (kTb * kSplit) steps x (kCb / kSplit) channels
 constexpr uint32_t kStageBytes = 3 * kArrayBytes;
 // kTeam warps per CTA, each taking every kTeam-th tile: 8 for sequences, 16 when the launch has no more strips
-// than the GPU has SMs (one CTA per SM then, and a strip's rate is set by how many tiles it has in flight),
-// 1 for a single tile (decode steps)
+// than the GPU has SMs (one CTA per SM then, and a strip's rate is set by how many tiles it has in flight)
 constexpr size_t smem_bytes(int team)
 {
     return 128 + (size_t)team * kStages * kStageBytes + (team * kStages + team) * 8 + 2 * kCb * 4 + 64;
@@ -82,6 +81,58 @@ __device__ __forceinline__ float sqrt_approx(float x)
 // two bf16 in one word -> packed fp32x2 (low half first)
 __device__ __forceinline__ uint64_t widen2(uint32_t w) { return pack_u32x2(w << 16, w & 0xffff0000u); }
 
+// The constants of a step's gates for two channels.
+struct GateConsts {
+    uint64_t k2h;                        // -4 softplus(a_param) log2(e)
+    uint64_t half2, quarter2, nquarter2, s1c, s2c, s3c, s4c;
+};
+
+__device__ __forceinline__ GateConsts gate_consts(const float *a_param, int c, bool live)
+{
+    // (1 - a^2) / 4 = -expm1(z) / 4 with z = w log2(a), w = 2 ln 2: series coefficients in log2(a), the quarter (which
+    // the square root turns into the half of sigmoid = 0.5 tanh + 0.5) folded in
+    constexpr float kW = 1.3862943611198906f;
+    GateConsts g;
+    uint64_t k2 = pack_f32x2(0.f, 0.f);                  // -8 softplus(a_param) log2(e)
+    if (live) {
+        const float2 lam = *reinterpret_cast<const float2 *>(a_param + c);
+        const float sp0 = lam.x > 15.f ? lam.x : log1pf(expf(lam.x));
+        const float sp1 = lam.y > 15.f ? lam.y : log1pf(expf(lam.y));
+        k2 = pack_f32x2(-8.f * 1.4426950408889634f * sp0, -8.f * 1.4426950408889634f * sp1);
+    }
+    g.half2 = pack_f32x2(0.5f, 0.5f);
+    g.k2h = mul_f32x2(k2, g.half2);
+    g.quarter2 = pack_f32x2(0.25f, 0.25f);
+    g.nquarter2 = pack_f32x2(-0.25f, -0.25f);
+    g.s1c = pack_f32x2(-kW / 4, -kW / 4);
+    g.s2c = pack_f32x2(-kW * kW / 8, -kW * kW / 8);
+    g.s3c = pack_f32x2(-kW * kW * kW / 24, -kW * kW * kW / 24);
+    g.s4c = pack_f32x2(-kW * kW * kW * kW / 96, -kW * kW * kW * kW / 96);
+    return g;
+}
+
+// A step's gates from the words of gate_x and gate_a: tanh(gate_x / 2), a and m / 2 of two channels.
+__device__ __forceinline__ void gates_of(const GateConsts &g, uint32_t gx, uint32_t ga, uint64_t &th_x, uint64_t &a, float &m0, float &m1)
+{
+    constexpr float kW = 1.3862943611198906f, kNearOne = -0.0625f / kW;
+    float g0, g1, r0, r1;
+    unpack_f32x2(mul_f32x2(widen2(gx), g.half2), g0, g1);
+    unpack_f32x2(mul_f32x2(widen2(ga), g.half2), r0, r1);
+    th_x = pack_f32x2(tanh_approx(g0), tanh_approx(g1));                       // sigmoid = 0.5 tanh(z/2) + 0.5
+    const uint64_t th_a = pack_f32x2(tanh_approx(r0), tanh_approx(r1));
+    const uint64_t la2 = fma_f32x2(th_a, g.k2h, g.k2h);                        // log2(a) = k2 * sigmoid(gate_a)
+    float l0, l1;
+    unpack_f32x2(la2, l0, l1);
+    a = pack_f32x2(fast_exp2(l0), fast_exp2(l1));
+    // m / 2 = sqrt((1 - a^2) / 4): a short series when a is close to 1, where 1 - a*a cancels
+    const uint64_t series = fma_f32x2(la2, fma_f32x2(la2, fma_f32x2(la2, g.s4c, g.s3c), g.s2c), g.s1c);
+    float s0, s1, d0, d1;
+    unpack_f32x2(mul_f32x2(la2, series), s0, s1);
+    unpack_f32x2(fma_f32x2(mul_f32x2(a, g.nquarter2), a, g.quarter2), d0, d1);
+    m0 = sqrt_approx(l0 > kNearOne ? s0 : d0);
+    m1 = sqrt_approx(l1 > kNearOne ? s1 : d1);
+}
+
 // kSeg: the launch is cut along the time axis (an instantiation of its own: the other launches are 8 % faster without its code)
 template <int kTeam, int kSplit, bool kSeg>
 __global__ void __launch_bounds__(kTeam * 32)
@@ -102,6 +153,16 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / kPairs, cp = lane % kPairs;   // this lane's sub-tile and channel pair
     const int b = blockIdx.y, c0 = blockIdx.x * kCw;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kTeam * kStages; ++s) mbar_init(&full[s], 1);
+        for (int w = 0; w < kTeam; ++w) mbar_init(&handed[w], 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+        fence_proxy_async_smem();
+    }
+    // everything above overlaps the tail of the kernel before; nothing is read before that has completed
+    grid_dependency_wait();
+    grid_launch_dependents();
     int L = p.seq_lens ? p.seq_lens[b] : p.T;
     L = L < 0 ? 0 : (L > p.T ? p.T : L);
     // this block's segment of the time axis: tiles [tile0, n_tiles) of the n_all tiles that the sequence has
@@ -112,13 +173,6 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int c = c0 + 2 * cp;
     const bool live = c < p.W;                           // W is even: both channels or neither
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kTeam * kStages; ++s) mbar_init(&full[s], 1);
-        for (int w = 0; w < kTeam; ++w) mbar_init(&handed[w], 1);
-        *abort_flag = 0;
-        fence_barrier_init();
-        fence_proxy_async_smem();
-    }
     if (warp == 0 && sub == 0) {
         // slot 0: the state that the block's first tile starts from (a later segment's: below)
         const float2 st = live && segment == 0 ? *reinterpret_cast<const float2 *>(p.state + (size_t)b * p.W + c) : make_float2(0.f, 0.f);
@@ -149,22 +203,8 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     }
     for (int k = 0; k < kStages; ++k) request(k);
 
-    uint64_t k2 = pack_f32x2(0.f, 0.f);                  // -8 softplus(a_param) log2(e), per channel
-    if (live) {
-        const float2 lam = *reinterpret_cast<const float2 *>(p.a_param + c);
-        const float sp0 = lam.x > 15.f ? lam.x : log1pf(expf(lam.x));
-        const float sp1 = lam.y > 15.f ? lam.y : log1pf(expf(lam.y));
-        k2 = pack_f32x2(-8.f * 1.4426950408889634f * sp0, -8.f * 1.4426950408889634f * sp1);
-    }
-    const uint64_t half2 = pack_f32x2(0.5f, 0.5f), one2 = pack_f32x2(1.f, 1.f), zero2 = pack_f32x2(0.f, 0.f);
-    const uint64_t k2h = mul_f32x2(k2, half2);
-    // (1 - a^2) / 4 = -expm1(z) / 4 with z = w log2(a), w = 2 ln 2: series coefficients in log2(a), the quarter (which
-    // the square root turns into the half of sigmoid = 0.5 tanh + 0.5) folded in
-    constexpr float kW = 1.3862943611198906f, kNearOne = -0.0625f / kW;
-    const uint64_t s1c = pack_f32x2(-kW / 4, -kW / 4), s2c = pack_f32x2(-kW * kW / 8, -kW * kW / 8);
-    const uint64_t s3c = pack_f32x2(-kW * kW * kW / 24, -kW * kW * kW / 24);
-    const uint64_t s4c = pack_f32x2(-kW * kW * kW * kW / 96, -kW * kW * kW * kW / 96);
-    const uint64_t quarter2 = pack_f32x2(0.25f, 0.25f), nquarter2 = pack_f32x2(-0.25f, -0.25f);
+    const GateConsts consts = gate_consts(p.a_param, c, live);
+    const uint64_t one2 = pack_f32x2(1.f, 1.f), zero2 = pack_f32x2(0.f, 0.f);
     uint32_t *yrow = reinterpret_cast<uint32_t *>(p.y + (size_t)b * p.T * p.W + c);
     const size_t y_step = (size_t)p.W / 2;               // 32-bit words between time steps
     // Positions of a tile's steps, one per lane and part, as loaded: the vote that turns them into a mask comes a whole
@@ -232,21 +272,9 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 #pragma unroll
             for (int t = 0; t < kTb; ++t) {
                 const uint64_t xv = widen2(xs[t * kPairs]);
-                float g0, g1, r0, r1;
-                unpack_f32x2(mul_f32x2(widen2(gxs[t * kPairs]), half2), g0, g1);
-                unpack_f32x2(mul_f32x2(widen2(gas[t * kPairs]), half2), r0, r1);
-                const uint64_t th_x = pack_f32x2(tanh_approx(g0), tanh_approx(g1));   // sigmoid = 0.5 tanh(z/2) + 0.5
-                const uint64_t th_a = pack_f32x2(tanh_approx(r0), tanh_approx(r1));
-                const uint64_t la2 = fma_f32x2(th_a, k2h, k2h);                        // log2(a) = k2 * sigmoid(gate_a)
-                float l0, l1;
-                unpack_f32x2(la2, l0, l1);
-                uint64_t a = pack_f32x2(fast_exp2(l0), fast_exp2(l1));
-                // m / 2 = sqrt((1 - a^2) / 4): a short series when a is close to 1, where 1 - a*a cancels
-                const uint64_t series = fma_f32x2(la2, fma_f32x2(la2, fma_f32x2(la2, s4c, s3c), s2c), s1c);
-                float s0, s1, d0, d1;
-                unpack_f32x2(mul_f32x2(la2, series), s0, s1);
-                unpack_f32x2(fma_f32x2(mul_f32x2(a, nquarter2), a, quarter2), d0, d1);
-                float m0 = sqrt_approx(l0 > kNearOne ? s0 : d0), m1 = sqrt_approx(l1 > kNearOne ? s1 : d1);
+                uint64_t th_x, a;
+                float m0, m1;
+                gates_of(consts, gxs[t * kPairs], gas[t * kPairs], th_x, a, m0, m1);
                 if constexpr (!kPlain) {
                     if ((resets >> t) & 1u) {                                          // uniform across a sub-tile's lanes
                         a = zero2;
@@ -329,6 +357,71 @@ rglru_scan_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status + kStatusErrWord, kErrScanWait);
 }
 
+// A few steps (decode, T <= kTb): a thread per channel pair walks them, straight from global memory. There is too little
+// work for a ring; the launch is one round trip to memory and a chain of gates. Against one warp and one TMA tile per 64
+// channels, which worked out sixteen steps whatever T was (launches back to back): 64 x 1 x 4096 10.3 -> 4.5 us, 16 x 1 x 2560
+// 6.2 -> 3.2, 8 x 16 x 2560 6.2 -> 3.8, 64 x 16 x 4096 12.3 -> 9.9, so it is taken up to sixteen steps.
+struct RglruStepParams {
+    const uint32_t *x, *gate_x, *gate_a;
+    const float *a_param;
+    const int32_t *position, *seq_lens;
+    float *state;
+    uint32_t *y;
+    int T, W;
+};
+
+template <int kAtOnce>
+__global__ void __launch_bounds__(128) rglru_steps_kernel(const RglruStepParams p)
+{
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const int b = blockIdx.y, pair = blockIdx.x * 128 + threadIdx.x, pairs = p.W / 2;
+    if (pair >= pairs) return;
+    const size_t row0 = (size_t)b * p.T;
+    int L = p.seq_lens ? __ldg(p.seq_lens + b) : p.T;
+    float2 *state = reinterpret_cast<float2 *>(p.state + (size_t)b * p.W) + pair;
+    const float2 st = *state;
+    uint64_t h = pack_f32x2(st.x, st.y);
+    const GateConsts consts = gate_consts(p.a_param, 2 * pair, true);
+    for (int t0 = 0; t0 < p.T; t0 += kAtOnce) {
+        // asked for together with the length (rows past it may hold anything, and are not used)
+        uint32_t xw[kAtOnce], gx[kAtOnce], ga[kAtOnce];
+        int pos[kAtOnce];
+#pragma unroll
+        for (int t = 0; t < kAtOnce; ++t) {
+            if (t0 + t < p.T) {
+                const size_t at = (row0 + t0 + t) * pairs + pair;
+                xw[t] = p.x[at];
+                gx[t] = p.gate_x[at];
+                ga[t] = p.gate_a[at];
+                pos[t] = p.position ? __ldg(p.position + row0 + t0 + t) : 1;
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kAtOnce; ++t) {
+            if (t0 + t < min(L, p.T)) {
+                uint64_t th_x, a;
+                float m0, m1;
+                gates_of(consts, gx[t], ga[t], th_x, a, m0, m1);
+                if (pos[t] == 0) {                                             // the first token of a segment
+                    a = pack_f32x2(0.f, 0.f);
+                    m0 = m1 = 0.5f;
+                }
+                const uint64_t mxh = mul_f32x2(pack_f32x2(m0, m1), widen2(xw[t]));
+                h = fma_f32x2(a, h, fma_f32x2(th_x, mxh, mxh));
+                float h0, h1;
+                unpack_f32x2(h, h0, h1);
+                p.y[(row0 + t0 + t) * pairs + pair] = pack_bf16x2(h0, h1);
+            }
+        }
+    }
+    if (L > 0) {
+        float h0, h1;
+        unpack_f32x2(h, h0, h1);
+        *state = make_float2(h0, h1);
+    }
+}
+
 }  // namespace
 
 // the status block and one counter per strip (of the narrowest width) where they fit the region that decode calls on
@@ -343,6 +436,25 @@ namespace {
 
 int tiles_of(int T, int split) { return (T + kTb * split - 1) / (kTb * split); }
 int tiles_per_segment(int tiles, int segments, int team) { return (tiles + segments * team - 1) / (segments * team) * team; }   // whole rounds of the team
+
+// A launch whose blocks may set themselves up under the tail of the kernel before: launches back to back 4 x 64 x 2560 6.2 -> 4.6 us,
+// 16 x 300 x 1024 14.4 -> 13.2, 64 x 100 x 2560 46.7 -> 44.5; nothing on 4 x 8192 x 2560 (147 us).
+struct Launch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    Launch(dim3 grid, int threads, size_t smem, cudaStream_t stream)
+    {
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    Launch(const Launch &) = delete;
+};
 
 template <int kTeam, int kSplit, bool kSeg = false>
 l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, RglruParams p, int segments, cudaStream_t stream)
@@ -369,8 +481,8 @@ l4l_status launch_shape(const void *x, const void *gate_x, const void *gate_a, R
     const int strips = (p.W + kCw - 1) / kCw, tiles = tiles_of(p.T, kSplit);
     p.seg_tiles = kSeg ? tiles_per_segment(tiles, segments, kTeam) : tiles;
     const dim3 grid(strips, p.B, (tiles + p.seg_tiles - 1) / p.seg_tiles);
-    rglru_scan_kernel<kTeam, kSplit, kSeg><<<grid, kTeam * 32, smem_bytes(kTeam), stream>>>(tx, tgx, tga, p);
-    return cudaGetLastError() == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
+    const Launch launch(grid, kTeam * 32, smem_bytes(kTeam), stream);
+    return cudaLaunchKernelEx(&launch.cfg, rglru_scan_kernel<kTeam, kSplit, kSeg>, tx, tgx, tga, p) == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
 }
 
 }  // namespace
@@ -385,7 +497,12 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
     p.status = static_cast<unsigned *>(workspace);
     p.B = B; p.T = T; p.W = W;
     p.progress = reinterpret_cast<int *>(static_cast<uint8_t *>(workspace) + kStatusBytes);
-    if (T <= kTb) return launch_shape<1, 1>(x, gate_x, gate_a, p, 1, stream);
+    if (T <= kTb) {
+        const RglruStepParams sp{static_cast<const uint32_t *>(x), static_cast<const uint32_t *>(gate_x), static_cast<const uint32_t *>(gate_a),
+                                 d_a_param, d_position, d_seq_lens, d_state, static_cast<uint32_t *>(y), T, W};
+        const Launch launch(dim3((W / 2 + 127) / 128, B), 128, 0, stream);
+        return cudaLaunchKernelEx(&launch.cfg, T == 1 ? rglru_steps_kernel<1> : rglru_steps_kernel<8>, sp) == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
+    }
     int segs = 1;
     const int split = rglru_shape(B, T, W, d_position != nullptr, ws_bytes, &segs);
     if (segs > 1)
@@ -398,8 +515,8 @@ l4l_status launch_rglru_scan(const void *x, const void *gate_x, const void *gate
     return launch_shape<8, 1>(x, gate_x, gate_a, p, 1, stream);
 }
 
-// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels (a single warp for a
-// single tile). *segments (when given): into how many segments the time axis is cut; positions: the launch has reset positions.
+// 0: 64-channel strips with teams of 16 warps; 1, 2, 4: teams of 8 warps on strips of 64, 32, 16 channels (sequences of at
+// most kTb steps have no tiles). *segments (when given): into how many segments the time axis is cut; positions: the launch has reset positions.
 static int rglru_strip_split(int B, int T, int W, int *segments, bool positions)
 {
     if (segments) *segments = 1;

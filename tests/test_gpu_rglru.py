@@ -75,6 +75,33 @@ def test_rglru_matches_oracle(B, T, W):
     assert (gy.t.cpu().view(torch.int16).numpy()[~valid] == SENTINEL).all()          # rows past seq_len untouched
 
 
+@pytest.mark.parametrize("B,T,W", [(1, 1, 8), (3, 1, 264), (70, 1, 256), (4, 2, 2560), (3, 7, 264), (3, 8, 256), (3, 9, 1032), (5, 16, 520)])
+def test_rglru_few_steps(B, T, W):
+    """Decode steps and short chunks (no tiles, a thread per channel pair): around the eight steps taken at once and the 128 pairs of a
+    block, with empty and ragged sequences, resets inside and rows past the end that hold NaN."""
+    x, gx, ga, ap, h0 = make(B, T, W, 77 + T)
+    # halved, so that all |y| < 4: half a bf16 ulp is 7.8e-3 there and 1.6e-2 above, beyond the absolute bound of check()
+    h0, x = 0.5 * h0, 0.5 * x
+    pos = torch.arange(5, 5 + T, dtype=torch.int32).repeat(B, 1)
+    pos[0] = torch.arange(T)
+    pos[-1, T // 2:] = torch.arange(T - T // 2)
+    lens = [T] + [(T - 2 * i) % (T + 1) for i in range(1, B)]
+    dead = torch.arange(T).view(1, T, 1) >= torch.tensor(lens).view(B, 1, 1)
+    nan = nan_bf16((1,))
+    x, gx, ga = torch.where(dead, nan, x), torch.where(dead, nan, gx), torch.where(dead, nan, ga)
+    y_ref, st_ref = orc.rglru(x, gx, ga, ap.numpy(), state=h0.double().numpy(), position=pos.numpy(), seq_len=lens)
+    gy = Guarded(torch.full((B, T, W), SENTINEL, dtype=torch.int16).view(torch.bfloat16))
+    gs = Guarded(h0)
+    ws = l4l.new_rglru_workspace(B, T, W)
+    l4l.l4l_rglru_scan(x.cuda(), gx.cuda(), ga.cuda(), ap.cuda(), gs.t, gy.t, ws, position=pos.cuda(),
+                       seq_lens=torch.tensor(lens, dtype=torch.int32).cuda())
+    torch.cuda.synchronize()
+    assert gy.margins_intact() and gs.margins_intact()
+    valid = np.broadcast_to(np.arange(T)[None, :, None] < np.array(lens)[:, None, None], (B, T, W))
+    check(gy.t, gs.t, y_ref, st_ref, valid)
+    assert (gy.t.cpu().view(torch.int16).numpy()[~valid] == SENTINEL).all()
+
+
 def test_rglru_chunks_carry_the_state():
     """A prompt of 200 steps, then single steps (the decode regime): same as one pass over all of it."""
     B, T, W = 2, 205, 128

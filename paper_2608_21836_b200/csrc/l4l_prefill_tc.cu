@@ -9,12 +9,20 @@
 //   warps 0-3   softmax of sub-tile 0: thread t owns row t (= TMEM lane t): reads S from TMEM,
 //               keeps the running max / sum in fp32, writes P (bf16) back into TMEM over S
 //   warps 4-7   the same for sub-tile 1
-//   warp  8     TMA producer: Q once, then K_j, V_j tiles (128 tokens, 128-byte swizzle) through a
-//               ring of shared-memory slots; afterwards copies the block's diagonal K/V tiles from
-//               shared memory into the KV cache (only for the first query head of a KV group)
+//   warp  8     TMA producer: Q, then K_j, V_j tiles (128 tokens, 128-byte swizzle) through a ring of shared-memory slots, item
+//               after item
 //   warp  9     MMA issuer (one lane): S_i = Q_i K_j^T from shared memory, O_i += P_i V_j with P read
 //               from TMEM and V as an MN-major shared-memory operand; owns the TMEM allocation
-//   warps 10-11 help with the cache copy, which runs beside the last iterations
+//   warps 10-11 what leaves: the block's diagonal K/V tiles into the KV cache (first query head of a KV group only), output rows
+//
+// A CTA that is through with its block goes on with blocks of the launch that have not started (cluster launch control), until none is
+// left: the next item's loads run ahead through the ring under the last tiles of the present one, and its first product follows the
+// last of this one. A block of its own for every item paid 5.7 us of launch, set-up, first loads and last stores around its tiles; an item
+// that follows another pays 1.3. The claim comes when the item's last loads are on their way, about two tile pairs ahead of its end: later
+// than that the loads would start late, earlier the order of the heaviest first would suffer. The MMA issuer's warp has uniform control flow
+// (values broadcast, one vote per tile, an elected lane): with branches per lane a tile pair took 3500-3640 cycles instead of 3250-3350,
+// which is more than the items gain. Figures (kept up, where the power cap sets the clock; start of one by one): four prompts of 8192 2188 -> 2110 us, one of 2048 44.8 -> 43.6, six of 517 to 1592 with the rotation
+// 138.2 -> 126.3, five paged chunks 116.3 -> 117.1, a prompt of one block per head pair 6.8 -> 7.1 (no claims; the longer way to the first item).
 //
 // The same kernel serves a chunk of new tokens over a populated cache. The key axis of a sequence is then two runs
 // of 128-token tiles: the `past` tokens cached before (tiles of the cache, contiguous or paged, aligned to slot 0;
@@ -22,7 +30,7 @@
 // to the chunk's first token, so the causal diagonal sits exactly as in a fresh prompt, which is the case past = 0).
 // The new tokens' K/V come from the caller's tensors (and are written to the cache in the same pass) or, when the
 // caller has appended them already, from the cache itself at slot past + row.
-// A whole sub-tile's output leaves through the shared memory that held its Q rows and TMA stores.
+// A whole sub-tile's output leaves through two slots of the ring and TMA stores.
 //
 // TMEM columns: S0 [0,128) S1 [128,256) O0 [256,256+D) O1 [256+D,256+2D); P_i aliases the first 64
 // columns of S_i. Causal tile skipping: sub-tile i only visits K/V tiles up to its diagonal.
@@ -38,6 +46,7 @@ namespace {
 constexpr int kRows = 128;                     // rows per sub-tile == tokens per K/V tile
 constexpr int kThreads = 384;                  // 3 warpgroups: softmax 0, softmax 1, {producer, MMA, 2 idle}
 constexpr uint32_t kHalfBytes = kRows * 128;   // [128 rows][64 bf16], 128-byte swizzled
+constexpr int kItemReaders = 11;               // warps that read an item: all but the producer's
 constexpr float kRescaleThreshold = 8.f;       // log2 domain: O is rescaled only if the max grew by > 2^8
 
 template <int D>
@@ -47,8 +56,8 @@ struct TcCfg {
     static constexpr int kSlots = (D == 128) ? 5 : 8;                    // ring of K/V tiles
     static constexpr uint32_t kTmemCols = 512;
     static constexpr uint32_t kColS0 = 0, kColS1 = 128, kColO0 = 256, kColO1 = 256 + D;
-    static constexpr int kNumBars = 1 + 2 * kSlots + 8;
-    static constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + (size_t)kSlots * kTileBytes + kNumBars * 8 + 64;
+    static constexpr int kNumBars = (2 * kSlots + 21 + 1) & ~1;          // even: what follows them is 16-byte aligned
+    static constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + (size_t)kSlots * kTileBytes + kNumBars * 8 + 16 + 2 * 64 + 16;
 };
 
 struct TcParams {
@@ -56,6 +65,8 @@ struct TcParams {
     int64_t o_sb, o_st, o_sh;
     __nv_bfloat16 *cache_k, *cache_v;   // destination of the fused cache write (null: nothing is written)
     int64_t c_sb, c_sh, c_st;           // its strides (paged: c_sb is the stride between pages)
+    const __nv_bfloat16 *k_new, *v_new; // the new tokens' K/V, for the rows that do not go to the cache from shared memory
+    int64_t k_sb, k_st, k_sh, v_sb, v_st, v_sh;
     int cache_slots;                    // token slots per sequence that may be written
     const int32_t *seq_lens;            // [B] new tokens per sequence (prompt or chunk length)
     const int32_t *past_lens;           // [B] tokens cached ahead of them, or null (none)
@@ -66,6 +77,8 @@ struct TcParams {
     float *lse;
     unsigned *status;
     int S_max, B, Hq, Hkv, G, n_qblocks;
+    int claims;                         // a CTA goes on with blocks that have not started
+    int cache_tma;                      // whole tiles are written to the cache by TMA, through the maps of the cache
     int pair_heads;                     // the two sub-tiles are two query heads of one KV group at the same 128 rows
     float scale_log2e;
     TmapCoord cq, ckv, co, ckc;         // ckv: maps of the new tokens' K/V; ckc: maps of the cache (tokens before)
@@ -83,13 +96,10 @@ __device__ __forceinline__ void order_coords(const TmapCoord &c, int t, int h, i
 // 64-element chunks along M/N.
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes)
 {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((1024u >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;                     // descriptor version for sm_100
-    d |= (uint64_t)2 << 61;                     // SWIZZLE_128B
-    return d;
+    constexpr uint32_t hi = (1024u >> 4) |      // stride between 8-row groups
+                            1u << 14 |          // descriptor version for sm_100
+                            2u << 29;           // SWIZZLE_128B
+    return pack_u32x2((smem_addr >> 4) | ((lbo_bytes >> 4) << 16), hi);
 }
 
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128.
@@ -128,6 +138,17 @@ __device__ __forceinline__ bool row_block_by_work(int len, int past_len, int S_m
     return true;
 }
 
+// One work item: 128 rows of two query heads of a KV group, or 256 rows of one head.
+struct Item {
+    int b, qb, h, kvh;           // sequence, row block, (first) query head and its KV head
+    int L, past;                 // new tokens of the sequence, tokens cached ahead of them
+    int n_cache;                 // key tiles of the past
+    int n_sub0, n_sub1, n_kv;    // key tiles that each sub-tile visits, and the longer of the two
+    int g;                       // ring entries used before it
+    int writes;                  // its diagonal tiles go to the cache
+    int valid;                   // 0: nothing to do (past the end of its sequence, or no item left)
+};
+
 // kRanked: row blocks in the order of their work, not of their place in the sequence (an instantiation of its own: fresh
 // prompts do not pay for it)
 template <int D, bool kRanked>
@@ -138,29 +159,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                   const TcParams p)
 {
     using C = TcCfg<D>;
-    // ---- which block: heaviest (longest causal span) blocks first, heads of a KV group adjacent
-    grid_dependency_wait();                       // seq_lens may have been written by the previous kernel
-    // pair mode: sub-tile i is query head h + i at rows q0 ..; else: head h at rows q0 + 128 i ..
-    const bool pair = p.pair_heads != 0;
-    const int heads = pair ? p.Hq / 2 : p.Hq;
-    const int per_block = heads * p.B;
-    int qb = p.n_qblocks - 1 - (int)(blockIdx.x / per_block);           // block of 128 (pair mode) or 256 rows
-    const int hb = blockIdx.x % per_block;
-    const int h = pair ? 2 * (hb % heads) : hb % heads;
-    int b = hb / heads;
-    const int kvh = h / p.G;
-    const int sub_rows = pair ? 0 : kRows;                // rows between the two sub-tiles
-    const int sub_heads = pair ? 1 : 0;                   // heads between them
-    // The two lengths are requested now and first looked at after the barrier / TMEM set-up below, so that
-    // their latency is hidden behind it.
-    int L_raw = __ldg(p.seq_lens + b);
-    int past_raw = p.past_lens ? __ldg(p.past_lens + b) : 0;
-    // Ranked row blocks: the lengths of all sequences (at most 32), requested with them.
-    int len_of = 0, past_of = 0;
-    if (kRanked && (int)(threadIdx.x & 31) < p.B) {
-        len_of = __ldg(p.seq_lens + (threadIdx.x & 31));
-        past_of = __ldg(p.past_lens + (threadIdx.x & 31));
-    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -168,121 +167,193 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     uint8_t *q_smem = smem;                                       // 2 sub-tiles
     uint8_t *ring = smem + 2 * C::kTileBytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(ring + (size_t)C::kSlots * C::kTileBytes);
-    uint64_t *q_full = bars;
-    uint64_t *kv_full = bars + 1;
-    uint64_t *kv_empty = kv_full + C::kSlots;
-    uint64_t *s_full = kv_empty + C::kSlots;      // [2]
-    uint64_t *p_full = s_full + 2;                // [2]
-    uint64_t *o_full = p_full + 2;                // [2]
-    uint64_t *o_staged = o_full + 2;              // [2] a sub-tile's output rows are in shared memory
-    uint32_t *tmem_base_smem = reinterpret_cast<uint32_t *>(o_staged + 2);
+    uint64_t *kv_full = bars;
+    uint64_t *kv_empty = kv_full + C::kSlots;     // two arrivals: the MMAs, and whoever else reads the slot (or the producer for them)
+    uint64_t *q_full = kv_empty + C::kSlots;
+    uint64_t *q_empty = q_full + 1;               // the last Q K^T of the item is done
+    uint64_t *claim_bar = q_empty + 1;
+    uint64_t *s_full = claim_bar + 1;             // [2]
+    uint64_t *o_full = s_full + 2;                // [2]
+    // One for even, one for odd items: a role may be a whole item behind another, and never two (the place of an item in shared
+    // memory is filled again only when all its readers have left it), so that a phase is never passed by unseen.
+    uint64_t *item_full = o_full + 2;             // [2] the item is known
+    uint64_t *loads_issued = item_full + 2;       // [2] all its tiles have been asked for
+    uint64_t *o_granted = loads_issued + 2;       // [2] the slots for its output rows are free
+    uint64_t *item_empty = o_granted + 2;         // [2] its readers have left it
+    uint64_t *p_full = item_empty + 2;            // [2]
+    uint64_t *o_staged = p_full + 2;              // [2][2] a sub-tile's output rows are in shared memory (or written directly)
+    uint4 *claim = reinterpret_cast<uint4 *>(bars + C::kNumBars);         // answer to the request for a block
+    Item *items = reinterpret_cast<Item *>(claim + 1);                    // [2]
+    uint32_t *tmem_base_smem = reinterpret_cast<uint32_t *>(items + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_base_smem + 1);
-    volatile int *copy_go = abort_flag + 1;       // producer -> helper warps: all loads issued
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    // The producer's lane sets the barriers up itself, so that it can start the first loads right away, while
-    // the other warps are still on their way to the block-wide barrier below (TMEM allocation included).
-    const bool producer_lane = threadIdx.x == 8 * 32;
-    if (producer_lane) {
-        mbar_init(q_full, 1);
-        for (int s = 0; s < C::kSlots; ++s) {
-            mbar_init(&kv_full[s], 1);
-            mbar_init(&kv_empty[s], 1);
+    // Set-up that depends on nothing the kernel before writes, and overlaps its tail. The producer's warp sets the barriers up itself,
+    // a lane each, so that its first loads need not wait for the other warps at the block-wide barrier below.
+    if (warp == 8) {
+        for (int i = lane; i < (int)(o_staged + 4 - bars); i += 32) {
+            uint64_t *bar = bars + i;
+            mbar_init(bar, bar >= p_full ? kRows : bar >= item_empty ? kItemReaders : bar >= kv_empty && bar < q_full ? 2 : 1);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&s_full[i], 1);
-            mbar_init(&p_full[i], kRows);
-            mbar_init(&o_full[i], 1);
-            mbar_init(&o_staged[i], kRows);
+        if (lane == 0) {
+            *abort_flag = 0;
+            tma_prefetch_desc(&tmap_q);
+            tma_prefetch_desc(&tmap_k);
+            tma_prefetch_desc(&tmap_v);
+            tma_prefetch_desc(&tmap_kc);
+            tma_prefetch_desc(&tmap_vc);
         }
-        *abort_flag = 0;
-        *copy_go = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
+        __syncwarp();
     }
-    // Ranked row blocks. With equal pasts (every fresh prompt) the order of places is the order of work, and this vote is all that
-    // the block pays for.
-    if (kRanked && __builtin_expect(!__all_sync(0xffffffffu, lane >= p.B || past_of == past_raw), 0)) {
-        if (!row_block_by_work(len_of, past_of, p.S_max, pair ? 7 : 8, pair ? 0 : 1, (int)(blockIdx.x / heads), b, qb)) return;
-        L_raw = __shfl_sync(0xffffffffu, len_of, b);
-        past_raw = __shfl_sync(0xffffffffu, past_of, b);
-        b = __shfl_sync(0xffffffffu, b, 0);                  // the same in every lane: in registers of the warp
-        qb = __shfl_sync(0xffffffffu, qb, 0);
+    if (warp == 9) {
+        tmem_alloc(tmem_base_smem, C::kTmemCols);
+        tmem_relinquish_alloc_permit();
     }
-    const int q0 = qb * (pair ? kRows : 2 * kRows);
-    const int diag0 = pair ? qb : 2 * qb;                 // tile (among the new tokens) of sub-tile 0's diagonal
-    // first use of the lengths. A block past the end of its sequence has nothing to do (decided before any
-    // TMEM is taken).
-    const int L = L_raw < 0 ? 0 : (L_raw > p.S_max ? p.S_max : L_raw);
-    if (q0 >= L) return;
-    // Tokens already in the cache ahead of these (0 for a fresh prompt): n_cache tiles, seen by every row.
-    const int past = past_raw < 0 ? 0 : past_raw;
-    const int n_cache = (past + kRows - 1) / kRows;
-    // sub-tile i (rows q0 + 128 i ..) visits the tiles of the past and the new tokens' tiles up to its diagonal
-    int n_sub[2];
-    n_sub[0] = n_cache + min(q0 + kRows - 1, L - 1) / kRows + 1;
-    n_sub[1] = (q0 + sub_rows < L) ? n_cache + min(q0 + sub_rows + kRows - 1, L - 1) / kRows + 1 : 0;
-    const int n_kv = max(n_sub[0], n_sub[1]);
-    // Q and the first ring-ful of K/V tiles need no waiting: requested before the block-wide barrier
-    const int n_pre = min(2 * n_kv, C::kSlots);
-    auto request_tile = [&](int idx) {
-        const uint32_t s = idx % C::kSlots;
+    grid_dependency_wait();                       // the lengths may have been written by the previous kernel
+
+    // pair mode: sub-tile i is query head h + i at rows q0 ..; else: head h at rows q0 + 128 i ..
+    const bool pair = p.pair_heads != 0;
+    const int heads = pair ? p.Hq / 2 : p.Hq;
+    const int sub_rows = pair ? 0 : kRows;                // rows between the two sub-tiles
+    const int sub_heads = pair ? 1 : 0;                   // heads between them
+    const int tiles_per_block = pair ? 1 : 2;             // new tiles from one row block to the next
+
+    // Up to 32 sequences: lane l of the producer's warp keeps the lengths of sequence l.
+    int len_of = 0, past_of = 0;
+    if (warp == 8 && lane < p.B && p.B > 1 && p.B <= 32) {
+        len_of = __ldg(p.seq_lens + lane);
+        past_of = p.past_lens ? __ldg(p.past_lens + lane) : 0;
+    }
+    // Block `index` of the launch: heaviest (longest causal span) blocks first, heads of a KV group adjacent. The whole warp calls this.
+    auto item_of = [&](int index) {
+        Item it = {};
+        const int per_block = heads * p.B;
+        it.qb = p.n_qblocks - 1 - index / per_block;      // block of 128 (pair mode) or 256 rows
+        const int hb = index % per_block;
+        it.h = pair ? 2 * (hb % heads) : hb % heads;
+        it.b = hb / heads;
+        it.kvh = it.h / p.G;
+        it.writes = p.cache_k != nullptr && it.kvh * p.G == it.h;
+        it.valid = 1;
+        int L_raw, past_raw;
+        if (kRanked) {
+            L_raw = __shfl_sync(0xffffffffu, len_of, it.b);
+            past_raw = __shfl_sync(0xffffffffu, past_of, it.b);
+            // With equal pasts (every fresh prompt) the order of places is the order of work, and this vote is all that is paid for.
+            if (__builtin_expect(!__all_sync(0xffffffffu, lane >= p.B || past_of == past_raw), 0)) {
+                it.valid = row_block_by_work(len_of, past_of, p.S_max, pair ? 7 : 8, pair ? 0 : 1, index / heads, it.b, it.qb);
+                it.b = it.valid ? it.b : 0;
+                L_raw = __shfl_sync(0xffffffffu, len_of, it.b);
+                past_raw = __shfl_sync(0xffffffffu, past_of, it.b);
+            }
+        } else if (p.B > 1 && p.B <= 32) {
+            // By place, the row blocks past the ends of their sequences left out (they would be passed over one by one, a request each): the
+            // place is the largest that has more than `left` row blocks at it or above, found by bisection.
+            const int blocks = (min(max(len_of, 0), p.S_max) + tiles_per_block * kRows - 1) / (tiles_per_block * kRows);
+            const int left = index / heads;
+            auto from = [&](int qb) { return (int)__reduce_add_sync(0xffffffffu, (unsigned)max(0, blocks - qb)); };
+            int lo = -1, hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)blocks), above = 0;        // from(hi) = above <= left
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1, n = from(mid);
+                if (n > left) lo = mid; else hi = mid, above = n;
+            }
+            it.qb = lo;
+            it.valid = lo >= 0;
+            unsigned who = __ballot_sync(0xffffffffu, blocks > lo);
+            for (int skip = it.valid ? left - above : 0; skip > 0; --skip) who &= who - 1;
+            it.b = it.valid ? __ffs(who) - 1 : 0;
+            L_raw = __shfl_sync(0xffffffffu, len_of, it.b);
+            past_raw = __shfl_sync(0xffffffffu, past_of, it.b);
+        } else {
+            L_raw = __ldg(p.seq_lens + it.b);
+            past_raw = p.past_lens ? __ldg(p.past_lens + it.b) : 0;
+        }
+        const int q0 = it.qb * tiles_per_block * kRows;
+        it.L = L_raw < 0 ? 0 : (L_raw > p.S_max ? p.S_max : L_raw);
+        if (q0 >= it.L || q0 < 0) it.valid = 0;                     // a block past the end of its sequence has nothing to do
+        // Tokens already in the cache ahead of these (0 for a fresh prompt): n_cache tiles, seen by every row.
+        it.past = past_raw < 0 ? 0 : past_raw;
+        it.n_cache = (it.past + kRows - 1) / kRows;
+        // sub-tile i (rows q0 + 128 i ..) visits the tiles of the past and the new tokens' tiles up to its diagonal
+        it.n_sub0 = it.n_cache + min(q0 + kRows - 1, it.L - 1) / kRows + 1;
+        it.n_sub1 = (q0 + sub_rows < it.L) ? it.n_cache + min(q0 + sub_rows + kRows - 1, it.L - 1) / kRows + 1 : 0;
+        it.n_kv = max(it.n_sub0, it.n_sub1);
+        return it;
+    };
+
+    // Whether key tile j goes to the cache from its slot in the ring, by TMA: a whole diagonal tile, contiguous cache. (What does not is
+    // copied from the caller's tensors, so that no slot waits for a copy row by row.)
+    auto leaves_ring = [&](const Item &x, int j) {
+        const int r_base = (j - x.n_cache) * kRows;
+        return x.writes && p.cache_tma && j >= x.n_cache + tiles_per_block * x.qb && min(x.L, p.cache_slots - x.past) - r_base >= kRows;
+    };
+    // ---- what the producer asks for (one lane: copies asked for by several lanes of a warp are issued one by one, at many times the
+    // cost). Ring entries of an item: K_0, V_0, K_1, V_1, ... then one for each sub-tile's output rows on their way out. `g` counts entries
+    // over all items of this block.
+    auto request_q = [&](const Item &x, int i) {
+        int c1, c2, c3;
+        order_coords(p.cq, x.qb * tiles_per_block * kRows + i * sub_rows, x.h + i * sub_heads, x.b, c1, c2, c3);
+#pragma unroll
+        for (int hf = 0; hf < C::kHalves; ++hf)
+            tma_load_4d(q_smem + i * C::kTileBytes + hf * kHalfBytes, &tmap_q, q_full, hf * 64, c1, c2, c3);
+    };
+    auto request_tile = [&](const Item &x, int g, int idx) {
+        const uint32_t s = g % C::kSlots;
         const int j = idx >> 1;
         uint8_t *dst = ring + (size_t)s * C::kTileBytes;
         int c1, c2, c3;
+        if (!leaves_ring(x, j)) mbar_arrive(&kv_empty[s]);        // no second reader
         mbar_arrive_expect_tx(&kv_full[s], C::kTileBytes);
-        if (j >= n_cache) {
+        if (j >= x.n_cache) {
             // a tile of the new tokens
-            order_coords(p.ckv, (p.new_at_past ? past : 0) + (j - n_cache) * kRows, kvh, b, c1, c2, c3);
+            order_coords(p.ckv, (p.new_at_past ? x.past : 0) + (j - x.n_cache) * kRows, x.kvh, x.b, c1, c2, c3);
             const CUtensorMap *tm = (idx & 1) ? &tmap_v : &tmap_k;
 #pragma unroll
             for (int hf = 0; hf < C::kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, &kv_full[s], hf * 64, c1, c2, c3);
         } else if (p.block_table == nullptr) {
             // a tile of the tokens cached before, contiguous cache
-            order_coords(p.ckc, j * kRows, kvh, b, c1, c2, c3);
+            order_coords(p.ckc, j * kRows, x.kvh, x.b, c1, c2, c3);
             const CUtensorMap *tm = (idx & 1) ? &tmap_vc : &tmap_kc;
 #pragma unroll
             for (int hf = 0; hf < C::kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, &kv_full[s], hf * 64, c1, c2, c3);
         } else {
-            // ... paged cache: one box per page that the tile touches (a page never straddles tiles or boxes). A
-            // table entry outside the pool becomes an out-of-range coordinate, which reads zeros.
+            // ... paged cache: one box per page that the tile touches (a page never straddles tiles or boxes), four look-ups at a
+            // time. A table entry outside the pool becomes an out-of-range coordinate, which reads zeros.
             const CUtensorMap *tm = (idx & 1) ? &tmap_vc : &tmap_kc;
-            const int32_t *row = p.block_table + (size_t)b * p.table_stride;
-            for (int r0 = 0; r0 < kRows; r0 += p.cache_box_t) {
-                const int slot0 = j * kRows + r0, entry = slot0 >> p.page_shift;
-                int page = entry < p.table_stride ? __ldg(row + entry) : -1;
-                if (page < 0 || page >= p.num_pages) page = p.num_pages;
-                order_coords(p.ckc, slot0 & (p.page_size - 1), kvh, page, c1, c2, c3);
+            const int32_t *row = p.block_table + (size_t)x.b * p.table_stride;
+            for (int at = 0; at < kRows; at += 4 * p.cache_box_t) {
+                int page[4];
 #pragma unroll
-                for (int hf = 0; hf < C::kHalves; ++hf)
-                    tma_load_4d(dst + hf * kHalfBytes + r0 * 128, tm, &kv_full[s], hf * 64, c1, c2, c3);
+                for (int u = 0; u < 4; ++u) {
+                    const int r0 = at + u * p.cache_box_t, entry = (j * kRows + r0) >> p.page_shift;
+                    page[u] = r0 < kRows && entry < p.table_stride ? __ldg(row + entry) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r0 = at + u * p.cache_box_t;
+                    if (r0 >= kRows) break;
+                    order_coords(p.ckc, (j * kRows + r0) & (p.page_size - 1), x.kvh, page[u] < 0 || page[u] >= p.num_pages ? p.num_pages : page[u], c1, c2, c3);
+#pragma unroll
+                    for (int hf = 0; hf < C::kHalves; ++hf)
+                        tma_load_4d(dst + hf * kHalfBytes + r0 * 128, tm, &kv_full[s], hf * 64, c1, c2, c3);
+                }
             }
         }
     };
-    if (producer_lane) {
-        tma_prefetch_desc(&tmap_q);
-        tma_prefetch_desc(&tmap_k);
-        tma_prefetch_desc(&tmap_v);
-        if (n_cache > 0) {
-            tma_prefetch_desc(&tmap_kc);
-            tma_prefetch_desc(&tmap_vc);
+    // What the first products need is requested before the block-wide barrier, the rest behind it
+    Item next = {};
+    if (warp == 8) {
+        next = item_of(blockIdx.x);
+        if (lane == 0 && next.valid) {
+            mbar_arrive_expect_tx(q_full, 2 * C::kTileBytes);
+            request_q(next, 0);
+            request_tile(next, 0, 0);                      // K_0 right behind Q_0: the first product needs both
+            request_q(next, 1);
+            next.g = 0;
+            items[0] = next;
+            mbar_arrive(&item_full[0]);
         }
-        int c1, c2, c3;
-        mbar_arrive_expect_tx(q_full, 2 * C::kTileBytes);
-        order_coords(p.cq, q0, h, b, c1, c2, c3);
-#pragma unroll
-        for (int hf = 0; hf < C::kHalves; ++hf) tma_load_4d(q_smem + hf * kHalfBytes, &tmap_q, q_full, hf * 64, c1, c2, c3);
-        request_tile(0);                                   // K_0 right behind Q_0: the first product needs both
-        order_coords(p.cq, q0 + sub_rows, h + sub_heads, b, c1, c2, c3);
-#pragma unroll
-        for (int hf = 0; hf < C::kHalves; ++hf)
-            tma_load_4d(q_smem + C::kTileBytes + hf * kHalfBytes, &tmap_q, q_full, hf * 64, c1, c2, c3);
-        for (int idx = 1; idx < n_pre; ++idx) request_tile(idx);
-    }
-    if (warp == 9) {
-        tmem_alloc(tmem_base_smem, C::kTmemCols);
-        tmem_relinquish_alloc_permit();
     }
     // Programmatic dependent launch: the next kernel of the stream may start its own prologue now.
     grid_launch_dependents();
@@ -291,76 +362,187 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     tcgen05_fence_after_sync();
     const uint32_t tmem_base = *tmem_base_smem;
 
-    // The block's diagonal K/V tiles (one or two tiles of the new tokens, from diag0 on) go to the cache, at slot past + row
-    // (first query head of a KV group only, so each row is written once). They are the last tiles loaded, so their
-    // ring slots are never refilled; the copy runs beside the last iterations, shared by three warps. Rows >= L
-    // and slots the cache does not have are not written.
-    const bool writes_cache = p.cache_k != nullptr && (h % p.G) == 0;
-    auto copy_diagonal_tiles = [&](int part) {
-        if (!writes_cache) return;
-        for (int j = n_cache + diag0; j < n_kv; ++j) {
-            const int r_base = (j - n_cache) * kRows;              // first row of the tile among the new tokens
-            for (int kv = 0; kv < 2; ++kv) {
-                const int idx = 2 * j + kv;
-                const uint32_t s = idx % C::kSlots, ph = (idx / C::kSlots) & 1u;
-                if (!mbar_wait(&kv_full[s], ph, abort_flag)) return;
-                const uint8_t *src = ring + (size_t)s * C::kTileBytes;
-                __nv_bfloat16 *dst_all = kv ? p.cache_v : p.cache_k;
-                constexpr int kChunks = D / 8;
-                const int rows = min(min(kRows, L - r_base), p.cache_slots - past - r_base);
-                for (int i = part * 32 + lane; i < rows * kChunks; i += 96) {
-                    const int r = i / kChunks, ch = i % kChunks;
-                    const int slot = past + r_base + r;
-                    __nv_bfloat16 *dst;
-                    if (p.block_table == nullptr) {
-                        dst = dst_all + b * p.c_sb + kvh * p.c_sh + (int64_t)slot * p.c_st;
-                    } else {
-                        const int page = __ldg(p.block_table + (size_t)b * p.table_stride + (slot >> p.page_shift));
-                        if (page < 0 || page >= p.num_pages) continue;          // no page behind this slot
-                        dst = dst_all + (int64_t)page * p.c_sb + kvh * p.c_sh + (int64_t)(slot & (p.page_size - 1)) * p.c_st;
-                    }
-                    const uint4 val = *reinterpret_cast<const uint4 *>(src + (ch >> 3) * kHalfBytes + swz128(r, ch & 7));
-                    *reinterpret_cast<uint4 *>(dst + ch * 8) = val;
-                }
-            }
+    // Every role but the producer takes its items like this, and reads them where the producer leaves them (a copy in registers
+    // would cost the softmax warps spills). An item is given back when the next one is asked for.
+    int n_read = 0;
+    auto all_wait = [&](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
+    auto next_item = [&]() {
+        if (n_read > 0) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&item_empty[(n_read - 1) & 1]);
         }
+        if (!all_wait(&item_full[n_read & 1], (n_read >> 1) & 1u)) return false;
+        ++n_read;
+        return items[(n_read - 1) & 1].valid != 0;
     };
+    auto item = [&]() { return items + ((n_read - 1) & 1); };
 
     // Register reallocation: the data-movement warpgroup gives registers to the softmax warpgroups,
     // whose threads hold a whole 128-column score row.
     if (warp >= 8) {
-    setmaxnreg_dec<64>();
+    setmaxnreg_dec<72>();
     if (warp == 8) {
-        // ============================================================ TMA producer (+ cache copy)
-        if (lane == 0) {
-            for (int idx = n_pre; idx < 2 * n_kv; ++idx) {
-                const uint32_t s = idx % C::kSlots, ph = (idx / C::kSlots) & 1u;
-                if (!mbar_wait(&kv_empty[s], ph ^ 1u, abort_flag)) break;
-                request_tile(idx);
+        // ============================================================ TMA producer; takes over blocks that have not started
+        int g = next.valid ? 1 : 0, idx = g, n_items = 0;
+        unsigned n_asked = 0;
+        bool ok = true;
+        auto wait_slot = [&]() { return mbar_wait(&kv_empty[g % C::kSlots], ((g / C::kSlots) & 1u) ^ 1u, abort_flag); };
+        while (true) {
+            // the others learn of the item first (of there being none only where nothing follows)
+            if (lane == 0 && idx == 0 && (next.valid || !p.claims || n_asked > 0)) {
+                next.g = g;
+                if (n_items >= 2) ok = mbar_wait(&item_empty[n_items & 1], ((n_items >> 1) - 1) & 1u, abort_flag);
+                items[n_items & 1] = next;
+                mbar_arrive(&item_full[n_items & 1]);
+            }
+            if (!next.valid && (!p.claims || n_asked > 0)) break;
+            if (next.valid) {
+                if (lane == 0) {
+                    if (ok && idx == 0) {
+                        ok = n_items == 0 || mbar_wait(q_empty, (n_items - 1) & 1u, abort_flag);
+                        if (ok) {
+                            mbar_arrive_expect_tx(q_full, 2 * C::kTileBytes);
+                            request_q(next, 0);
+                        }
+                    }
+                    for (; ok && idx < 2 * next.n_kv; ++idx, ++g) {
+                        ok = wait_slot();
+                        if (!ok) break;
+                        request_tile(next, g, idx);
+                        if (idx == 0) request_q(next, 1);
+                    }
+                    if (ok) mbar_arrive(&loads_issued[n_items & 1]);
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
+            }
+            // the next item: a block of the launch that no SM has started (those past the end of their sequence are passed over)
+            const bool had_item = next.valid;
+            next.valid = 0;
+            while (p.claims && !next.valid) {
+                int index = -1;
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(claim_bar, 16);
+                    clc_try_cancel(claim, claim_bar);
+                    if (mbar_wait(claim_bar, n_asked & 1u, abort_flag)) index = clc_answer(claim);
+                    fence_proxy_async_smem();              // the answer has been read before the next one is written
+                }
+                ++n_asked;
+                index = __shfl_sync(0xffffffffu, index, 0);
+                if (index < 0) break;
+                next = item_of(index);
+            }
+            if (had_item) {
+                // the slots that the outputs of the two sub-tiles leave through: theirs from here on
+                if (lane == 0) {
+                    for (int i = 0; ok && i < 2; ++i, ++g) {
+                        ok = wait_slot();
+                        if (ok) {
+                            mbar_arrive(&kv_empty[g % C::kSlots]);
+                            mbar_arrive(&kv_full[g % C::kSlots]);          // its phase, which nobody waits for
+                        }
+                    }
+                    if (ok) mbar_arrive(&o_granted[n_items & 1]);
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
+                ++n_items;
+                idx = 0;
             }
         }
-        // all loads are issued: the diagonal tiles' slots are in their last phase, the copy may start
-        if (lane == 0) {
-            __threadfence_block();
-            *copy_go = 1;
+        if (lane == 0 && !ok) {                            // a dead wait: the block leaves when what it asked for has landed
+            volatile int keep_waiting = 0;
+            for (int e = max(0, g - C::kSlots); e < g; ++e)
+                mbar_wait_budget(&kv_full[e % C::kSlots], (e / C::kSlots) & 1u, &keep_waiting, kWaitCycleBudget >> 6);
+            if (n_asked > 0) mbar_wait_budget(claim_bar, (n_asked - 1) & 1u, &keep_waiting, kWaitCycleBudget >> 6);
         }
-        __syncwarp();
-        copy_diagonal_tiles(0);
     } else if (warp == 10 || warp == 11) {
-        // otherwise idle warps. First: if an earlier CTA of this launch already reported a dead wait, do
-        // not repeat its time-out in every remaining CTA. Then: help the producer warp copy the diagonal
-        // tiles to the cache.
-        if (warp == 10 && lane == 0 && *reinterpret_cast<volatile unsigned *>(p.status + kStatusErrWord) != 0u)
+        // ============================================================ what leaves through shared memory
+        // Warp 10: the diagonal K tiles into the cache, output rows of sub-tile 0; warp 11: V and sub-tile 1. An item's diagonal
+        // tiles (one or two tiles of the new tokens, from its own rows on) go to the cache at slot past + row, from the first
+        // query head of a KV group only, so that each row is written once. Rows >= L and slots the cache does not have are not
+        // written.
+        // First: if an earlier CTA of this launch already reported a dead wait, do not repeat its time-out in every remaining CTA.
+        const int part = warp - 10;
+        if (part == 0 && lane == 0 && *reinterpret_cast<volatile unsigned *>(p.status + kStatusErrWord) != 0u)
             *abort_flag = 1;
-        if (writes_cache) {
-            const long long t0 = clock64();
-            bool go = true;
-            while (*copy_go == 0) {
-                if (*abort_flag || clock64() - t0 > kWaitCycleBudget) { go = false; break; }
-                __nanosleep(128);
+        bool ok = true;
+        while (next_item()) {
+            const int g = item()->g;
+            const int ev = (n_read - 1) & 1;                  // even or odd item, and its phase
+            const uint32_t item_ph = ((n_read - 1) >> 1) & 1u;
+            if (item()->writes) {
+                const int kvh = item()->kvh, past = item()->past, b = item()->b;
+                for (int j = item()->n_cache + tiles_per_block * item()->qb; j < item()->n_kv; ++j) {
+                    const int r_base = (j - item()->n_cache) * kRows;       // first row of the tile among the new tokens
+                    if (leaves_ring(*item(), j)) {
+                        // (before this the slot may be in an earlier phase, whose parity may be that of the one waited for)
+                        const int e = g + 2 * j + part;
+                        if (!all_wait(&loads_issued[ev], item_ph) || !all_wait(&kv_full[e % C::kSlots], (e / C::kSlots) & 1u)) { ok = false; break; }
+                        if (lane == 0) {
+                            const uint8_t *src = ring + (size_t)(e % C::kSlots) * C::kTileBytes;
+                            int c1, c2, c3;
+                            order_coords(p.ckc, past + r_base, kvh, b, c1, c2, c3);
+#pragma unroll
+                            for (int hf = 0; hf < C::kHalves; ++hf)
+                                tma_store_4d(part ? &tmap_vc : &tmap_kc, src + hf * kHalfBytes, hf * 64, c1, c2, c3);
+                            tma_store_commit();
+                            tma_store_wait_read_all();
+                            mbar_arrive(&kv_empty[e % C::kSlots]);
+                        }
+                        __syncwarp();
+                        continue;
+                    }
+                    // a lane keeps its 16-byte column and goes down the rows, four at a time; a new page is looked up where one begins
+                    constexpr int kChunks = D / 8, kStep = 32 / kChunks, kBatch = 4;
+                    const int rows = min(min(kRows, item()->L - r_base), p.cache_slots - past - r_base);
+                    const int ch = lane % kChunks;
+                    const __nv_bfloat16 *const src = (part ? p.v_new : p.k_new) + b * (part ? p.v_sb : p.k_sb) + kvh * (part ? p.v_sh : p.k_sh) +
+                                                     (int64_t)r_base * (part ? p.v_st : p.k_st) + ch * 8;
+                    const int64_t src_st = part ? p.v_st : p.k_st;
+                    __nv_bfloat16 *const base = (part ? p.cache_v : p.cache_k) + kvh * p.c_sh + ch * 8;
+                    __nv_bfloat16 *page_at = p.block_table ? nullptr : base + b * p.c_sb;
+                    int page_of = -1;
+                    for (int r0 = lane / kChunks; r0 < rows; r0 += kStep * kBatch) {
+                        uint4 val[kBatch];
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const int r = r0 + u * kStep;
+                            if (r < rows) val[u] = *reinterpret_cast<const uint4 *>(src + r * src_st);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const int r = r0 + u * kStep;
+                            if (r >= rows) break;
+                            int slot = past + r_base + r;
+                            if (p.block_table) {
+                                const int entry = slot >> p.page_shift;
+                                if (entry != page_of) {
+                                    page_of = entry;
+                                    const int pg = __ldg(p.block_table + (size_t)b * p.table_stride + entry);
+                                    page_at = pg < 0 || pg >= p.num_pages ? nullptr : base + (int64_t)pg * p.c_sb;   // null: no page behind this slot
+                                }
+                                slot &= p.page_size - 1;
+                            }
+                            if (page_at) *reinterpret_cast<uint4 *>(page_at + (int64_t)slot * p.c_st) = val[u];
+                        }
+                    }
+                    __syncwarp();
+                }
             }
-            __threadfence_block();
-            if (go) copy_diagonal_tiles(warp - 9);
+            if (!ok) break;
+            const int e = g + 2 * item()->n_kv + part, q0 = item()->qb * tiles_per_block * kRows + part * sub_rows;
+            if (!all_wait(&o_granted[ev], item_ph) || !all_wait(&o_staged[2 * ev + part], item_ph)) break;
+            if (q0 + kRows <= item()->L && lane == 0) {
+                const uint8_t *stage = ring + (size_t)(e % C::kSlots) * C::kTileBytes;
+                int c1, c2, c3;
+                order_coords(p.co, q0, item()->h + part * sub_heads, item()->b, c1, c2, c3);
+#pragma unroll
+                for (int hf = 0; hf < C::kHalves; ++hf) tma_store_4d(&tmap_o, stage + hf * kHalfBytes, hf * 64, c1, c2, c3);
+                tma_store_commit();
+                tma_store_wait_read_all();                         // shared memory must outlive the reads
+            }
+            if (lane == 0) mbar_arrive(&kv_empty[e % C::kSlots]);
         }
     } else if (warp == 9) {
         // ============================================================ MMA issuer
@@ -385,59 +567,77 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                                (first && k == 0) ? 0u : 1u);
         };
 
-        bool ok = mbar_wait(q_full, 0, abort_flag) && mbar_wait(&kv_full[0], 0, abort_flag);
-        if (ok) {
+        uint32_t q_ph = 0, p_ph[2] = {0, 0};
+        bool ok = true;
+        while (ok && next_item()) {
+            // (broadcast, so that the compiler knows them to be the same in all lanes)
+            const int n_kv = __shfl_sync(0xffffffffu, item()->n_kv, 0), g = __shfl_sync(0xffffffffu, item()->g, 0);
+            const int n_sub[2] = {__shfl_sync(0xffffffffu, item()->n_sub0, 0), __shfl_sync(0xffffffffu, item()->n_sub1, 0)};
+            const int n_cache = __shfl_sync(0xffffffffu, item()->n_cache, 0), past = __shfl_sync(0xffffffffu, item()->past, 0);
+            const int L = __shfl_sync(0xffffffffu, item()->L, 0);
+            ok = all_wait(q_full, q_ph) && all_wait(&kv_full[g % C::kSlots], (g / C::kSlots) & 1u);
+            q_ph ^= 1u;
+            if (!ok) break;
             tcgen05_fence_after_sync();
-            if (lane == 0) {
+            if (elect_one()) {
+#pragma unroll
                 for (int i = 0; i < 2; ++i)
                     if (n_sub[i] > 0) {
-                        issue_qk(i, ring_addr);
+                        issue_qk(i, ring_addr + (g % C::kSlots) * C::kTileBytes);
                         tcgen05_commit(&s_full[i]);
                     }
-                tcgen05_commit(&kv_empty[0]);
+                tcgen05_commit(&kv_empty[g % C::kSlots]);
+                if (n_kv == 1) tcgen05_commit(q_empty);
             }
             __syncwarp();
-        }
-        for (int j = 0; ok && j < n_kv; ++j) {
-            const int iv = 2 * j + 1, ik = 2 * j + 2;
-            const uint32_t sv = iv % C::kSlots, sk = ik % C::kSlots;
-            if (!mbar_wait(&kv_full[sv], (iv / C::kSlots) & 1u, abort_flag)) { ok = false; break; }
-            // V rows >= this hold no valid token (the partly filled last tile of the past, or of the new tokens)
-            const int first_dead = j < n_cache ? past - j * kRows : L - (j - n_cache) * kRows;
-            if (first_dead < kRows) {
-                // may hold any bits (NaN included): clear, so that a zero weight times garbage cannot appear
-                uint8_t *vt = ring + (size_t)sv * C::kTileBytes;
-                constexpr int kChunks = D / 8;
-                for (int i = lane; i < (kRows - first_dead) * kChunks; i += 32) {
-                    const int r = first_dead + i / kChunks, ch = i % kChunks;
-                    *reinterpret_cast<uint4 *>(vt + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) =
-                        make_uint4(0u, 0u, 0u, 0u);
-                }
-                fence_proxy_async_smem();
-                __syncwarp();
-            }
-            const bool have_next = j + 1 < n_kv;
-            if (have_next && !mbar_wait(&kv_full[sk], (ik / C::kSlots) & 1u, abort_flag)) { ok = false; break; }
-            for (int i = 0; i < 2 && ok; ++i) {
-                if (j >= n_sub[i]) continue;
-                if (!mbar_wait(&p_full[i], j & 1u, abort_flag)) { ok = false; break; }
-                tcgen05_fence_after_sync();
-                if (lane == 0) {
-                    issue_pv(i, ring_addr + sv * C::kTileBytes, j == 0);
-                    if (j + 1 < n_sub[i]) {
-                        issue_qk(i, ring_addr + sk * C::kTileBytes);
-                        tcgen05_commit(&s_full[i]);
-                    } else {
-                        tcgen05_commit(&o_full[i]);
+            for (int j = 0; j < n_kv; ++j) {
+                const int iv = g + 2 * j + 1, ik = g + 2 * j + 2;
+                const uint32_t sv = iv % C::kSlots, sk = ik % C::kSlots;
+                ok = mbar_wait(&kv_full[sv], (iv / C::kSlots) & 1u, abort_flag);
+                // V rows >= this hold no valid token (the partly filled last tile of the past, or of the new tokens)
+                const int first_dead = j < n_cache ? past - j * kRows : L - (j - n_cache) * kRows;
+                if (first_dead < kRows) {
+                    // may hold any bits (NaN included): clear, so that a zero weight times garbage cannot appear
+                    uint8_t *vt = ring + (size_t)sv * C::kTileBytes;
+                    constexpr int kChunks = D / 8;
+                    for (int i = lane; i < (kRows - first_dead) * kChunks; i += 32) {
+                        const int r = first_dead + i / kChunks, ch = i % kChunks;
+                        *reinterpret_cast<uint4 *>(vt + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) =
+                            make_uint4(0u, 0u, 0u, 0u);
                     }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                }
+                const bool have_next = j + 1 < n_kv;
+                if (have_next) ok = mbar_wait(&kv_full[sk], (ik / C::kSlots) & 1u, abort_flag) && ok;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    if (j >= n_sub[i]) continue;
+                    ok = mbar_wait(&p_full[i], p_ph[i], abort_flag) && ok;
+                    __syncwarp();
+                    p_ph[i] ^= 1u;
+                    tcgen05_fence_after_sync();
+                    if (elect_one()) {
+                        issue_pv(i, ring_addr + sv * C::kTileBytes, j == 0);
+                        if (j + 1 < n_sub[i]) {
+                            issue_qk(i, ring_addr + sk * C::kTileBytes);
+                            tcgen05_commit(&s_full[i]);
+                        } else {
+                            tcgen05_commit(&o_full[i]);
+                        }
+                    }
+                    __syncwarp();
+                }
+                // (one vote for the waits of the iteration: after a dead one its products are garbage, which the status word says)
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (elect_one()) {
+                    tcgen05_commit(&kv_empty[sv]);
+                    if (have_next) tcgen05_commit(&kv_empty[sk]);
+                    if (j + 2 == n_kv) tcgen05_commit(q_empty);
                 }
                 __syncwarp();
             }
-            if (ok && lane == 0) {
-                tcgen05_commit(&kv_empty[sv]);
-                if (have_next) tcgen05_commit(&kv_empty[sk]);
-            }
-            __syncwarp();
         }
     }
     } else {
@@ -445,22 +645,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         // ============================================================ softmax + epilogue warpgroups
         const int i = warp >> 2;                                   // sub-tile
         const int t = threadIdx.x & 127;                           // row within the sub-tile == TMEM lane
-        const int row = q0 + i * sub_rows + t;                     // token index of this thread's query row
-        const int hq = h + i * sub_heads;                          // ... and its query head
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tmem_s = tmem_base + lane_base + (i ? C::kColS1 : C::kColS0);
         const uint32_t tmem_o = tmem_base + lane_base + (i ? C::kColO1 : C::kColO0);
-        const int n_mine = n_sub[i];
-        // Tiles that need a mask: the last tile of the past when it is partly filled (columns past its end, the same
-        // for every row), and the sub-tile's diagonal tile among the new tokens (row t sees columns 0..t).
-        const int j_ragged = (past & (kRows - 1)) ? n_cache - 1 : -1;
-        const int j_diag = n_cache + (pair ? diag0 : diag0 + i);
         const float c = p.scale_log2e;
-        float m = -INFINITY, l = 0.f;
+        uint32_t phases = 0;                                       // bit 0: of s_full, bit 1: of o_full
         bool ok = true;
 
+        while (ok && next_item()) {
+        const int n_mine = i ? item()->n_sub1 : item()->n_sub0;
+        // Tiles that need a mask: the last tile of the past when it is partly filled (columns past its end, the same
+        // for every row), and the sub-tile's diagonal tile among the new tokens (row t sees columns 0..t).
+        const int j_ragged = (item()->past & (kRows - 1)) ? item()->n_cache - 1 : -1;
+        const int j_diag = item()->n_cache + (pair ? item()->qb : 2 * item()->qb + i);
+        float m = -INFINITY, l = 0.f;
+
         for (int j = 0; j < n_mine; ++j) {
-            if (!mbar_wait(&s_full[i], j & 1u, abort_flag)) { ok = false; break; }
+            if (!mbar_wait(&s_full[i], phases & 1u, abort_flag)) { ok = false; break; }
+            phases ^= 1u;
             tcgen05_fence_after_sync();
             uint32_t sr[4][32];
 #pragma unroll
@@ -473,7 +675,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             const bool diag = (j == j_ragged) || (j >= j_diag);
             float mx;
             if (diag) {
-                const int lim = (j == j_ragged) ? (past & (kRows - 1)) - 1 : t;   // columns > lim hold no visible key
+                const int lim = (j == j_ragged) ? (item()->past & (kRows - 1)) - 1 : t;   // columns > lim hold no visible key
                 float a0 = -INFINITY, a1 = -INFINITY, a2 = -INFINITY, a3 = -INFINITY;
 #pragma unroll
                 for (int qd = 0; qd < 4; ++qd)
@@ -568,16 +770,21 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             mbar_arrive(&p_full[i]);
         }
 
-        if (ok && n_mine > 0 && mbar_wait(&o_full[i], 0, abort_flag)) {
+        if (ok && n_mine > 0) {
+            ok = mbar_wait(&o_full[i], phases >> 1, abort_flag);
+            phases ^= 2u;
+            if (!ok) break;
             tcgen05_fence_after_sync();
+            const int q0 = item()->qb * tiles_per_block * kRows + i * sub_rows;         // first row of the sub-tile
+            const int row = q0 + t, hq = item()->h + i * sub_heads;                      // this thread's query row, its query head
             const float inv = 1.f / l;
-            const bool valid = row < L;
-            __nv_bfloat16 *orow = p.o + b * p.o_sb + (int64_t)row * p.o_st + hq * p.o_sh;
-            // A sub-tile whose 128 rows are all valid leaves through shared memory and one TMA store per 64
-            // columns (coalesced, asynchronous): the rows are staged where Q_i was, which no MMA reads any more
-            // (o_full follows the last of them). A ragged sub-tile writes its valid rows directly.
-            const bool whole = q0 + i * sub_rows + kRows <= L;
-            uint8_t *stage = q_smem + i * C::kTileBytes;
+            const bool valid = row < item()->L;
+            __nv_bfloat16 *orow = p.o + item()->b * p.o_sb + (int64_t)row * p.o_st + hq * p.o_sh;
+            // A sub-tile whose 128 rows are all valid leaves through a slot of the ring and one TMA store per 64
+            // columns (coalesced, asynchronous, issued by a helper warp). A ragged sub-tile writes its valid rows directly.
+            const bool whole = q0 + kRows <= item()->L;
+            uint8_t *stage = ring + (size_t)((item()->g + 2 * item()->n_kv + i) % C::kSlots) * C::kTileBytes;
+            if (whole && !mbar_wait(&o_granted[(n_read - 1) & 1], ((n_read - 1) >> 1) & 1u, abort_flag)) { ok = false; break; }
 #pragma unroll
             for (int qd = 0; qd < D / 32; ++qd) {
                 uint32_t orr[32];
@@ -606,20 +813,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                     }
                 }
             }
-            if (whole) {
-                fence_proxy_async_smem();                          // this thread's rows, for the TMA store
-                mbar_arrive(&o_staged[i]);
-                if (t == 0 && mbar_wait(&o_staged[i], 0, abort_flag)) {
-                    int c1, c2, c3;
-                    order_coords(p.co, q0 + i * sub_rows, hq, b, c1, c2, c3);
-#pragma unroll
-                    for (int hf = 0; hf < C::kHalves; ++hf) tma_store_4d(&tmap_o, stage + hf * kHalfBytes, hf * 64, c1, c2, c3);
-                    tma_store_commit();
-                    tma_store_wait_read_all();                     // shared memory must outlive the reads
-                }
-            }
+            if (whole) fence_proxy_async_smem();                   // this thread's rows, for the TMA store
             if (valid && p.lse)
-                p.lse[((size_t)b * p.Hq + hq) * p.S_max + row] = (m + log2f(l)) * 0.6931471805599453f;
+                p.lse[((size_t)item()->b * p.Hq + hq) * p.S_max + row] = (m + log2f(l)) * 0.6931471805599453f;
+        }
+        mbar_arrive(&o_staged[2 * ((n_read - 1) & 1) + i]);
         }
     }
 
@@ -729,11 +927,19 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     p.o = static_cast<__nv_bfloat16 *>(o.ptr);
     p.o_sb = o.stride_b; p.o_st = o.stride_t; p.o_sh = o.stride_h;
     if (kv.write) {
+        p.k_new = static_cast<const __nv_bfloat16 *>(kv.k_new.ptr);
+        p.v_new = static_cast<const __nv_bfloat16 *>(kv.v_new.ptr);
+        p.k_sb = kv.k_new.stride_b; p.k_st = kv.k_new.stride_t; p.k_sh = kv.k_new.stride_h;
+        p.v_sb = kv.v_new.stride_b; p.v_st = kv.v_new.stride_t; p.v_sh = kv.v_new.stride_h;
         p.cache_k = static_cast<__nv_bfloat16 *>(kv.write->k);
         p.cache_v = static_cast<__nv_bfloat16 *>(kv.write->v);
         p.c_sb = kv.write->stride_b; p.c_sh = kv.write->stride_h; p.c_st = kv.write->stride_t;
         const long long slots = kv.paged ? (long long)kv.paged->table_stride * kv.write->max_len : kv.write->max_len;
         p.cache_slots = slots > 0x7fffffffll ? 0x7fffffff : (int)slots;
+        // whole tiles of a contiguous cache leave by TMA (a cache whose strides no map can describe is written by the warps)
+        const l4l_kv_cache &c = *kv.write;
+        p.cache_tma = !kv.paged && (kv.past || (make_tmap_bf16(&tkc, &ckc, c.k, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows) &&
+                                                make_tmap_bf16(&tvc, &cvc, c.v, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows)));
     }
     if (kv.paged) {
         const int page_size = kv.past ? kv.past->max_len : kv.write->max_len;
@@ -752,6 +958,7 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     p.pair_heads = pairs_heads(p.G) ? 1 : 0;
     p.n_qblocks = row_blocks(S_max, p.G);
     p.scale_log2e = scale * 1.4426950408889634f;
+    p.claims = (long long)p.n_qblocks * (p.pair_heads ? Hq / 2 : Hq) * B > sm_count();
     p.cq = cq; p.ckv = ck; p.co = co; p.ckc = ckc;
     const long long slots = !kv.past ? 0 : kv.paged ? (long long)kv.paged->table_stride * kv.past->max_len : kv.past->max_len;
     const bool ranked = d_past_lens && row_blocks_by_work(S_max, slots, B, Hq, p.G);

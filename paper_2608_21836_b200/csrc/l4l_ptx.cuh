@@ -80,6 +80,31 @@ __device__ __forceinline__ void st_release_gpu(int *p, int v)
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Cluster launch control: asks for a block of this launch that has not started yet; if there is one it will not start, and
+// its work is the caller's. The 16-byte answer arrives in shared memory and is counted on `bar`.
+__device__ __forceinline__ void clc_try_cancel(void *answer, uint64_t *bar)
+{
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(smem_u32(answer)), "r"(smem_u32(bar))
+                 : "memory");
+}
+
+// The blockIdx.x that the answer hands over, or -1: no block left (do not ask again).
+__device__ __forceinline__ int clc_answer(const void *answer)
+{
+    int x;
+    asm volatile(
+        "{\n\t.reg .b128 R;\n\t.reg .pred P;\n\t"
+        "ld.shared.b128 R, [%1];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 P, R;\n\t"
+        "mov.s32 %0, -1;\n\t"
+        "@P clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, R;\n\t}"
+        : "=r"(x)
+        : "r"(smem_u32(answer))
+        : "memory");
+    return x;
+}
+
 // ----------------------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {

@@ -89,3 +89,36 @@ def test_where_the_order_is_by_place():
     assert order(1, 8192, 256) is None                                # one sequence
     assert order(33, 8192) is None and order(32, 8192) is not None
     assert order(4, 8192) is None                                     # 256 blocks: less than two per SM
+
+
+# several items per CTA (a CTA goes on with blocks that have not started) against launches of at most one block per SM
+@pytest.mark.parametrize("B,Hq,Hkv,D,S", [(7, 32, 8, 128, 520), (32, 6, 2, 128, 700), (33, 12, 4, 64, 300), (32, 12, 12, 64, 513), (2, 64, 8, 128, 2000)])
+def test_prompts_of_uneven_length_in_one_launch(B, Hq, Hkv, D, S):
+    """Fresh prompts, empty and short ones among them, with the cache written in the same launch (whole tiles and ragged ends, room behind
+    the prompt and too little of it): the same bits as one launch per sequence and group of heads."""
+    r = np.random.default_rng(B + S)
+    lens = r.integers(0, S + 1, B).astype(np.int32)
+    lens[:2] = S, 0 if B > 2 else 1
+    lens[-1] = min(256, S)
+    g = torch.Generator(device="cuda").manual_seed(B)
+    mk = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.bfloat16)  # noqa: E731
+    q, k, v = mk(B, S, Hq, D), mk(B, S, Hkv, D), mk(B, S, Hkv, D)
+    ws = l4l.new_workspace(l4l.L4L_OP_PREFILL, B, Hq, Hkv, D, S)
+    G, ln = Hq // Hkv, i32(lens)
+    for slots in (S + 37, S - 70):
+        outs = []
+        for whole in (True, False):
+            o = torch.full_like(q.view(torch.int16), SENTINEL).view(torch.bfloat16)
+            ck, cv = (torch.full((B, Hkv, slots, D), SENTINEL, dtype=torch.int16, device="cuda").view(torch.bfloat16) for _ in range(2))
+            if whole:
+                l4l.l4l_attn_prefill(q, k, v, o, ln, D ** -0.5, ws, cache_k=ck, cache_v=cv)
+            else:
+                for b in range(B):
+                    for h in range(Hkv):
+                        e, hq, hk = slice(b, b + 1), slice(h * G, (h + 1) * G), slice(h, h + 1)
+                        l4l.l4l_attn_prefill(q[e, :, hq], k[e, :, hk], v[e, :, hk], o[e, :, hq], ln[e], D ** -0.5, ws, cache_k=ck[e, hk],
+                                             cache_v=cv[e, hk])
+            assert l4l.l4l_last_device_error(ws) == 0
+            outs.append([t.view(torch.int16) for t in (o, ck, cv)])
+        for a, b in zip(*outs):
+            assert torch.equal(a, b)

@@ -901,6 +901,11 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
                              const int32_t *d_past_lens, int S_max, int B, int Hq, int Hkv, int D, float scale,
                              float *d_lse, void *workspace, cudaStream_t stream)
 {
+    // Up to 512 new tokens, and launches of at most one block per SM, are better off with a block per item (figures in
+    // l4l_prefill_blocks.cu: up to 400 tokens the one or the other is ahead by a tenth or more, from 700 on this kernel is).
+    const long long blocks = (long long)row_blocks(S_max, Hq / Hkv) * (pairs_heads(Hq / Hkv) ? Hq / 2 : Hq) * B;
+    if (S_max <= 512 || blocks <= sm_count())
+        return launch_prefill_blocks(q, o, kv, d_seq_lens, d_past_lens, S_max, B, Hq, Hkv, D, scale, d_lse, workspace, stream);
     CUtensorMap tq, tk, tv, to, tkc, tvc;
     TmapCoord cq, ck, cv, co, ckc, cvc;
     if (!make_tmap_bf16(&tq, &cq, q.ptr, D, S_max, Hq, B, q.stride_t, q.stride_h, q.stride_b, 64, kRows) ||

@@ -145,7 +145,7 @@ struct Item {
     int n_cache;                 // key tiles of the past
     int n_sub0, n_sub1, n_kv;    // key tiles that each sub-tile visits, and the longer of the two
     int g;                       // ring entries used before it
-    int writes;                  // its diagonal tiles go to the cache
+    int share, n_shares;         // which part of its diagonal tiles' rows goes to the cache from here, of how many (0: nothing is written)
     int valid;                   // 0: nothing to do (past the end of its sequence, or no item left)
 };
 
@@ -234,7 +234,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         it.h = pair ? 2 * (hb % heads) : hb % heads;
         it.b = hb / heads;
         it.kvh = it.h / p.G;
-        it.writes = p.cache_k != nullptr && it.kvh * p.G == it.h;
+        it.share = pair ? (it.h - it.kvh * p.G) >> 1 : it.h - it.kvh * p.G;
+        it.n_shares = p.cache_k == nullptr ? 0 : pair ? p.G >> 1 : p.G;
         it.valid = 1;
         int L_raw, past_raw;
         if (kRanked) {
@@ -282,12 +283,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         return it;
     };
 
-    // Whether key tile j goes to the cache from its slot in the ring, by TMA: a whole diagonal tile, contiguous cache. (What does not is
+    // Whether key tile j goes to the cache from a slot of the ring, by TMA: a whole diagonal tile, contiguous cache. (What does not is
     // copied from the caller's tensors, so that no slot waits for a copy row by row.)
-    auto leaves_ring = [&](const Item &x, int j) {
+    auto whole_by_tma = [&](const Item &x, int j) {
         const int r_base = (j - x.n_cache) * kRows;
-        return x.writes && p.cache_tma && j >= x.n_cache + tiles_per_block * x.qb && min(x.L, p.cache_slots - x.past) - r_base >= kRows;
+        return x.n_shares > 0 && p.cache_tma && j >= x.n_cache + tiles_per_block * x.qb && min(x.L, p.cache_slots - x.past) - r_base >= kRows;
     };
+    auto leaves_ring = [&](const Item &x, int j) { return x.share == 0 && whole_by_tma(x, j); };
     // ---- what the producer asks for (one lane: copies asked for by several lanes of a warp are issued one by one, at many times the
     // cost). Ring entries of an item: K_0, V_0, K_1, V_1, ... then one for each sub-tile's output rows on their way out. `g` counts entries
     // over all items of this block.
@@ -459,9 +461,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     } else if (warp == 10 || warp == 11) {
         // ============================================================ what leaves through shared memory
         // Warp 10: the diagonal K tiles into the cache, output rows of sub-tile 0; warp 11: V and sub-tile 1. An item's diagonal
-        // tiles (one or two tiles of the new tokens, from its own rows on) go to the cache at slot past + row, from the first
-        // query head of a KV group only, so that each row is written once. Rows >= L and slots the cache does not have are not
-        // written.
+        // tiles (one or two tiles of the new tokens, from its own rows on) go to the cache at slot past + row, each row once: a
+        // tile that leaves by TMA from the first query head of a KV group, the rows of the others in equal shares from all items of the
+        // group. Rows >= L and slots the cache does not have are not written.
         // First: if an earlier CTA of this launch already reported a dead wait, do not repeat its time-out in every remaining CTA.
         const int part = warp - 10;
         if (part == 0 && lane == 0 && *reinterpret_cast<volatile unsigned *>(p.status + kStatusErrWord) != 0u)
@@ -471,11 +473,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             const int g = item()->g;
             const int ev = (n_read - 1) & 1;                  // even or odd item, and its phase
             const uint32_t item_ph = ((n_read - 1) >> 1) & 1u;
-            if (item()->writes) {
+            if (item()->n_shares > 0) {
                 const int kvh = item()->kvh, past = item()->past, b = item()->b;
                 for (int j = item()->n_cache + tiles_per_block * item()->qb; j < item()->n_kv; ++j) {
                     const int r_base = (j - item()->n_cache) * kRows;       // first row of the tile among the new tokens
-                    if (leaves_ring(*item(), j)) {
+                    if (whole_by_tma(*item(), j)) {
+                        if (item()->share != 0) continue;
                         // (before this the slot may be in an earlier phase, whose parity may be that of the one waited for)
                         const int e = g + 2 * j + part;
                         if (!all_wait(&loads_issued[ev], item_ph) || !all_wait(&kv_full[e % C::kSlots], (e / C::kSlots) & 1u)) { ok = false; break; }
@@ -493,9 +496,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                         __syncwarp();
                         continue;
                     }
-                    // a lane keeps its 16-byte column and goes down the rows, four at a time; a new page is looked up where one begins
+                    // A lane keeps its 16-byte column and goes down the rows, four at a time; a new page is looked up where one begins. A tile
+                    // copied by one warp (sixteen round trips of 1 us for 128 rows) outlasted the products of short items; the rows
+                    // are shared out among the items of the KV group instead: 3 chunks of 300..600 over 64..300 in 64-token pages, 40/8 x 128
+                    // 60.2 -> 41.7 us, 32/8 35.8 -> 28.8, 64/8 53.6 -> 42.7. (More rows at a time: these warps then spill.)
                     constexpr int kChunks = D / 8, kStep = 32 / kChunks, kBatch = 4;
-                    const int rows = min(min(kRows, item()->L - r_base), p.cache_slots - past - r_base);
+                    const int all = max(0, min(min(kRows, item()->L - r_base), p.cache_slots - past - r_base));
+                    const int rows = all * (item()->share + 1) / item()->n_shares;
                     const int ch = lane % kChunks;
                     const __nv_bfloat16 *const src = (part ? p.v_new : p.k_new) + b * (part ? p.v_sb : p.k_sb) + kvh * (part ? p.v_sh : p.k_sh) +
                                                      (int64_t)r_base * (part ? p.v_st : p.k_st) + ch * 8;
@@ -503,7 +510,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                     __nv_bfloat16 *const base = (part ? p.cache_v : p.cache_k) + kvh * p.c_sh + ch * 8;
                     __nv_bfloat16 *page_at = p.block_table ? nullptr : base + b * p.c_sb;
                     int page_of = -1;
-                    for (int r0 = lane / kChunks; r0 < rows; r0 += kStep * kBatch) {
+                    for (int r0 = all * item()->share / item()->n_shares + lane / kChunks; r0 < rows; r0 += kStep * kBatch) {
                         uint4 val[kBatch];
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {

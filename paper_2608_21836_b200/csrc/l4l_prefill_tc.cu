@@ -357,8 +357,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             mbar_arrive(&item_full[0]);
         }
     }
-    // Programmatic dependent launch: the next kernel of the stream may start its own prologue now.
-    grid_launch_dependents();
     tcgen05_fence_before_sync();
     __syncthreads();
     tcgen05_fence_after_sync();
@@ -452,6 +450,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                 idx = 0;
             }
         }
+        // Programmatic dependent launch: the next kernel of the stream may set itself up from here on, while the last items end. (As soon
+        // as every block had started, its blocks settled on the SMs that fell idle first, in no order: 5 chunks of 202, 647, 129, 326 and
+        // 185 tokens over 563 to 3057, launches back to back 59.3 us, in this place 56.0, with a block per item 55.7.)
+        grid_launch_dependents();
         if (lane == 0 && !ok) {                            // a dead wait: the block leaves when what it asked for has landed
             volatile int keep_waiting = 0;
             for (int e = max(0, g - C::kSlots); e < g; ++e)

@@ -256,32 +256,31 @@ prefill_blocks_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         const uint32_t tmem_o[2] = {tmem_base + C::kColO0, tmem_base + C::kColO1};
         const uint32_t q_addr = smem_u32(q_smem), ring_addr = smem_u32(ring);
 
-        // (after a dead wait the lanes go on together, and none issues anything)
         bool ok = mbar_wait(q_full, 0, abort_flag) && mbar_wait(&kv_full[0], 0, abort_flag);
-        __syncwarp();
-        tcgen05_fence_after_sync();
-        if (lane == 0 && ok) {
-            for (int i = 0; i < 2; ++i)
-                if (n_sub[i] > 0) {
-                    issue_qk<D>(tmem_s[i], q_addr + i * C::kTileBytes, ring_addr);
-                    tcgen05_commit(&s_full[i]);
-                }
-            tcgen05_commit(&kv_empty[0]);
+        if (ok) {
+            tcgen05_fence_after_sync();
+            if (lane == 0) {
+                for (int i = 0; i < 2; ++i)
+                    if (n_sub[i] > 0) {
+                        issue_qk<D>(tmem_s[i], q_addr + i * C::kTileBytes, ring_addr);
+                        tcgen05_commit(&s_full[i]);
+                    }
+                tcgen05_commit(&kv_empty[0]);
+            }
+            __syncwarp();
         }
-        __syncwarp();
-        for (int j = 0; j < n_kv; ++j) {
+        for (int j = 0; ok && j < n_kv; ++j) {
             const int iv = 2 * j + 1, ik = 2 * j + 2;
             const uint32_t sv = iv % C::kSlots, sk = ik % C::kSlots;
-            ok = ok && mbar_wait(&kv_full[sv], (iv / C::kSlots) & 1u, abort_flag);
+            if (!mbar_wait(&kv_full[sv], (iv / C::kSlots) & 1u, abort_flag)) { ok = false; break; }
             clear_dead_rows<D>(ring + (size_t)sv * C::kTileBytes, j < n_cache ? past - j * kRows : L - (j - n_cache) * kRows, lane);
             const bool have_next = j + 1 < n_kv;
-            if (have_next) ok = ok && mbar_wait(&kv_full[sk], (ik / C::kSlots) & 1u, abort_flag);
-            for (int i = 0; i < 2; ++i) {
+            if (have_next && !mbar_wait(&kv_full[sk], (ik / C::kSlots) & 1u, abort_flag)) { ok = false; break; }
+            for (int i = 0; i < 2 && ok; ++i) {
                 if (j >= n_sub[i]) continue;
-                ok = ok && mbar_wait(&p_full[i], j & 1u, abort_flag);
-                __syncwarp();
+                if (!mbar_wait(&p_full[i], j & 1u, abort_flag)) { ok = false; break; }
                 tcgen05_fence_after_sync();
-                if (lane == 0 && ok) {
+                if (lane == 0) {
                     issue_pv<D>(tmem_o[i], tmem_s[i], ring_addr + sv * C::kTileBytes, j == 0);
                     if (j + 1 < n_sub[i]) {
                         issue_qk<D>(tmem_s[i], q_addr + i * C::kTileBytes, ring_addr + sk * C::kTileBytes);
@@ -316,22 +315,19 @@ prefill_blocks_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
         const int j_diag = n_cache + (pair ? diag0 : diag0 + i);
         const float c = p.scale_log2e;
         float m = -INFINITY, l = 0.f;
-        // After a dead wait the threads of a warp go on together (votes and tensor-memory accesses need whole warps), but count nowhere as
-        // arrived and write no row: the roles that wait for them give up in their turn.
         bool ok = true;
 
         for (int j = 0; j < n_mine; ++j) {
-            ok = ok && mbar_wait(&s_full[i], j & 1u, abort_flag);
+            if (!mbar_wait(&s_full[i], j & 1u, abort_flag)) { ok = false; break; }
             tcgen05_fence_after_sync();
             softmax_tile<D>(tmem_s, tmem_o, c, j == 0, j == j_ragged || j >= j_diag, [&] { return j == j_ragged ? (past & (kRows - 1)) - 1 : t; }, m, l);
-            if (ok) mbar_arrive(&p_full[i]);
+            mbar_arrive(&p_full[i]);
         }
 
-        if (n_mine > 0) {
-            ok = ok && mbar_wait(&o_full[i], 0, abort_flag);
+        if (ok && n_mine > 0 && mbar_wait(&o_full[i], 0, abort_flag)) {
             tcgen05_fence_after_sync();
             const float inv = 1.f / l;
-            const bool valid = ok && row < L;
+            const bool valid = row < L;
             __nv_bfloat16 *orow = p.o + b * p.o_sb + (int64_t)row * p.o_st + hq * p.o_sh;
             // A sub-tile whose 128 rows are all valid leaves through shared memory and one TMA store per 64
             // columns (coalesced, asynchronous): the rows are staged where Q_i was, which no MMA reads any more
@@ -340,8 +336,8 @@ prefill_blocks_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_c
             uint8_t *stage = q_smem + i * C::kTileBytes;
             put_row<D>(tmem_o, inv, whole, stage, t, valid, orow);
             if (whole) {
-                if (ok) mbar_arrive(&o_staged[i]);
-                if (t == 0 && ok && mbar_wait(&o_staged[i], 0, abort_flag)) {
+                mbar_arrive(&o_staged[i]);
+                if (t == 0 && mbar_wait(&o_staged[i], 0, abort_flag)) {
                     int c1, c2, c3;
                     order_coords(p.co, q0 + i * sub_rows, hq, b, c1, c2, c3);
 #pragma unroll

@@ -185,8 +185,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         }
         const int q0 = it.qb * tiles_per_block * kRows;
         it.L = L_raw < 0 ? 0 : (L_raw > p.S_max ? p.S_max : L_raw);
-        // a block past the end of its sequence has nothing to do (and no rows, for who still reads an item that a dead wait gave up)
-        if (q0 >= it.L || q0 < 0) it.valid = it.qb = it.L = 0;
+        if (q0 >= it.L || q0 < 0) it.valid = 0;                     // a block past the end of its sequence has nothing to do
         // Tokens already in the cache ahead of these (0 for a fresh prompt): n_cache tiles, seen by every row.
         it.past = past_raw < 0 ? 0 : past_raw;
         it.n_cache = (it.past + kRows - 1) / kRows;
@@ -301,7 +300,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                 if (lane == 0) {
                     mbar_arrive_expect_tx(claim_bar, 16);
                     clc_try_cancel(claim, claim_bar);
-                    if (mbar_wait(claim_bar, n_asked & 1u, abort_flag)) index = clc_answer(claim); else ok = false;
+                    if (mbar_wait(claim_bar, n_asked & 1u, abort_flag)) index = clc_answer(claim);
                     fence_proxy_async_smem();              // the answer has been read before the next one is written
                 }
                 ++n_asked;
@@ -506,11 +505,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         const uint32_t tmem_o = tmem_base + lane_base + (i ? C::kColO1 : C::kColO0);
         const float c = p.scale_log2e;
         uint32_t phases = 0;                                       // bit 0: of s_full, bit 1: of o_full
-        // After a dead wait the threads of a warp go on together (votes and tensor-memory accesses need whole warps), but count nowhere as
-        // arrived and write no row: the roles that wait for them give up in their turn.
         bool ok = true;
 
-        while (next_item()) {
+        while (ok && next_item()) {
         const int n_mine = i ? item()->n_sub1 : item()->n_sub0;
         // Tiles that need a mask: the last tile of the past when it is partly filled (columns past its end, the same
         // for every row), and the sub-tile's diagonal tile among the new tokens (row t sees columns 0..t).
@@ -519,33 +516,34 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         float m = -INFINITY, l = 0.f;
 
         for (int j = 0; j < n_mine; ++j) {
-            ok = ok && mbar_wait(&s_full[i], phases & 1u, abort_flag);
+            if (!mbar_wait(&s_full[i], phases & 1u, abort_flag)) { ok = false; break; }
             phases ^= 1u;
             tcgen05_fence_after_sync();
             softmax_tile<D>(tmem_s, tmem_o, c, j == 0, j == j_ragged || j >= j_diag,
                             [&] { return j == j_ragged ? (item()->past & (kRows - 1)) - 1 : t; }, m, l);
-            if (ok) mbar_arrive(&p_full[i]);
+            mbar_arrive(&p_full[i]);
         }
 
-        if (n_mine > 0) {
-            ok = ok && mbar_wait(&o_full[i], phases >> 1, abort_flag);
+        if (ok && n_mine > 0) {
+            ok = mbar_wait(&o_full[i], phases >> 1, abort_flag);
             phases ^= 2u;
+            if (!ok) break;
             tcgen05_fence_after_sync();
             const int q0 = item()->qb * tiles_per_block * kRows + i * sub_rows;         // first row of the sub-tile
             const int row = q0 + t, hq = item()->h + i * sub_heads;                      // this thread's query row, its query head
             const float inv = 1.f / l;
-            const bool valid = ok && row < item()->L;
+            const bool valid = row < item()->L;
             __nv_bfloat16 *orow = p.o + item()->b * p.o_sb + (int64_t)row * p.o_st + hq * p.o_sh;
             // A sub-tile whose 128 rows are all valid leaves through a slot of the ring and one TMA store per 64
             // columns (coalesced, asynchronous, issued by a helper warp). A ragged sub-tile writes its valid rows directly.
             const bool whole = q0 + kRows <= item()->L;
             uint8_t *stage = ring + (size_t)((item()->g + 2 * item()->n_kv + i) % C::kSlots) * C::kTileBytes;
-            if (whole) ok = ok && mbar_wait(&o_granted[(n_read - 1) & 1], ((n_read - 1) >> 1) & 1u, abort_flag);
+            if (whole && !mbar_wait(&o_granted[(n_read - 1) & 1], ((n_read - 1) >> 1) & 1u, abort_flag)) { ok = false; break; }
             put_row<D>(tmem_o, inv, whole, stage, t, valid, orow);
             if (valid && p.lse)
                 p.lse[((size_t)item()->b * p.Hq + hq) * p.S_max + row] = (m + log2f(l)) * 0.6931471805599453f;
         }
-        if (ok) mbar_arrive(&o_staged[2 * ((n_read - 1) & 1) + i]);
+        mbar_arrive(&o_staged[2 * ((n_read - 1) & 1) + i]);
         }
     }
 

@@ -178,5 +178,9 @@ int prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens,
 l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const PrefillKV &kv, const int32_t *d_seq_lens,
                              const int32_t *d_past_lens, int S_max, int B, int Hq, int Hkv, int D, float scale,
                              float *d_lse, void *workspace, cudaStream_t stream);
+// The same with a block per item (short sequences, few blocks); launch_prefill_tc hands such calls over.
+l4l_status launch_prefill_blocks(const l4l_tensor4 &q, const l4l_tensor4 &o, const PrefillKV &kv, const int32_t *d_seq_lens,
+                             const int32_t *d_past_lens, int S_max, int B, int Hq, int Hkv, int D, float scale,
+                             float *d_lse, void *workspace, cudaStream_t stream);
 
 }  // namespace l4l

@@ -36,20 +36,107 @@
 // columns of S_i. Causal tile skipping: sub-tile i only visits K/V tiles up to its diagonal.
 // The tensor pipe executes one thread's MMAs in issue order, which is what makes the S/P aliasing
 // safe: QK_{j+1} into S_i is issued after PV_j that reads P_i.
-#include "l4l_prefill.cuh"
+#include "l4l_internal.h"
+#include "l4l_ptx.cuh"
 
 namespace l4l {
 
 namespace {
 
+constexpr int kRows = 128;                     // rows per sub-tile == tokens per K/V tile
+constexpr int kThreads = 384;                  // 3 warpgroups: softmax 0, softmax 1, {producer, MMA, 2 idle}
+constexpr uint32_t kHalfBytes = kRows * 128;   // [128 rows][64 bf16], 128-byte swizzled
 constexpr int kItemReaders = 11;               // warps that read an item: all but the producer's
+constexpr float kRescaleThreshold = 8.f;       // log2 domain: O is rescaled only if the max grew by > 2^8
 
 template <int D>
-struct ItemsCfg : TcCfg<D> {
-    using TcCfg<D>::kSlots, TcCfg<D>::kTileBytes;
+struct TcCfg {
+    static constexpr int kHalves = D / 64;
+    static constexpr uint32_t kTileBytes = kHalves * kHalfBytes;        // one Q sub-tile, K tile or V tile
+    static constexpr int kSlots = (D == 128) ? 5 : 8;                    // ring of K/V tiles
+    static constexpr uint32_t kTmemCols = 512;
+    static constexpr uint32_t kColS0 = 0, kColS1 = 128, kColO0 = 256, kColO1 = 256 + D;
     static constexpr int kNumBars = (2 * kSlots + 21 + 1) & ~1;          // even: what follows them is 16-byte aligned
     static constexpr size_t kSmemBytes = 1024 + 2 * kTileBytes + (size_t)kSlots * kTileBytes + kNumBars * 8 + 16 + 2 * 64 + 16;
 };
+
+struct TcParams {
+    __nv_bfloat16 *o;
+    int64_t o_sb, o_st, o_sh;
+    __nv_bfloat16 *cache_k, *cache_v;   // destination of the fused cache write (null: nothing is written)
+    int64_t c_sb, c_sh, c_st;           // its strides (paged: c_sb is the stride between pages)
+    const __nv_bfloat16 *k_new, *v_new; // the new tokens' K/V, for the rows that do not go to the cache from shared memory
+    int64_t k_sb, k_st, k_sh, v_sb, v_st, v_sh;
+    int cache_slots;                    // token slots per sequence that may be written
+    const int32_t *seq_lens;            // [B] new tokens per sequence (prompt or chunk length)
+    const int32_t *past_lens;           // [B] tokens cached ahead of them, or null (none)
+    const int32_t *block_table;         // paged cache: [B, table_stride] page ids; null: contiguous cache
+    int table_stride, page_shift, page_size, num_pages;
+    int new_at_past;                    // the new tokens' K/V are read from the cache itself: row r is slot past + r
+    int cache_box_t;                    // token rows per TMA box of a cache tile (128, or the page size if smaller)
+    float *lse;
+    unsigned *status;
+    int S_max, B, Hq, Hkv, G, n_qblocks;
+    int claims;                         // a CTA goes on with blocks that have not started
+    int cache_tma;                      // whole tiles are written to the cache by TMA, through the maps of the cache
+    int pair_heads;                     // the two sub-tiles are two query heads of one KV group at the same 128 rows
+    float scale_log2e;
+    TmapCoord cq, ckv, co, ckc;         // ckv: maps of the new tokens' K/V; ckc: maps of the cache (tokens before)
+};
+
+__device__ __forceinline__ void order_coords(const TmapCoord &c, int t, int h, int b, int &c1, int &c2, int &c3)
+{
+    c1 = (c.pos_t == 1) ? t : (c.pos_h == 1) ? h : b;
+    c2 = (c.pos_t == 2) ? t : (c.pos_h == 2) ? h : b;
+    c3 = (c.pos_t == 3) ? t : (c.pos_h == 3) ? h : b;
+}
+
+// Shared-memory matrix descriptor, 128-byte swizzle, 8-row groups 1024 bytes apart.
+// K-major operands ignore the leading byte offset; MN-major ones use it as the stride between
+// 64-element chunks along M/N.
+__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes)
+{
+    constexpr uint32_t hi = (1024u >> 4) |      // stride between 8-row groups
+                            1u << 14 |          // descriptor version for sm_100
+                            2u << 29;           // SWIZZLE_128B
+    return pack_u32x2((smem_addr >> 4) | ((lbo_bytes >> 4) << 16), hi);
+}
+
+// Instruction descriptor: bf16 x bf16 -> fp32, M = 128.
+__host__ __device__ constexpr uint32_t make_idesc(int n, bool b_mn_major)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(kRows >> 4) << 24);
+}
+
+// Which row block the block group `g` (the blocks of all heads of one row block) works on when up to 32 sequences have different
+// pasts: row blocks are ranked by their work, i.e. the key tiles they visit, heaviest first. Row block qb of a sequence has
+// past + (qb + 1) << shift tiles, so the ranking needs no sort: the largest w with more than g row blocks of weight >= w is the
+// weight of rank g, found by bisection with a count over the sequences; equal weights go by sequence. A whole warp calls this,
+// lane l with the lengths of sequence l (0 past the last). Returns false past the last row block that holds rows.
+__device__ __forceinline__ bool row_block_by_work(int len, int past_len, int S_max, int row_shift, int shift, int g, int &b, int &qb)
+{
+    const int past = (max(past_len, 0) + kRows - 1) / kRows;
+    const int blocks = (min(max(len, 0), S_max) + (1 << row_shift) - 1) >> row_shift;
+    if (g >= (int)__reduce_add_sync(0xffffffffu, (unsigned)blocks)) return false;
+    auto at_least = [&](int w) {
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)max(0, blocks - max(0, ((w - past + (1 << shift) - 1) >> shift) - 1)));
+    };
+    const unsigned top = blocks > 0 ? (unsigned)(past + (blocks << shift)) : 0u;
+    int lo = 1, hi = (int)__reduce_max_sync(0xffffffffu, top) + 1;                     // at_least(lo) > g >= at_least(hi)
+    int above = 0;                                                                     // at_least(hi)
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1, n = at_least(mid);
+        if (n > g) lo = mid; else hi = mid, above = n;
+    }
+    // the row block of this very weight with g - above of them ahead (a sequence has one at most)
+    const int off = lo - past;
+    unsigned who = __ballot_sync(0xffffffffu, off > 0 && (off >> shift) << shift == off && off >> shift <= blocks);
+    for (int skip = g - above; skip > 0; --skip) who &= who - 1;
+    b = __ffs(who) - 1;
+    qb = (__shfl_sync(0xffffffffu, off, b) >> shift) - 1;
+    return true;
+}
 
 // One work item: 128 rows of two query heads of a KV group, or 256 rows of one head.
 struct Item {
@@ -71,7 +158,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                   const __grid_constant__ CUtensorMap tmap_kc, const __grid_constant__ CUtensorMap tmap_vc,
                   const TcParams p)
 {
-    using C = ItemsCfg<D>;
+    using C = TcCfg<D>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     extern __shared__ uint8_t smem_raw[];
@@ -215,9 +302,46 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     };
     auto request_tile = [&](const Item &x, int g, int idx) {
         const uint32_t s = g % C::kSlots;
-        if (!leaves_ring(x, idx >> 1)) mbar_arrive(&kv_empty[s]); // no second reader
+        const int j = idx >> 1;
+        uint8_t *dst = ring + (size_t)s * C::kTileBytes;
+        int c1, c2, c3;
+        if (!leaves_ring(x, j)) mbar_arrive(&kv_empty[s]);        // no second reader
         mbar_arrive_expect_tx(&kv_full[s], C::kTileBytes);
-        load_kv_tile<D>(p, tmap_k, tmap_v, tmap_kc, tmap_vc, x.b, x.kvh, x.past, x.n_cache, idx, ring + (size_t)s * C::kTileBytes, &kv_full[s]);
+        if (j >= x.n_cache) {
+            // a tile of the new tokens
+            order_coords(p.ckv, (p.new_at_past ? x.past : 0) + (j - x.n_cache) * kRows, x.kvh, x.b, c1, c2, c3);
+            const CUtensorMap *tm = (idx & 1) ? &tmap_v : &tmap_k;
+#pragma unroll
+            for (int hf = 0; hf < C::kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, &kv_full[s], hf * 64, c1, c2, c3);
+        } else if (p.block_table == nullptr) {
+            // a tile of the tokens cached before, contiguous cache
+            order_coords(p.ckc, j * kRows, x.kvh, x.b, c1, c2, c3);
+            const CUtensorMap *tm = (idx & 1) ? &tmap_vc : &tmap_kc;
+#pragma unroll
+            for (int hf = 0; hf < C::kHalves; ++hf) tma_load_4d(dst + hf * kHalfBytes, tm, &kv_full[s], hf * 64, c1, c2, c3);
+        } else {
+            // ... paged cache: one box per page that the tile touches (a page never straddles tiles or boxes), four look-ups at a
+            // time. A table entry outside the pool becomes an out-of-range coordinate, which reads zeros.
+            const CUtensorMap *tm = (idx & 1) ? &tmap_vc : &tmap_kc;
+            const int32_t *row = p.block_table + (size_t)x.b * p.table_stride;
+            for (int at = 0; at < kRows; at += 4 * p.cache_box_t) {
+                int page[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r0 = at + u * p.cache_box_t, entry = (j * kRows + r0) >> p.page_shift;
+                    page[u] = r0 < kRows && entry < p.table_stride ? __ldg(row + entry) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int r0 = at + u * p.cache_box_t;
+                    if (r0 >= kRows) break;
+                    order_coords(p.ckc, (j * kRows + r0) & (p.page_size - 1), x.kvh, page[u] < 0 || page[u] >= p.num_pages ? p.num_pages : page[u], c1, c2, c3);
+#pragma unroll
+                    for (int hf = 0; hf < C::kHalves; ++hf)
+                        tma_load_4d(dst + hf * kHalfBytes + r0 * 128, tm, &kv_full[s], hf * 64, c1, c2, c3);
+                }
+            }
+        }
     };
     // What the first products need is requested before the block-wide barrier, the rest behind it
     Item next = {};
@@ -265,13 +389,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         auto wait_slot = [&]() { return mbar_wait(&kv_empty[g % C::kSlots], ((g / C::kSlots) & 1u) ^ 1u, abort_flag); };
         while (true) {
             // the others learn of the item first (of there being none only where nothing follows)
-            if (lane == 0 && idx == 0 && (next.valid || n_asked > 0)) {
+            if (lane == 0 && idx == 0 && (next.valid || !p.claims || n_asked > 0)) {
                 next.g = g;
                 if (n_items >= 2) ok = mbar_wait(&item_empty[n_items & 1], ((n_items >> 1) - 1) & 1u, abort_flag);
                 items[n_items & 1] = next;
                 mbar_arrive(&item_full[n_items & 1]);
             }
-            if (!next.valid && n_asked > 0) break;
+            if (!next.valid && (!p.claims || n_asked > 0)) break;
             if (next.valid) {
                 if (lane == 0) {
                     if (ok && idx == 0) {
@@ -295,7 +419,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             // the next item: a block of the launch that no SM has started (those past the end of their sequence are passed over)
             const bool had_item = next.valid;
             next.valid = 0;
-            while (!next.valid) {
+            while (p.claims && !next.valid) {
                 int index = -1;
                 if (lane == 0) {
                     mbar_arrive_expect_tx(claim_bar, 16);
@@ -431,9 +555,26 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         }
     } else if (warp == 9) {
         // ============================================================ MMA issuer
+        constexpr uint32_t idesc_qk = make_idesc(kRows, false);
+        constexpr uint32_t idesc_pv = make_idesc(D, true);
         const uint32_t tmem_s[2] = {tmem_base + C::kColS0, tmem_base + C::kColS1};
         const uint32_t tmem_o[2] = {tmem_base + C::kColO0, tmem_base + C::kColO1};
         const uint32_t q_addr = smem_u32(q_smem), ring_addr = smem_u32(ring);
+
+        auto issue_qk = [&](int i, uint32_t k_addr) {
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k) {
+                const uint32_t off = (k >> 2) * kHalfBytes + (k & 3) * 32;
+                tcgen05_mma_ss(tmem_s[i], make_smem_desc(q_addr + i * C::kTileBytes + off, 0),
+                               make_smem_desc(k_addr + off, 0), idesc_qk, k > 0 ? 1u : 0u);
+            }
+        };
+        auto issue_pv = [&](int i, uint32_t v_addr, bool first) {
+#pragma unroll
+            for (int k = 0; k < kRows / 16; ++k)
+                tcgen05_mma_ts(tmem_o[i], tmem_s[i] + k * 8, make_smem_desc(v_addr + k * 2048, kHalfBytes), idesc_pv,
+                               (first && k == 0) ? 0u : 1u);
+        };
 
         uint32_t q_ph = 0, p_ph[2] = {0, 0};
         bool ok = true;
@@ -451,7 +592,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
                     if (n_sub[i] > 0) {
-                        issue_qk<D>(tmem_s[i], q_addr + i * C::kTileBytes, ring_addr + (g % C::kSlots) * C::kTileBytes);
+                        issue_qk(i, ring_addr + (g % C::kSlots) * C::kTileBytes);
                         tcgen05_commit(&s_full[i]);
                     }
                 tcgen05_commit(&kv_empty[g % C::kSlots]);
@@ -462,7 +603,20 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                 const int iv = g + 2 * j + 1, ik = g + 2 * j + 2;
                 const uint32_t sv = iv % C::kSlots, sk = ik % C::kSlots;
                 ok = mbar_wait(&kv_full[sv], (iv / C::kSlots) & 1u, abort_flag);
-                clear_dead_rows<D>(ring + (size_t)sv * C::kTileBytes, j < n_cache ? past - j * kRows : L - (j - n_cache) * kRows, lane);
+                // V rows >= this hold no valid token (the partly filled last tile of the past, or of the new tokens)
+                const int first_dead = j < n_cache ? past - j * kRows : L - (j - n_cache) * kRows;
+                if (first_dead < kRows) {
+                    // may hold any bits (NaN included): clear, so that a zero weight times garbage cannot appear
+                    uint8_t *vt = ring + (size_t)sv * C::kTileBytes;
+                    constexpr int kChunks = D / 8;
+                    for (int i = lane; i < (kRows - first_dead) * kChunks; i += 32) {
+                        const int r = first_dead + i / kChunks, ch = i % kChunks;
+                        *reinterpret_cast<uint4 *>(vt + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) =
+                            make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                }
                 const bool have_next = j + 1 < n_kv;
                 if (have_next) ok = mbar_wait(&kv_full[sk], (ik / C::kSlots) & 1u, abort_flag) && ok;
 #pragma unroll
@@ -473,9 +627,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
                     p_ph[i] ^= 1u;
                     tcgen05_fence_after_sync();
                     if (elect_one()) {
-                        issue_pv<D>(tmem_o[i], tmem_s[i], ring_addr + sv * C::kTileBytes, j == 0);
+                        issue_pv(i, ring_addr + sv * C::kTileBytes, j == 0);
                         if (j + 1 < n_sub[i]) {
-                            issue_qk<D>(tmem_s[i], q_addr + i * C::kTileBytes, ring_addr + sk * C::kTileBytes);
+                            issue_qk(i, ring_addr + sk * C::kTileBytes);
                             tcgen05_commit(&s_full[i]);
                         } else {
                             tcgen05_commit(&o_full[i]);
@@ -519,8 +673,109 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             if (!mbar_wait(&s_full[i], phases & 1u, abort_flag)) { ok = false; break; }
             phases ^= 1u;
             tcgen05_fence_after_sync();
-            softmax_tile<D>(tmem_s, tmem_o, c, j == 0, j == j_ragged || j >= j_diag,
-                            [&] { return j == j_ragged ? (item()->past & (kRows - 1)) - 1 : t; }, m, l);
+            uint32_t sr[4][32];
+#pragma unroll
+            for (int qd = 0; qd < 4; ++qd) tmem_ld_32x32b_x32(tmem_s + qd * 32, sr[qd]);
+            tcgen05_wait_ld();
+
+            // Row maximum of the scaled scores (log2 domain). Off the diagonal the maximum is taken over the
+            // raw scores with independent 3-input max chains and scaled once (min for a negative scale);
+            // on the diagonal tile the causal mask is applied to the scaled scores first.
+            const bool diag = (j == j_ragged) || (j >= j_diag);
+            float mx;
+            if (diag) {
+                const int lim = (j == j_ragged) ? (item()->past & (kRows - 1)) - 1 : t;   // columns > lim hold no visible key
+                float a0 = -INFINITY, a1 = -INFINITY, a2 = -INFINITY, a3 = -INFINITY;
+#pragma unroll
+                for (int qd = 0; qd < 4; ++qd)
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4) {
+                        float x[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            x[u] = __uint_as_float(sr[qd][e + u]) * c;
+                            x[u] = (qd * 32 + e + u > lim) ? -INFINITY : x[u];
+                            sr[qd][e + u] = __float_as_uint(x[u]);
+                        }
+                        a0 = fmaxf(a0, x[0]); a1 = fmaxf(a1, x[1]); a2 = fmaxf(a2, x[2]); a3 = fmaxf(a3, x[3]);
+                    }
+                mx = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3));
+            } else if (c >= 0.f) {
+                float a0 = -INFINITY, a1 = -INFINITY, a2 = -INFINITY, a3 = -INFINITY;
+#pragma unroll
+                for (int qd = 0; qd < 4; ++qd)
+#pragma unroll
+                    for (int e = 0; e < 32; e += 8) {
+                        a0 = max3(a0, __uint_as_float(sr[qd][e + 0]), __uint_as_float(sr[qd][e + 1]));
+                        a1 = max3(a1, __uint_as_float(sr[qd][e + 2]), __uint_as_float(sr[qd][e + 3]));
+                        a2 = max3(a2, __uint_as_float(sr[qd][e + 4]), __uint_as_float(sr[qd][e + 5]));
+                        a3 = max3(a3, __uint_as_float(sr[qd][e + 6]), __uint_as_float(sr[qd][e + 7]));
+                    }
+                mx = fmaxf(fmaxf(a0, a1), fmaxf(a2, a3)) * c;
+            } else {
+                float a0 = INFINITY, a1 = INFINITY, a2 = INFINITY, a3 = INFINITY;
+#pragma unroll
+                for (int qd = 0; qd < 4; ++qd)
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4) {
+                        a0 = fminf(a0, __uint_as_float(sr[qd][e + 0]));
+                        a1 = fminf(a1, __uint_as_float(sr[qd][e + 1]));
+                        a2 = fminf(a2, __uint_as_float(sr[qd][e + 2]));
+                        a3 = fminf(a3, __uint_as_float(sr[qd][e + 3]));
+                    }
+                mx = fminf(fminf(a0, a1), fminf(a2, a3)) * c;
+            }
+            // lazy rescale: keep the old reference max unless the new one is much larger
+            const bool grow = (mx > m + kRescaleThreshold) || (j == 0);
+            float alpha = 1.f;
+            if (grow) {
+                const float m_new = (mx == -INFINITY) ? 0.f : mx;
+                alpha = fast_exp2(m - m_new);                      // j == 0: exp2(-inf) = 0
+                m = m_new;
+                l *= alpha;
+            }
+            if (j > 0 && __any_sync(0xffffffffu, grow)) {
+                // PV_{j-1} has completed (s_full is committed after it), PV_j is not issued before p_full
+#pragma unroll
+                for (int qd = 0; qd < D / 32; ++qd) {
+                    uint32_t orr[32];
+                    tmem_ld_32x32b_x32(tmem_o + qd * 32, orr);
+                    tcgen05_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) orr[e] = __float_as_uint(__uint_as_float(orr[e]) * alpha);
+                    tmem_st_32x32b_x32(tmem_o + qd * 32, orr);
+                }
+            }
+            // p = 2^(x - m): packed fp32x2 FMA feeds the exp2 unit; sums in two independent packed chains
+            const float fc = diag ? 1.f : c;                       // diagonal scores are already scaled
+            const uint64_t c2 = pack_f32x2(fc, fc), nm2 = pack_f32x2(-m, -m);
+            uint64_t sum_a = pack_f32x2(0.f, 0.f), sum_b = sum_a;
+#pragma unroll
+            for (int qd = 0; qd < 4; ++qd) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int e = 0; e < 16; e += 2) {
+                    const uint64_t xa = fma_f32x2(pack_u32x2(sr[qd][2 * e], sr[qd][2 * e + 1]), c2, nm2);
+                    const uint64_t xb = fma_f32x2(pack_u32x2(sr[qd][2 * e + 2], sr[qd][2 * e + 3]), c2, nm2);
+                    float xa0, xa1, xb0, xb1;
+                    unpack_f32x2(xa, xa0, xa1);
+                    unpack_f32x2(xb, xb0, xb1);
+                    const float pa0 = fast_exp2(xa0), pa1 = fast_exp2(xa1);
+                    const float pb0 = fast_exp2(xb0), pb1 = fast_exp2(xb1);
+                    sum_a = add_f32x2(sum_a, pack_f32x2(pa0, pa1));
+                    sum_b = add_f32x2(sum_b, pack_f32x2(pb0, pb1));
+                    pk[e] = pack_bf16x2(pa0, pa1);
+                    pk[e + 1] = pack_bf16x2(pb0, pb1);
+                }
+                tmem_st_32x32b_x16(tmem_s + qd * 16, pk);
+            }
+            float sa0, sa1, sb0, sb1;
+            unpack_f32x2(sum_a, sa0, sa1);
+            unpack_f32x2(sum_b, sb0, sb1);
+            const float sum = (sa0 + sa1) + (sb0 + sb1);
+            l += sum;
+            tcgen05_wait_st();
+            tcgen05_fence_before_sync();
             mbar_arrive(&p_full[i]);
         }
 
@@ -539,7 +794,35 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             const bool whole = q0 + kRows <= item()->L;
             uint8_t *stage = ring + (size_t)((item()->g + 2 * item()->n_kv + i) % C::kSlots) * C::kTileBytes;
             if (whole && !mbar_wait(&o_granted[(n_read - 1) & 1], ((n_read - 1) >> 1) & 1u, abort_flag)) { ok = false; break; }
-            put_row<D>(tmem_o, inv, whole, stage, t, valid, orow);
+#pragma unroll
+            for (int qd = 0; qd < D / 32; ++qd) {
+                uint32_t orr[32];
+                tmem_ld_32x32b_x32(tmem_o + qd * 32, orr);
+                tcgen05_wait_ld();
+                if (whole) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint4 val;
+                        val.x = pack_bf16x2(__uint_as_float(orr[8 * e + 0]) * inv, __uint_as_float(orr[8 * e + 1]) * inv);
+                        val.y = pack_bf16x2(__uint_as_float(orr[8 * e + 2]) * inv, __uint_as_float(orr[8 * e + 3]) * inv);
+                        val.z = pack_bf16x2(__uint_as_float(orr[8 * e + 4]) * inv, __uint_as_float(orr[8 * e + 5]) * inv);
+                        val.w = pack_bf16x2(__uint_as_float(orr[8 * e + 6]) * inv, __uint_as_float(orr[8 * e + 7]) * inv);
+                        const int ch = qd * 4 + e;                 // 16-byte chunk of the row
+                        *reinterpret_cast<uint4 *>(stage + (ch >> 3) * kHalfBytes + swz128(t, ch & 7)) = val;
+                    }
+                } else if (valid) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint4 val;
+                        val.x = pack_bf16x2(__uint_as_float(orr[8 * e + 0]) * inv, __uint_as_float(orr[8 * e + 1]) * inv);
+                        val.y = pack_bf16x2(__uint_as_float(orr[8 * e + 2]) * inv, __uint_as_float(orr[8 * e + 3]) * inv);
+                        val.z = pack_bf16x2(__uint_as_float(orr[8 * e + 4]) * inv, __uint_as_float(orr[8 * e + 5]) * inv);
+                        val.w = pack_bf16x2(__uint_as_float(orr[8 * e + 6]) * inv, __uint_as_float(orr[8 * e + 7]) * inv);
+                        *reinterpret_cast<uint4 *>(orow + qd * 32 + e * 8) = val;
+                    }
+                }
+            }
+            if (whole) fence_proxy_async_smem();                   // this thread's rows, for the TMA store
             if (valid && p.lse)
                 p.lse[((size_t)item()->b * p.Hq + hq) * p.S_max + row] = (m + log2f(l)) * 0.6931471805599453f;
         }
@@ -558,6 +841,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
             p.status[kStatusInfoWord] = 0x20000u | (blockIdx.x & 0xffffu);
     }
 }
+
+bool pairs_heads(int G) { return G % 2 == 0; }
+int row_blocks(int S_max, int G) { return pairs_heads(G) ? (S_max + kRows - 1) / kRows : (S_max + 2 * kRows - 1) / (2 * kRows); }
 
 // Chunks over caches of different lengths: a row block's work is then set by the tokens cached ahead of it as much as by its
 // place, and with the last row blocks first whatever their length the launch ends on a few heavy blocks. Five chunks of
@@ -585,11 +871,37 @@ __global__ void row_block_order_kernel(const int32_t *past_lens, const int32_t *
     if (lane == 0) order[g] = rows ? make_int2(b, qb) : make_int2(-1, -1);
 }
 
-template <int D>
-l4l_status launch_items(const PrefillMaps &m, const TcParams &p, bool ranked, cudaStream_t stream)
+template <int D, bool kRanked>
+l4l_status launch_t(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const CUtensorMap &to,
+                    const CUtensorMap &tkc, const CUtensorMap &tvc, const TcParams &p, cudaStream_t stream)
 {
-    constexpr size_t smem = ItemsCfg<D>::kSmemBytes;
-    return ranked ? launch_prefill_kernel<prefill_tc_kernel<D, true>, smem>(m, p, stream) : launch_prefill_kernel<prefill_tc_kernel<D, false>, smem>(m, p, stream);
+    using C = TcCfg<D>;
+    static bool configured_on[kDeviceSlots] = {};
+    const int slot = device_slot();
+    if (slot < 0) return L4L_ERR_CUDA;
+    {
+        std::lock_guard<std::mutex> lock(setup_mutex());
+        bool &configured = configured_on[slot];
+        if (!configured) {
+            if (cudaFuncSetAttribute(prefill_tc_kernel<D, kRanked>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)C::kSmemBytes) != cudaSuccess)
+                return L4L_ERR_CUDA;
+            configured = true;
+        }
+    }
+    const long long grid = (long long)p.n_qblocks * (p.pair_heads ? p.Hq / 2 : p.Hq) * p.B;
+    if (grid > 0x7fffffffll) return L4L_ERR_UNSUPPORTED;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = C::kSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, kRanked>, tq, tk, tv, to, tkc, tvc, p) == cudaSuccess ? L4L_OK : L4L_ERR_CUDA;
 }
 
 }  // namespace
@@ -601,28 +913,29 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     // Up to 512 new tokens, and launches of at most one block per SM, are better off with a block per item (figures in
     // l4l_prefill_blocks.cu: up to 400 tokens the one or the other is ahead by a tenth or more, from 700 on this kernel is).
     const long long blocks = (long long)row_blocks(S_max, Hq / Hkv) * (pairs_heads(Hq / Hkv) ? Hq / 2 : Hq) * B;
-    const bool items = S_max > 512 && blocks > sm_count();
-    PrefillMaps m;
+    if (S_max <= 512 || blocks <= sm_count())
+        return launch_prefill_blocks(q, o, kv, d_seq_lens, d_past_lens, S_max, B, Hq, Hkv, D, scale, d_lse, workspace, stream);
+    CUtensorMap tq, tk, tv, to, tkc, tvc;
     TmapCoord cq, ck, cv, co, ckc, cvc;
-    if (!make_tmap_bf16(&m.q, &cq, q.ptr, D, S_max, Hq, B, q.stride_t, q.stride_h, q.stride_b, 64, kRows) ||
-        !make_tmap_bf16(&m.o, &co, o.ptr, D, S_max, Hq, B, o.stride_t, o.stride_h, o.stride_b, 64, kRows) ||
-        !make_tmap_bf16(&m.k, &ck, kv.k_new.ptr, D, kv.new_extent, Hkv, B, kv.k_new.stride_t, kv.k_new.stride_h,
+    if (!make_tmap_bf16(&tq, &cq, q.ptr, D, S_max, Hq, B, q.stride_t, q.stride_h, q.stride_b, 64, kRows) ||
+        !make_tmap_bf16(&to, &co, o.ptr, D, S_max, Hq, B, o.stride_t, o.stride_h, o.stride_b, 64, kRows) ||
+        !make_tmap_bf16(&tk, &ck, kv.k_new.ptr, D, kv.new_extent, Hkv, B, kv.k_new.stride_t, kv.k_new.stride_h,
                         kv.k_new.stride_b, 64, kRows) ||
-        !make_tmap_bf16(&m.v, &cv, kv.v_new.ptr, D, kv.new_extent, Hkv, B, kv.v_new.stride_t, kv.v_new.stride_h,
+        !make_tmap_bf16(&tv, &cv, kv.v_new.ptr, D, kv.new_extent, Hkv, B, kv.v_new.stride_t, kv.v_new.stride_h,
                         kv.v_new.stride_b, 64, kRows))
         return L4L_ERR_CUDA;
     if (ck.pos_t != cv.pos_t || ck.pos_h != cv.pos_h || ck.pos_b != cv.pos_b) return L4L_ERR_UNSUPPORTED;
     TcParams p = {};
     // the tokens cached before: tiles of the cache (one box per tile), or of the page pool (one box per page if the
     // pages are smaller than a tile); without a past the kernel never touches these two maps
-    m.kc = m.k; m.vc = m.v; ckc = ck;
+    tkc = tk; tvc = tv; ckc = ck;
     p.cache_box_t = kRows;
     if (kv.past) {
         const l4l_kv_cache &c = *kv.past;
         const int outer = kv.paged ? kv.paged->num_pages : B;
         if (kv.paged && c.max_len < kRows) p.cache_box_t = c.max_len;
-        if (!make_tmap_bf16(&m.kc, &ckc, c.k, D, c.max_len, Hkv, outer, c.stride_t, c.stride_h, c.stride_b, 64, p.cache_box_t) ||
-            !make_tmap_bf16(&m.vc, &cvc, c.v, D, c.max_len, Hkv, outer, c.stride_t, c.stride_h, c.stride_b, 64, p.cache_box_t))
+        if (!make_tmap_bf16(&tkc, &ckc, c.k, D, c.max_len, Hkv, outer, c.stride_t, c.stride_h, c.stride_b, 64, p.cache_box_t) ||
+            !make_tmap_bf16(&tvc, &cvc, c.v, D, c.max_len, Hkv, outer, c.stride_t, c.stride_h, c.stride_b, 64, p.cache_box_t))
             return L4L_ERR_CUDA;
     }
     p.o = static_cast<__nv_bfloat16 *>(o.ptr);
@@ -639,9 +952,8 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
         p.cache_slots = slots > 0x7fffffffll ? 0x7fffffff : (int)slots;
         // whole tiles of a contiguous cache leave by TMA (a cache whose strides no map can describe is written by the warps)
         const l4l_kv_cache &c = *kv.write;
-        p.cache_tma = items && !kv.paged &&
-                      (kv.past || (make_tmap_bf16(&m.kc, &ckc, c.k, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows) &&
-                                   make_tmap_bf16(&m.vc, &cvc, c.v, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows)));
+        p.cache_tma = !kv.paged && (kv.past || (make_tmap_bf16(&tkc, &ckc, c.k, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows) &&
+                                                make_tmap_bf16(&tvc, &cvc, c.v, D, c.max_len, Hkv, B, c.stride_t, c.stride_h, c.stride_b, 64, kRows)));
     }
     if (kv.paged) {
         const int page_size = kv.past ? kv.past->max_len : kv.write->max_len;
@@ -660,11 +972,13 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
     p.pair_heads = pairs_heads(p.G) ? 1 : 0;
     p.n_qblocks = row_blocks(S_max, p.G);
     p.scale_log2e = scale * 1.4426950408889634f;
+    p.claims = (long long)p.n_qblocks * (p.pair_heads ? Hq / 2 : Hq) * B > sm_count();
     p.cq = cq; p.ckv = ck; p.co = co; p.ckc = ckc;
     const long long slots = !kv.past ? 0 : kv.paged ? (long long)kv.paged->table_stride * kv.past->max_len : kv.past->max_len;
     const bool ranked = d_past_lens && row_blocks_by_work(S_max, slots, B, Hq, p.G);
-    if (!items) return launch_prefill_blocks(m, p, D, ranked, stream);
-    return D == 128 ? launch_items<128>(m, p, ranked, stream) : launch_items<64>(m, p, ranked, stream);
+    if (ranked)
+        return D == 128 ? launch_t<128, true>(tq, tk, tv, to, tkc, tvc, p, stream) : launch_t<64, true>(tq, tk, tv, to, tkc, tvc, p, stream);
+    return D == 128 ? launch_t<128, false>(tq, tk, tv, to, tkc, tvc, p, stream) : launch_t<64, false>(tq, tk, tv, to, tkc, tvc, p, stream);
 }
 
 int prefill_row_block_order(const int32_t *d_past_lens, const int32_t *d_q_lens, int S_max, long long slots, int B, int Hq, int Hkv,

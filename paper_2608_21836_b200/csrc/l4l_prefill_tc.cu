@@ -206,11 +206,17 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         fence_proxy_async_smem();
         __syncwarp();
     }
-    if (warp == 9) {
+    if (D == 128 && warp == 9) {
         tmem_alloc(tmem_base_smem, C::kTmemCols);
         tmem_relinquish_alloc_permit();
     }
     grid_dependency_wait();                       // the lengths may have been written by the previous kernel
+    // With 128-wide heads no other block fits beside this one, and tensor memory is there for the taking; with 64-wide heads one
+    // might, and if the kernel waited for lets its dependents start before it has taken its own, each would wait for the other.
+    if (D != 128 && warp == 9) {
+        tmem_alloc(tmem_base_smem, C::kTmemCols);
+        tmem_relinquish_alloc_permit();
+    }
 
     // pair mode: sub-tile i is query head h + i at rows q0 ..; else: head h at rows q0 + 128 i ..
     const bool pair = p.pair_heads != 0;

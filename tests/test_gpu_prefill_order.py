@@ -53,6 +53,36 @@ def test_row_blocks_by_work_cover_every_row_once(B, Hq, Hkv, D, page):
         assert torch.equal(o.view(torch.int16), outs[0][0])
 
 
+# the kernel with a block per item (S <= 512) ranks its row blocks too
+@pytest.mark.parametrize("page", [0, 64])
+@pytest.mark.parametrize("B,Hq,Hkv,D", [(12, 32, 8, 128), (32, 10, 2, 64), (31, 5, 5, 128)])
+def test_ranked_short_chunks(B, Hq, Hkv, D, page):
+    """The same bits as one launch per sequence, which has nothing to order."""
+    r = np.random.default_rng(B)
+    S, slots = 500, 1280
+    past, qlen = r.integers(0, slots - S + 1, B).astype(np.int32), r.integers(0, S + 1, B).astype(np.int32)
+    past[: B // 3], qlen[: B // 6], past[-1], qlen[-1] = 256, 0, 0, S
+    assert l4l.l4l_prefill_row_block_order(i32(past), i32(qlen), S, slots, Hq, Hkv, D) is not None
+    g = torch.Generator(device="cuda").manual_seed(B)
+    mk = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.bfloat16)  # noqa: E731
+    q, kn, vn = mk(B, S, Hq, D), mk(B, S, Hkv, D), mk(B, S, Hkv, D)
+    n = slots // page if page else 0
+    ck, cv = (mk(B * n, Hkv, page, D) if page else mk(B, Hkv, slots, D) for _ in range(2))
+    table = torch.randperm(B * n, generator=g, device="cuda").view(B, n).to(torch.int32) if page else None
+    ws = l4l.new_workspace(l4l.L4L_OP_PREFILL, B, Hq, Hkv, D, S)
+    outs = []
+    for step in (B, 1):
+        o, k2, v2 = torch.full_like(q.view(torch.int16), SENTINEL).view(torch.bfloat16), ck.clone(), cv.clone()
+        for b in range(0, B, step):
+            e = slice(b, b + step)
+            c = slice(None) if page else e
+            l4l.l4l_attn_prefill_chunk_append(q[e], kn[e], vn[e], o[e], k2[c], v2[c], i32(past)[e], i32(qlen)[e], D ** -0.5, ws,
+                                              block_table=table[e] if page else None)
+        assert l4l.l4l_last_device_error(ws) == 0
+        outs.append([t.view(torch.int16) for t in (o, k2, v2)])
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
 @pytest.mark.parametrize("G", [2, 3])
 @pytest.mark.parametrize("B", [2, 7, 31, 32])
 def test_the_order_is_by_work(B, G):
@@ -91,8 +121,10 @@ def test_where_the_order_is_by_place():
     assert order(4, 8192) is None                                     # 256 blocks: less than two per SM
 
 
-# several items per CTA (a CTA goes on with blocks that have not started) against launches of at most one block per SM
-@pytest.mark.parametrize("B,Hq,Hkv,D,S", [(7, 32, 8, 128, 520), (32, 6, 2, 128, 700), (33, 12, 4, 64, 300), (32, 12, 12, 64, 513), (2, 64, 8, 128, 2000)])
+# several items per CTA (S > 512: a CTA goes on with blocks that have not started; B = 33: empty row blocks are passed over one by one), and a
+# block per item, against launches of at most one block per SM
+@pytest.mark.parametrize("B,Hq,Hkv,D,S", [(7, 32, 8, 128, 520), (32, 6, 2, 128, 700), (33, 12, 4, 64, 300), (33, 12, 4, 64, 530), (32, 12, 12, 64, 513),
+                                          (2, 64, 8, 128, 2000)])
 def test_prompts_of_uneven_length_in_one_launch(B, Hq, Hkv, D, S):
     """Fresh prompts, empty and short ones among them, with the cache written in the same launch (whole tiles and ragged ends, room behind
     the prompt and too little of it): the same bits as one launch per sequence and group of heads."""
@@ -105,6 +137,7 @@ def test_prompts_of_uneven_length_in_one_launch(B, Hq, Hkv, D, S):
     q, k, v = mk(B, S, Hq, D), mk(B, S, Hkv, D), mk(B, S, Hkv, D)
     ws = l4l.new_workspace(l4l.L4L_OP_PREFILL, B, Hq, Hkv, D, S)
     G, ln = Hq // Hkv, i32(lens)
+    assert B * (-(-S // 128) * Hq // 2 if G % 2 == 0 else -(-S // 256) * Hq) > torch.cuda.get_device_properties(0).multi_processor_count
     for slots in (S + 37, S - 70):
         outs = []
         for whole in (True, False):

@@ -44,8 +44,8 @@ def check(y_gpu, st_gpu, y_ref, st_ref, valid):
 @pytest.mark.parametrize("B,T,W", [(2, 300, 2560), (1, 1237, 200), (3, 65, 40), (1, 1, 64), (5, 1000, 96), (1, 16, 64), (2, 17, 128),
                                    (4, 300, 2560), (4, 600, 2560), (5, 520, 2440), (19, 530, 512)])
 def test_rglru_matches_oracle(B, T, W):
-    """Sequences of many tiles (eight warps hand the state on from tile to tile), of exactly one tile (the one-warp
-    variant) and just past it; a second segment inside a sequence, ragged lengths, a channel count that does not fill
+    """Sequences of many tiles (eight warps hand the state on from tile to tile), of exactly one tile (sixteen steps, which
+    have a kernel of their own) and just past it; a second segment inside a sequence, ragged lengths, a channel count that does not fill
     the last strip; launches of 149 to 200 strips, which the library cuts into 32- or 16-channel strips (a warp
     then owns two or four consecutive time tiles)."""
     if (B, W) in ((4, 2560), (5, 2440), (19, 512)):                    # 160, 195 and 152 strips at 64 channels
@@ -85,7 +85,8 @@ def test_rglru_few_steps(B, T, W):
     pos = torch.arange(5, 5 + T, dtype=torch.int32).repeat(B, 1)
     pos[0] = torch.arange(T)
     pos[-1, T // 2:] = torch.arange(T - T // 2)
-    lens = [T] + [(T - 2 * i) % (T + 1) for i in range(1, B)]
+    lens = [T] + [(T - 2 * i) % (T + 1) if T > 1 else i % 2 for i in range(1, B)]    # (one step: empty and not in turn)
+    lens[-1] = 0 if B > 2 and T == 1 else lens[-1]
     dead = torch.arange(T).view(1, T, 1) >= torch.tensor(lens).view(B, 1, 1)
     nan = nan_bf16((1,))
     x, gx, ga = torch.where(dead, nan, x), torch.where(dead, nan, gx), torch.where(dead, nan, ga)

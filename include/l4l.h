@@ -294,6 +294,7 @@ size_t l4l_rglru_workspace_bytes(int B, int T, int W);
  * The choice also depends on whether there are reset positions and on the workspace; this answers for a launch with positions
  * on a workspace of l4l_rglru_workspace_bytes, l4l_rglru_launch_shape for the one that is described, with the number
  * of segments that the time axis is cut into in *segments (NULL: not asked for).
+ * Sequences of at most 16 steps have no strips (a thread per channel pair walks them): both answer 64 and one segment then.
  */
 int l4l_rglru_strip_channels(int B, int T, int W);
 int l4l_rglru_launch_shape(int B, int T, int W, int positions, size_t ws_bytes, int *segments);

@@ -1,8 +1,8 @@
 // Causal prefill on the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory).
 // A block per item, for launches of short sequences or of at most one block per SM; the longer ones go to l4l_prefill_tc.cu, whose CTAs
-// take item after item. Here three warps copy a ragged or paged diagonal tile into the cache and nothing waits for them, there one warp
-// per tensor does: 1 x 100 tokens (32/8 x 128) 9.1 us here, 13.3 there; 4 x 50..200 10.7 and 17.0; 16 x 50..100 18.1 and 25.3;
-// 8 x 100..700 (64/8) 92.5 and 75.0; 3 x 300..1000 (40/8) 40.8 and 36.0.
+// take item after item (where the line lies, and why: launch_prefill_tc). Here three warps copy a ragged or paged diagonal tile into the cache and
+// nothing waits for them. While one warp per tensor copied all rows of such a tile there: 1 x 100 tokens (32/8 x 128) 9.1 us here, 13.3 there;
+// 4 x 50..200 10.7 and 17.0; 16 x 50..100 18.1 and 25.3; 8 x 100..700 (64/8) 92.5 and 75.0; 3 x 300..1000 (40/8) 40.8 and 36.0.
 //
 // One CTA owns two 128-row sub-tiles whose S = Q K^T and O += P V products ping-pong on the tensor
 // pipe while the other sub-tile's softmax runs on the CUDA cores. The two sub-tiles are the same 128

@@ -21,8 +21,8 @@
 // that follows another pays 1.3. The claim comes when the item's last loads are on their way, about two tile pairs ahead of its end: later
 // than that the loads would start late, earlier the order of the heaviest first would suffer. The MMA issuer's warp has uniform control flow
 // (values broadcast, one vote per tile, an elected lane): with branches per lane a tile pair took 3500-3640 cycles instead of 3250-3350,
-// which is more than the items gain. Figures (kept up, where the power cap sets the clock; start of one by one): four prompts of 8192 2188 -> 2110 us, one of 2048 44.8 -> 43.6, six of 517 to 1592 with the rotation
-// 138.2 -> 126.3, five paged chunks 116.3 -> 117.1, a prompt of one block per head pair 6.8 -> 7.1 (no claims; the longer way to the first item).
+// which is more than the items gain. Figures (kept up, where the power cap sets the clock; a block per item first): four prompts of 8192 2198 and
+// 2129 us, one of 2048 45.1 and 43.5, six of 517 to 1592 with the rotation 139.7 and 128.0, five paged chunks 117.7 and 116.0.
 //
 // The same kernel serves a chunk of new tokens over a populated cache. The key axis of a sequence is then two runs
 // of 128-token tiles: the `past` tokens cached before (tiles of the cache, contiguous or paged, aligned to slot 0;
@@ -44,7 +44,7 @@ namespace l4l {
 namespace {
 
 constexpr int kRows = 128;                     // rows per sub-tile == tokens per K/V tile
-constexpr int kThreads = 384;                  // 3 warpgroups: softmax 0, softmax 1, {producer, MMA, 2 idle}
+constexpr int kThreads = 384;                  // 3 warpgroups: softmax 0, softmax 1, {producer, MMA, 2 that move rows to the cache and out}
 constexpr uint32_t kHalfBytes = kRows * 128;   // [128 rows][64 bf16], 128-byte swizzled
 constexpr int kItemReaders = 11;               // warps that read an item: all but the producer's
 constexpr float kRescaleThreshold = 8.f;       // log2 domain: O is rescaled only if the max grew by > 2^8
@@ -77,7 +77,7 @@ struct TcParams {
     float *lse;
     unsigned *status;
     int S_max, B, Hq, Hkv, G, n_qblocks;
-    int claims;                         // a CTA goes on with blocks that have not started
+    int claims;                         // a CTA goes on with blocks that have not started (every launch that comes here has them)
     int cache_tma;                      // whole tiles are written to the cache by TMA, through the maps of the cache
     int pair_heads;                     // the two sub-tiles are two query heads of one KV group at the same 128 rows
     float scale_log2e;
@@ -916,8 +916,11 @@ l4l_status launch_prefill_tc(const l4l_tensor4 &q, const l4l_tensor4 &o, const P
                              const int32_t *d_past_lens, int S_max, int B, int Hq, int Hkv, int D, float scale,
                              float *d_lse, void *workspace, cudaStream_t stream)
 {
-    // Up to 512 new tokens, and launches of at most one block per SM, are better off with a block per item (figures in
-    // l4l_prefill_blocks.cu: up to 400 tokens the one or the other is ahead by a tenth or more, from 700 on this kernel is).
+    // A launch of at most one block per SM has nothing to claim (one of 2 blocks 6.8 us with a block per item, 7.1 without), and up to
+    // 512 new tokens a block per item was ahead while one item copied all rows of a ragged or paged tile (figures in
+    // l4l_prefill_blocks.cu). Since the items share that copy this kernel is ahead in part of that range too: 40 x 512 (32/8 x 128)
+    // 192 us with a block per item, 145 here; 16 x 64..512 61 and 52; 12 x 17..64 over 64..500 27.3 and 29.1. Above: 4 x 300..540 with 40/8
+    // 36.7 and 34, 8 x 520..640 (32/8) 58.6 and 48.5.
     const long long blocks = (long long)row_blocks(S_max, Hq / Hkv) * (pairs_heads(Hq / Hkv) ? Hq / 2 : Hq) * B;
     if (S_max <= 512 || blocks <= sm_count())
         return launch_prefill_blocks(q, o, kv, d_seq_lens, d_past_lens, S_max, B, Hq, Hkv, D, scale, d_lse, workspace, stream);

@@ -278,7 +278,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         }
         const int q0 = it.qb * tiles_per_block * kRows;
         it.L = L_raw < 0 ? 0 : (L_raw > p.S_max ? p.S_max : L_raw);
-        if (q0 >= it.L || q0 < 0) it.valid = 0;                     // a block past the end of its sequence has nothing to do
+        // a block past the end of its sequence has nothing to do (and no rows, for a role that still reads an item whose place it takes after
+        // a dead wait)
+        if (q0 >= it.L || q0 < 0) it.valid = it.qb = it.L = 0;
         // Tokens already in the cache ahead of these (0 for a fresh prompt): n_cache tiles, seen by every row.
         it.past = past_raw < 0 ? 0 : past_raw;
         it.n_cache = (it.past + kRows - 1) / kRows;
